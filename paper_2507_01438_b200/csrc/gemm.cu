@@ -720,7 +720,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
           // tiles follow the dependency wait
           const int32_t npre = min(static_cast<int32_t>(nstages), tc.kb1 - tc.kb0);  // the ring is empty: no waits
           ptx::pdl_wait_prior_grids();
-          if (lane == 0)
+          if (ptx::elect_one())
             for (int32_t i = 0; i < npre; ++i)
               ptx::tma_load_2d(smem + static_cast<size_t>(i) * stage_bytes + r_bytes, mc, &full_bar[i],
                                (tc.kb0 + i) * kBlockK, tc.row_c);
@@ -733,7 +733,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
             ok = false;
             break;
           }
-          if (lane == 0) {
+          if (ptx::elect_one()) {
             uint8_t *sr = smem + static_cast<size_t>(stage) * stage_bytes;
             ptx::mbar_arrive_expect_tx(&full_bar[stage], tx_bytes);
             ptx::tma_load_2d(sr, mr, &full_bar[stage], kb * kBlockK, tc.row_r);
@@ -767,7 +767,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
             ok = false;
             break;
           }
-          if (lane == 0) {
+          if (ptx::elect_one()) {
             // The stage is free: let the builder write its half (it follows this warp, never the
             // stage barriers directly, so it cannot run ahead of the ring).
             ptx::mbar_arrive(&zgo_bar[stage]);
@@ -790,7 +790,9 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
-    if (lane == 0) {
+    // (elect.sync, not lane == 0: the compiler then knows that one thread issues, and the tensor and TMA
+    // instructions, which take their operands from uniform registers, need no loop over the lanes)
+    if (ptx::elect_one()) {
       const int lora_ksteps = p.R_pad / kUmmaK;
       uint32_t stage = 0, phase = 0, zphase = 0;  // zphase: one parity bit per stage
       bool ok = true, waited = p.mode == kModeSgmv;

@@ -77,7 +77,7 @@ __device__ __forceinline__ bool shrink_rows8(const CUtensorMap *tmap_a, const CU
   constexpr int kDsDepth = RingShape<NT, kDsDepthCfg>::kDepth;
   constexpr int kStage = RingShape<NT, kDsDepthCfg>::kStage;
   auto issue = [&](int step, int stage) {
-    if (lane == 0 && step < step1) {
+    if (step < step1 && ptx::elect_one()) {
       uint8_t *dst = ring + stage * kStage;
       ptx::mbar_arrive_expect_tx_relaxed(&bars[stage],
                                          (kQ8 ? 8 * (kQ8QBytes + kQ8DBytes) : 8 * kDsRowBytes) + NT * kDsRowBytes);
