@@ -9,6 +9,7 @@
 namespace edgelora {
 
 constexpr int kTileM = 128;        // UMMA M: rows of the TMEM accumulator (one per lane)
+constexpr int kListTile = 256;     // tokens of a prefill tile (two CTAs): the plan lists the adapters of each
 constexpr int kBlockK = 64;        // bf16 elements per K block = one 128-byte swizzled row
 constexpr int kUmmaK = 16;         // K of one tcgen05.mma for 16-bit inputs
 constexpr int kMaxStages = 12;
@@ -58,61 +59,35 @@ struct PlanView {
   int32_t *sgmv_tiles;     // [max_sgmv_tiles][4] {first token, tokens, slot, 0}
   int32_t *scratch;        // [maxT+1]
   int32_t *lg_adapter;     // [maxT]   distinct ids >= 0 of the batch, ascending (the LoRA groups)
-  int32_t *mt_count;       // [maxT/128+1] distinct ids >= 0 inside each 128-token tile
-  int32_t *mt_list;        // [ceil(maxT/128)*128] those ids, tile m at [128 m, 128 m + mt_count[m])
+  int32_t *mt_count;       // [ceil(maxT/256)+1] distinct ids >= 0 inside each 256-token tile
+  int32_t *mt_list;        // [ceil(maxT/256)*256] those ids, tile m at [256 m, 256 m + mt_count[m])
   int32_t *counts;         // [8]  0: n_groups, 1: n_segments, 2: n_sgmv_tiles, 3: short tokens,
                            //      4: LoRA groups, 5: K chunks used by the decode shrink
   uint32_t *status;        // device status word of the plan
   int32_t max_sgmv_tiles;
 };
 
-enum GemmMode : int32_t { kModePrefill = 0, kModeDecode = 1, kModeSgmv = 2 };
-
+// A decode launch of the tile kernel (gemm.cu).
 struct GemmParams {
-  int32_t mode;
   int32_t T, h_in, h_out;
-  int32_t BN;          // UMMA N = rows of the column-operand tile (multiple of 16, <= 256)
+  int32_t BN;          // UMMA N = tokens rounded up to a power of two (32 .. 256)
   int32_t stages;      // TMA pipeline depth
-  int32_t n_acc;       // TMEM accumulator buffers (1 or 2)
-  int32_t tmem_cols;   // power of two >= n_acc * acc_cols, >= 32
-  int32_t ring_rows;   // rows of the C region of a ring stage (>= BN; wider when gather passes need it)
-  int32_t acc_cols;    // TMEM columns between the accumulators (>= BN, >= gN)
-  int32_t y_tma;       // prefill: y leaves through a shared-memory stage and TMA stores (needs the y map)
-  int32_t fill_rounds; // prefill with a second job: how many of that job's tiles a CTA with a tile fewer (or none)
-                       // takes before the other CTAs get any: about (K blocks of a tile) / (K blocks of such an item)
-  int32_t heavy_first; // prefill: the first token tile holds the batch's decode tokens (many LoRA K blocks per
-                       // output tile): its tiles go to the CTAs that get one tile fewer (see heavy_slots)
+  int32_t tmem_cols;   // power of two >= BN
   int32_t kb_total;    // K blocks of 64 covering h_in
   int32_t kb_per;      // K blocks per split
   int32_t splits;
-  int32_t n_mtiles;    // prefill: token tiles; decode: W row tiles
-  int32_t n_ntiles;    // prefill: W row tiles of BN
+  int32_t n_mtiles;    // W row tiles
   int32_t R_pad;       // slot block rank stride
-  int32_t zsplits;     // partial z planes the consumer sums
-  int32_t expand_in_reduce;  // decode, small batches: B_a z is added by the owners of the cluster
+  int32_t expand_in_reduce;  // small batches: B_a z is added by the owners of the cluster
                              // reduction on the CUDA cores instead of by LoRA K blocks
-  int32_t max_tokens;  // row stride of the z / plan workspaces
+  int32_t max_tokens;  // row stride of the z workspace
   long long wait_cycles;  // limit of the bounded in-kernel waits, in SM clock cycles
-  // shrink jobs (mode sgmv): gather tiles for the tokens the segment tiles do not cover
-  int32_t gather;      // 1: the job also has gather tiles (stacked A rows x gathered token rows)
-  int32_t finalize;    // 1: whoever completes a gather tile last adds its K splits into the final z plane
-  int32_t gN;          // most token rows of one gather pass (multiple of 16, <= rows of the ring's C region)
-  const int32_t *perm_short;     // plan: tokens ordered by (id, token), short runs only
-  const int32_t *gs_short;       // plan: group boundaries inside perm_short
-  const int32_t *group_adapter;  // plan: adapter of each group (-1 first when present)
-  int32_t *tile_counters;        // [>= gather tiles] arrivals per gather tile, zero between launches
-  const int32_t *ids_valid;
-  const int32_t *ids;       // decode: the caller's ids (validated again inside the kernel)
+  const int32_t *ids;       // the caller's ids (validated again inside the kernel)
   int32_t n_slots;
   const SlotRow *slots;
   const uint16_t *B_pool;   // [S][h_out][R_pad]
-  const float *zws;         // [zsplits][max_tokens][R_pad]   (read by the prefill epilogue)
-  float *zws_out;           // same buffer, written by the segment shrink
+  const float *zws;         // [max_tokens][R_pad]: the summed z
   uint16_t *y;              // [T][h_out]
-  const int32_t *sgmv_tiles;
-  const int32_t *counts;
-  const int32_t *mt_count;    // prefill: per 128-token tile
-  const int32_t *mt_list;
   uint32_t *status;
 };
 
@@ -138,20 +113,13 @@ struct FusedDecode {
 void launch_plan(const int32_t *ids, int32_t T, int32_t n_slots, const PlanView &pv, bool pdl,
                  cudaStream_t stream);
 void init_plan_kernel();
-cudaError_t launch_gemm(const CUtensorMap &tmap_row, const CUtensorMap &tmap_col,
-                        const CUtensorMap &tmap_b, const GemmParams &p, int32_t grid,
-                        size_t smem_bytes, bool pdl, cudaStream_t stream, const CUtensorMap *tmap_y = nullptr);
-cudaError_t launch_gemm2(const CUtensorMap &tmap_row, const CUtensorMap &tmap_col,
-                         const CUtensorMap &tmap_b, const GemmParams &p, const CUtensorMap &tmap_row2,
-                         const CUtensorMap &tmap_col2, const CUtensorMap &tmap_g2, const GemmParams &p2,
-                         int32_t grid, size_t smem_bytes, bool pdl, cudaStream_t stream,
-                         const CUtensorMap *tmap_y = nullptr);
+cudaError_t launch_gemm(const CUtensorMap &tmap_row, const CUtensorMap &tmap_col, const CUtensorMap &tmap_b,
+                        const GemmParams &p, int32_t grid, size_t smem_bytes, bool pdl, cudaStream_t stream);
 // Decode job with the shrink in the same grid: grid = f.n_ctas + p.n_mtiles * p.splits CTAs.
 cudaError_t launch_gemm_fused(const CUtensorMap &tmap_row, const CUtensorMap &tmap_col, const GemmParams &p,
                               const FusedDecode &f, size_t smem_bytes, bool pdl, cudaStream_t stream);
 // How many CTAs of such a launch (in whole clusters) can be resident at once on the current device.
 int32_t gemm_fused_max_ctas(int32_t cluster, size_t smem_bytes);
-constexpr int kYStageBytes = 4 * 32 * 128;  // prefill epilogue: per epilogue warp 32 rows x 64 bf16
 cudaError_t gemm_set_smem_limit(size_t smem_bytes);
 cudaError_t shrink_set_smem_limit();
 cudaError_t launch_q8_to_block(const uint8_t *A_q8, const uint8_t *B_q8, uint16_t *A_blk, uint16_t *B_blk,

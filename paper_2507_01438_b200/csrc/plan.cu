@@ -8,7 +8,7 @@
 //   short lists the groups restricted to tokens the gather-by-token shrink handles,
 //   sgmv tiles  in batches above kDecodeMaxT tokens, for runs of >= kSegMin tokens on a real
 //               adapter: 128-token tiles of the run (work list of the segment shrink),
-//   tile lists  the distinct ids >= 0 inside every 128-token tile (the LoRA K blocks of that tile).
+//   tile lists  the distinct ids >= 0 inside every 256-token tile (the LoRA K blocks of that tile).
 // Tokens of one run stay together in the group order, so the runs are sorted, not the tokens: a
 // bitonic sort of the unique keys ((id + 1) << 16 | run index) in shared memory, exact and the
 // same on every launch.  Prefix sums run in rounds of one element per thread (warp shuffles plus
@@ -203,48 +203,40 @@ plan_kernel(const int32_t *__restrict__ ids, int32_t T, int32_t n_slots, PlanVie
   if (tid == 0) pv.counts[2] = min(n_tiles, pv.max_sgmv_tiles);
   __syncthreads();  // inv (in pv.mt_list) is dead from here
 
-  // 8. the distinct ids >= 0 inside every 128-token tile, in order of first appearance (the LoRA
-  // K blocks of that tile in the base-product kernel).  One warp per tile; lane l holds the ids
-  // of tokens l, l + 32, l + 64, l + 96 of the tile.
+  // 8. the distinct ids >= 0 inside every 256-token tile, in order of first appearance (the LoRA
+  // K blocks of that tile in the base-product kernel).  One warp per tile; lane l holds the ids of
+  // tokens l, l + 32, ... of the tile.  Only the first token of a run (inside the tile) can be a first
+  // appearance, so each of those is compared with the later ones: as many rounds as the tile has runs.
   {
     const int lane = tid & 31, warp = tid >> 5;
-    const int n_mt = (T + kTileM - 1) / kTileM;
+    const int n_mt = (T + kListTile - 1) / kListTile;
     for (int m = warp; m < n_mt; m += kPlanThreads / 32) {
-      int32_t id[4];
+      int32_t id[8];
+      uint32_t heads[8];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int t = m * kTileM + q * 32 + lane;
+      for (int q = 0; q < 8; ++q) {
+        const int t = m * kListTile + q * 32 + lane;
         id[q] = t < T ? pv.ids_valid[t] : -1;
+        const bool head = id[q] >= 0 && ((q == 0 && lane == 0) || pv.ids_valid[t - 1] != id[q]);
+        heads[q] = __ballot_sync(0xffffffffu, head);
       }
-      const int32_t id0 = __shfl_sync(0xffffffffu, id[0], 0);
-      bool same = true;
+      uint32_t dup = 0;  // bit q: this lane's q-th token is on an id seen before
 #pragma unroll
-      for (int q = 0; q < 4; ++q) same = same && (id[q] == id0);
-      if (__all_sync(0xffffffffu, same)) {  // the usual prefill tile: one run
-        if (lane == 0) {
-          pv.mt_count[m] = id0 >= 0 ? 1 : 0;
-          pv.mt_list[m * kTileM] = id0;
-        }
-        continue;
-      }
-      bool first[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) first[q] = id[q] >= 0;
-#pragma unroll
-      for (int qq = 0; qq < 4; ++qq) {
-        for (int src = 0; src < 32; ++src) {
+      for (int qq = 0; qq < 8; ++qq) {
+        for (uint32_t rest = heads[qq]; rest; rest &= rest - 1) {
+          const int src = __ffs(rest) - 1;
           const int32_t v = __shfl_sync(0xffffffffu, id[qq], src);
-          const int pos = qq * 32 + src;
 #pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (pos < q * 32 + lane && v == id[q]) first[q] = false;
+          for (int q = qq; q < 8; ++q)
+            if (v == id[q] && (q > qq || lane > src)) dup |= 1u << q;
         }
       }
       int base = 0;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const uint32_t b = __ballot_sync(0xffffffffu, first[q]);
-        if (first[q]) pv.mt_list[m * kTileM + base + __popc(b & ((1u << lane) - 1u))] = id[q];
+      for (int q = 0; q < 8; ++q) {
+        const bool first = ((heads[q] >> lane) & 1u) && !((dup >> q) & 1u);
+        const uint32_t b = __ballot_sync(0xffffffffu, first);
+        if (first) pv.mt_list[m * kListTile + base + __popc(b & ((1u << lane) - 1u))] = id[q];
         base += __popc(b);
       }
       if (lane == 0) pv.mt_count[m] = base;

@@ -13,11 +13,11 @@ namespace {
 
 constexpr int kStaticMaxTokens = EDGELORA_PLAN_STATIC_MAX_TOKENS;
 constexpr int kStaticMaxTiles = kStaticMaxTokens / kSegMin + 8;
-constexpr int kStaticTokenTiles = (kStaticMaxTokens + kTileM - 1) / kTileM;
+constexpr int kStaticTokenTiles = (kStaticMaxTokens + kListTile - 1) / kListTile;
 // tok_seg, perm_short, lg_adapter: T each; gs_short, scratch: T + 1 each; segment tile list;
 // per-token-tile adapter lists; counts[8]; status[4]
 constexpr int kStaticInts = 3 * kStaticMaxTokens + 2 * (kStaticMaxTokens + 1) + 4 * kStaticMaxTiles +
-                            (kStaticTokenTiles + 1) + kStaticTokenTiles * kTileM + 8 + 4;
+                            (kStaticTokenTiles + 1) + kStaticTokenTiles * kListTile + 8 + 4;
 constexpr int kMaxDevices = 64;
 
 // Held by every GPU that loads the library, until the process exits (about 100 KB).
@@ -78,7 +78,7 @@ extern "C" int edgelora_plan_build_static(const int32_t *adapter_id_dev, int32_t
   pv.sgmv_tiles = q; q += 4 * kStaticMaxTiles;
   pv.lg_adapter = q; q += kStaticMaxTokens;
   pv.mt_count = q; q += kStaticTokenTiles + 1;
-  pv.mt_list = q; q += kStaticTokenTiles * kTileM;
+  pv.mt_list = q; q += kStaticTokenTiles * kListTile;
   pv.counts = q; q += 8;
   pv.status = reinterpret_cast<uint32_t *>(q);
   pv.max_sgmv_tiles = kStaticMaxTiles;

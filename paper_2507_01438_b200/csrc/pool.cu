@@ -15,6 +15,8 @@
 
 #include "guard.h"
 #include "pool.h"
+#include "prefill.h"
+#include "shrink_tiles.h"
 
 using namespace edgelora;
 
@@ -42,7 +44,6 @@ constexpr int kMaxDecodeSplits = 8;  // K splits of a row tile form one (portabl
     }                                                    \
   } while (0)
 
-inline int round_up(int v, int m) { return (v + m - 1) / m * m; }
 inline int pad_rank(int r) { return r <= 16 ? 16 : (r <= 32 ? 32 : 64); }
 
 // ---- cuTensorMapEncodeTiled through the runtime's driver entry point (no link to libcuda) ----
@@ -163,10 +164,10 @@ int plan_alloc(edgelora_plan *pl) {
   const int max_tiles = pl->max_tokens / kSegMin + 8;
   // ids_valid, perm, group_adapter, seg_adapter, tok_seg, perm_short: mt each;
   // group_start, seg_start, gs_short, scratch: mt + 1 each; tiles; counts; status
-  // lg_adapter: mt; mt_count: n_mt + 1; mt_list: n_mt * 128
-  const size_t n_mt = (mt + kTileM - 1) / kTileM;
+  // lg_adapter: mt; mt_count: n_mt + 1; mt_list: n_mt * 256
+  const size_t n_mt = (mt + kListTile - 1) / kListTile;
   const size_t ints = 7 * mt + 4 * (mt + 1) + 4 * static_cast<size_t>(max_tiles) + (n_mt + 1) +
-                      n_mt * kTileM + 8 + 4;
+                      n_mt * kListTile + 8 + 4;
   CUDA_TRY(el_malloc(&pl->block, ints * 4));
   CUDA_TRY(cudaMemset(pl->block, 0, ints * 4));
   int32_t *q = static_cast<int32_t *>(pl->block);
@@ -184,7 +185,7 @@ int plan_alloc(edgelora_plan *pl) {
   v.sgmv_tiles = q; q += 4 * static_cast<size_t>(max_tiles);
   v.lg_adapter = q; q += mt;
   v.mt_count = q; q += n_mt + 1;
-  v.mt_list = q; q += n_mt * kTileM;
+  v.mt_list = q; q += n_mt * kListTile;
   v.counts = q; q += 8;
   v.status = reinterpret_cast<uint32_t *>(q);
   v.max_sgmv_tiles = max_tiles;
@@ -364,8 +365,15 @@ int edgelora_pool_create(const edgelora_pool_config *cfg, edgelora_pool_t **pool
   POOL_TRY(el_malloc(&p->zws, sizeof(float) * (kMaxZSplits + 1) * static_cast<size_t>(p->cfg.max_tokens) * p->R_pad));
   POOL_TRY(el_malloc(&p->group_counters, sizeof(int32_t) * (kDecodeMaxT * 8 + 32)));
   POOL_TRY(cudaMemset(p->group_counters, 0, sizeof(int32_t) * (kDecodeMaxT * 8 + 32)));
+  // an arrival counter per tile of the tensor-core shrink: segment tiles, then gather tiles
+  p->n_tile_counters = p->cfg.max_tokens / kSegMin + 8 +
+                       (std::min(p->cfg.max_tokens, p->cfg.n_slots) * p->R_pad + kTileM - 1) / kTileM;
+  POOL_TRY(el_malloc(&p->tile_counters, sizeof(int32_t) * p->n_tile_counters));
+  POOL_TRY(cudaMemset(p->tile_counters, 0, sizeof(int32_t) * p->n_tile_counters));
   POOL_TRY(gemm_set_smem_limit(kSmemBudget));
   POOL_TRY(shrink_set_smem_limit());
+  POOL_TRY(shrink_tiles_set_smem_limit());
+  POOL_TRY(pair_set_smem_limit());
   rc = edgelora_plan_create(p->cfg.max_tokens, cfg->n_slots, &p->plan);
   if (rc != EDGELORA_OK) {
     edgelora_pool_destroy(p);
@@ -393,6 +401,7 @@ int edgelora_pool_destroy(edgelora_pool_t *p) {
   if (p->zws) el_free(p->zws);
   if (p->q8_dev) el_free(p->q8_dev);
   if (p->group_counters) el_free(p->group_counters);
+  if (p->tile_counters) el_free(p->tile_counters);
   for (auto &r : p->prof) {
     cudaEventDestroy(r.start);
     cudaEventDestroy(r.stop);
@@ -702,8 +711,10 @@ int edgelora_pool_sync_status(edgelora_pool_t *p, uint32_t *bits_out) {
   const uint32_t bits = a | b;
   if (bits_out) *bits_out = bits;
   // a wait that ran out can leave arrival counters between their values: nothing is in flight now
-  if (bits & EDGELORA_STATUS_TIMEOUT)
+  if (bits & EDGELORA_STATUS_TIMEOUT) {
     CUDA_TRY(cudaMemset(p->group_counters, 0, sizeof(int32_t) * (kDecodeMaxT * 8 + 32)));
+    CUDA_TRY(cudaMemset(p->tile_counters, 0, sizeof(int32_t) * p->n_tile_counters));
+  }
   if (bits & EDGELORA_STATUS_BOUNDS) {  // checked build: which test failed first
     uint32_t site = 0;
     CUDA_TRY(cudaMemcpy(&site, p->status_dev + 1, 4, cudaMemcpyDeviceToHost));
@@ -747,9 +758,191 @@ int edgelora_pool_selftest_wait(edgelora_pool_t *p, void *stream) {
 }  // extern "C"
 
 namespace edgelora {
+
+// Orders a call behind every load issued so far, once per stream and load (a wait node between two
+// calls of one stream would also keep them from overlapping).  A captured call records no such wait:
+// see the header for what a graph's owner has to do instead.
+int wait_for_loads(edgelora_pool *p, cudaStream_t stream, bool capturing) {
+  if (p->load_seq == 0 || capturing) return EDGELORA_OK;
+  auto it = std::find_if(p->load_waited.begin(), p->load_waited.end(),
+                         [&](const std::pair<cudaStream_t, uint64_t> &e) { return e.first == stream; });
+  if (it == p->load_waited.end()) {
+    if (p->load_waited.size() >= 64) p->load_waited.clear();  // streams come and go: start over
+    p->load_waited.emplace_back(stream, 0);
+    it = p->load_waited.end() - 1;
+  }
+  if (it->second != p->load_seq) {
+    CUDA_TRY(cudaStreamWaitEvent(stream, p->load_ev, 0));
+    it->second = p->load_seq;
+  }
+  return EDGELORA_OK;
+}
+
+// ---- the tensor-core shrink (shrink_tiles.cu): what a site, its input and the plan contribute to a launch
+static int fill_shrink_site(edgelora_pool *q, ShrinkSite *s, int splits, int x_index) {
+  s->slots = q->slots_dev;
+  s->zws = q->zws;
+  s->tile_counters = q->tile_counters;
+  s->status = q->status_dev;
+  s->x_index = x_index;
+  s->kb_total = (q->cfg.h_in + kBlockK - 1) / kBlockK;
+  s->R_pad = q->R_pad;
+  s->max_tokens = q->cfg.max_tokens;
+  s->splits = splits;
+  // the A blocks as one 2D matrix [n_slots * R_pad][h_in]: slot a is rows [a R_pad, (a + 1) R_pad)
+  return get_tmap(q, &s->a, q->A_pool, q->cfg.h_in, static_cast<uint64_t>(q->R_pad) * q->cfg.n_slots, 0, q->R_pad);
+}
+static int fill_shrink_inputs(edgelora_pool *q, const uint16_t *x, int32_t T, CUtensorMap *mx, CUtensorMap *mg) {
+  const int rc = get_tmap(q, mx, x, q->cfg.h_in, T, 0, kTileM);
+  return rc ? rc : get_tmap(q, mg, x, q->cfg.h_in, T, 0, 1);
+}
+template <int kSites>
+static void fill_shrink_plan(const edgelora_plan *plan, int32_t T, long long wait_cycles, int n_sites, int z_bf16,
+                             ShrinkBatch<kSites> *b) {
+  b->n_sites = n_sites;
+  b->T = T;
+  b->n_slots = plan->n_slots;
+  b->z_bf16 = z_bf16;
+  b->sgmv_tiles = plan->pv.sgmv_tiles;
+  b->counts = plan->pv.counts;
+  b->perm_short = plan->pv.perm_short;
+  b->gs_short = plan->pv.gs_short;
+  b->group_adapter = plan->pv.group_adapter;
+  b->ids_valid = plan->pv.ids_valid;
+  b->wait_cycles = wait_cycles;
+}
+
+// K splits of a site's shrink tiles.  A single site is split until every SM has an item; in a run of sites the
+// items of all sites share the grid, and items of about 32 K blocks keep a wide input from making long ones.
+static int shrink_splits(const edgelora_pool *q, int32_t T, int n_sites) {
+  if (T <= kDecodeMaxT) return 1;
+  const int kbt = (q->cfg.h_in + kBlockK - 1) / kBlockK;
+  int z = n_sites > 1 ? std::min(8, std::max(1, kbt / 32)) : std::min(8, q->sms / std::max(1, T / kTileM));
+  z = std::max(1, std::min(z, kbt / 4));
+  const int kb_per = (kbt + z - 1) / z;
+  return (kbt + kb_per - 1) / kb_per;
+}
+
+// W rows of a pair tile.  A K block of a tile takes about max(2 BN + 60, 390) cycles (2 BN is the tensor pipe's
+// share; below BN = 160 the hand-over of a K block sets the pace: 385 cycles measured at BN = 64), so the width
+// whose last wave is fullest for the width's efficiency is taken; the sites' tiles form one list over all pairs.
+static int pair_width(const SiteCall *sites, int n, int n_mtiles, int units) {
+  int best = 0;
+  double best_cost = 0;
+  for (int BN = 256; BN >= 64; BN -= 32) {
+    double work = 0;
+    int64_t tiles = 0;
+    int kb_max = 0;
+    for (int i = 0; i < n; ++i) {
+      const int kb = (sites[i].p->cfg.h_in + kBlockK - 1) / kBlockK + 4;
+      const int64_t t = static_cast<int64_t>(n_mtiles) * ((sites[i].p->cfg.h_out + BN - 1) / BN);
+      tiles += t;
+      work += static_cast<double>(t) * kb;
+      kb_max = std::max(kb_max, kb);
+    }
+    const double waves = static_cast<double>((tiles + units - 1) / units);
+    // one site: whole waves; several: the list's total, and half a tile for its ragged end
+    const double k = n == 1 ? waves * kb_max : std::max(work / units + 0.5 * kb_max, static_cast<double>(kb_max));
+    const double cost = k * std::max(2 * BN + 60, 390) + 12.0 * BN;  // + the last tile's epilogue
+    if (best == 0 || cost < best_cost) {
+      best = BN;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
+template <int kSites>
+static int prefill_batch(const SiteCall *sites, int n, edgelora_plan *plan, int32_t T, cudaStream_t stream,
+                         bool pdl_shrink, bool pdl_base) {
+  edgelora_pool *p0 = sites[0].p;
+  const int n_mtiles = (T + kListTile - 1) / kListTile;
+  const int BN = pair_width(sites, n, n_mtiles, std::max(1, p0->sms / 2));
+  ShrinkBatch<kSites> sb{};
+  PairBatch<kSites> pb{};
+  fill_shrink_plan(plan, T, p0->wait_cycles, n, 1, &sb);
+  pb.n_sites = n;
+  pb.T = T;
+  pb.n_slots = plan->n_slots;
+  pb.BN = BN;
+  pb.stages = pair_stages(BN);
+  pb.n_mtiles = n_mtiles;
+  pb.ids_valid = plan->pv.ids_valid;
+  pb.mt_count = plan->pv.mt_count;
+  pb.mt_list = plan->pv.mt_list;
+  pb.wait_cycles = p0->wait_cycles;
+  const uint16_t *inputs[kPairInputs] = {};
+  int n_inputs = 0, tiles = 0;
+  for (int i = 0; i < n; ++i) {
+    edgelora_pool *q = sites[i].p;
+    int xi = 0;
+    while (xi < n_inputs && inputs[xi] != sites[i].x) ++xi;
+    if (xi == n_inputs) {
+      inputs[n_inputs++] = sites[i].x;
+      const int rc = fill_shrink_inputs(q, sites[i].x, T, &sb.x[xi], &sb.xg[xi]);
+      if (rc) return rc;
+      pb.x[xi] = sb.x[xi];
+    }
+    PairSite &s = pb.site[i];
+    int rc = fill_shrink_site(q, &sb.site[i], shrink_splits(q, T, n), xi);
+    if (!rc) rc = get_tmap(q, &s.w, sites[i].W, q->cfg.h_in, q->cfg.h_out, 0, BN / 2);
+    if (!rc) rc = get_tmap(q, &s.b, q->B_pool, q->R_pad, q->cfg.h_out, q->cfg.n_slots, BN / 2);
+    if (rc) return rc;
+    tiles += n_mtiles * ((q->cfg.h_out + BN - 1) / BN);
+    s.y = static_cast<uint16_t *>(sites[i].y);
+    s.slots = q->slots_dev;
+    s.zb = reinterpret_cast<const uint4 *>(q->zws + static_cast<size_t>(kMaxZSplits) * q->cfg.max_tokens * q->R_pad);
+    s.status = q->status_dev;
+    s.tile_end = tiles;
+    s.x_index = xi;
+    s.h_out = q->cfg.h_out;
+    s.kb_total = (q->cfg.h_in + kBlockK - 1) / kBlockK;
+    s.R_pad = q->R_pad;
+  }
+  {
+    ProfScope ps(p0, 2, stream);
+    CUDA_TRY(launch_shrink_tiles(sb, p0->sms, pdl_shrink, stream));
+  }
+  {
+    ProfScope ps(p0, 3, stream);
+    CUDA_TRY(launch_pair_gemm(pb, p0->sms, pdl_base, stream));
+  }
+  for (int i = 0; i < n; ++i) {
+    int64_t *info = sites[i].p->last_info;
+    info[1] = 2;
+    info[2] = 2 * std::max(1, std::min(p0->sms / 2, tiles));
+    info[3] = 1;
+    info[4] = pb.stages;
+    info[5] = BN;
+  }
+  return EDGELORA_OK;
+}
+
+// Large batches: plan (when ids are given), shrink, base product with the expand, for one site or for a run of
+// sites that share the plan: at most kPairSites sites on at most kPairInputs inputs, no pool twice.
+int prefill_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32_t *ids_dev, int32_t T,
+                  cudaStream_t stream, bool pdl_first) {
+  edgelora_pool *p0 = sites[0].p;
+  const bool pdl = p0->opt_pdl >= 1 && !p0->opt_profile;
+  int launches = 2;
+  if (ids_dev) {
+    ProfScope ps(p0, 0, stream);
+    plan->last_T = T;
+    launch_plan(ids_dev, T, plan->n_slots, plan->pv, pdl_first, stream);
+    CUDA_TRY(cudaGetLastError());
+    ++launches;
+  }
+  const bool pdl_shrink = ids_dev ? pdl : (pdl_first && pdl);
+  const int rc = n == 1 ? prefill_batch<1>(sites, n, plan, T, stream, pdl_shrink, pdl)
+                        : prefill_batch<kPairSites>(sites, n, plan, T, stream, pdl_shrink, pdl);
+  if (rc) return rc;
+  for (int i = 0; i < n; ++i) sites[i].p->last_info[0] = i == 0 ? launches : 0;
+  p0->total_launches += launches;
+  return EDGELORA_OK;
+}
+
 int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_dev, const void *W_dev,
-                     const void *x_dev, int32_t T, void *y_dev, cudaStream_t stream, bool skip_shrink,
-                     const NextShrink *next, bool independent) {
+                     const void *x_dev, int32_t T, void *y_dev, cudaStream_t stream, bool independent) {
   if (!p || !plan || T < 0) return EDGELORA_ERR_INVALID_ARG;
   if (T == 0) return EDGELORA_OK;
   if (!W_dev || !x_dev || !y_dev) return EDGELORA_ERR_INVALID_ARG;
@@ -768,22 +961,8 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
   const uint16_t *x = static_cast<const uint16_t *>(x_dev);
   int launches = 0;
 
-  // Order this call behind every load issued so far, once per stream and load (a wait node
-  // between two calls of one stream would also keep them from overlapping).  A captured call
-  // records no such wait: see the header for what a graph's owner has to do instead.
-  if (p->load_seq != 0 && !capturing) {
-    auto it = std::find_if(p->load_waited.begin(), p->load_waited.end(),
-                           [&](const std::pair<cudaStream_t, uint64_t> &e) { return e.first == stream; });
-    if (it == p->load_waited.end()) {
-      if (p->load_waited.size() >= 64) p->load_waited.clear();  // streams come and go: start over
-      p->load_waited.emplace_back(stream, 0);
-      it = p->load_waited.end() - 1;
-    }
-    if (it->second != p->load_seq) {
-      CUDA_TRY(cudaStreamWaitEvent(stream, p->load_ev, 0));
-      it->second = p->load_seq;
-    }
-  }
+  const int rc_loads = wait_for_loads(p, stream, capturing);
+  if (rc_loads) return rc_loads;
 
   int regime = (T <= kDecodeMaxT) ? 1 : 2;
   if (p->opt_regime == 2) regime = 2;
@@ -797,24 +976,18 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
   g.kb_total = kb_total;
   g.R_pad = R;
   g.max_tokens = p->cfg.max_tokens;
-  g.ids_valid = plan->pv.ids_valid;
   g.slots = p->slots_dev;
   g.B_pool = p->B_pool;
   g.zws = p->zws;
-  g.zws_out = p->zws;
   g.y = static_cast<uint16_t *>(y_dev);
-  g.sgmv_tiles = plan->pv.sgmv_tiles;
-  g.counts = plan->pv.counts;
   g.ids = ids_dev ? ids_dev : plan->pv.ids_valid;
   g.n_slots = p->cfg.n_slots;
-  g.mt_count = plan->pv.mt_count;
-  g.mt_list = plan->pv.mt_list;
   g.status = p->status_dev;
   g.wait_cycles = p->wait_cycles;
 
   auto smem_for = [](int stages, int BN, int extra = 0) {
-    // alignment slack + operand ring + barriers (512) + decode extras (3456, rounded up)
-    // (+ the prefill epilogue's staging area, 1024-aligned because every part before it is)
+    // alignment slack + operand ring + barriers (512) + adapter list and sort keys (3456, rounded up)
+    // (+ the staged rows of a one-launch call)
     return static_cast<size_t>(1024 + stages * (kTileM * kBlockK * 2 + BN * kBlockK * 2) + 4096 + extra);
   };
   auto stages_for = [&](int BN, int k_blocks_per_cta, size_t budget) {
@@ -827,87 +1000,6 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
     return c;
   };
 
-  // The shrink of a pool as a job of the tile kernel: segment tiles for the long runs of a large
-  // batch (tile list from the plan) and gather tiles for every other token.  `decode`: no segment
-  // tiles, the K split count is chosen on the device from the number of adapters the batch touches,
-  // and whoever completes a tile last adds its splits into the final z plane.
-  const bool sgmv = T > kDecodeMaxT;
-  struct ShrinkJob {
-    GemmParams s;
-    CUtensorMap mx, ma, mg;
-    int grid = 1;
-    size_t smem = 0;
-  };
-  // Inside a set of sites the shrink tiles ride on another site's base-product launch, where few
-  // large items fit into the slack of its last wave better than many small ones; on its own the
-  // shrink is split until every SM has an item.
-  const bool in_set = skip_shrink || next != nullptr;
-  auto zsplits_of = [&](const edgelora_pool *q) {
-    if (!sgmv) return 1;
-    const int kbt = (q->cfg.h_in + kBlockK - 1) / kBlockK;
-    const int tiles_est = std::max(1, T / kTileM);
-    // (inside a set: items of about 32 K blocks, so that a wide input does not make them long)
-    int z = std::max(1, std::min({in_set ? std::max(2, std::min(8, kbt / 32)) : 8, q->sms / tiles_est, kbt / 4}));
-    const int kb_per = (kbt + z - 1) / z;
-    return (kbt + kb_per - 1) / kb_per;
-  };
-  auto shrink_job = [&](edgelora_pool *q, const uint16_t *xq, bool decode, int ring_rows, ShrinkJob *out) -> int {
-    const int kbt = (q->cfg.h_in + kBlockK - 1) / kBlockK;
-    const int Rq = q->R_pad;
-    GemmParams s{};
-    s.mode = kModeSgmv;
-    s.T = T;
-    s.h_in = q->cfg.h_in;
-    s.h_out = q->cfg.h_out;
-    s.kb_total = kbt;
-    s.R_pad = Rq;
-    s.BN = Rq;
-    s.max_tokens = q->cfg.max_tokens;
-    s.zsplits = decode ? 1 : zsplits_of(q);
-    s.splits = decode ? q->opt_gather_splits : s.zsplits;  // 0: the kernel picks the gather tiles' split count
-    while (s.splits > 1 && (s.splits - 1) * ((kbt + s.splits - 1) / s.splits) >= kbt) --s.splits;  // no empty split
-    s.kb_per = (kbt + s.zsplits - 1) / s.zsplits;
-    s.gather = 1;
-    s.finalize = decode ? 1 : 0;
-    // token rows of one gather pass: what the ring's C region holds (given when the job rides on
-    // another job's ring), 64 on its own ring (deep pipeline; a tile rarely has more tokens)
-    s.gN = ring_rows > 0 ? std::min(256, ring_rows / 16 * 16) : std::min(64, round_up(T, 16));
-    s.ring_rows = ring_rows > 0 ? ring_rows : std::max(Rq, s.gN);
-    s.acc_cols = s.ring_rows;
-    s.stages = stages_for(s.ring_rows, std::max(s.kb_per, 8), kSmemBudget);
-    s.n_acc = 2;
-    s.tmem_cols = pow2_cols(2 * s.acc_cols);
-    // upper bound of its tiles (the true count is on the device): segment tiles x splits + one gather
-    // tile per 128 / R_pad adapters x splits
-    const int max_gt = (std::min(T, q->cfg.n_slots) * Rq + kTileM - 1) / kTileM;
-    s.n_mtiles = (plan->pv.max_sgmv_tiles + max_gt) * std::max(s.zsplits, 1);
-    s.ids_valid = plan->pv.ids_valid;
-    s.ids = plan->pv.ids_valid;
-    s.n_slots = q->cfg.n_slots;
-    s.slots = q->slots_dev;
-    s.B_pool = q->B_pool;
-    s.zws = q->zws;
-    s.zws_out = q->zws;
-    s.sgmv_tiles = plan->pv.sgmv_tiles;
-    s.counts = plan->pv.counts;
-    s.mt_count = plan->pv.mt_count;
-    s.mt_list = plan->pv.mt_list;
-    s.perm_short = plan->pv.perm_short;
-    s.gs_short = plan->pv.gs_short;
-    s.group_adapter = plan->pv.group_adapter;
-    s.tile_counters = q->group_counters;
-    s.status = q->status_dev;
-    s.wait_cycles = q->wait_cycles;
-    out->s = s;
-    out->grid = q->sms;
-    out->smem = smem_for(s.stages, s.ring_rows);
-    int rc2 = get_tmap(q, &out->mx, xq, q->cfg.h_in, T, 0, kTileM);
-    if (rc2) return rc2;
-    rc2 = get_tmap(q, &out->mg, xq, q->cfg.h_in, T, 0, 1);
-    if (rc2) return rc2;
-    // the A blocks as one 2D matrix [n_slots * R_pad][h_in]: slot a is rows [a R_pad, (a + 1) R_pad)
-    return get_tmap(q, &out->ma, q->A_pool, q->cfg.h_in, static_cast<uint64_t>(Rq) * q->cfg.n_slots, 0, Rq);
-  };
   // decode batches above this size take the plan kernel + tensor-core gather tiles; smaller ones
   // the single shrink kernel that derives the routing itself (a launch less)
   const int kGatherMinT = p->opt_gather_min_t;
@@ -927,11 +1019,17 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
           CUDA_TRY(cudaGetLastError());
           ++launches;
         }
-        ShrinkJob sj;
-        int rc = shrink_job(p, x, true, 0, &sj);
+        // gather tiles only, the K split count chosen on the device from the number of adapters the
+        // batch touches; the summed z as fp32
+        ShrinkBatch<1> sb{};
+        int splits = p->opt_gather_splits;
+        while (splits > 1 && (splits - 1) * ((kb_total + splits - 1) / splits) >= kb_total) --splits;  // no empty split
+        int rc = fill_shrink_site(p, &sb.site[0], splits, 0);
+        if (!rc) rc = fill_shrink_inputs(p, x, T, &sb.x[0], &sb.xg[0]);
         if (rc) return rc;
+        fill_shrink_plan(plan, T, p->wait_cycles, 1, 0, &sb);
         ProfScope ps(p, 2, stream);
-        CUDA_TRY(launch_gemm(sj.mx, sj.ma, sj.mg, sj.s, sj.grid, sj.smem, ids_dev ? pdl : pdl_first, stream));
+        CUDA_TRY(launch_shrink_tiles(sb, p->sms, ids_dev ? pdl : pdl_first, stream));
         ++launches;
       } else
       {
@@ -995,13 +1093,11 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
       splits >>= 1;
       kb_per = (kb_total + splits - 1) / splits;
     }
-    g.mode = kModeDecode;
     g.BN = N;
     g.splits = splits;
     g.kb_per = kb_per;
     g.n_mtiles = row_tiles;
-    g.n_ntiles = 1;
-    g.zsplits = 1;   // the decode shrink leaves the summed z in the plane after the partial ones
+    // the decode shrink leaves the summed z in the plane after the partial ones
     g.zws = p->zws + static_cast<size_t>(kMaxZSplits) * p->cfg.max_tokens * R;
     const size_t budget = ctas_per_sm == 2 ? kSmemBudget / 2 : kSmemBudget;
     g.stages = stages_for(N, kb_per + 8, budget);
@@ -1021,9 +1117,6 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
     // the cluster's reduction buffer (N x 128 fp32, plus z of the owner's tokens) overlays the ring
     while (splits > 1 && g.stages * stage_bytes < N * kTileM * 4 + (N / splits) * R * 4 && g.stages < kMaxStages)
       ++g.stages;
-    g.n_acc = 1;
-    g.ring_rows = N;
-    g.acc_cols = N;
     g.tmem_cols = pow2_cols(N);
     CUtensorMap mr, mc, mb;
     int rc = get_tmap(p, &mr, W_dev, h_in, h_out, 0, kTileM);
@@ -1103,91 +1196,17 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
     }
   } else {
     // ---------------------------------------------------------------- prefill
-    if (ids_dev) {
-      ProfScope ps(p, 0, stream);
-      plan->last_T = T;
-      launch_plan(ids_dev, T, plan->n_slots, plan->pv, pdl_first, stream);
-      CUDA_TRY(cudaGetLastError());
-      ++launches;
-    }
-    g.zsplits = zsplits_of(p);
-    if (!skip_shrink) {  // this site's shrink on its own, in front of its base product
-      ShrinkJob sj;
-      int rc = shrink_job(p, x, false, 0, &sj);
-      if (rc) return rc;
-      ProfScope ps(p, 2, stream);
-      CUDA_TRY(launch_gemm(sj.mx, sj.ma, sj.mg, sj.s, sj.grid, sj.smem, ids_dev ? pdl : pdl_first, stream));
-      ++launches;
-    }
-    CUtensorMap mx;
-    int rc = get_tmap(p, &mx, x, h_in, T, 0, kTileM);
+    const SiteCall call{p, W_dev, x, y_dev};
+    const int rc = prefill_sites(&call, 1, plan, ids_dev, T, stream, pdl_first);
     if (rc) return rc;
-    const int n_mtiles = (T + kTileM - 1) / kTileM;
-    const int tiles256 = n_mtiles * ((h_out + 255) / 256);
-    // 256-wide tiles unless they would leave three quarters of the SMs without a tile: a K block costs
-    // the producer warp about as much for a 128-wide W tile as for a 256-wide one, so narrow tiles
-    // only pay through parallelism
-    int BN = (tiles256 * 4 >= p->sms || h_out <= 128) ? 256 : 128;
-    BN = std::min(BN, round_up(h_out, 32));
-    g.mode = kModePrefill;
-    g.heavy_first = in_set ? 1 : 0;  // a serving batch: decode tokens first (see heavy_slots in gemm.cu)
-    g.BN = BN;
-    g.ring_rows = BN;
-    g.acc_cols = BN;
-    g.splits = 1;
-    g.kb_per = kb_total;
-    g.n_mtiles = n_mtiles;
-    g.n_ntiles = (h_out + BN - 1) / BN;
-    g.stages = stages_for(BN, kb_total, kSmemBudget - kYStageBytes);
-    g.n_acc = 2;
-    g.tmem_cols = pow2_cols(2 * BN);
-    g.y_tma = 1;
-    CUtensorMap mc, mb, my;
-    rc = get_tmap(p, &my, y_dev, h_out, T, 0, 32, kBlockK);  // y in boxes of 32 rows x 64 columns
-    if (rc) return rc;
-    rc = get_tmap(p, &mc, W_dev, h_in, h_out, 0, BN);
-    if (rc) return rc;
-    rc = get_tmap(p, &mb, p->B_pool, R, h_out, p->cfg.n_slots, BN);
-    if (rc) return rc;
-    int grid = std::min(p->sms, g.n_mtiles * g.n_ntiles);
-    // The next site of a set (independent of this one): its shrink rides on this site's
-    // base-product launch as extra tiles, on this launch's ring.
-    ShrinkJob nj;
-    bool fuse_next = false;
-    if (next && next->pool) {
-      edgelora_pool *q = next->pool;
-      if (q->cfg.max_tokens < T || q->cfg.n_slots != plan->n_slots) return EDGELORA_ERR_INVALID_ARG;
-      if (q->R_pad <= BN) {
-        rc = shrink_job(q, next->x, false, BN, &nj);
-        if (rc) return rc;
-        fuse_next = true;
-        grid = std::min(p->sms, g.n_mtiles * g.n_ntiles + nj.s.n_mtiles);
-        // CTAs that get one tile fewer (or none) are free for about a tile's time: that many shrink items
-        g.fill_rounds = std::max(1, std::min(8, kb_total / std::max(1, nj.s.kb_per)));
-      } else {  // cannot share the ring (a tiny site): on its own, before this site's base product
-        rc = shrink_job(q, next->x, false, 0, &nj);
-        if (rc) return rc;
-        ProfScope ps(q, 2, stream);
-        CUDA_TRY(launch_gemm(nj.mx, nj.ma, nj.mg, nj.s, nj.grid, nj.smem, pdl, stream));
-        ++launches;
-      }
+    if (!capturing) {
+      CUDA_TRY(cudaEventRecord(p->use_ev, stream));
+      p->use_recorded = true;
     }
-    {
-      ProfScope ps(p, 3, stream);
-      if (fuse_next)
-        CUDA_TRY(launch_gemm2(mx, mc, mb, g, nj.mx, nj.ma, nj.mg, nj.s, grid, smem_for(g.stages, BN, kYStageBytes), pdl,
-                              stream, &my));
-      else
-        CUDA_TRY(launch_gemm(mx, mc, mb, g, grid, smem_for(g.stages, BN, kYStageBytes), pdl, stream, &my));
-      ++launches;
-    }
-    p->last_info[2] = grid;
-    p->last_info[3] = 1;
+    return EDGELORA_OK;
   }
 
-  // (inside a set of sites the set records the events once, after its last site: an event between
-  // two kernels would keep them from overlapping)
-  if (!capturing && !next && !skip_shrink) {
+  if (!capturing) {
     CUDA_TRY(cudaEventRecord(p->use_ev, stream));
     p->use_recorded = true;
   }

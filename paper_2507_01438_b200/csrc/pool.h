@@ -77,6 +77,7 @@ struct edgelora_pool {
   edgelora_plan *plan = nullptr;
   float *zws = nullptr;
   int32_t *group_counters = nullptr;
+  int32_t *tile_counters = nullptr, n_tile_counters = 0;  // arrivals per tile of the tensor-core shrink
   int opt_decode_splits = 0, opt_shrink_items = 0, opt_gather_splits = 0, opt_gather_min_t = 256, opt_shrink_depth = 0;
   uint32_t *status_dev = nullptr;
   std::vector<TmapEntry> tmaps;
@@ -106,20 +107,20 @@ struct edgelora_pool {
 
 namespace edgelora {
 
-// What the next site of a set hands to this site's base-product launch: its segment shrink runs as
-// extra tiles of the same persistent kernel (sites are independent, so the tensor cores never
-// wait for a shrink of their own).
-struct NextShrink {
-  edgelora_pool *pool = nullptr;
-  const uint16_t *x = nullptr;
+// One linear site of a call: y = W x + s_a B_a A_a x over the batch of the call's plan.
+struct SiteCall {
+  edgelora_pool *p;
+  const void *W;
+  const uint16_t *x;
+  void *y;
 };
 
-// The layer (see pool.cu).  `skip_shrink`: this site's shrinks were already issued (as part of the
-// previous site's launches); `next`: issue the next site's shrinks along with this site's kernels;
-// `independent`: the call reads nothing the previous call on the stream writes, so its first
-// kernel may start under that call's tail.
+// The layer (see pool.cu).  `independent`: the call reads nothing the previous call on the stream
+// writes, so its first kernel may start under that call's tail.
 int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_dev, const void *W_dev,
-                     const void *x_dev, int32_t T, void *y_dev, cudaStream_t stream,
-                     bool skip_shrink = false, const NextShrink *next = nullptr, bool independent = false);
+                     const void *x_dev, int32_t T, void *y_dev, cudaStream_t stream, bool independent = false);
+int prefill_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32_t *ids_dev, int32_t T,
+                  cudaStream_t stream, bool pdl_first);
+int wait_for_loads(edgelora_pool *p, cudaStream_t stream, bool capturing);
 
 }  // namespace edgelora

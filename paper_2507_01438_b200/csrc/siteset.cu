@@ -1,10 +1,9 @@
 // A set of linear sites that see the same mixed batch (paper Section 3.4: every LoRA-augmented
 // linear layer of the model is evaluated over the same batch of requests; Section 4.3: the mapping
 // from adapter ids to samples is worked out once).  The set builds one routing plan per batch and
-// runs its sites back to back; because the sites are independent given their inputs, the shrink of
-// site i + 1 is issued together with the kernels of site i (its gather part as a light kernel that
-// runs beside them, its segment part as extra tiles of site i's base-product launch), so that only
-// the first site's shrink stands alone in front of a base product.
+// hands its sites to the device in runs: one launch computes the shrink of every site of a run, the next
+// one their base products with the expand, so that launches, ramp-ups and partly empty last waves are paid
+// per run and not per site.  Decode-sized batches go site by site.
 #include <cuda_runtime.h>
 
 #include <cstring>
@@ -13,6 +12,7 @@
 
 #include "guard.h"
 #include "pool.h"
+#include "prefill.h"
 
 using namespace edgelora;
 
@@ -52,25 +52,62 @@ int run_sites(edgelora_siteset *s, const void *const *x_dev, const int32_t *ids_
   int rc = edgelora_plan_build(s->plan, ids_dev, T, stream);
   if (rc != EDGELORA_OK) return rc;
   const int n = static_cast<int>(s->pools.size());
-  // The shrinks ride along only in the prefill regime (the decode regime has its own two-kernel
-  // form) and only when every pool runs in its default configuration.
-  bool pipelined = T > kDecodeMaxT;
-  for (auto *p : s->pools) pipelined = pipelined && p->opt_regime == 0 && p->opt_pdl >= 1;
-  for (int i = 0; i < n; ++i) {
-    NextShrink next;
-    if (pipelined && i + 1 < n) {
-      next.pool = s->pools[i + 1];
-      next.x = static_cast<const uint16_t *>(x_dev[s->input_of[i + 1]]);
+  const bool in_capture = capturing(stream);
+  // Large batches: the sites go to the device in runs that share one shrink launch and one base-product
+  // launch, when every pool runs in its default configuration.
+  bool runs = T > kDecodeMaxT;
+  for (auto *p : s->pools) runs = runs && p->opt_regime == 0 && p->opt_pdl >= 1 && !p->a_q8;
+  if (!runs) {
+    for (int i = 0; i < n; ++i) {
+      if (before && (*before)[i] && cudaStreamWaitEvent(stream, (*before)[i], 0) != cudaSuccess) return EDGELORA_ERR_CUDA;
+      // (decode-sized batches: the sites are independent given their inputs and results, so a
+      // site's shrink may start under the previous site's base product)
+      rc = lora_linear_impl(s->pools[i], s->plan, nullptr, s->W[i], x_dev[s->input_of[i]], T, y_dev[i], stream, i > 0);
+      if (rc != EDGELORA_OK) return rc;
+      if (after && (*after)[i] && cudaEventRecord((*after)[i], stream) != cudaSuccess) return EDGELORA_ERR_CUDA;
     }
-    if (before && (*before)[i] && cudaStreamWaitEvent(stream, (*before)[i], 0) != cudaSuccess) return EDGELORA_ERR_CUDA;
-    // (decode-sized batches: the sites are independent given their inputs and results, so a
-    // site's shrink may start under the previous site's base product)
-    rc = lora_linear_impl(s->pools[i], s->plan, nullptr, s->W[i], x_dev[s->input_of[i]], T, y_dev[i], stream,
-                          pipelined && i > 0, next.pool ? &next : nullptr, !pipelined && i > 0);
-    if (rc != EDGELORA_OK) return rc;
-    if (after && (*after)[i] && cudaEventRecord((*after)[i], stream) != cudaSuccess) return EDGELORA_ERR_CUDA;
+    return EDGELORA_OK;
   }
-  if (pipelined && !capturing(stream)) {  // slot loads issued later wait for this step
+  for (int i = 0; i < n; ++i) {
+    if ((reinterpret_cast<uintptr_t>(x_dev[s->input_of[i]]) | reinterpret_cast<uintptr_t>(s->W[i]) |
+         reinterpret_cast<uintptr_t>(y_dev[i])) & 15)
+      return EDGELORA_ERR_INVALID_ARG;
+    rc = wait_for_loads(s->pools[i], stream, in_capture);
+    if (rc != EDGELORA_OK) return rc;
+  }
+  for (int i0 = 0; i0 < n;) {
+    // A run ends where the launch's tables are full, where a pool would come twice (its z workspace holds one
+    // site's z), in front of a site whose input is still on its way, and behind about a decoder layer of
+    // sites when results are read back beside the sites that follow.  Profiled pools go one by one.
+    SiteCall calls[kPairSites];
+    const uint16_t *inputs[kPairInputs];
+    int m = 0, n_inputs = 0;
+    bool read_back = false;
+    for (int i = i0; i < n && m < kPairSites; ++i) {
+      edgelora_pool *p = s->pools[i];
+      const uint16_t *x = static_cast<const uint16_t *>(x_dev[s->input_of[i]]);
+      if (m > 0 && ((before && (*before)[i]) || p->opt_profile || calls[0].p->opt_profile || (read_back && m >= 7))) break;
+      bool again = false;
+      for (int k = 0; k < m; ++k) again = again || calls[k].p == p;
+      if (again) break;
+      int xi = 0;
+      while (xi < n_inputs && inputs[xi] != x) ++xi;
+      if (xi == kPairInputs) break;
+      if (xi == n_inputs) inputs[n_inputs++] = x;
+      if (m == 0 && before && (*before)[i] && cudaStreamWaitEvent(stream, (*before)[i], 0) != cudaSuccess)
+        return EDGELORA_ERR_CUDA;
+      calls[m++] = SiteCall{p, s->W[i], x, y_dev[i]};
+      read_back = read_back || (after && (*after)[i]);
+    }
+    // (the kernel in front of a run is the plan kernel, launched behind everything before it, or the base
+    // product of the run before)
+    rc = prefill_sites(calls, m, s->plan, nullptr, T, stream, true);
+    if (rc != EDGELORA_OK) return rc;
+    for (int i = i0; i < i0 + m; ++i)
+      if (after && (*after)[i] && cudaEventRecord((*after)[i], stream) != cudaSuccess) return EDGELORA_ERR_CUDA;
+    i0 += m;
+  }
+  if (!in_capture) {  // slot loads issued later wait for this step
     for (auto *p : s->pools) {
       if (cudaEventRecord(p->use_ev, stream) != cudaSuccess) return EDGELORA_ERR_CUDA;
       p->use_recorded = true;
