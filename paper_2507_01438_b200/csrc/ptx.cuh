@@ -338,6 +338,35 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t *bar) {
       : "memory");
 }
 
+// ---------------------------------------------------------------- cluster launch control
+// Takes a cluster of this grid that has not started yet: its launch is cancelled and the caller does its work
+// instead.  The answer (16 bytes) is written to `dst`, and counted on `bar`, at these offsets in every CTA of
+// the caller's cluster.
+__device__ __forceinline__ void cluster_try_cancel(void *dst, uint64_t *bar) {
+  asm volatile(
+      "clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.multicast::cluster::all.b128 "
+      "[%0], [%1];" ::"r"(smem_u32(dst)),
+      "r"(smem_u32(bar))
+      : "memory");
+}
+// The first CTA of the cluster that was taken, or -1 when none was left.
+__device__ __forceinline__ int32_t cluster_taken(const void *answer) {
+  uint64_t lo, hi;
+  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "r"(smem_u32(answer)) : "memory");
+  int32_t first = -1;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b128 h;\n\tmov.b128 h, {%1, %2};\n\t"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\t"
+      "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, h;\n\t}"
+      : "+r"(first)
+      : "l"(lo), "l"(hi));
+  return first;
+}
+// arrive + expect on a barrier of another CTA of the cluster
+__device__ __forceinline__ void mbar_arrive_expect_tx_cluster(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+
 // ---------------------------------------------------------------- programmatic dependent launch
 __device__ __forceinline__ void pdl_wait_prior_grids() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
