@@ -57,14 +57,242 @@ __device__ __forceinline__ int scan_rounds(int n, int *wt, Value value, Consume 
   return base;
 }
 
+// The distinct ids >= 0 inside every 256-token tile, in order of first appearance (the LoRA K blocks of that tile
+// in the base-product kernel).  One warp per tile; lane l holds the ids of tokens l, l + 32, ... of the tile.
+// Only the first token of a run (inside the tile) can be a first appearance, so each of those is compared with
+// the later ones: as many rounds as the tile has runs.
+__device__ __forceinline__ void list_tiles(const int32_t *valid, int32_t T, const PlanView &pv) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n_mt = (T + kListTile - 1) / kListTile;
+  for (int m = warp; m < n_mt; m += kPlanThreads / 32) {
+    int32_t id[8];
+    uint32_t heads[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int t = m * kListTile + q * 32 + lane;
+      id[q] = t < T ? valid[t] : -1;
+      const bool head = id[q] >= 0 && ((q == 0 && lane == 0) || valid[t - 1] != id[q]);
+      heads[q] = __ballot_sync(0xffffffffu, head);
+    }
+    uint32_t dup = 0;  // bit q: this lane's q-th token is on an id seen before
+#pragma unroll
+    for (int qq = 0; qq < 8; ++qq) {
+      for (uint32_t rest = heads[qq]; rest; rest &= rest - 1) {
+        const int src = __ffs(rest) - 1;
+        const int32_t v = __shfl_sync(0xffffffffu, id[qq], src);
+#pragma unroll
+        for (int q = qq; q < 8; ++q)
+          if (v == id[q] && (q > qq || lane > src)) dup |= 1u << q;
+      }
+    }
+    int base = 0;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const bool first = ((heads[q] >> lane) & 1u) && !((dup >> q) & 1u);
+      const uint32_t b = __ballot_sync(0xffffffffu, first);
+      if (first) pv.mt_list[m * kListTile + base + __popc(b & ((1u << lane) - 1u))] = id[q];
+      base += __popc(b);
+    }
+    if (lane == 0) pv.mt_count[m] = base;
+  }
+}
+
+// Batches up to kPlanSmallT tokens with up to 1024 runs (every serving batch of ordinary make): the same plan,
+// worked out in shared memory with one thread per run.  The general form below keeps its intermediate arrays
+// in global memory and goes through them in about thirty barrier-separated passes, each a round trip to L2;
+// here the runs are ordered by counting smaller keys instead of by a sorting network, and the four prefix sums
+// over the runs are one scan of four packed 16-bit fields.
+constexpr int kPlanSmallT = 4096;
+constexpr int kPlanTok = kPlanSmallT / kPlanThreads;  // tokens per thread, consecutive
+struct PlanSmall {
+  int32_t ids[kPlanSmallT];
+  int32_t seg_start[kPlanThreads + 1], seg_id[kPlanThreads];
+  alignas(16) uint32_t key[kPlanThreads];
+  int32_t run[kPlanThreads];                      // run at each place of the order
+  int32_t out[kPlanThreads], out_short[kPlanThreads];  // by run: where it begins in perm and perm_short
+  unsigned long long wt[kPlanThreads / 32];
+};
+static_assert(sizeof(PlanSmall) >= kPlanSmallT * 4, "the general form's keys fit too");
+
+// Exclusive prefix sum over the block (one synchronisation; wt must not be in use by an earlier scan).
+__device__ __forceinline__ unsigned long long scan_block(unsigned long long v, unsigned long long *wt,
+                                                         unsigned long long &total) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned long long incl = v;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const unsigned long long o = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += o;
+  }
+  if (lane == 31) wt[warp] = incl;
+  __syncthreads();
+  unsigned long long w = wt[lane];  // every warp adds up the 32 warps' sums for itself
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const unsigned long long o = __shfl_up_sync(0xffffffffu, w, d);
+    if (lane >= d) w += o;
+  }
+  total = __shfl_sync(0xffffffffu, w, 31);
+  const unsigned long long before = __shfl_sync(0xffffffffu, w, max(warp - 1, 0));
+  return (warp > 0 ? before : 0ull) + incl - v;
+}
+
+// Returns false, with nothing but ids_valid written, when the batch has more than 1024 runs.
+__device__ __forceinline__ bool plan_small(const int32_t *__restrict__ ids, int32_t T, int32_t n_slots,
+                                           const PlanView &pv, PlanSmall &sh) {
+  const int tid = threadIdx.x;
+  // validate; segments = maximal runs of equal id in token order
+  bool bad = false;
+  int32_t id[kPlanTok];
+#pragma unroll
+  for (int q = 0; q < kPlanTok; ++q) {
+    const int t = q * kPlanThreads + tid;
+    if (t < T) {
+      int32_t a = ids[t];
+      if (a < -1 || a >= n_slots) {
+        a = -1;
+        bad = true;
+      }
+      sh.ids[t] = a;
+      pv.ids_valid[t] = a;
+    }
+  }
+  if (__syncthreads_or(bad ? 1 : 0) && tid == 0) atomicOr(pv.status, EDGELORA_STATUS_BAD_ADAPTER_ID);
+  const int per = (T + kPlanThreads - 1) / kPlanThreads;  // tokens of this thread: [tid per, tid per + per)
+  int heads = 0;
+  uint32_t is_head = 0;
+#pragma unroll
+  for (int q = 0; q < kPlanTok; ++q) {
+    const int t = tid * per + q;
+    if (q < per && t < T) {
+      id[q] = sh.ids[t];
+      if (t == 0 || sh.ids[t - 1] != id[q]) {
+        is_head |= 1u << q;
+        ++heads;
+      }
+    }
+  }
+  unsigned long long total;
+  int s = static_cast<int>(scan_block(heads, sh.wt, total)) - 1;
+  const int n_segs = static_cast<int>(total);
+  if (n_segs > kPlanThreads) return false;
+#pragma unroll
+  for (int q = 0; q < kPlanTok; ++q) {
+    const int t = tid * per + q;
+    if (q < per && t < T) {
+      if ((is_head >> q) & 1u) {
+        ++s;
+        sh.seg_start[s] = t;
+        sh.seg_id[s] = id[q];
+        pv.seg_start[s] = t;
+        pv.seg_adapter[s] = id[q];
+      }
+      pv.tok_seg[t] = s;
+    }
+  }
+  if (tid == 0) {
+    sh.seg_start[n_segs] = T;
+    pv.seg_start[n_segs] = T;
+    pv.counts[1] = n_segs;
+  }
+  __syncthreads();
+
+  // the runs ordered by (id, run index): -1 first, token order kept.  Keys are unique.
+  const int n4 = (n_segs + 3) & ~3;
+  uint32_t key = 0xFFFFFFFFu;
+  int len = 0;
+  if (tid < n_segs) {
+    key = (static_cast<uint32_t>(sh.seg_id[tid] + 1) << 16) | static_cast<uint32_t>(tid);
+    len = sh.seg_start[tid + 1] - sh.seg_start[tid];
+  }
+  if (tid < n4) sh.key[tid] = key;
+  __syncthreads();
+  if (tid < n_segs) {
+    int place = 0;
+    for (int i = 0; i < n4; i += 4) {
+      const uint4 k = *reinterpret_cast<const uint4 *>(&sh.key[i]);
+      place += (k.x < key) + (k.y < key) + (k.z < key) + (k.w < key);
+    }
+    sh.run[place] = tid;
+  }
+  __syncthreads();
+
+  // one scan: tokens and short tokens (runs the gather-by-token shrink handles: every run of a small batch,
+  // otherwise those below kSegMin) and group heads in the order of the runs, segment tiles in token order
+  const bool all_short = T <= kDecodeMaxT;
+  int my_run = 0, my_len = 0, my_short = 0, my_head = 0, my_tiles = 0, my_id = -1;
+  if (tid < n_segs) {
+    my_run = sh.run[tid];
+    my_len = sh.seg_start[my_run + 1] - sh.seg_start[my_run];
+    my_short = (all_short || my_len < kSegMin) ? my_len : 0;
+    my_id = sh.seg_id[my_run];
+    my_head = (tid == 0 || sh.seg_id[sh.run[tid - 1]] != my_id) ? 1 : 0;
+    my_tiles = (!all_short && sh.seg_id[tid] >= 0 && len >= kSegMin) ? (len + kTileM - 1) / kTileM : 0;
+  }
+  const unsigned long long packed = static_cast<unsigned long long>(my_len) | (static_cast<unsigned long long>(my_short) << 16) |
+                                    (static_cast<unsigned long long>(my_head) << 32) |
+                                    (static_cast<unsigned long long>(my_tiles) << 48);
+  const unsigned long long pre = scan_block(packed, sh.wt, total);  // (the barriers above lie behind the first scan)
+  const int p_len = static_cast<int>(pre & 0xFFFF), p_short = static_cast<int>((pre >> 16) & 0xFFFF);
+  const int g = static_cast<int>((pre >> 32) & 0xFFFF) + my_head - 1, p_tiles = static_cast<int>(pre >> 48);
+  const int n_groups = static_cast<int>((total >> 32) & 0xFFFF), n_short = static_cast<int>((total >> 16) & 0xFFFF);
+  const int has_base = (n_segs > 0 && sh.seg_id[sh.run[0]] < 0) ? 1 : 0;  // the group of id -1 comes first
+  if (tid < n_segs) {
+    sh.out[my_run] = p_len;
+    sh.out_short[my_run] = my_short > 0 ? p_short : -1;
+    if (my_head) {
+      pv.group_start[g] = p_len;
+      pv.gs_short[g] = p_short;
+      pv.group_adapter[g] = my_id;
+      if (my_id >= 0) pv.lg_adapter[g - has_base] = my_id;
+    }
+    for (int i = 0; i < my_tiles; ++i) {  // 128-token tiles of this thread's (long) run
+      const int tile = p_tiles + i;
+      if (tile < pv.max_sgmv_tiles) {
+        pv.sgmv_tiles[4 * tile + 0] = sh.seg_start[tid] + i * kTileM;
+        pv.sgmv_tiles[4 * tile + 1] = min(kTileM, len - i * kTileM);
+        pv.sgmv_tiles[4 * tile + 2] = sh.seg_id[tid];
+        pv.sgmv_tiles[4 * tile + 3] = 0;
+      }
+    }
+  }
+  if (tid == 0) {
+    pv.group_start[n_groups] = T;
+    pv.gs_short[n_groups] = n_short;
+    pv.counts[0] = n_groups;
+    pv.counts[2] = min(static_cast<int>(total >> 48), pv.max_sgmv_tiles);
+    pv.counts[3] = n_short;
+    pv.counts[4] = n_groups - has_base;
+    pv.counts[5] = 0;
+  }
+  __syncthreads();
+  // groups: the runs in order, concatenated (s is the run of this thread's last token)
+#pragma unroll
+  for (int q = kPlanTok - 1; q >= 0; --q) {
+    const int t = tid * per + q;
+    if (q < per && t < T) {
+      const int off = t - sh.seg_start[s], pos = sh.out[s] + off;
+      if (EL_CHECK(pv.status, s >= 0 && s < n_segs && pos >= 0 && pos < T, 30)) pv.perm[pos] = t;
+      if (sh.out_short[s] >= 0 && EL_CHECK(pv.status, sh.out_short[s] + off < T, 31)) pv.perm_short[sh.out_short[s] + off] = t;
+      if ((is_head >> q) & 1u) --s;
+    }
+  }
+  list_tiles(sh.ids, T, pv);
+  return true;
+}
+
 __global__ void __launch_bounds__(kPlanThreads)
 plan_kernel(const int32_t *__restrict__ ids, int32_t T, int32_t n_slots, PlanView pv) {
-  extern __shared__ uint32_t keys[];  // one key per run, padded to a power of two
+  extern __shared__ __align__(16) uint32_t keys[];  // one key per run, padded to a power of two
   __shared__ int wt[34];
   const int tid = threadIdx.x;
 
   ptx::pdl_launch_dependents();
   ptx::pdl_wait_prior_grids();  // earlier kernels on the stream may still read the plan arrays
+  if (T <= kPlanSmallT) {
+    if (plan_small(ids, T, n_slots, pv, *reinterpret_cast<PlanSmall *>(keys))) return;
+    __syncthreads();
+  }
 
   // 1. validate
   bool bad = false;
@@ -203,53 +431,16 @@ plan_kernel(const int32_t *__restrict__ ids, int32_t T, int32_t n_slots, PlanVie
   if (tid == 0) pv.counts[2] = min(n_tiles, pv.max_sgmv_tiles);
   __syncthreads();  // inv (in pv.mt_list) is dead from here
 
-  // 8. the distinct ids >= 0 inside every 256-token tile, in order of first appearance (the LoRA
-  // K blocks of that tile in the base-product kernel).  One warp per tile; lane l holds the ids of
-  // tokens l, l + 32, ... of the tile.  Only the first token of a run (inside the tile) can be a first
-  // appearance, so each of those is compared with the later ones: as many rounds as the tile has runs.
-  {
-    const int lane = tid & 31, warp = tid >> 5;
-    const int n_mt = (T + kListTile - 1) / kListTile;
-    for (int m = warp; m < n_mt; m += kPlanThreads / 32) {
-      int32_t id[8];
-      uint32_t heads[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int t = m * kListTile + q * 32 + lane;
-        id[q] = t < T ? pv.ids_valid[t] : -1;
-        const bool head = id[q] >= 0 && ((q == 0 && lane == 0) || pv.ids_valid[t - 1] != id[q]);
-        heads[q] = __ballot_sync(0xffffffffu, head);
-      }
-      uint32_t dup = 0;  // bit q: this lane's q-th token is on an id seen before
-#pragma unroll
-      for (int qq = 0; qq < 8; ++qq) {
-        for (uint32_t rest = heads[qq]; rest; rest &= rest - 1) {
-          const int src = __ffs(rest) - 1;
-          const int32_t v = __shfl_sync(0xffffffffu, id[qq], src);
-#pragma unroll
-          for (int q = qq; q < 8; ++q)
-            if (v == id[q] && (q > qq || lane > src)) dup |= 1u << q;
-        }
-      }
-      int base = 0;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const bool first = ((heads[q] >> lane) & 1u) && !((dup >> q) & 1u);
-        const uint32_t b = __ballot_sync(0xffffffffu, first);
-        if (first) pv.mt_list[m * kListTile + base + __popc(b & ((1u << lane) - 1u))] = id[q];
-        base += __popc(b);
-      }
-      if (lane == 0) pv.mt_count[m] = base;
-    }
-  }
+  // 8. the adapters of every 256-token tile
+  list_tiles(pv.ids_valid, T, pv);
 }
 
 void launch_plan(const int32_t *ids, int32_t T, int32_t n_slots, const PlanView &pv, bool pdl,
                  cudaStream_t stream) {
   int npow2 = 32;  // the number of runs is only known on the device: size for the worst case
   while (npow2 < T) npow2 <<= 1;
-  launch_ex(plan_kernel, dim3(1), dim3(kPlanThreads), static_cast<size_t>(npow2) * 4, stream, pdl, 1,
-            ids, T, n_slots, pv);
+  const size_t smem = T <= kPlanSmallT ? sizeof(PlanSmall) : static_cast<size_t>(npow2) * 4;
+  launch_ex(plan_kernel, dim3(1), dim3(kPlanThreads), smem, stream, pdl, 1, ids, T, n_slots, pv);
 }
 
 void init_plan_kernel() {

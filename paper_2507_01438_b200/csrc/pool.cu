@@ -899,14 +899,13 @@ static int prefill_batch(const SiteCall *sites, int n, edgelora_plan *plan, int3
     s.kb_total = (q->cfg.h_in + kBlockK - 1) / kBlockK;
     s.R_pad = q->R_pad;
   }
-  pb.steal = tiles > p0->sms / 2 ? 1 : 0;
   {
     ProfScope ps(p0, 2, stream);
     CUDA_TRY(launch_shrink_tiles(sb, p0->sms, pdl_shrink, stream));
   }
   {
     ProfScope ps(p0, 3, stream);
-    CUDA_TRY(launch_pair_gemm(pb, pdl_base, stream));
+    CUDA_TRY(launch_pair_gemm(pb, p0->sms, pdl_base, stream));
   }
   for (int i = 0; i < n; ++i) {
     int64_t *info = sites[i].p->last_info;

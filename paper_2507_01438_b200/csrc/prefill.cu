@@ -93,11 +93,13 @@ __device__ __forceinline__ Tile tile_at(const Batch &b, int32_t tile, int32_t &s
 // What every role does between two tiles: the answer of the launch queue is read and handed back to the thread
 // that asks (`nempty`: its barrier's cluster address), by whole warps (kWarp: one arrival per warp) or by single
 // threads.  `tile` becomes the next tile, -1 when none is left.  Returns false when the wait ran out.
-template <bool kWarp>
-__device__ __forceinline__ bool next_tile(Barriers &sh, int32_t it, uint32_t nempty, int32_t steal, long long wl,
+// Without kSteal the tiles are dealt round-robin to the pairs of the grid.
+template <bool kWarp, bool kSteal>
+__device__ __forceinline__ bool next_tile(Barriers &sh, int32_t it, uint32_t nempty, int32_t n_tiles, long long wl,
                                           int32_t &tile) {
-  if (!steal) {
-    tile = -1;
+  if (!kSteal) {
+    tile += static_cast<int32_t>(gridDim.x >> 1);
+    if (tile >= n_tiles) tile = -1;
     return true;
   }
   const bool got = ptx::mbar_wait_cluster(&sh.nfull, it & 1, wl);
@@ -112,7 +114,7 @@ constexpr int kAnswerReaders = 10 + 9;  // TMA, MMA, 4 epilogue and 4 builder wa
 
 }  // namespace
 
-template <int kSites>
+template <int kSites, bool kSteal>
 __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_constant__ PairBatch<kSites> b) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -124,7 +126,7 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = ptx::cluster_rank();
   const bool leader = rank == 0;
-  const int32_t tile0 = static_cast<int32_t>(blockIdx.x >> 1);
+  const int32_t tile0 = static_cast<int32_t>(blockIdx.x >> 1), n_tiles = b.site[b.n_sites - 1].tile_end;
   const long long wl = b.wait_cycles;
 
   if (threadIdx.x == 0) {
@@ -190,7 +192,7 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
             ok = false;
             break;
           }
-          if (!leader && kb == kb_ask) ptx::mbar_arrive(&sh.ask);
+          if (kSteal && !leader && kb == kb_ask) ptx::mbar_arrive(&sh.ask);
           uint8_t *sr = smem + static_cast<size_t>(stage) * stage_bytes;
           const uint32_t bar = full0 + stage * 8;
           if (leader) ptx::mbar_arrive_expect_tx(&sh.full[stage], 2 * (kXBytes + w_bytes));
@@ -221,7 +223,7 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
         }
         if (!ok) break;
         ptx::mbar_arrive(&sh.lempty[buf]);
-        ok = next_tile<false>(sh, it, nempty1, b.steal, wl, tile);
+        ok = next_tile<false, kSteal>(sh, it, nempty1, n_tiles, wl, tile);
         if (!ok) break;
       }
       // the commits that hand the last stages back arrive in this CTA's shared memory: wait for them
@@ -287,14 +289,14 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
         if (!ok) break;
         ptx::mbar_arrive(&sh.lempty[buf]);
         ptx::umma_commit_pair(&sh.tfull[acc]);  // accumulator complete
-        ok = next_tile<false>(sh, it, nempty1, b.steal, wl, tile);
+        ok = next_tile<false, kSteal>(sh, it, nempty1, n_tiles, wl, tile);
         if (!ok) break;
       }
-    } else if (!leader && b.steal && ptx::elect_one()) {
+    } else if (kSteal && !leader && ptx::elect_one()) {
       // The pair's requests to the launch queue, one tile ahead: asked once every role has read the answer before,
-      // and not before the loads of the tile at hand are nearly through.  (At the start of a launch that begins
-      // under the one before it, clusters still wait for their SMs; taking those tiles at once left the SMs
-      // that came free a moment later without work: 47.8 against 37.5 us on 4096 -> 4096, T = 300.)
+      // and not before the loads of the tile at hand are nearly through (at the start of a launch clusters still
+      // wait for their SMs; taking those tiles at once would leave the SMs that come free a moment later without
+      // work).
       const uint32_t nfull0 = ptx::map_to_rank(ptx::smem_u32(&sh.nfull), 0);
       for (int32_t it = 0;; ++it) {
         if (!ptx::mbar_wait(&sh.ask, it & 1, wl) ||
@@ -365,7 +367,7 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
         }
         __syncwarp();
       }
-      ok = __all_sync(0xffffffffu, next_tile<true>(sh, it, nempty1, b.steal, wl, tile));
+      ok = __all_sync(0xffffffffu, next_tile<true, kSteal>(sh, it, nempty1, n_tiles, wl, tile));
       if (!ok) break;
     }
   } else {
@@ -448,7 +450,7 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive_cluster(zfull0 + stage * 8);
       }
-      const bool got = next_tile<true>(sh, it, nempty1, b.steal, wl, tile);
+      const bool got = next_tile<true, kSteal>(sh, it, nempty1, n_tiles, wl, tile);
       if (named_bar_any(2, 128, !ok || !got)) {
         ok = false;
         break;
@@ -478,18 +480,30 @@ int pair_stages(int BN) {
 
 cudaError_t pair_set_smem_limit() {
   const int bytes = static_cast<int>(kPairSmemBudget);
-  cudaError_t e = cudaFuncSetAttribute(pair_gemm_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(pair_gemm_kernel<kPairSites>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  cudaError_t e = cudaSuccess;
+#define EDGELORA_SMEM(N, ST)                                                                                      \
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(pair_gemm_kernel<N, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  EDGELORA_SMEM(1, false)
+  EDGELORA_SMEM(1, true)
+  EDGELORA_SMEM(kPairSites, false)
+  EDGELORA_SMEM(kPairSites, true)
+#undef EDGELORA_SMEM
   return e;
 }
 
+// Tiles come off the launch queue when the pairs run through more than four waves of them; shorter launches have
+// no time to drift, and a kernel that uses the launch queue does not start under the tail of the kernel in front
+// of it (4096 -> 4096, T = 300: 46 us per call against 37.5 us; 3080 -> 5000, T = 1111: 88 against 82 us).
 template <int kSites>
-cudaError_t launch_pair_gemm(const PairBatch<kSites> &b, bool pdl, cudaStream_t stream) {
-  return launch_ex(pair_gemm_kernel<kSites>, dim3(2 * b.site[b.n_sites - 1].tile_end), dim3(kThreads), pair_smem_bytes(b.stages, b.BN), stream, pdl,
-                   2, b);
+cudaError_t launch_pair_gemm(const PairBatch<kSites> &b, int32_t sms, bool pdl, cudaStream_t stream) {
+  const int32_t tiles = b.site[b.n_sites - 1].tile_end, units = std::max(1, sms / 2);
+  const size_t smem = pair_smem_bytes(b.stages, b.BN);
+  if (tiles > 4 * units)
+    return launch_ex(pair_gemm_kernel<kSites, true>, dim3(2 * tiles), dim3(kThreads), smem, stream, pdl, 2, b);
+  return launch_ex(pair_gemm_kernel<kSites, false>, dim3(2 * std::min(tiles, units)), dim3(kThreads), smem, stream, pdl, 2,
+                   b);
 }
-template cudaError_t launch_pair_gemm<1>(const PairBatch<1> &, bool, cudaStream_t);
-template cudaError_t launch_pair_gemm<kPairSites>(const PairBatch<kPairSites> &, bool, cudaStream_t);
+template cudaError_t launch_pair_gemm<1>(const PairBatch<1> &, int32_t, bool, cudaStream_t);
+template cudaError_t launch_pair_gemm<kPairSites>(const PairBatch<kPairSites> &, int32_t, bool, cudaStream_t);
 
 }  // namespace edgelora

@@ -31,7 +31,6 @@ struct PairBatch {
   int32_t n_sites, T, n_slots;
   int32_t BN;        // W rows of a tile, a multiple of 32 up to 256
   int32_t stages, n_mtiles;
-  int32_t steal;     // 1: more tiles than pairs fit the device, so pairs take further tiles off the launch queue
   const int32_t *ids_valid, *mt_count, *mt_list;  // of the plan all sites share
   long long wait_cycles;
 };
@@ -39,6 +38,6 @@ struct PairBatch {
 int pair_stages(int BN);
 cudaError_t pair_set_smem_limit();
 template <int kSites>
-cudaError_t launch_pair_gemm(const PairBatch<kSites> &b, bool pdl, cudaStream_t stream);
+cudaError_t launch_pair_gemm(const PairBatch<kSites> &b, int32_t sms, bool pdl, cudaStream_t stream);
 
 }  // namespace edgelora

@@ -447,28 +447,53 @@ __global__ void __launch_bounds__(kThreads, 1) shrink_tiles_kernel(const __grid_
       if (!(ok = ep_sync())) break;
       if (sh.last) {
         __threadfence();
-        const int nch = R >> 3, n_tok = tc.gather ? tc.ntok : tc.nrows;
-        for (int i = etid; i < n_tok * nch; i += 128) {
-          const int k = i / nch, c = i - k * nch;
-          int32_t t = tc.gather ? b.perm_short[tc.tok0 + k] : tc.row + k;
-          if (!EL_CHECK(st.status, t >= 0 && t < b.T, 7)) continue;
-          const int32_t rank = st.slots[tc.gather ? b.ids_valid[t] : tc.slot].rank;
-          if (rank <= 0) continue;  // nothing loaded: nobody reads this z
-          const size_t off = static_cast<size_t>(t) * R + c * 8;
-          float *out = st.zws + static_cast<size_t>(kMaxZSplits) * plane;
-          if (b.z_bf16) {
-            reinterpret_cast<uint4 *>(out)[static_cast<size_t>(t) * nch + c] =
-                z_chunk(st.zws + off, plane, tc.splits, c * 8, rank);
-          } else {
-            float4 u = make_float4(0.f, 0.f, 0.f, 0.f), w = u;
-            for (int32_t sp = 0; sp < tc.splits; ++sp) {
-              const float4 *zp = reinterpret_cast<const float4 *>(st.zws + sp * plane + off);
-              const float4 p = __ldcg(zp), q = __ldcg(zp + 1);
-              u.x += p.x; u.y += p.y; u.z += p.z; u.w += p.w;
-              w.x += q.x; w.y += q.y; w.z += q.z; w.w += q.w;
+        // Four chunks of eight values per thread and round, their loads of a plane in flight together: with one
+        // chunk at a time the sum of seven planes of 128 x 64 took 20 us.
+        const int nch = R >> 3, n_chunks = (tc.gather ? tc.ntok : tc.nrows) * nch;
+        float *out = st.zws + static_cast<size_t>(kMaxZSplits) * plane;
+        for (int i0 = etid; i0 < n_chunks; i0 += 4 * 128) {
+          int32_t tok[4], rank[4];
+          float acc[4][8];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int i = i0 + q * 128, k = i / nch;
+            tok[q] = i < n_chunks ? (tc.gather ? b.perm_short[tc.tok0 + k] : tc.row + k) : -1;
+            if (!EL_CHECK(st.status, tok[q] < b.T, 7)) tok[q] = -1;
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            rank[q] = 0;  // nothing loaded: nobody reads this z
+            if (tok[q] >= 0) rank[q] = st.slots[tc.gather ? b.ids_valid[tok[q]] : tc.slot].rank;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[q][e] = 0.f;
+          }
+#pragma unroll 2
+          for (int32_t sp = 0; sp < tc.splits; ++sp) {
+            float4 u[4], w[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const int c = (i0 + q * 128) % nch;
+              const float4 *zp = reinterpret_cast<const float4 *>(st.zws + sp * plane + static_cast<size_t>(max(tok[q], 0)) * R + c * 8);
+              u[q] = tok[q] >= 0 ? __ldcg(zp) : make_float4(0.f, 0.f, 0.f, 0.f);
+              w[q] = tok[q] >= 0 ? __ldcg(zp + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
-            *reinterpret_cast<float4 *>(out + off) = u;
-            *reinterpret_cast<float4 *>(out + off + 4) = w;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              acc[q][0] += u[q].x; acc[q][1] += u[q].y; acc[q][2] += u[q].z; acc[q][3] += u[q].w;
+              acc[q][4] += w[q].x; acc[q][5] += w[q].y; acc[q][6] += w[q].z; acc[q][7] += w[q].w;
+            }
+          }
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if (rank[q] <= 0) continue;
+            const int c = (i0 + q * 128) % nch;
+            if (b.z_bf16) {
+              reinterpret_cast<uint4 *>(out)[static_cast<size_t>(tok[q]) * nch + c] = pack_z_chunk(acc[q], c * 8, rank[q]);
+            } else {
+              float4 *o = reinterpret_cast<float4 *>(out + static_cast<size_t>(tok[q]) * R + c * 8);
+              o[0] = make_float4(acc[q][0], acc[q][1], acc[q][2], acc[q][3]);
+              o[1] = make_float4(acc[q][4], acc[q][5], acc[q][6], acc[q][7]);
+            }
           }
         }
       }
