@@ -141,8 +141,9 @@ def _check(rc: int, what: str) -> None:
 
 def _stream_ptr(stream) -> int:
     if stream is None:
+        # the handle of torch.cuda.current_stream(), without the Stream object around it (0.2 us against 3.4 us)
         import torch
-        stream = torch.cuda.current_stream()
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     return int(stream.cuda_stream) if hasattr(stream, "cuda_stream") else int(stream)
 
 
@@ -203,10 +204,11 @@ def edgelora_pool_wait_loads(pool) -> None:
 def edgelora_lora_linear(pool, W, x, adapter_id, y, stream=None) -> None:
     """W [h_out,h_in], x [T,h_in], y [T,h_out]: torch bf16 CUDA tensors; adapter_id: int32 [T]."""
     T = int(x.shape[0])
-    _check(lib().edgelora_lora_linear(pool, _dev_ptr(W, 2, "W"), _dev_ptr(x, 2, "x") if T else None,
-                                      _dev_ptr(adapter_id, 4, "ids") if T else None, T,
-                                      _dev_ptr(y, 2, "y") if T else None, _stream_ptr(stream)),
-           "lora_linear")
+    rc = (_lib or lib()).edgelora_lora_linear(pool, _dev_ptr(W, 2, "W"), _dev_ptr(x, 2, "x") if T else None,
+                                              _dev_ptr(adapter_id, 4, "ids") if T else None, T,
+                                              _dev_ptr(y, 2, "y") if T else None, _stream_ptr(stream))
+    if rc != OK:
+        raise EdgeLoraError(rc, "lora_linear")
 
 
 def edgelora_lora_linear_planned(pool, plan, W, x, y, stream=None) -> None:
