@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -812,20 +813,25 @@ static void fill_shrink_plan(const edgelora_plan *plan, int32_t T, long long wai
   b->wait_cycles = wait_cycles;
 }
 
-// K splits of a site's shrink tiles.  A single site is split until every SM has an item; in a run of sites the
-// items of all sites share the grid, and items of about 32 K blocks keep a wide input from making long ones.
+// K splits of a site's shrink tiles.  A single site is split until every SM has an item, but not further than the
+// sum of the planes at the end of a tile (1.6 us per plane of 128 x 64) gains over the K blocks (0.25 us each): the
+// sum of both is least near sqrt(10 kb / R).  In a run of sites the items of all sites share the grid, and items
+// of about 32 K blocks keep a wide input from making long ones.
 static int shrink_splits(const edgelora_pool *q, int32_t T, int n_sites) {
   if (T <= kDecodeMaxT) return 1;
   const int kbt = (q->cfg.h_in + kBlockK - 1) / kBlockK;
   int z = n_sites > 1 ? std::min(8, std::max(1, kbt / 32)) : std::min(8, q->sms / std::max(1, T / kTileM));
+  if (n_sites == 1) z = std::min(z, static_cast<int>(std::sqrt(10.0 * kbt / q->R_pad) + 0.5));
   z = std::max(1, std::min(z, kbt / 4));
   const int kb_per = (kbt + z - 1) / z;
   return (kbt + kb_per - 1) / kb_per;
 }
 
-// W rows of a pair tile.  A K block of a tile takes about max(2 BN + 60, 390) cycles (2 BN is the tensor pipe's
-// share; below BN = 160 the hand-over of a K block sets the pace: 385 cycles measured at BN = 64), so the width
-// whose last wave is fullest for the width's efficiency is taken; the sites' tiles form one list over all pairs.
+// W rows of a pair tile.  A K block of a tile takes about 2 BN + 140 cycles (2 BN is the tensor pipe's share),
+// below BN = 160 about 480 (the hand-over of a K block sets the pace), so the width whose last wave is fullest for
+// the width's efficiency is taken; the sites' tiles form one list over all pairs.  Measured per call:
+// 14336 -> 4096, T = 4096: 367 us at 256, 381 at 192; 4096 -> 4096, T = 300: 32 us at 160, 37 at 128 and 256;
+// 3080 -> 5000, T = 1111: 68 us at 192, 72 at 256, 80 at 128.
 static int pair_width(const SiteCall *sites, int n, int n_mtiles, int units) {
   int best = 0;
   double best_cost = 0;
@@ -843,7 +849,7 @@ static int pair_width(const SiteCall *sites, int n, int n_mtiles, int units) {
     const double waves = static_cast<double>((tiles + units - 1) / units);
     // one site: whole waves; several: the list's total, and half a tile for its ragged end
     const double k = n == 1 ? waves * kb_max : std::max(work / units + 0.5 * kb_max, static_cast<double>(kb_max));
-    const double cost = k * std::max(2 * BN + 60, 390) + 12.0 * BN;  // + the last tile's epilogue
+    const double cost = k * (BN >= 160 ? 2 * BN + 140 : 480) + 12.0 * BN;  // + the last tile's epilogue
     if (best == 0 || cost < best_cost) {
       best = BN;
       best_cost = cost;

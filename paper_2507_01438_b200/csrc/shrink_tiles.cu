@@ -136,10 +136,9 @@ __device__ __forceinline__ int32_t passes_of(const Item &c) {
 
 // The copies of one pass over a gather tile, K blocks [kb0, kb1).  A K block needs one copy per
 // group of the tile (its A block, R_pad rows of the R operand) and one per token quad (four rows of
-// x into the C operand).  A warp issues its lanes' TMA copies one after the other at roughly a hundred
-// cycles each, so the copies of a K block are dealt out to kGatherParts warps (the producer warp is
+// x into the C operand).  The copies of a K block are dealt out to kGatherParts warps (the producer warp is
 // part 0 and also posts the byte count; the four helper warps are parts 1..4): copy i goes to part
-// i % kGatherParts, lane i / kGatherParts.
+// i % kGatherParts, looked up by lane i / kGatherParts.
 // The parts other than the producer follow it: the producer announces a free stage on the stage's
 // "go" barrier, every other part waits for that, issues its copies and arrives on the stage's
 // "z full" barrier, which the MMA warp waits for beside the byte count.  (Waiting on the stage's
@@ -147,6 +146,7 @@ __device__ __forceinline__ int32_t passes_of(const Item &c) {
 // ring revolutions ahead, and a parity wait cannot tell revolutions apart.)  A copy that lands before
 // the byte count is posted only drives the barrier's transaction count below zero for a moment.
 constexpr int kGatherParts = 5;
+constexpr int kGatherItems = (kTileM / 16 + kTileGatherN / 4 + kGatherParts - 1) / kGatherParts;  // copies of a part
 template <typename Batch>
 __device__ __forceinline__ bool gather_pass_copies(const Batch &b, const ShrinkSite &st, const Item &tc, int32_t t0,
                                                    uint8_t *smem, Barriers &sh, int part, int lane, uint32_t &stage,
@@ -177,37 +177,53 @@ __device__ __forceinline__ bool gather_pass_copies(const Batch &b, const ShrinkS
       if (!EL_CHECK(st.status, tok[i] >= 0 && tok[i] < b.T, 5)) tok[i] = 0;
     }
   }
-  for (int32_t kb = tc.kb0; kb < tc.kb1; ++kb) {
-    int got = 1;
-    if (lane == 0) {
-      if (part == 0)
-        got = (ptx::mbar_wait(&sh.empty[stage], phase ^ 1, b.wait_cycles) && !sh.abort_flag) ? 1 : 0;
-      else
-        got = (ptx::mbar_wait(&sh.zgo[stage], (gophase >> stage) & 1u, b.wait_cycles) && !sh.abort_flag) ? 1 : 0;
-    }
-    if (!__shfl_sync(0xffffffffu, got, 0)) return false;
-    gophase ^= 1u << stage;
-    uint8_t *sr = smem + static_cast<size_t>(stage) * kStageBytes;
-    if (part == 0 && lane == 0) {
-      ptx::mbar_arrive(&sh.zgo[stage]);
-      ptx::mbar_arrive_expect_tx(&sh.full[stage], tx);
-    }
-    if (my_slot >= 0)
-      ptx::tma_load_2d(sr + static_cast<size_t>(item) * a_bytes, &st.a, &sh.full[stage], kb * kBlockK,
-                       my_slot * st.R_pad);
-    if (my_quad >= 0)
-      ptx::tma_gather4_2d(sr + kRBytes + static_cast<size_t>(my_quad) * (4 * kBlockK * 2), mg, &sh.full[stage],
-                          kb * kBlockK, tok[0], tok[1], tok[2], tok[3]);
-    if (part != 0) {
-      __syncwarp();
-      if (lane == 0) ptx::mbar_arrive(&sh.zfull[stage]);
-    }
-    if (++stage == kTileStages) {
-      stage = 0;
-      phase ^= 1;
+  // One thread walks the K blocks and issues all of the part's copies (lane after lane, a warp-wide issue cost a
+  // hundred cycles per copy): it takes over what the lanes have looked up.
+  int32_t slot_j[kGatherItems], quad_j[kGatherItems], tok_j[kGatherItems][4];
+#pragma unroll
+  for (int j = 0; j < kGatherItems; ++j) {
+    slot_j[j] = __shfl_sync(0xffffffffu, my_slot, j);
+    quad_j[j] = __shfl_sync(0xffffffffu, my_quad, j);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) tok_j[j][i] = __shfl_sync(0xffffffffu, tok[i], j);
+  }
+  const bool issuer = ptx::elect_one() != 0;
+  const int src = __ffs(__ballot_sync(0xffffffffu, issuer)) - 1;
+  int good = 1;
+  if (issuer) {
+    for (int32_t kb = tc.kb0; kb < tc.kb1; ++kb) {
+      const bool got = part == 0 ? ptx::mbar_wait(&sh.empty[stage], phase ^ 1, b.wait_cycles)
+                                 : ptx::mbar_wait(&sh.zgo[stage], (gophase >> stage) & 1u, b.wait_cycles);
+      if (!got || sh.abort_flag) {
+        good = 0;
+        break;
+      }
+      gophase ^= 1u << stage;
+      uint8_t *sr = smem + static_cast<size_t>(stage) * kStageBytes;
+      if (part == 0) {
+        ptx::mbar_arrive(&sh.zgo[stage]);
+        ptx::mbar_arrive_expect_tx(&sh.full[stage], tx);
+      }
+#pragma unroll
+      for (int j = 0; j < kGatherItems; ++j) {
+        if (slot_j[j] >= 0)
+          ptx::tma_load_2d(sr + static_cast<size_t>(part + kGatherParts * j) * a_bytes, &st.a, &sh.full[stage],
+                           kb * kBlockK, slot_j[j] * st.R_pad);
+        if (quad_j[j] >= 0)
+          ptx::tma_gather4_2d(sr + kRBytes + static_cast<size_t>(quad_j[j]) * (4 * kBlockK * 2), mg, &sh.full[stage],
+                              kb * kBlockK, tok_j[j][0], tok_j[j][1], tok_j[j][2], tok_j[j][3]);
+      }
+      if (part != 0) ptx::mbar_arrive(&sh.zfull[stage]);
+      if (++stage == kTileStages) {
+        stage = 0;
+        phase ^= 1;
+      }
     }
   }
-  return true;
+  stage = __shfl_sync(0xffffffffu, stage, src);
+  phase = __shfl_sync(0xffffffffu, phase, src);
+  gophase = __shfl_sync(0xffffffffu, gophase, src);
+  return __shfl_sync(0xffffffffu, good, src) != 0;
 }
 
 }  // namespace
