@@ -236,9 +236,8 @@ int edgelora_plan_sync_status(edgelora_plan_t *plan, void *stream, uint32_t *bit
  * (pools[i], W_dev[i]) and reads input number input_of_site[i] (sites with the same input width
  * may share an input, e.g. q/k/v/o/gate/up of a decoder layer); all pools have the same n_slots
  * and max_tokens >= the set's.  A run builds ONE routing plan from the ids and evaluates the sites
- * in order; the sites are independent given their inputs, so in batches above 256 tokens the
- * shrink of site i + 1 is issued with the kernels of site i and only the first site's shrink stands
- * alone.  The set borrows the pools and W (the caller keeps them alive) and owns its plan and the
+ * in order; the sites are independent given their inputs, so in batches above 256 tokens runs of up
+ * to 32 sites share one shrink launch and one base-product launch.  The set borrows the pools and W (the caller keeps them alive) and owns its plan and the
  * device mirrors of the host-buffer call.  One thread at a time per set; runs of one set (and of
  * its pools) must not overlap on the GPU. */
 typedef struct edgelora_siteset edgelora_siteset_t;

@@ -44,6 +44,11 @@ bool capturing(cudaStream_t s) {
   return st != cudaStreamCaptureStatusNone;
 }
 
+bool overlap(const void *a, size_t na, const void *b, size_t nb) {
+  const uintptr_t pa = reinterpret_cast<uintptr_t>(a), pb = reinterpret_cast<uintptr_t>(b);
+  return pa < pb + nb && pb < pa + na;
+}
+
 // after: optional, one event per site (or null): recorded on the stream behind that site's launch.
 // before: optional, one event per site (or null): the stream waits for it in front of that site's launch.
 int run_sites(edgelora_siteset *s, const void *const *x_dev, const int32_t *ids_dev, int32_t T,
@@ -57,12 +62,20 @@ int run_sites(edgelora_siteset *s, const void *const *x_dev, const int32_t *ids_
   // launch, when every pool runs in its default configuration.
   bool runs = T > kDecodeMaxT;
   for (auto *p : s->pools) runs = runs && p->opt_regime == 0 && p->opt_pdl >= 1 && !p->a_q8;
+  // A result that lies in an input's memory is written in the order of the sites: one by one, nothing overlapped.
+  const size_t row = static_cast<size_t>(T) * 2;
+  bool chained = false;
+  for (int k = 0; runs && k < s->n_inputs; ++k)
+    for (int i = 0; s->in_width[k] && i < n; ++i)
+      chained = chained || overlap(x_dev[k], row * s->in_width[k], y_dev[i], row * s->pools[i]->cfg.h_out);
+  runs = runs && !chained;
   if (!runs) {
     for (int i = 0; i < n; ++i) {
       if (before && (*before)[i] && cudaStreamWaitEvent(stream, (*before)[i], 0) != cudaSuccess) return EDGELORA_ERR_CUDA;
       // (decode-sized batches: the sites are independent given their inputs and results, so a
       // site's shrink may start under the previous site's base product)
-      rc = lora_linear_impl(s->pools[i], s->plan, nullptr, s->W[i], x_dev[s->input_of[i]], T, y_dev[i], stream, i > 0);
+      rc = lora_linear_impl(s->pools[i], s->plan, nullptr, s->W[i], x_dev[s->input_of[i]], T, y_dev[i], stream,
+                            i > 0 && !chained);
       if (rc != EDGELORA_OK) return rc;
       if (after && (*after)[i] && cudaEventRecord((*after)[i], stream) != cudaSuccess) return EDGELORA_ERR_CUDA;
     }
@@ -77,7 +90,8 @@ int run_sites(edgelora_siteset *s, const void *const *x_dev, const int32_t *ids_
   }
   for (int i0 = 0; i0 < n;) {
     // A run ends where the launch's tables are full, where a pool would come twice (its z workspace holds one
-    // site's z), in front of a site whose input is still on its way, and behind about a decoder layer of
+    // site's z), where two sites write the same memory (the later one is to be seen; results that the host call
+    // does not read back share a buffer nobody looks at), in front of a site whose input is still on its way, and behind about a decoder layer of
     // sites when results are read back beside the sites that follow.  Profiled pools go one by one.
     SiteCall calls[kPairSites];
     const uint16_t *inputs[kPairInputs];
@@ -88,7 +102,10 @@ int run_sites(edgelora_siteset *s, const void *const *x_dev, const int32_t *ids_
       const uint16_t *x = static_cast<const uint16_t *>(x_dev[s->input_of[i]]);
       if (m > 0 && ((before && (*before)[i]) || p->opt_profile || calls[0].p->opt_profile || (read_back && m >= 7))) break;
       bool again = false;
-      for (int k = 0; k < m; ++k) again = again || calls[k].p == p;
+      for (int k = 0; k < m; ++k)
+        again = again || calls[k].p == p ||
+                (!(after && !(*after)[i] && !(*after)[i0 + k]) &&
+                 overlap(y_dev[i], row * p->cfg.h_out, calls[k].y, row * calls[k].p->cfg.h_out));
       if (again) break;
       int xi = 0;
       while (xi < n_inputs && inputs[xi] != x) ++xi;

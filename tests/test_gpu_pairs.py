@@ -74,3 +74,31 @@ def test_one_pool_at_two_sites_of_a_set():
     finally:
         B.edgelora_siteset_destroy(s)
         pool.close()
+
+
+@pytest.mark.parametrize("what", ["results", "input"])
+def test_sites_of_a_set_that_share_memory(what):
+    # two sites with one result buffer: the later one is seen; a result in an input's memory: the sites in order
+    import torch
+    ids = mixed_ids(8, 20, [(0, 300)], 3)
+    T = len(ids)
+    _, sites = make_sites(13, T, [(128, 128)] * 3, [16, 8, 4], 16, ids)
+    pools = [make_pool(w) for w in sites]
+    Ws = [to_dev_bf16(w.W) for w in sites]
+    second = 1 if what == "input" else 0
+    s = B.edgelora_siteset_create([p.handle for p in pools], Ws, [0, 0, second], 2, T)
+    try:
+        x = to_dev_bf16(sites[0].x)
+        y = [torch.empty((T, 128), dtype=torch.bfloat16, device="cuda") for _ in range(3)]
+        if what == "results":
+            y[2] = y[0]
+        B.edgelora_siteset_run(s, [x, y[0]], torch.from_numpy(ids).cuda(), y)
+        if what == "input":
+            sites[2].x = y[0].view(torch.int16).cpu().numpy().view(np.uint16)
+        for i in ([1, 2] if what == "results" else [0, 1, 2]):
+            assert_parity(from_dev_bf16(y[i]), oracle_of(sites[i]), sites[i].name)
+        assert all(p.status() == (0, 0) for p in pools)
+    finally:
+        B.edgelora_siteset_destroy(s)
+        for p in pools:
+            p.close()
