@@ -645,8 +645,7 @@ def bench_full_set(ctx, steps=None, warmup=None, cpu_budget=12.0, layers=wl.LLAM
     widths = (4096, 14336)
     xs = [to_bf16(batch.x4096), to_bf16(batch.x14336)]
     ids = torch.from_numpy(batch.ids).cuda()
-    ybuf = {h: torch.empty((T, h), dtype=torch.bfloat16, device="cuda") for h in (1024, 4096, 14336)}
-    ys = [ybuf[s[2]] for s in sites]
+    ys = [torch.empty((T, s[2]), dtype=torch.bfloat16, device="cuda") for s in sites]
     sset = B.edgelora_siteset_create([s[4].handle for s in sites], [s[3] for s in sites],
                                      [widths.index(s[1]) for s in sites], 2, T)
     stream = torch.cuda.Stream()
@@ -784,7 +783,7 @@ def bench_full_set(ctx, steps=None, warmup=None, cpu_budget=12.0, layers=wl.LLAM
     B.edgelora_siteset_destroy(sset)
     for s in sites:
         s[4].close()
-    del sites, xs, ys, ybuf
+    del sites, xs, ys
     torch.cuda.empty_cache()
     return res
 
@@ -817,7 +816,7 @@ def bench_serving(ctx, layers=wl.LLAMA8B_LAYERS):
         sites.append((sname, h_in, h_out, W, pool))
     widths = (4096, 14336)
     xs = [(torch.randn((max_tokens, w_), generator=gen, device="cuda", dtype=torch.float32)).to(torch.bfloat16) for w_ in widths]
-    ybuf = {h: torch.empty((max_tokens, h), dtype=torch.bfloat16, device="cuda") for h in (1024, 4096, 14336)}
+    ybuf = [torch.empty((max_tokens, s[2]), dtype=torch.bfloat16, device="cuda") for s in sites]
     sset = B.edgelora_siteset_create([s[4].handle for s in sites], [s[3] for s in sites],
                                      [widths.index(s[1]) for s in sites], 2, max_tokens)
     cache = B.edgelora_cache_create(n_blocks)
@@ -854,7 +853,7 @@ def bench_serving(ctx, layers=wl.LLAMA8B_LAYERS):
         with torch.cuda.stream(stream):
             ids_dev[:T].copy_(ids_host[:T], non_blocking=True)
             e0.record(stream)
-            B.edgelora_siteset_run(sset, [x[:T] for x in xs], ids_dev[:T], [ybuf[s[2]][:T] for s in sites], stream)
+            B.edgelora_siteset_run(sset, [x[:T] for x in xs], ids_dev[:T], [y[:T] for y in ybuf], stream)
             e1.record(stream)
         stream.synchronize()
         ms = e0.elapsed_time(e1)
