@@ -101,7 +101,8 @@ __device__ __forceinline__ void list_tiles(const int32_t *valid, int32_t T, cons
 // worked out in shared memory with one thread per run.  The general form below keeps its intermediate arrays
 // in global memory and goes through them in about thirty barrier-separated passes, each a round trip to L2;
 // here the runs are ordered by counting smaller keys instead of by a sorting network, and the four prefix sums
-// over the runs are one scan of four packed 16-bit fields.
+// over the runs are one scan of four packed 16-bit fields (8 runs in 4096 tokens: 8.5 us against 13; 64 decode tokens
+// and two runs: 11 against 18).
 constexpr int kPlanSmallT = 4096;
 constexpr int kPlanTok = kPlanSmallT / kPlanThreads;  // tokens per thread, consecutive
 struct PlanSmall {
