@@ -877,14 +877,14 @@ static int prefill_batch(const SiteCall *sites, int n, edgelora_plan *plan, int3
   pb.mt_count = plan->pv.mt_count;
   pb.mt_list = plan->pv.mt_list;
   pb.wait_cycles = p0->wait_cycles;
-  const uint16_t *inputs[kPairInputs] = {};
+  const SiteCall *inputs[kPairInputs] = {};  // the first site on each input
   int n_inputs = 0, tiles = 0;
   for (int i = 0; i < n; ++i) {
     edgelora_pool *q = sites[i].p;
     int xi = 0;
-    while (xi < n_inputs && inputs[xi] != sites[i].x) ++xi;
+    while (xi < n_inputs && !inputs[xi]->same_input(sites[i])) ++xi;
     if (xi == n_inputs) {
-      inputs[n_inputs++] = sites[i].x;
+      inputs[n_inputs++] = &sites[i];
       const int rc = fill_shrink_inputs(q, sites[i].x, T, &sb.x[xi], &sb.xg[xi]);
       if (rc) return rc;
       pb.x[xi] = sb.x[xi];

@@ -113,6 +113,8 @@ struct SiteCall {
   const void *W;
   const uint16_t *x;
   void *y;
+  // Two inputs of a set may lie at one address and still be read in rows of different widths.
+  bool same_input(const SiteCall &o) const { return x == o.x && p->cfg.h_in == o.p->cfg.h_in; }
 };
 
 // The layer (see pool.cu).  `independent`: the call reads nothing the previous call on the stream

@@ -94,12 +94,12 @@ int run_sites(edgelora_siteset *s, const void *const *x_dev, const int32_t *ids_
     // does not read back share a buffer nobody looks at), in front of a site whose input is still on its way, and behind about a decoder layer of
     // sites when results are read back beside the sites that follow.  Profiled pools go one by one.
     SiteCall calls[kPairSites];
-    const uint16_t *inputs[kPairInputs];
+    SiteCall inputs[kPairInputs];  // the first site on each input
     int m = 0, n_inputs = 0;
     bool read_back = false;
     for (int i = i0; i < n && m < kPairSites; ++i) {
       edgelora_pool *p = s->pools[i];
-      const uint16_t *x = static_cast<const uint16_t *>(x_dev[s->input_of[i]]);
+      const SiteCall call{p, s->W[i], static_cast<const uint16_t *>(x_dev[s->input_of[i]]), y_dev[i]};
       if (m > 0 && ((before && (*before)[i]) || p->opt_profile || calls[0].p->opt_profile || (read_back && m >= 7))) break;
       bool again = false;
       for (int k = 0; k < m; ++k)
@@ -108,12 +108,12 @@ int run_sites(edgelora_siteset *s, const void *const *x_dev, const int32_t *ids_
                  overlap(y_dev[i], row * p->cfg.h_out, calls[k].y, row * calls[k].p->cfg.h_out));
       if (again) break;
       int xi = 0;
-      while (xi < n_inputs && inputs[xi] != x) ++xi;
+      while (xi < n_inputs && !inputs[xi].same_input(call)) ++xi;
       if (xi == kPairInputs) break;
-      if (xi == n_inputs) inputs[n_inputs++] = x;
+      if (xi == n_inputs) inputs[n_inputs++] = call;
       if (m == 0 && before && (*before)[i] && cudaStreamWaitEvent(stream, (*before)[i], 0) != cudaSuccess)
         return EDGELORA_ERR_CUDA;
-      calls[m++] = SiteCall{p, s->W[i], x, y_dev[i]};
+      calls[m++] = call;
       read_back = read_back || (after && (*after)[i]);
     }
     // (the kernel in front of a run is the plan kernel, launched behind everything before it, or the base

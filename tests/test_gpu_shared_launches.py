@@ -1,0 +1,60 @@
+"""Sets of sites whose launches are shared, in the forms that the ordinary set tests do not take: inputs of different
+widths at one address.  Against the CPU oracle, element by element.
+"""
+import numpy as np
+import pytest
+
+from paper_2507_01438_b200 import binding as B
+from paper_2507_01438_b200 import workloads as wl
+from helpers import assert_parity, oracle_of
+from gpu_helpers import from_dev_bf16, make_pool, to_dev_bf16
+from test_gpu_siteset import make_sites, mixed_ids
+
+pytestmark = pytest.mark.gpu
+
+
+class SetOf:
+    """Pools, weights and the set of some sites; ``inputs`` gives each site's input number."""
+
+    def __init__(self, sites, inputs, max_tokens=0):
+        import torch
+        self.sites = sites
+        T = sites[0].T
+        self.pools = [make_pool(w, max_tokens or T) for w in sites]
+        self.Ws = [to_dev_bf16(w.W) for w in sites]
+        self.ids = torch.from_numpy(sites[0].ids).cuda()
+        self.ys = [torch.full((T, w.h_out), float("nan"), dtype=torch.bfloat16, device="cuda") for w in sites]
+        self.handle = B.edgelora_siteset_create([p.handle for p in self.pools], self.Ws, inputs, max(inputs) + 1,
+                                                max_tokens or T)
+
+    def __enter__(self):
+        return self
+
+    def __exit__(self, *exc):
+        B.edgelora_siteset_destroy(self.handle)
+        for p in self.pools:
+            p.close()
+
+    def run(self, xs, stream=None):
+        B.edgelora_siteset_run(self.handle, xs, self.ids, self.ys, stream)
+
+    def check(self, what="", rows=None):
+        for p in self.pools:
+            assert p.status() == (0, 0)
+        for w, y in zip(self.sites, self.ys):
+            got = from_dev_bf16(y)
+            assert_parity(got if rows is None else got[rows], oracle_of(w, rows), f"{what} {w.name}")
+
+
+def test_inputs_of_different_widths_at_one_address():
+    # input 0 is [T][128], input 1 the first T * 64 values of the same buffer as [T][64]
+    ids = mixed_ids(21, 20, [(0, 300)], 3)
+    T = len(ids)
+    xs, sites = make_sites(22, T, [(128, 136), (64, 72), (128, 64), (64, 264)], [16, 8, 4], 16, ids)
+    for w in sites:
+        if w.h_in == 64:
+            w.x = np.ascontiguousarray(xs[128].reshape(-1)[:T * 64].reshape(T, 64))
+    with SetOf(sites, [0, 1, 0, 1]) as s:
+        wide = to_dev_bf16(xs[128])
+        s.run([wide, wide.view(-1)[:T * 64].view(T, 64)])
+        s.check()
