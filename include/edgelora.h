@@ -237,9 +237,12 @@ int edgelora_plan_sync_status(edgelora_plan_t *plan, void *stream, uint32_t *bit
  * may share an input, e.g. q/k/v/o/gate/up of a decoder layer); all pools have the same n_slots
  * and max_tokens >= the set's.  A run builds ONE routing plan from the ids and evaluates the sites
  * in order; the sites are independent given their inputs, so in batches above 256 tokens runs of up
- * to 32 sites share one shrink launch and one base-product launch.  The set borrows the pools and W (the caller keeps them alive) and owns its plan and the
- * device mirrors of the host-buffer call.  One thread at a time per set; runs of one set (and of
- * its pools) must not overlap on the GPU. */
+ * to 32 sites share one shrink launch and one base-product launch.  A site's result may lie in the memory of
+ * an input: the sites behind it that read this input read the result (they start when it is written, one
+ * launch per site, also with EDGELORA_OPT_PDL = 2); only a site's own input must not overlap its result.  The set
+ * borrows the pools and W (the caller keeps them alive) and owns its plan and the device mirrors of the
+ * host-buffer call.  One thread at a time per set; runs of one set (and of its pools) must not overlap on
+ * the GPU. */
 typedef struct edgelora_siteset edgelora_siteset_t;
 int edgelora_siteset_create(int32_t n_sites, edgelora_pool_t *const *pools, const void *const *W_dev,
                             const int32_t *input_of_site, int32_t n_inputs, int32_t max_tokens,

@@ -948,7 +948,7 @@ int prefill_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32
 }
 
 int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_dev, const void *W_dev,
-                     const void *x_dev, int32_t T, void *y_dev, cudaStream_t stream, bool independent) {
+                     const void *x_dev, int32_t T, void *y_dev, cudaStream_t stream, Order order) {
   if (!p || !plan || T < 0) return EDGELORA_ERR_INVALID_ARG;
   if (T == 0) return EDGELORA_OK;
   if (!W_dev || !x_dev || !y_dev) return EDGELORA_ERR_INVALID_ARG;
@@ -961,9 +961,10 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
   const int h_in = p->cfg.h_in, h_out = p->cfg.h_out, R = p->R_pad;
   const bool capturing = stream_capturing(stream);
   const bool pdl = p->opt_pdl >= 1 && !p->opt_profile;        // between the kernels of this call
-  // first kernel vs earlier stream work: when the pool's option says so, or when the caller (a set
-  // of sites) knows that this call does not consume what the call before it produces
-  const bool pdl_first = (p->opt_pdl >= 2 || (independent && p->opt_pdl >= 1)) && !p->opt_profile;
+  // first kernel vs earlier stream work (see Order): a set of sites knows whether a call consumes what the calls
+  // before it produce
+  const bool pdl_first = !p->opt_profile && ((order == Order::kPool && p->opt_pdl >= 2) ||
+                                             (order == Order::kIndependent && p->opt_pdl >= 1));
   const uint16_t *x = static_cast<const uint16_t *>(x_dev);
   int launches = 0;
 

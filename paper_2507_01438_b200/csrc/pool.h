@@ -117,10 +117,13 @@ struct SiteCall {
   bool same_input(const SiteCall &o) const { return x == o.x && p->cfg.h_in == o.p->cfg.h_in; }
 };
 
-// The layer (see pool.cu).  `independent`: the call reads nothing the previous call on the stream
-// writes, so its first kernel may start under that call's tail.
+// How a call's first kernel stands to the work in front of it on the stream: as the pool's EDGELORA_OPT_PDL says;
+// under that work's tail (the call reads nothing the call before it writes); or behind it, whatever the option says.
+enum class Order { kPool, kIndependent, kAfter };
+
+// The layer (see pool.cu).
 int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_dev, const void *W_dev,
-                     const void *x_dev, int32_t T, void *y_dev, cudaStream_t stream, bool independent = false);
+                     const void *x_dev, int32_t T, void *y_dev, cudaStream_t stream, Order order = Order::kPool);
 int prefill_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32_t *ids_dev, int32_t T,
                   cudaStream_t stream, bool pdl_first);
 int wait_for_loads(edgelora_pool *p, cudaStream_t stream, bool capturing);

@@ -22,6 +22,7 @@ struct edgelora_siteset {
   std::vector<int32_t> input_of;
   int32_t n_inputs = 0, max_tokens = 0;
   std::vector<int32_t> in_width;          // h_in of every input
+  std::vector<int32_t> first_writer;      // per input, of the call at hand: the first site that writes into its memory
   edgelora_plan *plan = nullptr;
   // host-buffer path (allocated on first use)
   std::vector<uint16_t *> dx;             // [n_inputs] device mirrors of the inputs
@@ -58,24 +59,27 @@ int run_sites(edgelora_siteset *s, const void *const *x_dev, const int32_t *ids_
   if (rc != EDGELORA_OK) return rc;
   const int n = static_cast<int>(s->pools.size());
   const bool in_capture = capturing(stream);
-  // Large batches: the sites go to the device in runs that share one shrink launch and one base-product
-  // launch, when every pool runs in its default configuration.
-  bool runs = T > kDecodeMaxT;
-  for (auto *p : s->pools) runs = runs && p->opt_regime == 0 && p->opt_pdl >= 1 && !p->a_q8;
-  // A result that lies in an input's memory is written in the order of the sites: one by one, nothing overlapped.
+  // A result that lies in an input's memory is seen by the sites behind it: a site that reads such an input starts
+  // when the site in front of it is done (which is when all before that are), whatever overlap the pools allow.
   const size_t row = static_cast<size_t>(T) * 2;
   bool chained = false;
-  for (int k = 0; runs && k < s->n_inputs; ++k)
-    for (int i = 0; s->in_width[k] && i < n; ++i)
-      chained = chained || overlap(x_dev[k], row * s->in_width[k], y_dev[i], row * s->pools[i]->cfg.h_out);
-  runs = runs && !chained;
+  for (int k = 0; k < s->n_inputs; ++k) {
+    int i = 0;
+    while (i < n && !(s->in_width[k] && overlap(x_dev[k], row * s->in_width[k], y_dev[i], row * s->pools[i]->cfg.h_out))) ++i;
+    s->first_writer[k] = i;
+    chained = chained || i < n;
+  }
+  // Large batches: the sites go to the device in runs that share one shrink launch and one base-product
+  // launch, when every pool runs in its default configuration and no result is an input.
+  bool runs = T > kDecodeMaxT && !chained;
+  for (auto *p : s->pools) runs = runs && p->opt_regime == 0 && p->opt_pdl >= 1 && !p->a_q8;
   if (!runs) {
     for (int i = 0; i < n; ++i) {
       if (before && (*before)[i] && cudaStreamWaitEvent(stream, (*before)[i], 0) != cudaSuccess) return EDGELORA_ERR_CUDA;
-      // (decode-sized batches: the sites are independent given their inputs and results, so a
-      // site's shrink may start under the previous site's base product)
-      rc = lora_linear_impl(s->pools[i], s->plan, nullptr, s->W[i], x_dev[s->input_of[i]], T, y_dev[i], stream,
-                            i > 0 && !chained);
+      // (otherwise the sites are independent given their inputs and results, so a site's shrink may start under the
+      // previous site's base product)
+      const Order order = s->first_writer[s->input_of[i]] < i ? Order::kAfter : i > 0 ? Order::kIndependent : Order::kPool;
+      rc = lora_linear_impl(s->pools[i], s->plan, nullptr, s->W[i], x_dev[s->input_of[i]], T, y_dev[i], stream, order);
       if (rc != EDGELORA_OK) return rc;
       if (after && (*after)[i] && cudaEventRecord((*after)[i], stream) != cudaSuccess) return EDGELORA_ERR_CUDA;
     }
@@ -148,6 +152,7 @@ int edgelora_siteset_create(int32_t n_sites, edgelora_pool_t *const *pools, cons
   s->n_inputs = n_inputs;
   s->max_tokens = max_tokens;
   s->in_width.assign(n_inputs, 0);
+  s->first_writer.assign(n_inputs, n_sites);
   for (int i = 0; i < n_sites; ++i) {
     edgelora_pool *p = pools[i];
     const int in = input_of_site[i];

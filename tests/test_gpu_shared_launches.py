@@ -1,5 +1,5 @@
 """Sets of sites whose launches are shared, in the forms that the ordinary set tests do not take: inputs of different
-widths at one address.  Against the CPU oracle, element by element.
+widths at one address, results that are inputs.  Against the CPU oracle, element by element.
 """
 import numpy as np
 import pytest
@@ -58,3 +58,21 @@ def test_inputs_of_different_widths_at_one_address():
         wide = to_dev_bf16(xs[128])
         s.run([wide, wide.view(-1)[:T * 64].view(T, 64)])
         s.check()
+
+
+@pytest.mark.parametrize("options", [{}, {B.OPT_PDL: 2}, {B.OPT_PDL: 0}, {B.OPT_REGIME: 2}])
+@pytest.mark.parametrize("T", [20, 200, 320])
+def test_a_result_that_is_an_input_of_later_sites(T, options):
+    import torch
+    # site 0 streams a wide W and writes into input 1, which sites 1 and 3 read; site 2 does not
+    ids = mixed_ids(23, 20, [(0, T - 20)], 3)
+    xs, sites = make_sites(24, T, [(4096, 256), (256, 264), (4096, 136), (256, 72)], [16, 8, 4], 16, ids)
+    with SetOf(sites, [0, 1, 0, 1]) as s:
+        for p in s.pools:
+            for option, value in options.items():
+                B.edgelora_pool_set_option(p.handle, option, value)
+        for _ in range(3):
+            s.ys[0].fill_(float("nan"))   # a site that reads too early reads these
+            s.run([to_dev_bf16(xs[4096]), s.ys[0]])
+            sites[1].x = sites[3].x = s.ys[0].view(torch.int16).cpu().numpy().view(np.uint16)
+            s.check(f"T={T}")
