@@ -28,6 +28,7 @@
 #include "launch.cuh"
 #include "prefill.h"
 #include "ptx.cuh"
+#include "tile_order.h"
 
 namespace edgelora {
 
@@ -71,24 +72,6 @@ __device__ __forceinline__ bool named_bar_any(int id, int threads, bool v) {
       : "r"(id), "r"(threads), "r"(v ? 1u : 0u)
       : "memory");
   return r != 0;
-}
-
-// The tile of a position of the launch's list: site, token tile, W tile.  Token tiles run fastest, so that
-// neighbouring pairs share a W tile; the first token tile of a column moves with the column, because in a
-// serving batch the first token tile holds the decode tokens (many adapters, many LoRA K blocks) and a
-// fixed order would hand it to the same pairs again and again.
-struct Tile {
-  int32_t s, m, n;
-};
-template <typename Batch>
-__device__ __forceinline__ Tile tile_at(const Batch &b, int32_t tile, int32_t &site) {
-  while (tile >= b.site[site].tile_end) ++site;
-  const int32_t local = tile - (site > 0 ? b.site[site - 1].tile_end : 0);
-  Tile t;
-  t.s = site;
-  t.n = local / b.n_mtiles;
-  t.m = (local + t.n) % b.n_mtiles;
-  return t;
 }
 
 // What every role does between two tiles: the answer of the launch queue is read and handed back to the thread

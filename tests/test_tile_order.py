@@ -1,0 +1,57 @@
+"""The order in which the pair kernel's roles walk a launch's tiles, on the CPU: csrc/tile_order.h is plain C++ and is
+compiled here with the host compiler.
+"""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+SOURCE = r"""
+#include "tile_order.h"
+struct Site { int32_t tile_end; };
+struct Batch { Site site[32]; int32_t n_sites, n_mtiles; };
+extern "C" void walk(int32_t n_sites, const int32_t *tile_end, int32_t n_mtiles, int32_t n, const int32_t *tiles, int32_t *out) {
+  Batch b;
+  b.n_sites = n_sites;
+  b.n_mtiles = n_mtiles;
+  for (int i = 0; i < n_sites; ++i) b.site[i].tile_end = tile_end[i];
+  int32_t site = 0;
+  for (int i = 0; i < n; ++i) {
+    const edgelora::Tile t = edgelora::tile_at(b, tiles[i], site);
+    out[3 * i] = t.s; out[3 * i + 1] = t.m; out[3 * i + 2] = t.n;
+  }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def lib(tmp_path_factory):
+    d = tmp_path_factory.mktemp("tile_order")
+    src, out = d / "t.cpp", d / "t.so"
+    src.write_text(SOURCE)
+    subprocess.run(["g++", "-O1", "-std=c++17", "-fPIC", "-shared", "-I",
+                    os.path.join(ROOT, "paper_2507_01438_b200", "csrc"), str(src), "-o", str(out)], check=True)
+    return ctypes.CDLL(str(out))
+
+
+@pytest.mark.parametrize("n_mtiles,w_tiles", [(1, [3]), (2, [16, 1, 4]), (9, [16, 4, 4, 16, 56, 56, 16]), (3, [1] * 32)])
+@pytest.mark.parametrize("order", ["rising", "falling", "shuffled"])
+def test_every_tile_is_found_in_any_order(lib, n_mtiles, w_tiles, order):
+    # the launch queue promises no order of its answers
+    ends = np.cumsum(np.array(w_tiles) * n_mtiles).astype(np.int32)
+    tiles = np.arange(ends[-1], dtype=np.int32)
+    if order == "falling":
+        tiles = tiles[::-1].copy()
+    elif order == "shuffled":
+        np.random.default_rng(len(w_tiles)).shuffle(tiles)
+    out = np.full((len(tiles), 3), -99, np.int32)
+    ptr = lambda a: a.ctypes.data_as(ctypes.POINTER(ctypes.c_int32))
+    lib.walk(len(ends), ptr(ends), n_mtiles, len(tiles), ptr(tiles), ptr(out))
+    site = np.searchsorted(ends, tiles, side="right")
+    local = tiles - np.concatenate([[0], ends[:-1]])[site]
+    n = local // n_mtiles
+    assert np.array_equal(out, np.stack([site, (local + n) % n_mtiles, n], axis=1))
