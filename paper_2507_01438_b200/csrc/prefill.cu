@@ -211,7 +211,10 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
         if (!ok) break;
       }
       // the commits that hand the last stages back arrive in this CTA's shared memory: wait for them
-      for (uint32_t i = 0; ok && i < min(used, nstages); ++i) {
+      const RingPos last = ring_drain(used, nstages);
+      stage = last.stage;
+      phase = last.phase;
+      for (uint32_t i = min(used, nstages); ok && i > 0; --i) {
         ok = ptx::mbar_wait(&sh.empty[stage], phase ^ 1, wl);
         advance();
       }

@@ -1,5 +1,5 @@
 // The arithmetic of the pair kernel's walks that can be worked out without a GPU (plain C++, also compiled by the host
-// compiler): the order of the tiles of a launch.
+// compiler): the order of the tiles of a launch, the end of an operand ring.
 #pragma once
 #include <stdint.h>
 
@@ -30,6 +30,18 @@ EDGELORA_HD Tile tile_at(const Batch &b, int32_t tile, int32_t &site) {
   t.n = local / b.n_mtiles;
   t.m = (local + t.n) % b.n_mtiles;
   return t;
+}
+
+// Where in its ring a producer that has filled `used` stages in all begins to wait for the last use of each stage that
+// it has filled: `stage` with parity `phase` ^ 1, then on around the ring, min(used, nstages) times.  A ring that was
+// never filled once is waited for from its beginning (the stages behind the last one used were never filled, and a wait
+// for them would pass at once).
+struct RingPos {
+  uint32_t stage, phase;
+};
+EDGELORA_HD RingPos ring_drain(uint32_t used, uint32_t nstages) {
+  if (used < nstages) return RingPos{0u, 1u};
+  return RingPos{used % nstages, (used / nstages) & 1u};
 }
 
 }  // namespace edgelora

@@ -1,4 +1,4 @@
-"""The order in which the pair kernel's roles walk a launch's tiles, on the CPU: csrc/tile_order.h is plain C++ and is
+"""The order in which the pair kernel's roles walk a launch's tiles, and the end of its operand ring, on the CPU: csrc/tile_order.h is plain C++ and is
 compiled here with the host compiler.
 """
 import ctypes
@@ -24,6 +24,12 @@ extern "C" void walk(int32_t n_sites, const int32_t *tile_end, int32_t n_mtiles,
     const edgelora::Tile t = edgelora::tile_at(b, tiles[i], site);
     out[3 * i] = t.s; out[3 * i + 1] = t.m; out[3 * i + 2] = t.n;
   }
+}
+extern "C" int32_t drain(uint32_t used, uint32_t nstages, uint32_t *stage, uint32_t *phase) {
+  const edgelora::RingPos p = edgelora::ring_drain(used, nstages);
+  *stage = p.stage;
+  *phase = p.phase;
+  return 0;
 }
 """
 
@@ -55,3 +61,23 @@ def test_every_tile_is_found_in_any_order(lib, n_mtiles, w_tiles, order):
     local = tiles - np.concatenate([[0], ends[:-1]])[site]
     n = local // n_mtiles
     assert np.array_equal(out, np.stack([site, (local + n) % n_mtiles, n], axis=1))
+
+
+@pytest.mark.parametrize("nstages", [1, 2, 6, 8])
+def test_the_drain_waits_for_the_last_use_of_every_stage(lib, nstages):
+    # a stage's barrier after k completed uses: a wait with parity p passes when the phase of parity p is over,
+    # that is when (k - 1) % 2 == p, and on a barrier never used (k = 0) for parity 1
+    for used in range(0, 4 * nstages + 1):
+        stage, phase = ctypes.c_uint32(), ctypes.c_uint32()
+        lib.drain(ctypes.c_uint32(used), ctypes.c_uint32(nstages), ctypes.byref(stage), ctypes.byref(phase))
+        s, ph = stage.value, phase.value
+        waited = []
+        for _ in range(min(used, nstages)):
+            uses = (used - s + nstages - 1) // nstages      # fills of this stage
+            passes_after = lambda k: (k - 1) % 2 == (ph ^ 1)
+            assert uses >= 1 and passes_after(uses) and not passes_after(uses - 1), (used, s, ph)
+            waited.append(s)
+            s += 1
+            if s == nstages:
+                s, ph = 0, ph ^ 1
+        assert sorted(waited) == list(range(min(used, nstages)))
