@@ -450,6 +450,8 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
   }
   __syncwarp();
   ptx::tc_fence_before_sync();
+  __syncthreads();
+  if (sh.abort_flag) ptx::settle();
   ptx::cluster_sync_all();  // nothing of the other CTA touches this one's memory from here on
   if (warp == 1) {
     ptx::tc_fence_after_sync();

@@ -68,6 +68,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity,
   return true;
 }
 
+// After a wait that ran out, copies, tensor operations and launch-queue answers issued earlier may still be on their way
+// into this CTA's shared and tensor memory, and which of them will never be counted on a barrier depends on where each
+// role gave up.  They take microseconds; the CTA stays for about half a millisecond before it frees its memory.
+constexpr long long kSettleCycles = 1LL << 20;
+__device__ __forceinline__ void settle() {
+  const long long t0 = clock64();
+  while (clock64() - t0 < kSettleCycles) __nanosleep(1000);
+}
+
 // ---------------------------------------------------------------- TMA
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *m) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");

@@ -408,7 +408,10 @@ decode_shrink_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
     const int last_ticket = warps_total + (n_items - first_round) + first_round - 1;
     if (item == last_ticket) *ticket = 0;
   }
-  if (!ok && lane == 0) atomicOr(status, EDGELORA_STATUS_TIMEOUT);
+  if (!ok) {
+    if (lane == 0) atomicOr(status, EDGELORA_STATUS_TIMEOUT);
+    ptx::settle();
+  }
 }
 
 // The shared-memory limit is an attribute of (function, device): set for the current device, by

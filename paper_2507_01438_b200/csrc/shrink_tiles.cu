@@ -539,6 +539,7 @@ __global__ void __launch_bounds__(kThreads, 1) shrink_tiles_kernel(const __grid_
   __syncwarp();
   ptx::tc_fence_before_sync();
   __syncthreads();
+  if (sh.abort_flag) ptx::settle();
   if (warp == 1) {
     ptx::tc_fence_after_sync();
     ptx::tmem_dealloc(tmem_base, 2 * kAccCols);

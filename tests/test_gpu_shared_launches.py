@@ -1,5 +1,5 @@
 """Sets of sites whose launches are shared, in the forms that the ordinary set tests do not take: inputs of different
-widths at one address, results that are inputs.  Against the CPU oracle, element by element.
+widths at one address, results that are inputs, waits that run out.  Against the CPU oracle, element by element.
 """
 import numpy as np
 import pytest
@@ -8,6 +8,7 @@ from paper_2507_01438_b200 import binding as B
 from paper_2507_01438_b200 import workloads as wl
 from helpers import assert_parity, oracle_of
 from gpu_helpers import from_dev_bf16, make_pool, to_dev_bf16
+from test_gpu_parity import random_workload
 from test_gpu_siteset import make_sites, mixed_ids
 
 pytestmark = pytest.mark.gpu
@@ -76,3 +77,37 @@ def test_a_result_that_is_an_input_of_later_sites(T, options):
             s.run([to_dev_bf16(xs[4096]), s.ys[0]])
             sites[1].x = sites[3].x = s.ys[0].view(torch.int16).cpu().numpy().view(np.uint16)
             s.check(f"T={T}")
+
+
+def shorten_waits(pool, on=True):
+    # 1024 cycles, and what a single try of a barrier may take: far less than the longest waits of these calls.  The
+    # kernels give up, wait for what they have in flight, report and return; sync_status brings the pool back
+    B.edgelora_pool_set_option(pool.handle, B.OPT_WAIT_CYCLES, 1 if on else 0)
+
+
+@pytest.mark.parametrize("T,h_in,h_out,options", [
+    (300, 2048, 264, {}),                        # shrink and pair kernel, tiles dealt out
+    (513, 1032, 40000, {}),                      # tiles off the launch queue
+    (40, 2048, 264, {B.OPT_REGIME: 2}),          # gather tiles only
+    (24, 4096, 512, {}),                         # decode in one launch
+    (200, 14336, 520, {}),                       # decode with LoRA K blocks
+])
+def test_a_call_whose_waits_run_out_reports_and_leaves_the_pool_usable(T, h_in, h_out, options):
+    import torch
+    w = random_workload(31, T, h_in, h_out, ranks=[16, 8, 4], max_rank=16)
+    rows = np.unique(np.linspace(0, T - 1, 24).astype(int))
+    pool = make_pool(w)
+    try:
+        for option, value in options.items():
+            B.edgelora_pool_set_option(pool.handle, option, value)
+        W, x, ids = to_dev_bf16(w.W), to_dev_bf16(w.x), torch.from_numpy(w.ids).cuda()
+        for _ in range(2):
+            shorten_waits(pool)
+            pool.linear(W, x, ids)
+            assert pool.status() == (B.ERR_TIMEOUT, B.STATUS_TIMEOUT)
+            shorten_waits(pool, False)
+            y = pool.linear(W, x, ids)
+            assert pool.status() == (0, 0)
+            assert_parity(from_dev_bf16(y)[rows], oracle_of(w, rows), "after the time-out")
+    finally:
+        pool.close()
