@@ -444,9 +444,9 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
       }
     }
   }
-  if (!ok) {
+  if (!ok) {  // the tiles that this pair leaves undone may belong to any site
     sh.abort_flag = 1;
-    if (lane == 0) atomicOr(b.site[min(site, b.n_sites - 1)].status, EDGELORA_STATUS_TIMEOUT);
+    for (int32_t s = 0; s < b.n_sites; ++s) atomicOr(b.site[s].status, EDGELORA_STATUS_TIMEOUT);
   }
   __syncwarp();
   ptx::tc_fence_before_sync();

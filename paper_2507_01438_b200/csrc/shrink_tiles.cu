@@ -532,9 +532,9 @@ __global__ void __launch_bounds__(kThreads, 1) shrink_tiles_kernel(const __grid_
       }
     }
   }
-  if (!ok) {
+  if (!ok) {  // the items that this CTA leaves undone may belong to any site, and leave its arrival counters short
     sh.abort_flag = 1;
-    if (lane == 0) atomicOr(b.site[min(max(cur.s, 0), b.n_sites - 1)].status, EDGELORA_STATUS_TIMEOUT);
+    for (int32_t s = 0; s < b.n_sites; ++s) atomicOr(b.site[s].status, EDGELORA_STATUS_TIMEOUT);
   }
   __syncwarp();
   ptx::tc_fence_before_sync();
