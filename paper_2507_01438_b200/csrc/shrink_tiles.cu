@@ -431,7 +431,9 @@ __global__ void __launch_bounds__(kThreads, 1) shrink_tiles_kernel(const __grid_
       } else {
         // segment tile: row = token of the run, columns = rank index; z partial = scale * acc
         const uint32_t acc = it & 1;
-        const float scale = st.slots[tc.slot].scale;
+        const SlotRow slot = st.slots[tc.slot];
+        const float scale = slot.scale;
+        if (slot.rank <= 0 && tc.nrows > 0 && tc.split == 0 && etid == 0) atomicOr(st.status, EDGELORA_STATUS_SLOT_EMPTY);
         ok = wait_acc(acc);
         if (!ok) break;
         ++it;

@@ -132,3 +132,18 @@ def test_a_wait_that_runs_out_in_a_shared_launch_is_reported_by_every_site():
             for _ in range(2):
                 s.run([xs[1024], xs[256], xs[4096]])
                 s.check("after the time-out", np.array([0, 17, 29, 30, 111, 512]))
+
+
+@pytest.mark.parametrize("sites", [1, 3])
+def test_a_long_run_on_an_empty_slot_raises_the_status(sites):
+    # 300 tokens of one prompt on a slot with nothing loaded: base-only, and the pool says so
+    ids = mixed_ids(41, 10, [(0, 60), (1, 300), (2, 40)], 3)
+    ids[:10] = 0
+    _, ws = make_sites(42, len(ids), [(256, 136), (256, 72), (4096, 64)][:sites], [16, 0, 8], 16, ids)
+    xs = [to_dev_bf16(ws[i].x) for i in ([0] if sites == 1 else [0, 2])]
+    with SetOf(ws, [0, 0, 1][:sites]) as s:
+        s.run(xs)
+        assert [p.status() for p in s.pools] == [(B.ERR_SLOT_EMPTY, B.STATUS_SLOT_EMPTY)] * sites
+        for w in ws:
+            w.ids = np.where(ids == 1, -1, ids).astype(np.int32)
+        s.check()
