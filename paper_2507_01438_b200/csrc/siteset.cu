@@ -95,8 +95,9 @@ int run_sites(edgelora_siteset *s, const void *const *x_dev, const int32_t *ids_
   for (int i0 = 0; i0 < n;) {
     // A run ends where the launch's tables are full, where a pool would come twice (its z workspace holds one
     // site's z), where two sites write the same memory (the later one is to be seen; results that the host call
-    // does not read back share a buffer nobody looks at), in front of a site whose input is still on its way, and behind about a decoder layer of
-    // sites when results are read back beside the sites that follow.  Profiled pools go one by one.
+    // does not read back share a buffer nobody looks at), where the pools' wait limits differ (a launch has one), in
+    // front of a site whose input is still on its way, and behind about a decoder layer of sites when results are read
+    // back beside the sites that follow.  Profiled pools go one by one.
     SiteCall calls[kPairSites];
     SiteCall inputs[kPairInputs];  // the first site on each input
     int m = 0, n_inputs = 0;
@@ -104,7 +105,9 @@ int run_sites(edgelora_siteset *s, const void *const *x_dev, const int32_t *ids_
     for (int i = i0; i < n && m < kPairSites; ++i) {
       edgelora_pool *p = s->pools[i];
       const SiteCall call{p, s->W[i], static_cast<const uint16_t *>(x_dev[s->input_of[i]]), y_dev[i]};
-      if (m > 0 && ((before && (*before)[i]) || p->opt_profile || calls[0].p->opt_profile || (read_back && m >= 7))) break;
+      if (m > 0 && ((before && (*before)[i]) || p->opt_profile || calls[0].p->opt_profile ||
+                    p->wait_cycles != calls[0].p->wait_cycles || (read_back && m >= 7)))
+        break;
       bool again = false;
       for (int k = 0; k < m; ++k)
         again = again || calls[k].p == p ||

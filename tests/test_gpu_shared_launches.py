@@ -147,3 +147,13 @@ def test_a_long_run_on_an_empty_slot_raises_the_status(sites):
         for w in ws:
             w.ids = np.where(ids == 1, -1, ids).astype(np.int32)
         s.check()
+
+
+def test_pools_with_their_own_wait_limits_do_not_share_a_launch():
+    ids = mixed_ids(43, 20, [(0, 300)], 3)
+    _, ws = make_sites(44, len(ids), [(128, 72)] * 4, [16, 8, 4], 16, ids)
+    with SetOf(ws, [0] * 4) as s:
+        B.edgelora_pool_set_option(s.pools[2].handle, B.OPT_WAIT_CYCLES, 1 << 20)
+        s.run([to_dev_bf16(ws[0].x)])
+        s.check()
+        assert [B.edgelora_pool_last_launch(p.handle)["launches"] for p in s.pools] == [2, 0, 2, 2]
