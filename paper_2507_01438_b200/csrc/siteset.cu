@@ -262,9 +262,8 @@ int edgelora_siteset_run_host(edgelora_siteset_t *s, const uint16_t *const *x_ho
       y_dev[i] = buf;
     }
   }
-  // An input that the first launches do not need is uploaded on the second stream, beside them; the
-  // launch in front of its first consumer waits for it (a launch also carries the next site's shrink,
-  // hence one launch earlier).
+  // An input that the first sites do not need is uploaded on the second stream, beside them; the launches of its
+  // first consumer wait for it.
   if (!s->copy_stream) SET_TRY(cudaStreamCreateWithFlags(&s->copy_stream, cudaStreamNonBlocking));
   if (s->up_ev.empty()) s->up_ev.assign(s->n_inputs, nullptr);
   std::vector<cudaEvent_t> before(n, nullptr);
@@ -277,15 +276,14 @@ int edgelora_siteset_run_host(edgelora_siteset_t *s, const uint16_t *const *x_ho
         first = k;
         break;
       }
-    const int at = first - 1;  // the launch that may already read it
     const size_t bytes = static_cast<size_t>(T) * s->in_width[i] * 2;
-    if (at <= 0 || first >= n || before[at]) {
+    if (first == 0 || first == n) {
       SET_TRY(cudaMemcpyAsync(s->dx[i], x_host[i], bytes, cudaMemcpyHostToDevice, st));
     } else {
       if (!s->up_ev[i]) SET_TRY(cudaEventCreateWithFlags(&s->up_ev[i], cudaEventDisableTiming));
       SET_TRY(cudaMemcpyAsync(s->dx[i], x_host[i], bytes, cudaMemcpyHostToDevice, s->copy_stream));
       SET_TRY(cudaEventRecord(s->up_ev[i], s->copy_stream));
-      before[at] = s->up_ev[i];
+      before[first] = s->up_ev[i];
     }
   }
   std::vector<const void *> xd(s->dx.begin(), s->dx.end());

@@ -157,3 +157,15 @@ def test_pools_with_their_own_wait_limits_do_not_share_a_launch():
         s.run([to_dev_bf16(ws[0].x)])
         s.check()
         assert [B.edgelora_pool_last_launch(p.handle)["launches"] for p in s.pools] == [2, 0, 2, 2]
+
+
+def test_an_input_still_on_its_way_ends_a_run_in_front_of_its_first_reader():
+    import torch
+    ids = mixed_ids(45, 20, [(0, 300)], 3)
+    xs, ws = make_sites(46, len(ids), [(256, 72), (256, 64), (128, 72), (256, 136)], [16, 8, 4], 16, ids)
+    pin = lambda a, dt: torch.from_numpy(np.ascontiguousarray(a).view(dt)).pin_memory()
+    with SetOf(ws, [0, 0, 1, 0]) as s:
+        ys = [None] * 3 + [torch.zeros((len(ids), 136), dtype=torch.int16).pin_memory()]
+        B.edgelora_siteset_run_host(s.handle, [pin(xs[256], np.int16), pin(xs[128], np.int16)], pin(ids, np.int32), ys)
+        assert [B.edgelora_pool_last_launch(p.handle)["launches"] for p in s.pools] == [2, 0, 2, 0]
+        assert_parity(wl.bf16_bits_to_f32(ys[3].numpy().view(np.uint16)), oracle_of(ws[3]), ws[3].name)
