@@ -1138,8 +1138,7 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
     // reduction wait for its arrival counter.  CTAs of one grid wait for one another here, so every
     // cluster of the launch must be resident at once: checked against the device's occupancy figure.
     bool fused = false;
-    static const bool log_launches = getenv("EDGELORA_LOG") != nullptr;
-    if (log_launches)
+    if (getenv("EDGELORA_LOG"))
       fprintf(stderr, "edgelora: decode T %d N %d splits %d grid %d expand_in_reduce %d ctas_per_sm %d\n", T, N, splits,
               grid, g.expand_in_reduce, ctas_per_sm);
     // (Calls that may overlap the call before them keep the two launches: a one-launch grid holds every

@@ -169,3 +169,20 @@ def test_load_from_page_locked_memory():
         assert B.edgelora_pool_load_slot_pinned(pool.handle, 0, 8, 1.0, keep[0], keep[1]) == B.ERR_INVALID_ARG
     finally:
         pool.close()
+
+
+def test_the_log_switch_is_read_at_every_decode_call(monkeypatch, capfd):
+    import torch
+    w = random_workload(47, 20, 256, 256, ranks=[16, 8], max_rank=16)
+    pool = make_pool(w)
+    try:
+        W, x, ids = to_dev_bf16(w.W), to_dev_bf16(w.x), torch.from_numpy(w.ids).cuda()
+        for on in (False, True, False):
+            if on:
+                monkeypatch.setenv("EDGELORA_LOG", "1")
+            else:
+                monkeypatch.delenv("EDGELORA_LOG", raising=False)
+            pool.linear(W, x, ids)
+            assert ("edgelora: decode T 20" in capfd.readouterr().err) == on
+    finally:
+        pool.close()
