@@ -8,8 +8,8 @@
 // rows [c BN/2, (c + 1) BN/2), so a K block costs an SM 32 KB of operand fill for 512 tensor cycles where
 // a tile of 128 x 256 per SM costs 48 KB (4096 -> 14336, T = 4096: 289 us, 1.66 PFLOP/s, against 371 us; the tensor
 // pipe is busy 87 % of the cycles, and what bounds a loop of calls is the power limit).  After the K blocks of h_in come the LoRA K blocks, one per
-// adapter of the tile's 256 tokens: B_a rows (TMA, each CTA its half) against z in bf16, masked to that
-// adapter's tokens (each CTA builds the rows of its own tokens).
+// adapter of the tile's 256 tokens: B_a rows (TMA, each CTA its half) against z in bf16 (each CTA writes the
+// rows of its own tokens), added to the accumulator rows of that adapter's tokens only.
 //
 // Warp roles, in both CTAs: warp 0 issues TMA, warp 1 owns tensor memory (and, in CTA 0 only, issues the
 // MMAs of the pair), warps 2..5 are the epilogue of the CTA's 128 tokens, warps 6..9 list the tile's adapters
@@ -41,7 +41,8 @@ constexpr int kListMax = kListTile;                 // adapters of a tile at mos
 struct Barriers {
   uint64_t full[kPairMaxStages];   // CTA 0: loads of both CTAs -> MMA
   uint64_t empty[kPairMaxStages];  // MMA -> TMA (own CTA)
-  uint64_t zfull[kPairMaxStages];  // CTA 0: builder warps of both CTAs -> MMA (LoRA K blocks)
+  uint64_t zfull[kPairMaxStages];  // CTA 0: builder warps of CTA 1 -> MMA: their rows of z (first LoRA K blocks of a tile)
+  uint64_t mfull[kPairMaxStages];  // builder -> MMA (own CTA): the rows that the LoRA K block is for, and CTA 0's rows of z
   uint64_t zgo[kPairMaxStages];    // TMA warp -> builder (own CTA): the stage is free
   uint64_t tfull[2];               // MMA -> epilogue (own CTA)
   uint64_t tempty[2];              // CTA 0: epilogue warps of both CTAs -> MMA
@@ -51,6 +52,7 @@ struct Barriers {
   uint64_t nempty;                 // CTA 1: every role of both CTAs has read it
   uint64_t ask;                    // CTA 1: its TMA thread is near the end of the tile's K blocks
   alignas(16) uint32_t answer[4];
+  alignas(16) uint32_t off[kPairMaxStages][8];  // CTA 0: per LoRA K block, the rows of the tile that are not on its adapter
   uint32_t tmem_slot;
   volatile uint32_t abort_flag;
   int32_t wcount[8];
@@ -119,7 +121,8 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
     for (uint32_t s = 0; s < nstages; ++s) {
       ptx::mbar_init(&sh.full[s], 1);
       ptx::mbar_init(&sh.empty[s], 1);
-      ptx::mbar_init(&sh.zfull[s], 8);  // one arrival per builder warp of the pair
+      ptx::mbar_init(&sh.zfull[s], 4);  // one arrival per builder warp of CTA 1
+      ptx::mbar_init(&sh.mfull[s], 4);  // one arrival per builder warp
       ptx::mbar_init(&sh.zgo[s], 1);
     }
     for (int i = 0; i < 2; ++i) {
@@ -199,7 +202,7 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
           }
           // The stage is free: let the builder write its half (it follows this warp, never the stage
           // barriers directly, so it cannot run ahead of the ring).
-          ptx::mbar_arrive(&sh.zgo[stage]);
+          if (leader || e < static_cast<int32_t>(nstages)) ptx::mbar_arrive(&sh.zgo[stage]);
           if (leader) ptx::mbar_arrive_expect_tx(&sh.full[stage], 2 * w_bytes);
           ptx::tma_load_3d_pair(smem + static_cast<size_t>(stage) * stage_bytes + kXBytes, &st.b, full0 + stage * 8, 0,
                                 row_w, a);
@@ -223,7 +226,7 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
     // ------------------------------------------------------------ MMA issuer (of the pair)
     if (leader && ptx::elect_one()) {
       const uint32_t idesc = ptx::umma_idesc_bf16(2 * kTileM, static_cast<uint32_t>(b.BN));
-      uint32_t stage = 0, phase = 0, zphase = 0;  // zphase: one parity bit per stage
+      uint32_t stage = 0, phase = 0, zphase = 0, mphase = 0;  // zphase, mphase: one parity bit per stage
       int32_t it = 0;
       for (int32_t tile = tile0; tile >= 0; ++it) {
         const Tile t = tile_at(b, tile, site);
@@ -235,14 +238,8 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
         }
         ptx::tc_fence_after_sync();
         const uint32_t tmem_d = tmem_base + acc * 256;
-        auto mma_block = [&](int ksteps, bool first) {
-          const uint32_t sr = ptx::smem_u32(smem + static_cast<size_t>(stage) * stage_bytes);
-          const uint64_t da = ptx::umma_desc_k128(sr), db = ptx::umma_desc_k128(sr + kXBytes);
-          // advancing 16 bf16 along K inside the swizzled row = 32 bytes = 2 descriptor units
-#pragma unroll
-          for (int k = 0; k < kBlockK / kUmmaK; ++k)
-            if (k < ksteps) ptx::umma_bf16_pair(tmem_d, da + 2 * k, db + 2 * k, idesc, (!first || k > 0) ? 1u : 0u);
-          ptx::umma_commit_pair(&sh.empty[stage]);  // frees the stage in both CTAs once these MMAs are done
+        auto commit = [&]() {  // frees the stage in both CTAs once its MMAs are done
+          ptx::umma_commit_pair(&sh.empty[stage]);
           if (++stage == nstages) {
             stage = 0;
             phase ^= 1;
@@ -254,7 +251,13 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
             break;
           }
           ptx::tc_fence_after_sync();
-          mma_block(kBlockK / kUmmaK, kb == 0);
+          const uint32_t sr = ptx::smem_u32(smem + static_cast<size_t>(stage) * stage_bytes);
+          const uint64_t da = ptx::umma_desc_k128(sr), db = ptx::umma_desc_k128(sr + kXBytes);
+          // advancing 16 bf16 along K inside the swizzled row = 32 bytes = 2 descriptor units
+#pragma unroll
+          for (int k = 0; k < kBlockK / kUmmaK; ++k)
+            ptx::umma_bf16_pair(tmem_d, da + 2 * k, db + 2 * k, idesc, (kb > 0 || k > 0) ? 1u : 0u);
+          commit();
         }
         if (!ok) break;
         const int buf = it & 1;
@@ -263,15 +266,24 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
           break;
         }
         const int32_t cnt = sh.count[buf];
+        const int lora_ksteps = st.R_pad / kUmmaK;
         for (int32_t e = 0; e < cnt; ++e) {
-          if (!ptx::mbar_wait(&sh.full[stage], phase, wl) ||
-              !ptx::mbar_wait_cluster(&sh.zfull[stage], (zphase >> stage) & 1u, wl) || sh.abort_flag) {
+          const bool has_z = e < static_cast<int32_t>(nstages);  // (later blocks find z in the stage, see the builder)
+          if (!ptx::mbar_wait(&sh.full[stage], phase, wl) || !ptx::mbar_wait(&sh.mfull[stage], (mphase >> stage) & 1u, wl) ||
+              (has_z && !ptx::mbar_wait_cluster(&sh.zfull[stage], (zphase >> stage) & 1u, wl)) || sh.abort_flag) {
             ok = false;
             break;
           }
-          zphase ^= 1u << stage;
+          mphase ^= 1u << stage;
+          if (has_z) zphase ^= 1u << stage;
           ptx::tc_fence_after_sync();
-          mma_block(st.R_pad / kUmmaK, false);
+          const uint4 off_lo = *reinterpret_cast<const uint4 *>(&sh.off[stage][0]);
+          const uint4 off_hi = *reinterpret_cast<const uint4 *>(&sh.off[stage][4]);
+          const uint32_t sr = ptx::smem_u32(smem + static_cast<size_t>(stage) * stage_bytes);
+          const uint64_t da = ptx::umma_desc_k128(sr), db = ptx::umma_desc_k128(sr + kXBytes);
+          for (int k = 0; k < lora_ksteps; ++k)
+            ptx::umma_bf16_pair_rows(tmem_d, da + 2 * k, db + 2 * k, idesc, off_lo, off_hi);
+          commit();
         }
         if (!ok) break;
         ptx::mbar_arrive(&sh.lempty[buf]);
@@ -382,6 +394,8 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
       const int32_t tok = t.m * (2 * kTileM) + static_cast<int32_t>(rank) * kTileM + btid;
       int32_t id = tok < b.T ? b.ids_valid[tok] : -1;
       if (!EL_CHECK(st.status, id >= -1 && id < b.n_slots, 2)) id = -1;
+      int32_t id1 = leader && tok + kTileM < b.T ? b.ids_valid[tok + kTileM] : -1;  // of a token of CTA 1
+      if (!EL_CHECK(st.status, id1 >= -1 && id1 < b.n_slots, 2)) id1 = -1;
       // z of the thread's token, in flight while the list is made
       const int nch = st.R_pad >> 3;  // 16-byte chunks of one operand row that the MMAs read
       uint4 z[8];
@@ -419,23 +433,41 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
       if (btid == 0) ptx::mbar_arrive(&sh.lfull[buf]);
 
       count += static_cast<uint32_t>(st.kb_total);
+      // A LoRA K block multiplies the z of all tokens with one adapter's B, and the tensor core leaves the rows of the
+      // tokens that are not on this adapter as they are: an infinity or NaN in one adapter's B stays away from the tokens
+      // on others, which a product with zeros of z would not see to.  So z is the same for every block of the tile: it is
+      // written once per stage of the ring, and what a block needs beyond that is its eight words of rows.
       for (int32_t e = 0; e < total; ++e) {
-        const bool m = sh.list[buf][e] == id;
+        const bool write_z = e < static_cast<int32_t>(nstages);
         const uint32_t stage = count % nstages;
         ++count;
+        if (!leader && !write_z) continue;
         ok = __all_sync(0xffffffffu, ptx::mbar_wait(&sh.zgo[stage], (gophase >> stage) & 1u, wl) && !sh.abort_flag);
         if (!ok) break;
         gophase ^= 1u << stage;
-        // 128-byte swizzle: the 16-byte chunk index is XORed with the row index modulo 8.  Every row is
-        // written: z of the tokens on this adapter, zeros for the others.
-        uint8_t *drow = smem + static_cast<size_t>(stage) * stage_bytes + btid * 128;
+        if (write_z) {
+          // 128-byte swizzle: the 16-byte chunk index is XORed with the row index modulo 8
+          uint8_t *drow = smem + static_cast<size_t>(stage) * stage_bytes + btid * 128;
 #pragma unroll
-        for (int c = 0; c < 8; ++c)
-          if (c < nch)
-            *reinterpret_cast<uint4 *>(drow + ((c ^ (btid & 7)) << 4)) = m ? z[c] : make_uint4(0u, 0u, 0u, 0u);
-        ptx::fence_proxy_async();  // make the generic-proxy writes visible to the tensor core
+          for (int c = 0; c < 8; ++c)
+            if (c < nch) *reinterpret_cast<uint4 *>(drow + ((c ^ (btid & 7)) << 4)) = z[c];
+          ptx::fence_proxy_async();  // make the generic-proxy writes visible to the tensor core
+        }
+        if (leader) {
+          const int32_t a = sh.list[buf][e];
+          const uint32_t on0 = __ballot_sync(0xffffffffu, id == a), on1 = __ballot_sync(0xffffffffu, id1 == a);
+          if (lane == 0) {
+            sh.off[stage][bwarp] = ~on0;
+            sh.off[stage][4 + bwarp] = ~on1;
+          }
+        }
         __syncwarp();
-        if (lane == 0) ptx::mbar_arrive_cluster(zfull0 + stage * 8);
+        if (lane == 0) {
+          if (leader)
+            ptx::mbar_arrive(&sh.mfull[stage]);
+          else
+            ptx::mbar_arrive_cluster(zfull0 + stage * 8);
+        }
       }
       const bool got = next_tile<true, kSteal>(sh, it, nempty1, n_tiles, wl, tile);
       if (named_bar_any(2, 128, !ok || !got)) {

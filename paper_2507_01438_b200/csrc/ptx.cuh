@@ -308,6 +308,17 @@ __device__ __forceinline__ void umma_bf16_pair(uint32_t tmem_d, uint64_t desc_a,
       "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(accumulate)
       : "memory");
 }
+// The same for some of the 256 rows of D only: bit i of off[0..7] set leaves row i (lane i of the first CTA's tensor
+// memory, lane i - 128 of the second's) as it is, whatever the product would add to it.
+__device__ __forceinline__ void umma_bf16_pair_rows(uint32_t tmem_d, uint64_t desc_a, uint64_t desc_b, uint32_t idesc,
+                                                    const uint4 &off_lo, const uint4 &off_hi) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, 1, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, {%4, %5, %6, %7, %8, %9, %10, %11}, p;\n\t}" ::"r"(tmem_d),
+      "l"(desc_a), "l"(desc_b), "r"(idesc), "r"(off_lo.x), "r"(off_lo.y), "r"(off_lo.z), "r"(off_lo.w), "r"(off_hi.x),
+      "r"(off_hi.y), "r"(off_hi.z), "r"(off_hi.w)
+      : "memory");
+}
 // Arrive on the barrier at this offset in both CTAs once the MMAs issued so far are finished.
 __device__ __forceinline__ void umma_commit_pair(uint64_t *bar) {
   asm volatile(

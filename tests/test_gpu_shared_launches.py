@@ -169,3 +169,26 @@ def test_an_input_still_on_its_way_ends_a_run_in_front_of_its_first_reader():
         B.edgelora_siteset_run_host(s.handle, [pin(xs[256], np.int16), pin(xs[128], np.int16)], pin(ids, np.int32), ys)
         assert [B.edgelora_pool_last_launch(p.handle)["launches"] for p in s.pools] == [2, 0, 2, 0]
         assert_parity(wl.bf16_bits_to_f32(ys[3].numpy().view(np.uint16)), oracle_of(ws[3]), ws[3].name)
+
+
+@pytest.mark.parametrize("rank", [16, 32, 64])
+@pytest.mark.parametrize("T,n_adapters", [(300, 3), (513, 40), (700, 300)])
+def test_a_non_finite_adapter_reaches_its_own_tokens_only(T, n_adapters, rank):
+    import torch
+    # every third adapter has an infinity or NaN in its B; the others share token tiles with it
+    rng = np.random.Generator(np.random.PCG64(T + rank))
+    w = random_workload(T, T, 264, 392, ranks=[rank] * n_adapters, max_rank=rank)
+    w.ids = rng.permutation(np.arange(T) % (n_adapters + 1) - 1).astype(np.int32)
+    w.ids[60:100] = 1                                     # and a run of its own, in the first tile
+    bad = np.isin(w.ids, np.arange(0, n_adapters, 3))
+    want = oracle_of(w)
+    for a in range(0, n_adapters, 3):
+        w.adapters[a].B[:, a % rank] = 0x7F80 if a % 2 else 0x7FC0   # bfloat16 infinity, NaN
+    pool = make_pool(w)
+    try:
+        got = from_dev_bf16(pool.linear(to_dev_bf16(w.W), to_dev_bf16(w.x), torch.from_numpy(w.ids).cuda()))
+        assert pool.status() == (0, 0)
+        assert_parity(got[~bad], want[~bad], "tokens on finite adapters and on none")
+        assert not np.isfinite(got[bad]).any()
+    finally:
+        pool.close()
