@@ -24,6 +24,7 @@
 #include "internal.cuh"
 #include "launch.cuh"
 #include "ptx.cuh"
+#include "tile_order.h"
 #include "zload.cuh"
 
 namespace edgelora {
@@ -298,10 +299,11 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer
     if (ptx::elect_one()) {
-      uint32_t stage = 0, phase = 0;
+      uint32_t stage = 0, phase = 0, used = 0;
       bool ok = true;
       auto wait_empty = [&]() { return ptx::mbar_wait(&empty_bar[stage], phase ^ 1, wl) && !*abort_flag; };
       auto advance = [&]() {
+        ++used;
         if (++stage == nstages) {
           stage = 0;
           phase ^= 1;
@@ -353,6 +355,14 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
       if (!ok) {
         *abort_flag = 1;
         atomicOr(p.status, EDGELORA_STATUS_TIMEOUT);
+      }
+      // What was requested lands before the CTA frees its memory, also when a wait of some role ran out.
+      const RingPos last = ring_drain(used, nstages);
+      stage = last.stage;
+      phase = last.phase;
+      for (uint32_t i = min(used, nstages); i > 0; --i) {
+        ptx::mbar_wait(&full_bar[stage], phase ^ 1);
+        advance();
       }
     }
   } else if (warp == 1) {
@@ -406,12 +416,13 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
           }
         }
       }
-      if (ok) {
-        ptx::umma_commit(tfull_bar);  // accumulator complete
-      } else {
+      if (!ok) {
         *abort_flag = 1;
         atomicOr(p.status, EDGELORA_STATUS_TIMEOUT);
       }
+      ptx::umma_commit(tfull_bar);  // accumulator complete, or as far as it came (the flag says which)
+      ptx::mbar_wait(tfull_bar, 0);  // this warp frees the tensor memory: nothing writes to it any more
+
     }
   } else if (warp < 6) {
     // ------------------------------------------------------------ epilogue (warps 2..5)
@@ -663,9 +674,10 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
         if (!EL_CHECK(p.status, a >= 0 && a < p.n_slots, 1)) continue;
         const uint32_t stage = count % nstages;
         ++count;
-        // (the lanes of a warp leave together: the cluster barriers behind this loop take whole warps)
-        ok = __all_sync(0xffffffffu, ptx::mbar_wait(&zgo_bar[stage], (gophase >> stage) & 1u, wl) && !*abort_flag);
-        if (!ok) break;
+        if (!ptx::mbar_wait(&zgo_bar[stage], (gophase >> stage) & 1u, wl) || *abort_flag) {
+          ok = false;
+          break;
+        }
         gophase ^= 1u << stage;
         uint8_t *dst = smem + static_cast<size_t>(stage) * stage_bytes + r_bytes;
         // 128-byte swizzle: the 16-byte chunk index is XORed with the row index modulo 8.
@@ -717,7 +729,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
     const bool wide = !p.expand_in_reduce;
     const bool sender = epi || (wide && warp >= 6);
     const int c_first = (wide && warp >= 6) ? 32 : 0, c_step = wide ? 64 : 32;
-    const bool have_acc = __all_sync(0xffffffffu, sender && !*abort_flag);  // this CTA's accumulator is complete (tfull waited)
+    const bool have_acc = sender && !*abort_flag;  // this CTA's accumulator is complete (tfull waited)
     const bool z_ok = fused_z_ok;  // fused launches: the wait for the shrink teams ended in time
     float4 *z_stage = reinterpret_cast<float4 *>(b_stage + static_cast<size_t>(cols_per) * kTileM * p.R_pad * 2);
     // The partial tiles land in the operand ring, which is idle once every CTA of the cluster is past
@@ -812,9 +824,8 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
         bool b_ok = true;
         {
           int got = 1;
-          if (lane == 0) got = ptx::mbar_wait(ep_bar, 0, wl) ? 1 : 0;  // the staged B_a rows
+          if (lane == 0) got = ptx::mbar_wait(ep_bar, 0, max(wl, ptx::kSettleCycles)) ? 1 : 0;  // the staged B_a rows
           if (!__shfl_sync(0xffffffffu, got, 0)) {
-            *abort_flag = 1;
             if (lane == 0) atomicOr(p.status, EDGELORA_STATUS_TIMEOUT);
             b_ok = false;
           }
@@ -947,7 +958,6 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
 
   ptx::tc_fence_before_sync();
   __syncthreads();
-  if (*abort_flag) ptx::settle();
   if (warp == 1) {
     ptx::tc_fence_after_sync();
     ptx::tmem_dealloc(tmem_base, static_cast<uint32_t>(p.tmem_cols));

@@ -482,8 +482,6 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
   }
   __syncwarp();
   ptx::tc_fence_before_sync();
-  __syncthreads();
-  if (sh.abort_flag) ptx::settle();
   ptx::cluster_sync_all();  // nothing of the other CTA touches this one's memory from here on
   if (warp == 1) {
     ptx::tc_fence_after_sync();
@@ -503,6 +501,7 @@ cudaError_t pair_set_smem_limit() {
   const int bytes = static_cast<int>(kPairSmemBudget);
   cudaError_t e = cudaSuccess;
 #define EDGELORA_SMEM(N, ST)                                                                                      \
+    ptx::settle();
   if (e == cudaSuccess) e = cudaFuncSetAttribute(pair_gemm_kernel<N, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   EDGELORA_SMEM(1, false)
   EDGELORA_SMEM(1, true)

@@ -68,14 +68,16 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity,
   return true;
 }
 
-// After a wait that ran out, copies, tensor operations and launch-queue answers issued earlier may still be on their way
-// into this CTA's shared and tensor memory, and which of them will never be counted on a barrier depends on where each
-// role gave up.  They take microseconds; the CTA stays for about half a millisecond before it frees its memory.
+// For a role that gives up a wait, behind the last thing it issued: copies, tensor operations and launch-queue answers
+// may still be on their way into shared and tensor memory, and which of them will ever be counted on a barrier depends on
+// where each role gave up.  They take microseconds; the role stays for about half a millisecond before it goes to the
+// barrier behind which the CTA frees its memory.
 constexpr long long kSettleCycles = 1LL << 20;
-__device__ __forceinline__ void settle() {
+__device__ __forceinline__ void settle_inline() {
   const long long t0 = clock64();
   while (clock64() - t0 < kSettleCycles) __nanosleep(1000);
 }
+static __device__ __noinline__ void settle() { settle_inline(); }  // (a kernel of few microseconds pays for the fetch of cold code)
 
 // ---------------------------------------------------------------- TMA
 __device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *m) {

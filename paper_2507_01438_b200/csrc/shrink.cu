@@ -410,7 +410,7 @@ decode_shrink_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
   }
   if (!ok) {
     if (lane == 0) atomicOr(status, EDGELORA_STATUS_TIMEOUT);
-    ptx::settle();
+    ptx::settle_inline();
   }
 }
 

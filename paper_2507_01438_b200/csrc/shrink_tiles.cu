@@ -541,7 +541,6 @@ __global__ void __launch_bounds__(kThreads, 1) shrink_tiles_kernel(const __grid_
   __syncwarp();
   ptx::tc_fence_before_sync();
   __syncthreads();
-  if (sh.abort_flag) ptx::settle();
   if (warp == 1) {
     ptx::tc_fence_after_sync();
     ptx::tmem_dealloc(tmem_base, 2 * kAccCols);
@@ -559,6 +558,7 @@ cudaError_t shrink_tiles_set_smem_limit() {
 }
 
 template <int kSites>
+    ptx::settle();
 cudaError_t launch_shrink_tiles(const ShrinkBatch<kSites> &b, int32_t grid, bool pdl, cudaStream_t stream) {
   return launch_ex(shrink_tiles_kernel<kSites>, dim3(grid), dim3(kThreads), kShrinkTilesSmem, stream, pdl, 1, b);
 }
