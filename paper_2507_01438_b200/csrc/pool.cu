@@ -65,8 +65,8 @@ EncodeTiledFn get_encode_fn() {
 }
 
 // bf16 row-major [d2][d1][d0] (d2 == 0 => 2D), box = {box_cols, box_rows, 1}; out-of-range
-// elements read as zero.  box_cols == 64: the 128-byte-swizzled operand tiles of the GEMM;
-// otherwise (the shrink's row segments) no swizzle.
+// elements read as zero.  box_cols 64, 32, 16: operand tiles of the tensor core, rows of 128, 64 or 32 bytes with the
+// swizzle of that width; otherwise (the decode shrink's row segments) no swizzle.
 int encode_tmap(CUtensorMap *out, const void *base, uint64_t d0, uint64_t d1, uint64_t d2,
                 uint32_t box_rows, uint32_t box_cols, uint64_t s1 = 0, uint64_t s2 = 0) {
   EncodeTiledFn fn = get_encode_fn();
@@ -78,7 +78,10 @@ int encode_tmap(CUtensorMap *out, const void *base, uint64_t d0, uint64_t d1, ui
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = fn(out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank, const_cast<void *>(base), dims,
                   strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  box_cols == static_cast<uint32_t>(kBlockK) ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                  box_cols == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
+                  : box_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
+                  : box_cols == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
+                                   : CU_TENSOR_MAP_SWIZZLE_NONE,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     snprintf(g_last_error, sizeof g_last_error, "cuTensorMapEncodeTiled failed (%d)", (int)r);
@@ -892,7 +895,7 @@ static int prefill_batch(const SiteCall *sites, int n, edgelora_plan *plan, int3
     PairSite &s = pb.site[i];
     int rc = fill_shrink_site(q, &sb.site[i], shrink_splits(q, T, n), xi);
     if (!rc) rc = get_tmap(q, &s.w, sites[i].W, q->cfg.h_in, q->cfg.h_out, 0, BN / 2);
-    if (!rc) rc = get_tmap(q, &s.b, q->B_pool, q->R_pad, q->cfg.h_out, q->cfg.n_slots, BN / 2);
+    if (!rc) rc = get_tmap(q, &s.b, q->B_pool, q->R_pad, q->cfg.h_out, q->cfg.n_slots, BN / 2, q->R_pad);
     if (rc) return rc;
     tiles += n_mtiles * ((q->cfg.h_out + BN - 1) / BN);
     s.y = static_cast<uint16_t *>(sites[i].y);

@@ -21,7 +21,7 @@ void set_last_cuda_error(cudaError_t e, const char *what);
 struct TmapKey {
   const void *base;
   uint64_t d0, d1, d2;
-  uint32_t b1, b0;  // box rows, box columns (64 => 128-byte swizzle, otherwise no swizzle)
+  uint32_t b1, b0;  // box rows, box columns (which also say the swizzle)
   uint64_t s1, s2;  // byte strides of dimensions 1 and 2 (0 = dense)
   bool operator==(const TmapKey &o) const {
     return base == o.base && d0 == o.d0 && d1 == o.d1 && d2 == o.d2 && b1 == o.b1 && b0 == o.b0 && s1 == o.s1 &&

@@ -7,9 +7,10 @@
 // and half in the other's.  CTA c of the pair holds the tokens [128 c, 128 c + 128) of the tile and the W
 // rows [c BN/2, (c + 1) BN/2), so a K block costs an SM 32 KB of operand fill for 512 tensor cycles where
 // a tile of 128 x 256 per SM costs 48 KB (4096 -> 14336, T = 4096: 289 us, 1.66 PFLOP/s, against 371 us; the tensor
-// pipe is busy 87 % of the cycles, and what bounds a loop of calls is the power limit).  After the K blocks of h_in come the LoRA K blocks, one per
-// adapter of the tile's 256 tokens: B_a rows (TMA, each CTA its half) against z in bf16 (each CTA writes the
-// rows of its own tokens), added to the accumulator rows of that adapter's tokens only.
+// pipe is busy 87 % of the cycles, and what bounds a loop of calls is the power limit).  After the K blocks of h_in come
+// the LoRA K blocks for the adapters of the tile's 256 tokens, 64 / R_pad adapters in a block: B_a rows (TMA, each CTA
+// its half) against z in bf16 (each CTA writes the rows of its own tokens), where the MMA of an adapter adds to the
+// accumulator rows of its tokens only.
 //
 // Warp roles, in both CTAs: warp 0 issues TMA, warp 1 owns tensor memory (and, in CTA 0 only, issues the
 // MMAs of the pair), warps 2..5 are the epilogue of the CTA's 128 tokens, warps 6..9 list the tile's adapters
@@ -42,7 +43,7 @@ struct Barriers {
   uint64_t full[kPairMaxStages];   // CTA 0: loads of both CTAs -> MMA
   uint64_t empty[kPairMaxStages];  // MMA -> TMA (own CTA)
   uint64_t zfull[kPairMaxStages];  // CTA 0: builder warps of CTA 1 -> MMA: their rows of z (first LoRA K blocks of a tile)
-  uint64_t mfull[kPairMaxStages];  // builder -> MMA (own CTA): the rows that the LoRA K block is for, and CTA 0's rows of z
+  uint64_t mfull[kPairMaxStages];  // builder -> MMA (own CTA): whose rows the LoRA K block is for, and CTA 0's rows of z
   uint64_t zgo[kPairMaxStages];    // TMA warp -> builder (own CTA): the stage is free
   uint64_t tfull[2];               // MMA -> epilogue (own CTA)
   uint64_t tempty[2];              // CTA 0: epilogue warps of both CTAs -> MMA
@@ -52,7 +53,8 @@ struct Barriers {
   uint64_t nempty;                 // CTA 1: every role of both CTAs has read it
   uint64_t ask;                    // CTA 1: its TMA thread is near the end of the tile's K blocks
   alignas(16) uint32_t answer[4];
-  alignas(16) uint32_t off[kPairMaxStages][8];  // CTA 0: per LoRA K block, the rows of the tile that are not on its adapter
+  // CTA 0: per adapter of a LoRA K block, the rows of the tile that are not on it
+  alignas(16) uint32_t off[kPairMaxStages][kBlockK / kUmmaK][8];
   uint32_t tmem_slot;
   volatile uint32_t abort_flag;
   int32_t wcount[8];
@@ -194,18 +196,21 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
           break;
         }
         const int32_t cnt = sh.count[buf];
-        for (int32_t e = 0; e < cnt; ++e) {
-          const int32_t a = sh.list[buf][e];
+        const int32_t per = kBlockK / st.R_pad;  // adapters of a LoRA K block
+        const uint32_t b_bytes = static_cast<uint32_t>(b.BN * st.R_pad);  // a CTA's half of one adapter's rows
+        for (int32_t e0 = 0, blk = 0; e0 < cnt; e0 += per, ++blk) {
+          const int32_t n = min(per, cnt - e0);
           if (!wait_empty()) {
             ok = false;
             break;
           }
           // The stage is free: let the builder write its half (it follows this warp, never the stage
           // barriers directly, so it cannot run ahead of the ring).
-          if (leader || e < static_cast<int32_t>(nstages)) ptx::mbar_arrive(&sh.zgo[stage]);
-          if (leader) ptx::mbar_arrive_expect_tx(&sh.full[stage], 2 * w_bytes);
-          ptx::tma_load_3d_pair(smem + static_cast<size_t>(stage) * stage_bytes + kXBytes, &st.b, full0 + stage * 8, 0,
-                                row_w, a);
+          if (leader || blk < static_cast<int32_t>(nstages)) ptx::mbar_arrive(&sh.zgo[stage]);
+          if (leader) ptx::mbar_arrive_expect_tx(&sh.full[stage], 2 * n * b_bytes);
+          uint8_t *dst = smem + static_cast<size_t>(stage) * stage_bytes + kXBytes;
+          for (int32_t j = 0; j < n; ++j)
+            ptx::tma_load_3d_pair(dst + j * b_bytes, &st.b, full0 + stage * 8, 0, row_w, sh.list[buf][e0 + j]);
           advance();
         }
         if (!ok) break;
@@ -266,23 +271,36 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
           break;
         }
         const int32_t cnt = sh.count[buf];
-        const int lora_ksteps = st.R_pad / kUmmaK;
-        for (int32_t e = 0; e < cnt; ++e) {
-          const bool has_z = e < static_cast<int32_t>(nstages);  // (later blocks find z in the stage, see the builder)
-          if (!ptx::mbar_wait(&sh.full[stage], phase, wl) || !ptx::mbar_wait(&sh.mfull[stage], (mphase >> stage) & 1u, wl) ||
-              (has_z && !ptx::mbar_wait_cluster(&sh.zfull[stage], (zphase >> stage) & 1u, wl)) || sh.abort_flag) {
+        const int32_t per = kBlockK / st.R_pad;
+        const uint32_t b_bytes = static_cast<uint32_t>(b.BN * st.R_pad), row_bytes = static_cast<uint32_t>(st.R_pad) * 2;
+        const int ksteps = st.R_pad / kUmmaK;
+        for (int32_t e0 = 0, blk = 0; e0 < cnt; e0 += per, ++blk) {
+          const bool has_z = blk < static_cast<int32_t>(nstages);  // (later blocks find z in the stage, see the builder)
+          ok = ptx::mbar_wait(&sh.mfull[stage], (mphase >> stage) & 1u, wl);
+          // (the builder is ahead of the loads as a rule: the first adapter's rows are read while those are on their way)
+          uint4 off_lo = *reinterpret_cast<const uint4 *>(&sh.off[stage][0][0]);
+          uint4 off_hi = *reinterpret_cast<const uint4 *>(&sh.off[stage][0][4]);
+          if (!ok || (has_z && !ptx::mbar_wait_cluster(&sh.zfull[stage], (zphase >> stage) & 1u, wl)) ||
+              !ptx::mbar_wait(&sh.full[stage], phase, wl) || sh.abort_flag) {
             ok = false;
             break;
           }
           mphase ^= 1u << stage;
           if (has_z) zphase ^= 1u << stage;
           ptx::tc_fence_after_sync();
-          const uint4 off_lo = *reinterpret_cast<const uint4 *>(&sh.off[stage][0]);
-          const uint4 off_hi = *reinterpret_cast<const uint4 *>(&sh.off[stage][4]);
           const uint32_t sr = ptx::smem_u32(smem + static_cast<size_t>(stage) * stage_bytes);
-          const uint64_t da = ptx::umma_desc_k128(sr), db = ptx::umma_desc_k128(sr + kXBytes);
-          for (int k = 0; k < lora_ksteps; ++k)
-            ptx::umma_bf16_pair_rows(tmem_d, da + 2 * k, db + 2 * k, idesc, off_lo, off_hi);
+          const uint64_t da = ptx::umma_desc_k128(sr);
+          uint64_t db = ptx::umma_desc_rows(sr + kXBytes, row_bytes);
+          const int32_t n = min(per, cnt - e0);
+          for (int32_t j = 0; j < n; ++j, db += b_bytes >> 4) {
+            if (j > 0) {
+              off_lo = *reinterpret_cast<const uint4 *>(&sh.off[stage][j][0]);
+              off_hi = *reinterpret_cast<const uint4 *>(&sh.off[stage][j][4]);
+            }
+#pragma unroll
+            for (int k = 0; k < kBlockK / kUmmaK; ++k)
+              if (k < ksteps) ptx::umma_bf16_pair_rows(tmem_d, da + 2 * k, db + 2 * k, idesc, off_lo, off_hi);
+          }
           commit();
         }
         if (!ok) break;
@@ -433,12 +451,16 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
       if (btid == 0) ptx::mbar_arrive(&sh.lfull[buf]);
 
       count += static_cast<uint32_t>(st.kb_total);
-      // A LoRA K block multiplies the z of all tokens with one adapter's B, and the tensor core leaves the rows of the
-      // tokens that are not on this adapter as they are: an infinity or NaN in one adapter's B stays away from the tokens
-      // on others, which a product with zeros of z would not see to.  So z is the same for every block of the tile: it is
-      // written once per stage of the ring, and what a block needs beyond that is its eight words of rows.
-      for (int32_t e = 0; e < total; ++e) {
-        const bool write_z = e < static_cast<int32_t>(nstages);
+      // The MMA of an adapter multiplies the z of all tokens with its B, and the tensor core leaves the rows of the tokens
+      // that are not on it as they are.  So z is the same for every block of the tile: it is written once per stage of
+      // the ring, and what a block needs beyond that is eight words of rows per adapter.  It also keeps an infinity or NaN
+      // in one adapter's B away from the tokens on others, which a product with zeros of z would not.  What bounds a tile
+      // of many adapters is the hand-over of a stage with the latency of its B_a rows, hence 64 / R_pad adapters to a
+      // stage: 300 tokens on 300 adapters of rank 16, 4096 -> 4096: 61 us, 115 with one adapter to a stage, 123 with z
+      // masked and written anew for every adapter.
+      const int32_t per = kBlockK / st.R_pad;
+      for (int32_t e0 = 0, blk = 0; e0 < total; e0 += per, ++blk) {
+        const bool write_z = blk < static_cast<int32_t>(nstages);
         const uint32_t stage = count % nstages;
         ++count;
         if (!leader && !write_z) continue;
@@ -454,11 +476,13 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
           ptx::fence_proxy_async();  // make the generic-proxy writes visible to the tensor core
         }
         if (leader) {
-          const int32_t a = sh.list[buf][e];
-          const uint32_t on0 = __ballot_sync(0xffffffffu, id == a), on1 = __ballot_sync(0xffffffffu, id1 == a);
-          if (lane == 0) {
-            sh.off[stage][bwarp] = ~on0;
-            sh.off[stage][4 + bwarp] = ~on1;
+          for (int32_t j = 0; j < min(per, total - e0); ++j) {
+            const int32_t a = sh.list[buf][e0 + j];
+            const uint32_t on0 = __ballot_sync(0xffffffffu, id == a), on1 = __ballot_sync(0xffffffffu, id1 == a);
+            if (lane == 0) {
+              sh.off[stage][j][bwarp] = ~on0;
+              sh.off[stage][j][4 + bwarp] = ~on1;
+            }
           }
         }
         __syncwarp();
@@ -479,6 +503,7 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
   if (!ok) {  // the tiles that this pair leaves undone may belong to any site
     sh.abort_flag = 1;
     for (int32_t s = 0; s < b.n_sites; ++s) atomicOr(b.site[s].status, EDGELORA_STATUS_TIMEOUT);
+    ptx::settle();
   }
   __syncwarp();
   ptx::tc_fence_before_sync();
@@ -501,7 +526,6 @@ cudaError_t pair_set_smem_limit() {
   const int bytes = static_cast<int>(kPairSmemBudget);
   cudaError_t e = cudaSuccess;
 #define EDGELORA_SMEM(N, ST)                                                                                      \
-    ptx::settle();
   if (e == cudaSuccess) e = cudaFuncSetAttribute(pair_gemm_kernel<N, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   EDGELORA_SMEM(1, false)
   EDGELORA_SMEM(1, true)

@@ -10,12 +10,12 @@ constexpr int kPairMaxStages = 8;
 constexpr int kPairSites = 32;   // sites of one launch at most
 constexpr int kPairInputs = 4;   // distinct inputs of one launch at most
 constexpr int kYStageBytes = 4 * 32 * 128;  // epilogue: per warp 32 tokens x 64 bf16
-constexpr size_t kPairTailBytes = 3072;
+constexpr size_t kPairTailBytes = 4096;
 constexpr size_t kPairSmemBudget = 226 * 1024;
 
 struct PairSite {
   CUtensorMap w;         // W [h_out][h_in], boxes of BN / 2 rows x 64
-  CUtensorMap b;         // the pool's B blocks [S][h_out][R_pad], boxes of BN / 2 rows x 64
+  CUtensorMap b;         // the pool's B blocks [S][h_out][R_pad], boxes of BN / 2 rows x R_pad
   uint16_t *y;           // [T][h_out]
   const SlotRow *slots;
   const uint4 *zb;       // z as bf16 [max_tokens][R_pad], zero at and past the true rank

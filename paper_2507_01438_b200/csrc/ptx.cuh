@@ -157,6 +157,13 @@ __device__ __forceinline__ uint64_t umma_desc_k128(uint32_t smem_addr) {
   d |= static_cast<uint64_t>(2) << 61;
   return d;
 }
+// The same for a tile stored as rows of `row_bytes` = 32, 64 or 128 with the swizzle of that width (a TMA box of row_bytes
+// with SWIZZLE_32B, 64B or 128B): 8-row groups are 8 * row_bytes apart; swizzle modes 6 (32B), 4 (64B), 2 (128B).
+__device__ __forceinline__ uint64_t umma_desc_rows(uint32_t smem_addr, uint32_t row_bytes) {
+  const uint64_t mode = row_bytes == 128 ? 2 : row_bytes == 64 ? 4 : 6;
+  return static_cast<uint64_t>((smem_addr & 0x3FFFFu) >> 4) | (static_cast<uint64_t>(1) << 16) |
+         (static_cast<uint64_t>(row_bytes >> 1) << 32) | (static_cast<uint64_t>(1) << 46) | (mode << 61);
+}
 // Instruction descriptor for kind::f16 with bf16 A and B (both K-major), fp32 accumulate:
 // D format f32 (1) in bits 4-5, A format bf16 (1) in 7-9, B format bf16 (1) in 10-12,
 // N >> 3 in 17-22, M >> 4 in 24-28.
