@@ -114,23 +114,24 @@ def test_a_call_whose_waits_run_out_reports_and_leaves_the_pool_usable(T, h_in, 
 
 
 def test_a_wait_that_runs_out_in_a_shared_launch_is_reported_by_every_site():
-    # more items and tiles than the first round of CTAs takes: those of the last site (two K parts per shrink tile) are
-    # never reached.  Its pool reports all the same, and its arrival counters are back in place for the next run
+    # more items and tiles than the first round of CTAs takes, in a launch that deals its tiles out: those of the last
+    # site (two K parts per shrink tile) need not be reached.  Its pool reports all the same, and its arrival counters are
+    # back in place for the next run
     T = 513
     ids = mixed_ids(33, 30, [(i % 3, 40) for i in range(11)] + [(0, 43)], 3)
-    shapes = [(1024, 32768)] + [(256, 72)] * 18 + [(4096, 64)]
+    shapes = [(2048, 8192)] + [(256, 72)] * 18 + [(4096, 64)]
     _, sites = make_sites(34, T, shapes, [16, 8, 4], 16, ids)
     xs = {w.h_in: to_dev_bf16(w.x) for w in sites}
     with SetOf(sites, [0] + [1] * 18 + [2]) as s:
         for _ in range(2):
             for p in s.pools:
                 shorten_waits(p)
-            s.run([xs[1024], xs[256], xs[4096]])
+            s.run([xs[2048], xs[256], xs[4096]])
             assert [p.status() for p in s.pools] == [(B.ERR_TIMEOUT, B.STATUS_TIMEOUT)] * len(sites)
             for p in s.pools:
                 shorten_waits(p, False)
             for _ in range(2):
-                s.run([xs[1024], xs[256], xs[4096]])
+                s.run([xs[2048], xs[256], xs[4096]])
                 s.check("after the time-out", np.array([0, 17, 29, 30, 111, 512]))
 
 
