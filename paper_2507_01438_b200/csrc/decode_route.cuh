@@ -97,6 +97,7 @@ __device__ __forceinline__ void publish_decode_plan(const PlanView &pv, int a, i
     pv.counts[3] = T;
     pv.counts[4] = n_groups - has_base;
     pv.counts[5] = KS;
+    pv.counts[6] = 0;
   }
 }
 

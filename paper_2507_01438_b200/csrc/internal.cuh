@@ -62,7 +62,8 @@ struct PlanView {
   int32_t *mt_count;       // [ceil(maxT/256)+1] distinct ids >= 0 inside each 256-token tile
   int32_t *mt_list;        // [ceil(maxT/256)*256] those ids, tile m at [256 m, 256 m + mt_count[m])
   int32_t *counts;         // [8]  0: n_groups, 1: n_segments, 2: n_sgmv_tiles, 3: short tokens,
-                           //      4: LoRA groups, 5: K chunks used by the decode shrink
+                           //      4: LoRA groups, 5: K chunks used by the decode shrink,
+                           //      6: short tokens with an adapter (0: not counted)
   uint32_t *status;        // device status word of the plan
   int32_t max_sgmv_tiles;
 };

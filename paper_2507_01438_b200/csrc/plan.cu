@@ -9,10 +9,9 @@
 //   sgmv tiles  in batches above kDecodeMaxT tokens, for runs of >= kSegMin tokens on a real
 //               adapter: 128-token tiles of the run (work list of the segment shrink),
 //   tile lists  the distinct ids >= 0 inside every 256-token tile (the LoRA K blocks of that tile).
-// Tokens of one run stay together in the group order, so the runs are sorted, not the tokens: a
-// bitonic sort of the unique keys ((id + 1) << 16 | run index) in shared memory, exact and the
-// same on every launch.  Prefix sums run in rounds of one element per thread (warp shuffles plus
-// one shared-memory stage), so nothing but the outputs goes through global memory.
+// Tokens of one run stay together in the group order, so the runs are sorted, not the tokens, by the
+// unique keys ((id + 1) << 16 | run index) in shared memory: exact and the same on every launch.
+// Batches up to 4096 tokens keep everything but the outputs in shared memory (plan_small).
 #include "internal.cuh"
 #include "launch.cuh"
 #include "ptx.cuh"
@@ -58,62 +57,61 @@ __device__ __forceinline__ int scan_rounds(int n, int *wt, Value value, Consume 
 }
 
 // The distinct ids >= 0 inside every 256-token tile, in order of first appearance (the LoRA K blocks of that tile
-// in the base-product kernel).  One warp per tile; lane l holds the ids of tokens l, l + 32, ... of the tile.
-// Only the first token of a run (inside the tile) can be a first appearance, so each of those is compared with
-// the later ones: as many rounds as the tile has runs.
-__device__ __forceinline__ void list_tiles(const int32_t *valid, int32_t T, const PlanView &pv) {
+// in the base-product kernel).  One warp per tile; `first` has a bit per token, set for the heads of runs whose id does
+// not occur earlier in their tile.  A tile's first token is a first appearance in any case.
+__device__ __forceinline__ void list_tiles(const int32_t *valid, int32_t T, const PlanView &pv, const uint32_t *first) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int n_mt = (T + kListTile - 1) / kListTile;
   for (int m = warp; m < n_mt; m += kPlanThreads / 32) {
     int32_t id[8];
-    uint32_t heads[8];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
       const int t = m * kListTile + q * 32 + lane;
       id[q] = t < T ? valid[t] : -1;
-      const bool head = id[q] >= 0 && ((q == 0 && lane == 0) || valid[t - 1] != id[q]);
-      heads[q] = __ballot_sync(0xffffffffu, head);
-    }
-    uint32_t dup = 0;  // bit q: this lane's q-th token is on an id seen before
-#pragma unroll
-    for (int qq = 0; qq < 8; ++qq) {
-      for (uint32_t rest = heads[qq]; rest; rest &= rest - 1) {
-        const int src = __ffs(rest) - 1;
-        const int32_t v = __shfl_sync(0xffffffffu, id[qq], src);
-#pragma unroll
-        for (int q = qq; q < 8; ++q)
-          if (v == id[q] && (q > qq || lane > src)) dup |= 1u << q;
-      }
     }
     int base = 0;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const bool first = ((heads[q] >> lane) & 1u) && !((dup >> q) & 1u);
-      const uint32_t b = __ballot_sync(0xffffffffu, first);
-      if (first) pv.mt_list[m * kListTile + base + __popc(b & ((1u << lane) - 1u))] = id[q];
-      base += __popc(b);
+      uint32_t bits = m * kListTile + q * 32 < T ? first[m * 8 + q] : 0u;
+      if (q == 0) bits |= __shfl_sync(0xffffffffu, id[0], 0) >= 0 ? 1u : 0u;
+      if ((bits >> lane) & 1u) pv.mt_list[m * kListTile + base + __popc(bits & ((1u << lane) - 1u))] = id[q];
+      base += __popc(bits);
     }
     if (lane == 0) pv.mt_count[m] = base;
   }
 }
+// Marks the head of a run (first token t0, id >= 0) for list_tiles.  prev_end: where the run in front of it with the same
+// id ends (0: there is none); in the order of the runs by (id, run index) that is the neighbour.
+__device__ __forceinline__ void mark_first(uint32_t *first, int t0, int prev_end) {
+  if (prev_end <= (t0 & ~(kListTile - 1))) atomicOr(&first[t0 >> 5], 1u << (t0 & 31));
+}
 
-// Batches up to kPlanSmallT tokens with up to 1024 runs (every serving batch of ordinary make): the same plan,
-// worked out in shared memory with one thread per run.  The general form below keeps its intermediate arrays
-// in global memory and goes through them in about thirty barrier-separated passes, each a round trip to L2;
-// here the runs are ordered by counting smaller keys instead of by a sorting network, and the four prefix sums
-// over the runs are one scan of four packed 16-bit fields (8 runs in 4096 tokens: 8.5 us against 13; 64 decode tokens
-// and two runs: 11 against 18).
+// Batches up to kPlanSmallT tokens: the plan is worked out in shared memory.  The general form below keeps its
+// intermediate arrays in global memory and goes through them in about thirty barrier-separated passes, each a round trip
+// to L2; here each thread looks after T / 1024 consecutive tokens and n_segs / 1024 consecutive places of the order of
+// the runs, and the four prefix sums over the runs are one scan of four packed 16-bit fields.  Per build, back to back:
+// 8 runs in 512 tokens 4.4 us (general form 11), 66 runs in 2112 tokens 5.6 (21), 2048 runs in 2048 tokens 17 (39), 4096 in
+// 4096 34 (76).  Up to kCountRuns runs are ordered by counting smaller keys, more of them by a sorting network: 512 runs
+// in 1024 tokens 9.4 us counted, 10.7 sorted; 1024 runs 11.8 sorted, 20 and more counted.
 constexpr int kPlanSmallT = 4096;
 constexpr int kPlanTok = kPlanSmallT / kPlanThreads;  // tokens per thread, consecutive
+constexpr int kCountRuns = 512;
 struct PlanSmall {
-  int32_t ids[kPlanSmallT];
-  int32_t seg_start[kPlanThreads + 1], seg_id[kPlanThreads];
-  alignas(16) uint32_t key[kPlanThreads];
-  int32_t run[kPlanThreads];                      // run at each place of the order
-  int32_t out[kPlanThreads], out_short[kPlanThreads];  // by run: where it begins in perm and perm_short
-  unsigned long long wt[kPlanThreads / 32];
+  int32_t *ids, *seg_start, *seg_id;
+  uint32_t *key;             // (id + 1) << 16 | run: of every run, then in order
+  int32_t *out, *out_short;  // by run: where it begins in perm and perm_short (-1: nowhere)
+  static __host__ __device__ int32_t stride(int32_t T) { return (T + 4) & ~3; }  // T + 1 entries each
+  static __host__ __device__ size_t bytes(int32_t T) { return 6 * sizeof(int32_t) * stride(T); }
+  __device__ PlanSmall(uint32_t *mem, int32_t T) {
+    const int32_t n = stride(T);
+    ids = reinterpret_cast<int32_t *>(mem);
+    seg_start = ids + n;
+    seg_id = seg_start + n;
+    key = reinterpret_cast<uint32_t *>(seg_id + n);
+    out = seg_id + 2 * n;
+    out_short = out + n;
+  }
 };
-static_assert(sizeof(PlanSmall) >= kPlanSmallT * 4, "the general form's keys fit too");
 
 // Exclusive prefix sum over the block (one synchronisation; wt must not be in use by an earlier scan).
 __device__ __forceinline__ unsigned long long scan_block(unsigned long long v, unsigned long long *wt,
@@ -138,9 +136,28 @@ __device__ __forceinline__ unsigned long long scan_block(unsigned long long v, u
   return (warp > 0 ? before : 0ull) + incl - v;
 }
 
-// Returns false, with nothing but ids_valid written, when the batch has more than 1024 runs.
-__device__ __forceinline__ bool plan_small(const int32_t *__restrict__ ids, int32_t T, int32_t n_slots,
-                                           const PlanView &pv, PlanSmall &sh) {
+// Sorts n keys (a power of two, at least 32) in shared memory, ascending; the caller synchronises before and after.
+// A warp's pairs of a step with j <= 32 lie in blocks of 64 keys that no other warp touches in such a step.
+__device__ __forceinline__ void sort_keys(uint32_t *key, int n) {
+  for (int k = 2; k <= n; k <<= 1) {
+    for (int j = k >> 1; j > 0; j >>= 1) {
+      for (int i = threadIdx.x; i < (n >> 1); i += kPlanThreads) {
+        const int lo = 2 * i - (i & (j - 1)), hi = lo + j;
+        const uint32_t a = key[lo], b = key[hi];
+        if ((a > b) == ((lo & k) == 0)) {
+          key[lo] = b;
+          key[hi] = a;
+        }
+      }
+      if (j > 32 || (j == 1 && k >= 64)) __syncthreads();  // (j == 1: the next step is 2 k / 2 = k apart)
+      else __syncwarp();
+    }
+  }
+}
+
+__device__ __forceinline__ void plan_small(const int32_t *__restrict__ ids, int32_t T, int32_t n_slots,
+                                           const PlanView &pv, const PlanSmall &sh, uint32_t *first,
+                                           unsigned long long (&wt)[2][kPlanThreads / 32]) {
   const int tid = threadIdx.x;
   // validate; segments = maximal runs of equal id in token order
   bool bad = false;
@@ -158,6 +175,7 @@ __device__ __forceinline__ bool plan_small(const int32_t *__restrict__ ids, int3
       pv.ids_valid[t] = a;
     }
   }
+  for (int i = tid; i < kPlanSmallT / 32; i += kPlanThreads) first[i] = 0;
   if (__syncthreads_or(bad ? 1 : 0) && tid == 0) atomicOr(pv.status, EDGELORA_STATUS_BAD_ADAPTER_ID);
   const int per = (T + kPlanThreads - 1) / kPlanThreads;  // tokens of this thread: [tid per, tid per + per)
   int heads = 0;
@@ -174,9 +192,11 @@ __device__ __forceinline__ bool plan_small(const int32_t *__restrict__ ids, int3
     }
   }
   unsigned long long total;
-  int s = static_cast<int>(scan_block(heads, sh.wt, total)) - 1;
+  int s = static_cast<int>(scan_block(heads, wt[0], total)) - 1;
   const int n_segs = static_cast<int>(total);
-  if (n_segs > kPlanThreads) return false;
+  const bool counted = n_segs <= kCountRuns;
+  int npow2 = 32;
+  while (!counted && npow2 < n_segs) npow2 <<= 1;
 #pragma unroll
   for (int q = 0; q < kPlanTok; ++q) {
     const int t = tid * per + q;
@@ -185,12 +205,15 @@ __device__ __forceinline__ bool plan_small(const int32_t *__restrict__ ids, int3
         ++s;
         sh.seg_start[s] = t;
         sh.seg_id[s] = id[q];
+        sh.key[s] = (static_cast<uint32_t>(id[q] + 1) << 16) | static_cast<uint32_t>(s);
         pv.seg_start[s] = t;
         pv.seg_adapter[s] = id[q];
       }
       pv.tok_seg[t] = s;
     }
   }
+  // (n_segs <= T and the network's next power of two may lie past the key array: out and out_short follow it, unused yet)
+  for (int i = n_segs + tid; i < (counted ? (n_segs + 3) & ~3 : npow2); i += kPlanThreads) sh.key[i] = 0xFFFFFFFFu;
   if (tid == 0) {
     sh.seg_start[n_segs] = T;
     pv.seg_start[n_segs] = T;
@@ -199,60 +222,72 @@ __device__ __forceinline__ bool plan_small(const int32_t *__restrict__ ids, int3
   __syncthreads();
 
   // the runs ordered by (id, run index): -1 first, token order kept.  Keys are unique.
-  const int n4 = (n_segs + 3) & ~3;
-  uint32_t key = 0xFFFFFFFFu;
-  int len = 0;
-  if (tid < n_segs) {
-    key = (static_cast<uint32_t>(sh.seg_id[tid] + 1) << 16) | static_cast<uint32_t>(tid);
-    len = sh.seg_start[tid + 1] - sh.seg_start[tid];
-  }
-  if (tid < n4) sh.key[tid] = key;
-  __syncthreads();
-  if (tid < n_segs) {
+  if (counted) {
+    const uint32_t key = tid < n_segs ? sh.key[tid] : 0u;
     int place = 0;
-    for (int i = 0; i < n4; i += 4) {
-      const uint4 k = *reinterpret_cast<const uint4 *>(&sh.key[i]);
-      place += (k.x < key) + (k.y < key) + (k.z < key) + (k.w < key);
-    }
-    sh.run[place] = tid;
+    if (tid < n_segs)
+      for (int i = 0; i < n_segs; i += 4) {
+        const uint4 k = *reinterpret_cast<const uint4 *>(&sh.key[i]);
+        place += (k.x < key) + (k.y < key) + (k.z < key) + (k.w < key);
+      }
+    __syncthreads();
+    if (tid < n_segs) sh.key[place] = key;
+  } else {
+    sort_keys(sh.key, npow2);
   }
   __syncthreads();
 
   // one scan: tokens and short tokens (runs the gather-by-token shrink handles: every run of a small batch,
   // otherwise those below kSegMin) and group heads in the order of the runs, segment tiles in token order
   const bool all_short = T <= kDecodeMaxT;
-  int my_run = 0, my_len = 0, my_short = 0, my_head = 0, my_tiles = 0, my_id = -1;
-  if (tid < n_segs) {
-    my_run = sh.run[tid];
-    my_len = sh.seg_start[my_run + 1] - sh.seg_start[my_run];
-    my_short = (all_short || my_len < kSegMin) ? my_len : 0;
-    my_id = sh.seg_id[my_run];
-    my_head = (tid == 0 || sh.seg_id[sh.run[tid - 1]] != my_id) ? 1 : 0;
-    my_tiles = (!all_short && sh.seg_id[tid] >= 0 && len >= kSegMin) ? (len + kTileM - 1) / kTileM : 0;
+  const int rper = (n_segs + kPlanThreads - 1) / kPlanThreads;  // places, and runs, of this thread: [tid rper, ...)
+  auto len_of = [&](int r) { return sh.seg_start[r + 1] - sh.seg_start[r]; };
+  auto short_of = [&](int len) { return (all_short || len < kSegMin) ? len : 0; };
+  auto id_at = [&](int i) { return static_cast<int32_t>(sh.key[i] >> 16) - 1; };
+  auto head_at = [&](int i) { return (i == 0 || (sh.key[i - 1] >> 16) != (sh.key[i] >> 16)) ? 1 : 0; };
+  auto tiles_of = [&](int r) {
+    const int len = len_of(r);
+    return (!all_short && sh.seg_id[r] >= 0 && len >= kSegMin) ? (len + kTileM - 1) / kTileM : 0;
+  };
+  auto pack = [](int len, int sh_len, int head, int tiles) {
+    return static_cast<unsigned long long>(len) | (static_cast<unsigned long long>(sh_len) << 16) |
+           (static_cast<unsigned long long>(head) << 32) | (static_cast<unsigned long long>(tiles) << 48);
+  };
+  unsigned long long mine = 0;
+  for (int q = 0; q < rper; ++q) {
+    const int i = tid * rper + q;
+    if (i < n_segs) {
+      const int len = len_of(static_cast<int>(sh.key[i] & 0xFFFFu));
+      mine += pack(len, short_of(len), head_at(i), tiles_of(i));
+    }
   }
-  const unsigned long long packed = static_cast<unsigned long long>(my_len) | (static_cast<unsigned long long>(my_short) << 16) |
-                                    (static_cast<unsigned long long>(my_head) << 32) |
-                                    (static_cast<unsigned long long>(my_tiles) << 48);
-  const unsigned long long pre = scan_block(packed, sh.wt, total);  // (the barriers above lie behind the first scan)
-  const int p_len = static_cast<int>(pre & 0xFFFF), p_short = static_cast<int>((pre >> 16) & 0xFFFF);
-  const int g = static_cast<int>((pre >> 32) & 0xFFFF) + my_head - 1, p_tiles = static_cast<int>(pre >> 48);
+  unsigned long long pre = scan_block(mine, wt[1], total);
   const int n_groups = static_cast<int>((total >> 32) & 0xFFFF), n_short = static_cast<int>((total >> 16) & 0xFFFF);
-  const int has_base = (n_segs > 0 && sh.seg_id[sh.run[0]] < 0) ? 1 : 0;  // the group of id -1 comes first
-  if (tid < n_segs) {
-    sh.out[my_run] = p_len;
-    sh.out_short[my_run] = my_short > 0 ? p_short : -1;
-    if (my_head) {
+  const int has_base = id_at(0) < 0 ? 1 : 0;  // the group of id -1 comes first
+  for (int q = 0; q < rper; ++q) {
+    const int i = tid * rper + q;
+    if (i >= n_segs) break;
+    const int r = static_cast<int>(sh.key[i] & 0xFFFFu), len = len_of(r), my_short = short_of(len), my_id = id_at(i);
+    const int head = head_at(i), n_tiles = tiles_of(i);
+    const int p_len = static_cast<int>(pre & 0xFFFF), p_short = static_cast<int>((pre >> 16) & 0xFFFF);
+    const int g = static_cast<int>((pre >> 32) & 0xFFFF) + head - 1, p_tiles = static_cast<int>(pre >> 48);
+    pre += pack(len, my_short, head, n_tiles);
+    sh.out[r] = p_len;
+    sh.out_short[r] = my_short > 0 ? p_short : -1;
+    if (my_id >= 0) mark_first(first, sh.seg_start[r], head ? 0 : sh.seg_start[(sh.key[i - 1] & 0xFFFFu) + 1]);
+    if (head) {
       pv.group_start[g] = p_len;
       pv.gs_short[g] = p_short;
       pv.group_adapter[g] = my_id;
       if (my_id >= 0) pv.lg_adapter[g - has_base] = my_id;
+      if (g == has_base) pv.counts[6] = n_short - p_short;
     }
-    for (int i = 0; i < my_tiles; ++i) {  // 128-token tiles of this thread's (long) run
-      const int tile = p_tiles + i;
+    for (int k = 0; k < n_tiles; ++k) {  // 128-token tiles of the (long) run i
+      const int tile = p_tiles + k;
       if (tile < pv.max_sgmv_tiles) {
-        pv.sgmv_tiles[4 * tile + 0] = sh.seg_start[tid] + i * kTileM;
-        pv.sgmv_tiles[4 * tile + 1] = min(kTileM, len - i * kTileM);
-        pv.sgmv_tiles[4 * tile + 2] = sh.seg_id[tid];
+        pv.sgmv_tiles[4 * tile + 0] = sh.seg_start[i] + k * kTileM;
+        pv.sgmv_tiles[4 * tile + 1] = min(kTileM, len_of(i) - k * kTileM);
+        pv.sgmv_tiles[4 * tile + 2] = sh.seg_id[i];
         pv.sgmv_tiles[4 * tile + 3] = 0;
       }
     }
@@ -265,6 +300,7 @@ __device__ __forceinline__ bool plan_small(const int32_t *__restrict__ ids, int3
     pv.counts[3] = n_short;
     pv.counts[4] = n_groups - has_base;
     pv.counts[5] = 0;
+    if (n_groups == has_base) pv.counts[6] = 0;
   }
   __syncthreads();
   // groups: the runs in order, concatenated (s is the run of this thread's last token)
@@ -278,25 +314,27 @@ __device__ __forceinline__ bool plan_small(const int32_t *__restrict__ ids, int3
       if ((is_head >> q) & 1u) --s;
     }
   }
-  list_tiles(sh.ids, T, pv);
-  return true;
+  list_tiles(sh.ids, T, pv, first);
 }
 
-__global__ void __launch_bounds__(kPlanThreads)
+__global__ void __launch_bounds__(kPlanThreads, 1)
 plan_kernel(const int32_t *__restrict__ ids, int32_t T, int32_t n_slots, PlanView pv) {
-  extern __shared__ __align__(16) uint32_t keys[];  // one key per run, padded to a power of two
+  extern __shared__ __align__(16) uint32_t keys[];  // one key per run, padded to a power of two; or the small form's arrays
   __shared__ int wt[34];
+  __shared__ unsigned long long wt_small[2][kPlanThreads / 32];
+  __shared__ uint32_t first[kMaxTokensLimit / 32];  // see list_tiles
   const int tid = threadIdx.x;
 
   ptx::pdl_launch_dependents();
   ptx::pdl_wait_prior_grids();  // earlier kernels on the stream may still read the plan arrays
   if (T <= kPlanSmallT) {
-    if (plan_small(ids, T, n_slots, pv, *reinterpret_cast<PlanSmall *>(keys))) return;
-    __syncthreads();
+    plan_small(ids, T, n_slots, pv, PlanSmall(keys, T), first, wt_small);
+    return;
   }
 
   // 1. validate
   bool bad = false;
+  for (int i = tid; i < kMaxTokensLimit / 32; i += kPlanThreads) first[i] = 0;
   for (int t = tid; t < T; t += kPlanThreads) {
     int32_t a = ids[t];
     if (a < -1 || a >= n_slots) {
@@ -332,22 +370,8 @@ plan_kernel(const int32_t *__restrict__ ids, int32_t T, int32_t n_slots, PlanVie
     keys[i] = i < n_segs ? ((static_cast<uint32_t>(pv.seg_adapter[i] + 1) << 16) | static_cast<uint32_t>(i))
                          : 0xFFFFFFFFu;
   __syncthreads();
-  for (int k = 2; k <= npow2; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = tid; i < npow2; i += kPlanThreads) {
-        const int ixj = i ^ j;
-        if (ixj > i) {
-          const uint32_t a = keys[i], b = keys[ixj];
-          const bool up = (i & k) == 0;
-          if ((a > b) == up) {
-            keys[i] = b;
-            keys[ixj] = a;
-          }
-        }
-      }
-      __syncthreads();
-    }
-  }
+  sort_keys(keys, npow2);
+  __syncthreads();
 
   // 4. groups: the runs in sorted order, concatenated.  out_start[j] (in pv.scratch) is where the
   // j-th sorted run begins in perm; inv (borrowing pv.mt_list until step 8) maps a run to j.
@@ -372,8 +396,9 @@ plan_kernel(const int32_t *__restrict__ ids, int32_t T, int32_t n_slots, PlanVie
     const int head = is_ghead(j);
     const int g = before + head - 1;
     gidx[j] = g;
+    const int32_t a = static_cast<int32_t>(keys[j] >> 16) - 1;
+    if (a >= 0) mark_first(first, pv.seg_start[run_of(j)], head ? 0 : pv.seg_start[run_of(j - 1) + 1]);
     if (head) {
-      const int32_t a = static_cast<int32_t>(keys[j] >> 16) - 1;
       pv.group_start[g] = out_start[j];
       pv.group_adapter[g] = a;
       if (a >= 0) pv.lg_adapter[g - has_base] = a;
@@ -408,6 +433,7 @@ plan_kernel(const int32_t *__restrict__ ids, int32_t T, int32_t n_slots, PlanVie
   if (tid == 0) {
     pv.gs_short[n_groups] = n_short;
     pv.counts[3] = n_short;
+    pv.counts[6] = n_short - pv.gs_short[has_base];  // (written behind the barriers of the scan; n_short when no id >= 0 is there)
   }
 
   // 7. 128-token tiles of the long runs (segment shrink work list), in token order
@@ -433,14 +459,14 @@ plan_kernel(const int32_t *__restrict__ ids, int32_t T, int32_t n_slots, PlanVie
   __syncthreads();  // inv (in pv.mt_list) is dead from here
 
   // 8. the adapters of every 256-token tile
-  list_tiles(pv.ids_valid, T, pv);
+  list_tiles(pv.ids_valid, T, pv, first);
 }
 
 void launch_plan(const int32_t *ids, int32_t T, int32_t n_slots, const PlanView &pv, bool pdl,
                  cudaStream_t stream) {
   int npow2 = 32;  // the number of runs is only known on the device: size for the worst case
   while (npow2 < T) npow2 <<= 1;
-  const size_t smem = T <= kPlanSmallT ? sizeof(PlanSmall) : static_cast<size_t>(npow2) * 4;
+  const size_t smem = T <= kPlanSmallT ? PlanSmall::bytes(T) : static_cast<size_t>(npow2) * 4;
   launch_ex(plan_kernel, dim3(1), dim3(kPlanThreads), smem, stream, pdl, 1, ids, T, n_slots, pv);
 }
 

@@ -102,3 +102,19 @@ def test_sites_of_a_set_that_share_memory(what):
         B.edgelora_siteset_destroy(s)
         for p in pools:
             p.close()
+
+
+@pytest.mark.parametrize("T,n_runs", [
+    (700, 511), (700, 512), (700, 513),    # runs ordered by counting, and by the sorting network
+    (1030, 1030), (2049, 2047),            # more than one run per thread; the network's padding lies past the keys
+    (4095, 4095), (4098, 4098),            # the last batch of the shared-memory form, the general form
+])
+def test_plan_orders(T, n_runs):
+    w = random_workload(T + n_runs, T, 64, 64, ranks=[8, 16, 4, 0, 16, 2, 5], max_rank=16)
+    rng = np.random.Generator(np.random.PCG64(n_runs))
+    per_run = np.cumsum(rng.integers(1, 7, size=n_runs)) % 7     # neighbours differ
+    w.ids = np.array([-1, 0, 1, 2, 4, 5, 6], np.int32)[per_run][np.arange(T) * n_runs // T]
+    assert 1 + np.count_nonzero(np.diff(w.ids)) == n_runs
+    y, plan = run_gpu(w, return_plan=True)
+    assert_parity(y, oracle_of(w), f"T={T}")
+    check_plan(plan, w.ids, w.n_slots)
