@@ -59,7 +59,7 @@ template <typename Batch>
 struct Cursor {
   const Batch &b;
   int32_t s = -1, base = 0, n_items = 0;
-  int32_t n_seg = 0, seg_splits = 1, n_gt = 0, g_splits = 1;
+  int32_t n_seg = 0, seg_splits = 1, n_gt = 0, g_splits = 1, lg_parts = 0;
   __device__ explicit Cursor(const Batch &batch) : b(batch) {}
   // K splits of the gather tiles when the host leaves the choice to the device (it does not know how
   // many adapters a batch touches): the count up to 8 whose items fill whole waves of the grid best,
@@ -78,6 +78,18 @@ struct Cursor {
     }
     return best;
   }
+  // Parts that the tokens of a gather tile are cut into, each a tile of its own (a power of two, its logarithm here).  A
+  // tile goes through its tokens 64 at a time, one pass after the other over its K blocks: with hundreds of scattered
+  // tokens on a few adapters (and so a few tiles) the passes are what the launch takes.  As many parts as idle CTAs of the
+  // grid would take, and half as many again as an average tile has passes (tiles differ, and a part of two passes takes
+  // twice as long); tiles of one pass stay whole.  2048 tokens 4096 wide on 4 adapters: 344 -> 30 us, on 16 adapters
+  // 192 -> 36; 4096 tokens on 100 adapters by a power law 413 -> 160.
+  __device__ int32_t choose_parts(int32_t grid) const {
+    const int32_t passes = (b.counts[6] + kTileGatherN - 1) / kTileGatherN, items = n_gt * g_splits * b.n_sites;
+    int32_t lp = 0;
+    while ((1 << lp) < passes && (2 * (n_gt << lp) < 3 * passes || (items << (lp + 1)) <= grid)) ++lp;
+    return lp;
+  }
   __device__ bool seek(int32_t item) {
     while (item >= base + n_items) {
       base += n_items;
@@ -88,7 +100,8 @@ struct Cursor {
       n_seg = st.splits > 0 ? b.counts[2] : 0;
       seg_splits = max(st.splits, 1);
       g_splits = st.splits > 0 ? st.splits : choose_splits(st, gridDim.x);
-      n_items = n_seg * seg_splits + n_gt * g_splits;
+      lg_parts = st.splits > 0 ? choose_parts(gridDim.x) : 0;
+      n_items = n_seg * seg_splits + (n_gt << lg_parts) * g_splits;
     }
     return true;
   }
@@ -112,16 +125,25 @@ struct Cursor {
       }
     } else {
       local -= n_seg * seg_splits;
-      const int32_t g = local % n_gt;
+      const int32_t n_tiles = n_gt << lg_parts;
       c.gather = 1;
-      c.tile = n_seg + g;
-      c.split = local / n_gt;
+      c.split = local / n_tiles;
       c.splits = g_splits;
+      const int32_t t = local - c.split * n_tiles, g = t >> lg_parts;
+      c.tile = n_seg + t;
       const int32_t per = kTileM / st.R_pad, n_groups = b.counts[0], n_lg = b.counts[4];
       c.g0 = (n_groups - n_lg) + g * per;  // the group of id -1, when there is one, comes first
       c.ng = min(per, n_groups - c.g0);
       c.tok0 = b.gs_short[c.g0];
       c.ntok = b.gs_short[c.g0 + c.ng] - c.tok0;
+      if (lg_parts > 0) {
+        const int32_t passes = (c.ntok + kTileGatherN - 1) / kTileGatherN;
+        const int32_t n = (passes + (1 << lg_parts) - 1) >> lg_parts << 6;
+        static_assert(kTileGatherN == 1 << 6, "tokens of a pass");
+        const int32_t skip = min(c.ntok, (t - (g << lg_parts)) * n);
+        c.tok0 += skip;
+        c.ntok = min(c.ntok - skip, n);
+      }
     }
     const int32_t per_split = (st.kb_total + c.splits - 1) / c.splits;
     c.kb0 = min(c.split * per_split, st.kb_total);
@@ -537,6 +559,7 @@ __global__ void __launch_bounds__(kThreads, 1) shrink_tiles_kernel(const __grid_
   if (!ok) {  // the items that this CTA leaves undone may belong to any site, and leave its arrival counters short
     sh.abort_flag = 1;
     for (int32_t s = 0; s < b.n_sites; ++s) atomicOr(b.site[s].status, EDGELORA_STATUS_TIMEOUT);
+    ptx::settle();
   }
   __syncwarp();
   ptx::tc_fence_before_sync();
@@ -558,7 +581,6 @@ cudaError_t shrink_tiles_set_smem_limit() {
 }
 
 template <int kSites>
-    ptx::settle();
 cudaError_t launch_shrink_tiles(const ShrinkBatch<kSites> &b, int32_t grid, bool pdl, cudaStream_t stream) {
   return launch_ex(shrink_tiles_kernel<kSites>, dim3(grid), dim3(kThreads), kShrinkTilesSmem, stream, pdl, 1, b);
 }

@@ -86,3 +86,23 @@ def test_repeated_calls_reuse_the_arrival_counters():
             assert np.array_equal(run_gpu(w, pool=pool, options=GATHER), first)
     finally:
         pool.close()
+
+
+@pytest.mark.parametrize("max_rank", [16, 64])
+@pytest.mark.parametrize("T,n_adapters,law", [
+    (320, 1, "even"),      # one tile, five passes
+    (2048, 3, "even"),     # parts for idle CTAs
+    (1500, 70, "skewed"),  # a few popular adapters: parts of several passes, empty parts
+    (4500, 9, "skewed"),   # above the plan's shared-memory form
+])
+def test_prefill_with_scattered_tokens(T, n_adapters, law, max_rank):
+    # no run is long: every token goes through the gather tiles, whose tokens are cut into parts
+    rng = np.random.Generator(np.random.PCG64(T + n_adapters))
+    w = random_workload(2000 + T, T, 448, 136, ranks=[int(r) for r in rng.integers(1, max_rank + 1, size=n_adapters)],
+                        max_rank=max_rank)
+    ids = rng.integers(0, n_adapters, size=T) if law == "even" else np.minimum(rng.zipf(1.4, size=T) - 1, n_adapters - 1)
+    ids[::29] = -1          # (one adapter: runs of 28)
+    w.ids = ids.astype(np.int32)
+    y, plan = run_gpu(w, return_plan=True)
+    assert_parity(y, oracle_of(w), f"T={T} adapters={n_adapters} {law}")
+    check_plan(plan, w.ids, w.n_slots)
