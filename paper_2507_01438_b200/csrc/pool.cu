@@ -921,7 +921,7 @@ static int prefill_batch(const SiteCall *sites, int n, edgelora_plan *plan, int3
   for (int i = 0; i < n; ++i) {
     int64_t *info = sites[i].p->last_info;
     info[1] = 2;
-    info[2] = 2 * std::max(1, std::min(p0->sms / 2, tiles));
+    info[2] = pair_grid(tiles, p0->sms);
     info[3] = 1;
     info[4] = pb.stages;
     info[5] = BN;

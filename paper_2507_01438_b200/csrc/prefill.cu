@@ -535,17 +535,18 @@ cudaError_t pair_set_smem_limit() {
   return e;
 }
 
-// Tiles come off the launch queue when the pairs run through more than four waves of them; shorter launches have
-// no time to drift, and a kernel that uses the launch queue does not start under the tail of the kernel in front
-// of it (4096 -> 4096, T = 300: 46 us per call against 37.5 us; 3080 -> 5000, T = 1111: 88 against 82 us).
+// Tiles come off the launch queue when the pairs run through more than four waves of them.  Shorter launches have no time
+// to drift, and a kernel that uses the launch queue does not start under the tail of the kernel in front of it: 1 to 3 us
+// per call in favour of the static deal up to four waves (4096 -> 6144, T = 2112, 2.9 waves: 96 against 99 us).  At five
+// to seven waves the two differ by less than runs of one do (4096 -> 20480, T = 1024: 133-152 against 144-152 us), from
+// nine on the queue is ahead (14 sites, T = 300: 398-459 against 428-536 us; T = 1024: 757-792 against 823-868 us).
 template <int kSites>
 cudaError_t launch_pair_gemm(const PairBatch<kSites> &b, int32_t sms, bool pdl, cudaStream_t stream) {
-  const int32_t tiles = b.site[b.n_sites - 1].tile_end, units = std::max(1, sms / 2);
+  const int32_t tiles = b.site[b.n_sites - 1].tile_end, grid = pair_grid(tiles, sms);
   const size_t smem = pair_smem_bytes(b.stages, b.BN);
-  if (tiles > 4 * units)
-    return launch_ex(pair_gemm_kernel<kSites, true>, dim3(2 * tiles), dim3(kThreads), smem, stream, pdl, 2, b);
-  return launch_ex(pair_gemm_kernel<kSites, false>, dim3(2 * std::min(tiles, units)), dim3(kThreads), smem, stream, pdl, 2,
-                   b);
+  if (pair_queued(tiles, sms))
+    return launch_ex(pair_gemm_kernel<kSites, true>, dim3(grid), dim3(kThreads), smem, stream, pdl, 2, b);
+  return launch_ex(pair_gemm_kernel<kSites, false>, dim3(grid), dim3(kThreads), smem, stream, pdl, 2, b);
 }
 template cudaError_t launch_pair_gemm<1>(const PairBatch<1> &, int32_t, bool, cudaStream_t);
 template cudaError_t launch_pair_gemm<kPairSites>(const PairBatch<kPairSites> &, int32_t, bool, cudaStream_t);

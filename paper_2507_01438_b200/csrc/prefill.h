@@ -36,6 +36,12 @@ struct PairBatch {
 };
 
 int pair_stages(int BN);
+// Launches of more than four tiles per pair take them off the launch queue (a cluster per tile); the others deal them to
+// the pairs that fit the device (see launch_pair_gemm).
+inline bool pair_queued(int32_t tiles, int32_t sms) { return tiles > 4 * std::max(1, sms / 2); }
+inline int32_t pair_grid(int32_t tiles, int32_t sms) {  // CTAs
+  return 2 * (pair_queued(tiles, sms) ? tiles : std::min(tiles, std::max(1, sms / 2)));
+}
 cudaError_t pair_set_smem_limit();
 template <int kSites>
 cudaError_t launch_pair_gemm(const PairBatch<kSites> &b, int32_t sms, bool pdl, cudaStream_t stream);

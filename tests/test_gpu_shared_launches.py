@@ -193,3 +193,18 @@ def test_a_non_finite_adapter_reaches_its_own_tokens_only(T, n_adapters, rank):
         assert not np.isfinite(got[bad]).any()
     finally:
         pool.close()
+
+
+@pytest.mark.parametrize("T,h_out", [(300, 264), (513, 40000)])
+def test_the_reported_grid_is_the_launch(T, h_out):
+    # a tile per pair while the pairs of the device hold them, a cluster per tile off the launch queue
+    import torch
+    w = random_workload(51, T, 64, h_out, ranks=[16], max_rank=16)
+    pool = make_pool(w)
+    try:
+        pool.linear(to_dev_bf16(w.W), to_dev_bf16(w.x), torch.from_numpy(w.ids).cuda())
+        info = B.edgelora_pool_last_launch(pool.handle)
+        tiles = -(-T // 256) * -(-h_out // info["n_tile"])
+        assert info["gemm_grid"] == 2 * tiles
+    finally:
+        pool.close()
