@@ -208,3 +208,58 @@ def test_the_reported_grid_is_the_launch(T, h_out):
         assert info["gemm_grid"] == 2 * tiles
     finally:
         pool.close()
+
+
+def test_sites_of_different_rank_strides_off_the_launch_queue():
+    T = 513
+    ids = mixed_ids(61, 40, [(0, 200), (2, 31), (1, 242)], 4)
+    sites = []
+    for i, (h_in, h_out, rank) in enumerate([(264, 16384, 16), (72, 16384, 64), (1032, 2056, 32), (264, 136, 64)]):
+        sites += make_sites(62 + i, T, [(h_in, h_out)], [rank, rank // 2, 4, rank], rank, ids)[1]
+    with SetOf(sites, [0, 1, 2, 3]) as s:
+        s.run([to_dev_bf16(w.x) for w in sites])
+        info = B.edgelora_pool_last_launch(s.pools[0].handle)
+        assert info["launches"] == 2 and info["gemm_grid"] > 148     # one run, a cluster per tile
+        s.check(rows=np.array([0, 7, 39, 40, 239, 240, 255, 256, 270, 271, 400, 512]))
+
+
+def test_more_sites_than_one_launch_takes_on_few_inputs():
+    ids = mixed_ids(65, 20, [(1, 250), (0, 40)], 3)
+    shapes = [((64, 128, 72)[i % 3], 64 + 8 * i) for i in range(35)]   # 35 sites on three inputs: 32 and 3
+    xs, sites = make_sites(66, len(ids), shapes, [16, 8, 4], 16, ids)
+    with SetOf(sites, [i % 3 for i in range(35)]) as s:
+        s.run([to_dev_bf16(xs[h]) for h in (64, 128, 72)])
+        s.check()
+        assert [B.edgelora_pool_last_launch(p.handle)["launches"] for p in s.pools] == [2] + [0] * 31 + [2, 0, 0]
+
+
+def test_a_captured_set_of_a_large_batch():
+    import torch
+    ids = mixed_ids(67, 30, [(1, 250), (0, 60)], 3)
+    xs, sites = make_sites(68, len(ids), [(256, 264), (512, 128), (256, 520)], [16, 8, 4], 16, ids)
+    rng = np.random.Generator(np.random.PCG64(69))
+    with SetOf(sites, [0, 1, 0]) as s:
+        x = [to_dev_bf16(xs[256]), to_dev_bf16(xs[512])]
+        for p in s.pools:
+            B.edgelora_pool_wait_loads(p.handle)
+        stream = torch.cuda.Stream()
+        stream.wait_stream(torch.cuda.current_stream())
+        s.run(x, stream)
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            s.run(x, stream)
+        for _ in range(2):                 # the replay reads what the buffers hold now
+            for i, h in ((0, 256), (1, 512)):
+                new = wl.normal_bf16(rng, xs[h].shape, 1.0)
+                x[i].copy_(to_dev_bf16(new))
+                for w in sites:
+                    if w.h_in == h:
+                        w.x = new
+            for y in s.ys:
+                y.fill_(float("nan"))
+            torch.cuda.synchronize()
+            with torch.cuda.stream(stream):
+                graph.replay()
+            stream.synchronize()
+            s.check("replay")
