@@ -54,6 +54,39 @@ struct Item {
   int32_t tile, split, splits, kb0, kb1;  // tile: index of its arrival counter
 };
 
+// The two choices below are made once per site and role, most of the time not at all, and kept out of line: four roles
+// walk the items, and the fetch of their code is part of a launch of ten microseconds.
+//
+// K splits of the gather tiles when the host leaves the choice to the device (it does not know how
+// many adapters a batch touches): the count up to 8 whose items fill whole waves of the grid best,
+// each split keeping at least four K blocks.
+__device__ __noinline__ int32_t choose_splits(int32_t kb_total, int32_t n_gt, int32_t grid) {
+  int32_t best = 1;
+  float best_eff = 0.f;
+  for (int32_t sp = 1; sp <= 8 && kb_total / sp >= 4; ++sp) {
+    if ((sp - 1) * ((kb_total + sp - 1) / sp) >= kb_total) continue;  // every split needs a K block
+    const int32_t items = n_gt * sp, waves = (items + grid - 1) / grid;
+    const float eff = waves > 0 ? static_cast<float>(items) / static_cast<float>(waves * grid) : 0.f;
+    if (eff > best_eff + 0.02f) {
+      best_eff = eff;
+      best = sp;
+    }
+  }
+  return best;
+}
+// Parts that the tokens of a gather tile are cut into, each a tile of its own (a power of two, its logarithm here).  A
+// tile goes through its tokens 64 at a time, one pass after the other over its K blocks: with hundreds of scattered
+// tokens on a few adapters (and so a few tiles) the passes are what the launch takes.  As many parts as idle CTAs of the
+// grid would take, and half as many again as an average tile has passes (tiles differ, and a part of two passes takes
+// twice as long); tiles of one pass stay whole.  2048 tokens 4096 wide on 4 adapters: 344 -> 30 us, on 16 adapters
+// 192 -> 36; 4096 tokens on 100 adapters by a power law 413 -> 160.
+__device__ __noinline__ int32_t choose_parts(int32_t n_tok, int32_t n_gt, int32_t items, int32_t grid) {
+  const int32_t passes = (n_tok + kTileGatherN - 1) / kTileGatherN;
+  int32_t lp = 0;
+  while ((1 << lp) < passes && (2 * (n_gt << lp) < 3 * passes || (items << (lp + 1)) <= grid)) ++lp;
+  return lp;
+}
+
 // Walks the items of all sites in order.
 template <typename Batch>
 struct Cursor {
@@ -61,35 +94,6 @@ struct Cursor {
   int32_t s = -1, base = 0, n_items = 0;
   int32_t n_seg = 0, seg_splits = 1, n_gt = 0, g_splits = 1, lg_parts = 0;
   __device__ explicit Cursor(const Batch &batch) : b(batch) {}
-  // K splits of the gather tiles when the host leaves the choice to the device (it does not know how
-  // many adapters a batch touches): the count up to 8 whose items fill whole waves of the grid best,
-  // each split keeping at least four K blocks.
-  __device__ int32_t choose_splits(const ShrinkSite &st, int32_t grid) const {
-    int32_t best = 1;
-    float best_eff = 0.f;
-    for (int32_t sp = 1; sp <= 8 && st.kb_total / sp >= 4; ++sp) {
-      if ((sp - 1) * ((st.kb_total + sp - 1) / sp) >= st.kb_total) continue;  // every split needs a K block
-      const int32_t items = n_gt * sp, waves = (items + grid - 1) / grid;
-      const float eff = waves > 0 ? static_cast<float>(items) / static_cast<float>(waves * grid) : 0.f;
-      if (eff > best_eff + 0.02f) {
-        best_eff = eff;
-        best = sp;
-      }
-    }
-    return best;
-  }
-  // Parts that the tokens of a gather tile are cut into, each a tile of its own (a power of two, its logarithm here).  A
-  // tile goes through its tokens 64 at a time, one pass after the other over its K blocks: with hundreds of scattered
-  // tokens on a few adapters (and so a few tiles) the passes are what the launch takes.  As many parts as idle CTAs of the
-  // grid would take, and half as many again as an average tile has passes (tiles differ, and a part of two passes takes
-  // twice as long); tiles of one pass stay whole.  2048 tokens 4096 wide on 4 adapters: 344 -> 30 us, on 16 adapters
-  // 192 -> 36; 4096 tokens on 100 adapters by a power law 413 -> 160.
-  __device__ int32_t choose_parts(int32_t grid) const {
-    const int32_t passes = (b.counts[6] + kTileGatherN - 1) / kTileGatherN, items = n_gt * g_splits * b.n_sites;
-    int32_t lp = 0;
-    while ((1 << lp) < passes && (2 * (n_gt << lp) < 3 * passes || (items << (lp + 1)) <= grid)) ++lp;
-    return lp;
-  }
   __device__ bool seek(int32_t item) {
     while (item >= base + n_items) {
       base += n_items;
@@ -99,8 +103,9 @@ struct Cursor {
       n_gt = (b.counts[4] + per - 1) / per;
       n_seg = st.splits > 0 ? b.counts[2] : 0;
       seg_splits = max(st.splits, 1);
-      g_splits = st.splits > 0 ? st.splits : choose_splits(st, gridDim.x);
-      lg_parts = st.splits > 0 ? choose_parts(gridDim.x) : 0;
+      g_splits = st.splits > 0 ? st.splits : choose_splits(st.kb_total, n_gt, gridDim.x);
+      const int32_t n_tok = st.splits > 0 ? b.counts[6] : 0;
+      lg_parts = n_tok > kTileGatherN ? choose_parts(n_tok, n_gt, n_gt * g_splits * b.n_sites, gridDim.x) : 0;
       n_items = n_seg * seg_splits + (n_gt << lg_parts) * g_splits;
     }
     return true;
@@ -414,7 +419,6 @@ __global__ void __launch_bounds__(kThreads, 1) shrink_tiles_kernel(const __grid_
           scale = row.scale;
           c_lo = b.gs_short[tc.g0 + gi] - tc.tok0;
           c_hi = b.gs_short[tc.g0 + gi + 1] - tc.tok0;
-          if (!live && r == 0 && tc.split == 0 && c_hi > c_lo) atomicOr(st.status, EDGELORA_STATUS_SLOT_EMPTY);
         }
         const int32_t n_pass = passes_of(tc);
         for (int32_t pass = 0; ok && pass < n_pass; ++pass, ++it) {
@@ -453,9 +457,7 @@ __global__ void __launch_bounds__(kThreads, 1) shrink_tiles_kernel(const __grid_
       } else {
         // segment tile: row = token of the run, columns = rank index; z partial = scale * acc
         const uint32_t acc = it & 1;
-        const SlotRow slot = st.slots[tc.slot];
-        const float scale = slot.scale;
-        if (slot.rank <= 0 && tc.nrows > 0 && tc.split == 0 && etid == 0) atomicOr(st.status, EDGELORA_STATUS_SLOT_EMPTY);
+        const float scale = st.slots[tc.slot].scale;
         ok = wait_acc(acc);
         if (!ok) break;
         ++it;
@@ -525,7 +527,10 @@ __global__ void __launch_bounds__(kThreads, 1) shrink_tiles_kernel(const __grid_
           }
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
-            if (rank[q] <= 0) continue;
+            if (rank[q] <= 0) {
+              if (tok[q] >= 0) atomicOr(st.status, EDGELORA_STATUS_SLOT_EMPTY);
+              continue;
+            }
             const int c = (i0 + q * 128) % nch;
             if (b.z_bf16) {
               reinterpret_cast<uint4 *>(out)[static_cast<size_t>(tok[q]) * nch + c] = pack_z_chunk(acc[q], c * 8, rank[q]);
