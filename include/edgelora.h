@@ -112,8 +112,11 @@ typedef struct {
                                         such grids could each hold SMs the other needs, and the wait would
                                         end in EDGELORA_ERR_TIMEOUT */
 #define EDGELORA_OPT_WAIT_CYCLES 6   /* limit of every bounded in-kernel wait of the layer, in units
-                                        of 1024 SM clock cycles; 0 = default (about two seconds).
-                                        A wait that runs out raises EDGELORA_STATUS_TIMEOUT           */
+                                        of 1024 SM clock cycles; 0 = default (about two seconds).  One
+                                        try of a barrier may last some microseconds whatever the limit,
+                                        and the copies of the decode shrink keep the default.  A wait
+                                        that runs out raises EDGELORA_STATUS_TIMEOUT, in every pool of a
+                                        launch that several pools share                               */
 
 /* Bytes of device memory the slot blocks need for this geometry (what arena_bytes must
  * be at least).  Host-only arithmetic. */

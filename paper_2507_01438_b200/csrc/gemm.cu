@@ -515,7 +515,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
           }
         }
         if (!got) atomicOr(p.status, EDGELORA_STATUS_TIMEOUT);
-        *s_last = got;  // (the gather tiles' flag: unused in this launch)
+        *s_last = got;
       }
       named_bar_sync(1, 128);
       fused_z_ok = *s_last != 0;

@@ -1,8 +1,8 @@
 // Shrink for small decode batches: z[t] = s_a * A_a x[t] for tokens scattered across adapters
 // (paper Section 2.1 for A: r x h_in; Section 4.3: tokens that share an adapter are handled as one
 // sub-batch so the adapter is fetched once), with the routing derived inside the kernel so that a
-// step of a few microseconds needs no routing launch.  Larger batches take the tensor-core gather
-// tiles of the tile kernel (gemm.cu).
+// step of a few microseconds needs no routing launch.  Larger batches take the tensor-core tiles of
+// shrink_tiles.cu.
 #include <cuda_fp16.h>
 
 #include "decode_route.cuh"

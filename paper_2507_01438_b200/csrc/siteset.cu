@@ -45,6 +45,13 @@ bool capturing(cudaStream_t s) {
   return st != cudaStreamCaptureStatusNone;
 }
 
+// Sites of a run that holds a result to be read back: the copy starts behind the run, so a long run delays it, and a short
+// one pays for its own launches.  28 sites of four decoder layers, host call, us for runs of 1 / 4 / 7 / 14 / 32 sites:
+// T = 2112, last layer read back 6512 / 6509 / 6857 / 6858 / 7161, the down projections 4092 / 4109 / 4214 / 4397 / 5015, k
+// and v 3839 / 3836 / 3779 / 3932 / 4209; T = 320, last layer 1412 / 1322 / 1444 / 1438 / 1449, the down projections 1081 /
+// 1083 / 1028 / 1055 / 1173, k and v 1264 / 1100 / 1013 / 1034 / 1061; all results: no difference.
+constexpr int kReadBackRun = 7;
+
 bool overlap(const void *a, size_t na, const void *b, size_t nb) {
   const uintptr_t pa = reinterpret_cast<uintptr_t>(a), pb = reinterpret_cast<uintptr_t>(b);
   return pa < pb + nb && pb < pa + na;
@@ -96,8 +103,8 @@ int run_sites(edgelora_siteset *s, const void *const *x_dev, const int32_t *ids_
     // A run ends where the launch's tables are full, where a pool would come twice (its z workspace holds one
     // site's z), where two sites write the same memory (the later one is to be seen; results that the host call
     // does not read back share a buffer nobody looks at), where the pools' wait limits differ (a launch has one), in
-    // front of a site whose input is still on its way, and behind about a decoder layer of sites when results are read
-    // back beside the sites that follow.  Profiled pools go one by one.
+    // front of a site whose input is still on its way, and behind kReadBackRun sites when results are read back beside
+    // the sites that follow.  Profiled pools go one by one.
     SiteCall calls[kPairSites];
     SiteCall inputs[kPairInputs];  // the first site on each input
     int m = 0, n_inputs = 0;
@@ -106,7 +113,7 @@ int run_sites(edgelora_siteset *s, const void *const *x_dev, const int32_t *ids_
       edgelora_pool *p = s->pools[i];
       const SiteCall call{p, s->W[i], static_cast<const uint16_t *>(x_dev[s->input_of[i]]), y_dev[i]};
       if (m > 0 && ((before && (*before)[i]) || p->opt_profile || calls[0].p->opt_profile ||
-                    p->wait_cycles != calls[0].p->wait_cycles || (read_back && m >= 7)))
+                    p->wait_cycles != calls[0].p->wait_cycles || (read_back && m >= kReadBackRun)))
         break;
       bool again = false;
       for (int k = 0; k < m; ++k)

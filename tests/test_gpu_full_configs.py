@@ -81,8 +81,8 @@ def full_set_rows(batch):
 
 @pytest.mark.parametrize("layer", [0, 15, 31])
 def test_full_projection_set_whole_layers_through_the_site_set(layer):
-    # the seven projections of a decoder layer as one set of sites: one plan, the sites back to
-    # back with the next site's shrink riding on the current site's launches (what bench.py times)
+    # the seven projections of a decoder layer as one set of sites: one plan, the sites in shared
+    # launches (what bench.py times, there with 32 sites to a launch)
     import torch
     batch = wl.full_set_batch()
     assert batch.ids.shape[0] == 2112

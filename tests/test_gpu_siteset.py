@@ -1,5 +1,5 @@
-"""A set of linear sites over one batch (edgelora_siteset_*): one routing plan, the sites run back
-to back with the next site's shrink issued alongside the current site's kernels.  Every site's
+"""A set of linear sites over one batch (edgelora_siteset_*): one routing plan, the sites of a large
+batch in shared launches, those of a decode-sized batch one after the other.  Every site's
 result is compared with the CPU oracle of that site, element by element; the plan bit for bit.
 """
 import numpy as np
@@ -78,8 +78,8 @@ def check_plan(plan, ids, n_slots):
 
 @pytest.mark.parametrize("host", [False, True])
 def test_prefill_sized_set_with_ragged_ranks(host):
-    # 40 scattered tokens, then runs of 300 / 70 / 20 tokens (long runs go through the segment shrink
-    # that rides on the previous site's launch, the short ones through the gather shrink beside it)
+    # 40 scattered tokens, then runs of 300 / 70 / 20 tokens (long runs go through the segment tiles
+    # of the shrink, the short ones through its gather tiles)
     ranks = [8, 16, 32, 4, 0, 32, 12]
     ids = mixed_ids(3, 40, [(2, 300), (5, 70), (0, 20), (-1, 37)], len(ranks))
     ids[ids == 4] = -1                                   # slot 4 is empty
