@@ -98,6 +98,8 @@ __device__ __forceinline__ bool next_tile(Barriers &sh, int32_t it, uint32_t nem
   if (!kWarp || (threadIdx.x & 31) == 0) ptx::mbar_arrive_cluster(nempty);
   return got;
 }
+// Adapters of a LoRA K block: 64 / R_pad (16, 32 or 64), without the division.
+__device__ __forceinline__ int32_t lora_per(int32_t R_pad) { return kBlockK >> (31 - __clz(R_pad)); }
 constexpr int kAnswerReaders = 10 + 9;  // TMA, MMA, 4 epilogue and 4 builder warps of CTA 0; CTA 1 issues no MMAs
 
 }  // namespace
@@ -196,7 +198,7 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
           break;
         }
         const int32_t cnt = sh.count[buf];
-        const int32_t per = kBlockK / st.R_pad;  // adapters of a LoRA K block
+        const int32_t per = lora_per(st.R_pad);  // adapters of a LoRA K block
         const uint32_t b_bytes = static_cast<uint32_t>(b.BN * st.R_pad);  // a CTA's half of one adapter's rows
         for (int32_t e0 = 0, blk = 0; e0 < cnt; e0 += per, ++blk) {
           const int32_t n = min(per, cnt - e0);
@@ -271,9 +273,9 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
           break;
         }
         const int32_t cnt = sh.count[buf];
-        const int32_t per = kBlockK / st.R_pad;
+        const int32_t per = lora_per(st.R_pad);
         const uint32_t b_bytes = static_cast<uint32_t>(b.BN * st.R_pad), row_bytes = static_cast<uint32_t>(st.R_pad) * 2;
-        const int ksteps = st.R_pad / kUmmaK;
+        const int ksteps = st.R_pad >> 4;  // K steps of 16
         for (int32_t e0 = 0, blk = 0; e0 < cnt; e0 += per, ++blk) {
           const bool has_z = blk < static_cast<int32_t>(nstages);  // (later blocks find z in the stage, see the builder)
           ok = ptx::mbar_wait(&sh.mfull[stage], (mphase >> stage) & 1u, wl);
@@ -458,7 +460,7 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
       // of many adapters is the hand-over of a stage with the latency of its B_a rows, hence 64 / R_pad adapters to a
       // stage: 300 tokens on 300 adapters of rank 16, 4096 -> 4096: 61 us, 115 with one adapter to a stage, 123 with z
       // masked and written anew for every adapter.
-      const int32_t per = kBlockK / st.R_pad;
+      const int32_t per = lora_per(st.R_pad);
       for (int32_t e0 = 0, blk = 0; e0 < total; e0 += per, ++blk) {
         const bool write_z = blk < static_cast<int32_t>(nstages);
         const uint32_t stage = count % nstages;
