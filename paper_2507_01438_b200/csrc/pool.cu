@@ -18,6 +18,7 @@
 #include "pool.h"
 #include "prefill.h"
 #include "shrink_tiles.h"
+#include "tile_order.h"
 
 using namespace edgelora;
 
@@ -369,11 +370,10 @@ int edgelora_pool_create(const edgelora_pool_config *cfg, edgelora_pool_t **pool
   POOL_TRY(el_malloc(&p->zws, sizeof(float) * (kMaxZSplits + 1) * static_cast<size_t>(p->cfg.max_tokens) * p->R_pad));
   POOL_TRY(el_malloc(&p->group_counters, sizeof(int32_t) * (kDecodeMaxT * 8 + 32)));
   POOL_TRY(cudaMemset(p->group_counters, 0, sizeof(int32_t) * (kDecodeMaxT * 8 + 32)));
-  // an arrival counter per tile of the tensor-core shrink: segment tiles, then gather tiles in parts (a power of two: up
-  // to twice the passes of an average tile, or a part per CTA of the grid)
+  // an arrival counter per tile of the tensor-core shrink: segment tiles, then gather tiles (in parts)
+  const int max_gather = (std::min(p->cfg.max_tokens, p->cfg.n_slots) * p->R_pad + kTileM - 1) / kTileM;
   p->n_tile_counters = p->cfg.max_tokens / kSegMin + 8 +
-                       (std::min(p->cfg.max_tokens, p->cfg.n_slots) * p->R_pad + kTileM - 1) / kTileM +
-                       2 * (p->cfg.max_tokens / kTileGatherN + 1) + p->sms;
+                       static_cast<int32_t>(gather_tiles_max(p->cfg.max_tokens, max_gather, p->sms));
   POOL_TRY(el_malloc(&p->tile_counters, sizeof(int32_t) * p->n_tile_counters));
   POOL_TRY(cudaMemset(p->tile_counters, 0, sizeof(int32_t) * p->n_tile_counters));
   POOL_TRY(gemm_set_smem_limit(kSmemBudget));

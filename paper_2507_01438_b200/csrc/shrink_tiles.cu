@@ -22,12 +22,14 @@
 #include "launch.cuh"
 #include "ptx.cuh"
 #include "shrink_tiles.h"
+#include "tile_order.h"
 #include "zload.cuh"
 
 namespace edgelora {
 
 namespace {
 
+static_assert(kTileGatherN == kGatherPass, "tokens of a pass");
 constexpr int kThreads = 320;
 constexpr uint32_t kRBytes = kTileM * kBlockK * 2;
 constexpr uint32_t kStageBytes = kRBytes + kTileGatherN * kBlockK * 2;  // C: up to 64 rows (A_a, or gathered tokens)
@@ -74,17 +76,8 @@ __device__ __noinline__ int32_t choose_splits(int32_t kb_total, int32_t n_gt, in
   }
   return best;
 }
-// Parts that the tokens of a gather tile are cut into, each a tile of its own (a power of two, its logarithm here).  A
-// tile goes through its tokens 64 at a time, one pass after the other over its K blocks: with hundreds of scattered
-// tokens on a few adapters (and so a few tiles) the passes are what the launch takes.  As many parts as idle CTAs of the
-// grid would take, and half as many again as an average tile has passes (tiles differ, and a part of two passes takes
-// twice as long); tiles of one pass stay whole.  2048 tokens 4096 wide on 4 adapters: 344 -> 30 us, on 16 adapters
-// 192 -> 36; 4096 tokens on 100 adapters by a power law 413 -> 160.
 __device__ __noinline__ int32_t choose_parts(int32_t n_tok, int32_t n_gt, int32_t items, int32_t grid) {
-  const int32_t passes = (n_tok + kTileGatherN - 1) / kTileGatherN;
-  int32_t lp = 0;
-  while ((1 << lp) < passes && (2 * (n_gt << lp) < 3 * passes || (items << (lp + 1)) <= grid)) ++lp;
-  return lp;
+  return gather_parts_lg(n_tok, n_gt, items, grid);
 }
 
 // Walks the items of all sites in order.
@@ -142,12 +135,9 @@ struct Cursor {
       c.tok0 = b.gs_short[c.g0];
       c.ntok = b.gs_short[c.g0 + c.ng] - c.tok0;
       if (lg_parts > 0) {
-        const int32_t passes = (c.ntok + kTileGatherN - 1) / kTileGatherN;
-        const int32_t n = (passes + (1 << lg_parts) - 1) >> lg_parts << 6;
-        static_assert(kTileGatherN == 1 << 6, "tokens of a pass");
-        const int32_t skip = min(c.ntok, (t - (g << lg_parts)) * n);
-        c.tok0 += skip;
-        c.ntok = min(c.ntok - skip, n);
+        const GatherPart part = gather_part(c.ntok, t - (g << lg_parts), lg_parts);
+        c.tok0 += part.skip;
+        c.ntok = part.n;
       }
     }
     const int32_t per_split = (st.kb_total + c.splits - 1) / c.splits;

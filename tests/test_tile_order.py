@@ -1,4 +1,5 @@
-"""The order in which the pair kernel's roles walk a launch's tiles, and the end of its operand ring, on the CPU: csrc/tile_order.h is plain C++ and is
+"""The order in which the pair kernel's roles walk a launch's tiles, the end of its operand ring, and the parts of the
+shrink's gather tiles, on the CPU: csrc/tile_order.h is plain C++ and is
 compiled here with the host compiler.
 """
 import ctypes
@@ -30,6 +31,17 @@ extern "C" int32_t drain(uint32_t used, uint32_t nstages, uint32_t *stage, uint3
   *stage = p.stage;
   *phase = p.phase;
   return 0;
+}
+extern "C" int32_t parts_lg(int32_t n_tok, int32_t n_tiles, int32_t items, int32_t grid) {
+  return edgelora::gather_parts_lg(n_tok, n_tiles, items, grid);
+}
+extern "C" void part(int32_t n_tok, int32_t p, int32_t lg, int32_t *out) {
+  const edgelora::GatherPart g = edgelora::gather_part(n_tok, p, lg);
+  out[0] = g.skip;
+  out[1] = g.n;
+}
+extern "C" int64_t tiles_max(int32_t max_tokens, int32_t max_tiles, int32_t grid) {
+  return edgelora::gather_tiles_max(max_tokens, max_tiles, grid);
 }
 """
 
@@ -81,3 +93,34 @@ def test_the_drain_waits_for_the_last_use_of_every_stage(lib, nstages):
             if s == nstages:
                 s, ph = 0, ph ^ 1
         assert sorted(waited) == list(range(min(used, nstages)))
+
+
+def test_the_parts_of_a_gather_tile_are_its_tokens_in_whole_passes(lib):
+    out = (ctypes.c_int32 * 2)()
+    for n_tok in (0, 1, 63, 64, 65, 300, 1024, 1025, 32768):
+        for lg in range(0, 10):
+            at = 0
+            for p in range(1 << lg):
+                lib.part(n_tok, p, lg, out)
+                assert out[0] == at and out[1] >= 0
+                assert out[1] % 64 == 0 or out[0] + out[1] == n_tok
+                at += out[1]
+            assert at == n_tok
+
+
+def test_the_gather_tiles_of_a_batch_fit_the_arrival_counters(lib):
+    lib.tiles_max.restype = ctypes.c_int64
+    grid = 148
+    for max_tokens in (257, 1000, 4096, 9500, 32768):
+        for n_slots in (1, 3, 100, 65534):
+            for r_pad in (16, 32, 64):
+                max_tiles = -(-min(max_tokens, n_slots) * r_pad // 128)
+                bound = lib.tiles_max(max_tokens, max_tiles, grid)
+                for n_tok in sorted({1, 64, 65, 300, max_tokens // 3, max_tokens}):
+                    for n_tiles in sorted({1, 2, 3, 7, max_tiles // 5, max_tiles}):
+                        if not 1 <= n_tiles <= min(max_tiles, n_tok):
+                            continue
+                        for splits, n_sites in ((1, 1), (8, 1), (2, 32)):
+                            lg = lib.parts_lg(n_tok, n_tiles, n_tiles * splits * n_sites, grid)
+                            assert (n_tiles << lg) <= bound and (1 << lg) < 2 * max(1, -(-n_tok // 64))
+                            assert lg == 0 or n_tok > 64
