@@ -278,12 +278,8 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
         const int ksteps = st.R_pad >> 4;  // K steps of 16
         for (int32_t e0 = 0, blk = 0; e0 < cnt; e0 += per, ++blk) {
           const bool has_z = blk < static_cast<int32_t>(nstages);  // (later blocks find z in the stage, see the builder)
-          ok = ptx::mbar_wait(&sh.mfull[stage], (mphase >> stage) & 1u, wl);
-          // (the builder is ahead of the loads as a rule: the first adapter's rows are read while those are on their way)
-          uint4 off_lo = *reinterpret_cast<const uint4 *>(&sh.off[stage][0][0]);
-          uint4 off_hi = *reinterpret_cast<const uint4 *>(&sh.off[stage][0][4]);
-          if (!ok || (has_z && !ptx::mbar_wait_cluster(&sh.zfull[stage], (zphase >> stage) & 1u, wl)) ||
-              !ptx::mbar_wait(&sh.full[stage], phase, wl) || sh.abort_flag) {
+          if (!ptx::mbar_wait(&sh.full[stage], phase, wl) || !ptx::mbar_wait(&sh.mfull[stage], (mphase >> stage) & 1u, wl) ||
+              (has_z && !ptx::mbar_wait_cluster(&sh.zfull[stage], (zphase >> stage) & 1u, wl)) || sh.abort_flag) {
             ok = false;
             break;
           }
@@ -295,10 +291,8 @@ __global__ void __launch_bounds__(kThreads, 1) pair_gemm_kernel(const __grid_con
           uint64_t db = ptx::umma_desc_rows(sr + kXBytes, row_bytes);
           const int32_t n = min(per, cnt - e0);
           for (int32_t j = 0; j < n; ++j, db += b_bytes >> 4) {
-            if (j > 0) {
-              off_lo = *reinterpret_cast<const uint4 *>(&sh.off[stage][j][0]);
-              off_hi = *reinterpret_cast<const uint4 *>(&sh.off[stage][j][4]);
-            }
+            const uint4 off_lo = *reinterpret_cast<const uint4 *>(&sh.off[stage][j][0]);
+            const uint4 off_hi = *reinterpret_cast<const uint4 *>(&sh.off[stage][j][4]);
 #pragma unroll
             for (int k = 0; k < kBlockK / kUmmaK; ++k)
               if (k < ksteps) ptx::umma_bf16_pair_rows(tmem_d, da + 2 * k, db + 2 * k, idesc, off_lo, off_hi);
