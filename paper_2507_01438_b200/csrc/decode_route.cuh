@@ -101,4 +101,137 @@ __device__ __forceinline__ void publish_decode_plan(const PlanView &pv, int a, i
   }
 }
 
+// The u-batches of a decode batch, in shared memory: adapters in order of first appearance, the tokens of each in token
+// order, and the tokens of an adapter in blocks.
+struct Groups {
+  alignas(16) int32_t id[kDecodeMaxT];  // validated id of each token
+  int32_t adapter[kDecodeMaxT];  // of each group
+  int32_t cnt[kDecodeMaxT];      // scratch: tokens of each group
+  int32_t wt[9];                 // scratch of the prefix sums
+  int32_t n_groups, n_blocks;
+  int16_t start[kDecodeMaxT + 1];    // groups' first positions in tok
+  int16_t block_pos[kDecodeMaxT];    // blocks' first positions in tok
+  uint8_t tok[kDecodeMaxT], block_group[kDecodeMaxT];
+  uint8_t group[kDecodeMaxT];        // of each token with an adapter
+  int16_t pos[kDecodeMaxT];          // its position in tok
+};
+// Exclusive prefix sums of a value per element, elements i = k * kN + tid, over kN threads that meet on barrier kBar.
+template <int kBar, int kN, int kPer>
+__device__ __forceinline__ int32_t group_scan(const int32_t (&v)[kPer], int32_t *wt, int tid, int32_t (&out)[kPer]) {
+  const int lane = tid & 31, warp = tid >> 5;
+  int32_t incl[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    incl[k] = v[k];
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int32_t o = __shfl_up_sync(0xffffffffu, incl[k], d);
+      if (lane >= d) incl[k] += o;
+    }
+    if (lane == 31) wt[k * (kN / 32) + warp] = incl[k];
+  }
+  asm volatile("bar.sync %0, %1;" ::"n"(kBar), "n"(kN) : "memory");
+  int32_t total = 0;
+#pragma unroll
+  for (int i = 0; i < kPer * kN / 32; ++i) {
+#pragma unroll
+    for (int k = 0; k < kPer; ++k)
+      if (i == k * (kN / 32) + warp) out[k] = total + incl[k] - v[k];
+    total += wt[i];
+  }
+  return total;
+}
+// kN threads (128 or 256, a multiple of 32) call it with their number `tid`; they meet on the named barrier kBar.  Blocks
+// hold at most kBlockTok tokens.  Returns whether one of this thread's ids was out of range (-1 is kept for it).
+template <int kBlockTok, int kBar, int kN>
+__device__ __forceinline__ bool derive_groups(Groups &s, const int32_t *ids, int T, int32_t n_slots, int tid) {
+  constexpr int kPer = kDecodeMaxT / kN;
+  const auto sync = [] { asm volatile("bar.sync %0, %1;" ::"n"(kBar), "n"(kN) : "memory"); };
+  int32_t a[kPer], pos[kPer], first[kPer], v[kPer], out[kPer];
+  bool bad = false;
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int t = k * kN + tid;
+    a[k] = t < T ? ids[t] : -1;
+    if (a[k] < -1 || a[k] >= n_slots) {
+      a[k] = -1;
+      bad = true;
+    }
+    s.id[t] = a[k];
+    s.cnt[t] = 0;
+  }
+  sync();
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int t = k * kN + tid;
+    pos[k] = 0;
+    first[k] = t;
+    if (a[k] >= 0) {  // earlier tokens on the same adapter, four ids per shared-memory load
+      auto see = [&](int id, int u) {
+        if (id == a[k]) {
+          if (pos[k] == 0) first[k] = u;
+          ++pos[k];
+        }
+      };
+      const int full = t & ~3;
+#pragma unroll 4
+      for (int u = 0; u < full; u += 4) {
+        const int4 w = *reinterpret_cast<const int4 *>(&s.id[u]);
+        see(w.x, u);
+        see(w.y, u + 1);
+        see(w.z, u + 2);
+        see(w.w, u + 3);
+      }
+      for (int u = full; u < t; ++u) see(s.id[u], u);
+    }
+    v[k] = a[k] >= 0 && pos[k] == 0 ? 1 : 0;
+  }
+  const int32_t G = group_scan<kBar, kN, kPer>(v, s.wt, tid, out);
+#pragma unroll
+  for (int k = 0; k < kPer; ++k)
+    if (v[k]) {
+      s.group[k * kN + tid] = static_cast<uint8_t>(out[k]);
+      s.adapter[out[k]] = a[k];
+    }
+  sync();
+#pragma unroll
+  for (int k = 0; k < kPer; ++k)
+    if (a[k] >= 0) {
+      first[k] = s.group[first[k]];  // its group from here on
+      atomicAdd(&s.cnt[first[k]], 1);
+    }
+  sync();
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {  // tokens in the low half, blocks in the high half
+    const int g = k * kN + tid, n = g < G ? s.cnt[g] : 0;
+    v[k] = n | ((n + kBlockTok - 1) / kBlockTok) << 16;
+  }
+  const int32_t total = group_scan<kBar, kN, kPer>(v, s.wt, tid, out);
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int g = k * kN + tid, start = out[k] & 0xFFFF, b0 = out[k] >> 16;
+    if (g < G) s.start[g] = static_cast<int16_t>(start);
+    for (int b = 0; b < v[k] >> 16; ++b) {
+      s.block_group[b0 + b] = static_cast<uint8_t>(g);
+      s.block_pos[b0 + b] = static_cast<int16_t>(start + b * kBlockTok);
+    }
+  }
+  if (tid == 0) {
+    s.start[G] = static_cast<int16_t>(total & 0xFFFF);
+    s.n_groups = G;
+    s.n_blocks = total >> 16;
+  }
+  sync();
+#pragma unroll
+  for (int k = 0; k < kPer; ++k)
+    if (a[k] >= 0) {
+      const int p = s.start[first[k]] + pos[k];
+      s.tok[p] = static_cast<uint8_t>(k * kN + tid);
+      s.pos[k * kN + tid] = static_cast<int16_t>(p);
+      s.group[k * kN + tid] = static_cast<uint8_t>(first[k]);
+    }
+  sync();
+  return bad;
+}
+
 }  // namespace edgelora

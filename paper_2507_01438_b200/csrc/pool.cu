@@ -14,6 +14,7 @@
 #include <utility>
 #include <vector>
 
+#include "decode_sites.h"
 #include "guard.h"
 #include "pool.h"
 #include "prefill.h"
@@ -380,6 +381,7 @@ int edgelora_pool_create(const edgelora_pool_config *cfg, edgelora_pool_t **pool
   POOL_TRY(shrink_set_smem_limit());
   POOL_TRY(shrink_tiles_set_smem_limit());
   POOL_TRY(pair_set_smem_limit());
+  POOL_TRY(decode_sites_set_smem_limit());
   rc = edgelora_plan_create(p->cfg.max_tokens, cfg->n_slots, &p->plan);
   if (rc != EDGELORA_OK) {
     edgelora_pool_destroy(p);
@@ -949,6 +951,102 @@ int prefill_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32
   if (rc) return rc;
   for (int i = 0; i < n; ++i) sites[i].p->last_info[0] = i == 0 ? launches : 0;
   p0->total_launches += launches;
+  return EDGELORA_OK;
+}
+
+// ---- decode-sized batches of a run of sites (decode_sites.cu)
+static int32_t decode_columns(int32_t T) { return std::max(16, (T + 15) / 16 * 16); }
+
+size_t decode_workspace_bytes(int32_t sms, int32_t max_tokens, size_t *arrivals_at) {
+  const size_t planes = static_cast<size_t>(sms) * 2 * kTileM * decode_columns(std::min(max_tokens, kDecodeMaxT)) * sizeof(float);
+  *arrivals_at = planes;
+  return planes + static_cast<size_t>(sms) * 4 * sizeof(int32_t);
+}
+
+static int fill_decode_site(const SiteCall &c, int x_index, DecSite *d) {
+  edgelora_pool *q = c.p;
+  const int h_in = q->cfg.h_in, h_out = q->cfg.h_out, R = q->R_pad;
+  const int rc = get_tmap(q, &d->w, c.W, h_in, h_out, 0, kTileM);
+  if (rc) return rc;
+  d->slots = q->slots_dev;
+  d->z = q->zws + static_cast<size_t>(kMaxZSplits) * q->cfg.max_tokens * R;
+  d->status = q->status_dev;
+  d->x_index = x_index;
+  d->R_pad = R;
+  d->y = static_cast<uint16_t *>(c.y);
+  d->h_out = h_out;
+  d->kb = (h_in + kBlockK - 1) / kBlockK;
+  return get_tmap(q, &d->b, q->B_pool, R, h_out, q->cfg.n_slots, kTileM, R);
+}
+
+int decode_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32_t *ids_dev, int32_t T,
+                 const DecodeWorkspace &ws, cudaStream_t stream, bool pdl_first) {
+  edgelora_pool *p0 = sites[0].p;
+  const int32_t N = decode_columns(T);
+  int32_t R_max = 0;
+  for (int i = 0; i < n; ++i) R_max = std::max(R_max, sites[i].p->R_pad);
+  const DecShape shape = decode_sites_shape(N, R_max);
+  DecShrinkBatch sb{};
+  DecBatch db{};
+  sb.n_sites = db.n_sites = n;
+  sb.T = T;
+  sb.n_slots = db.n_slots = plan->n_slots;
+  sb.ids = ids_dev;
+  sb.pv = plan->pv;
+  sb.zero = db.arrivals = ws.arrivals;
+  sb.n_zero = 4 * p0->sms;
+  db.T = T;
+  db.N = N;
+  db.ids = ids_dev;
+  db.stages = shape.stages;
+  db.exp_stages = shape.exp_stages;
+  db.exp_bytes = shape.exp_bytes;
+  db.n_acc = shape.n_acc;
+  db.tmem_cols = shape.tmem_cols;
+  db.partial = ws.partial;
+  db.wait_cycles = p0->wait_cycles;
+  const SiteCall *inputs[kDecInputs] = {};  // the first site on each input
+  int n_inputs = 0;
+  for (int i = 0; i < n; ++i) {
+    edgelora_pool *q = sites[i].p;
+    const int h_in = q->cfg.h_in, R = q->R_pad;
+    int xi = 0, rc = EDGELORA_OK;
+    while (xi < n_inputs && !inputs[xi]->same_input(sites[i])) ++xi;
+    if (xi == n_inputs) {
+      inputs[n_inputs++] = &sites[i];
+      rc = get_tmap(q, &sb.x[xi], sites[i].x, h_in, T, 0, 1, kShrinkStepElems);
+      if (!rc) rc = get_tmap(q, &db.x[xi], sites[i].x, h_in, T, 0, N);
+      if (rc) return rc;
+    }
+    DecShrinkSite &s = sb.site[i];
+    rc = get_tmap(q, &s.a, q->A_pool, h_in, R, q->cfg.n_slots, 8, kShrinkStepElems);
+    if (!rc) rc = fill_decode_site(sites[i], xi, &db.site[i]);
+    if (rc) return rc;
+    s.slots = q->slots_dev;
+    s.zws = q->zws;
+    s.counters = q->group_counters;
+    s.status = q->status_dev;
+    s.x_index = xi;
+    s.n_ksteps = (h_in + kShrinkStepElems - 1) / kShrinkStepElems;
+    // K chunks of eight steps or more, 32 KB of A per item (four and sixteen: within 1 us of 335)
+    s.ks = std::max(1, std::min(kMaxZSplits, s.n_ksteps / 8));
+    s.R_pad = R;
+    s.max_tokens = q->cfg.max_tokens;
+  }
+  plan->last_T = T;
+  // (two CTAs of the shrink per SM, 98 KB of ring each: 333 us for the 28 sites, 336 with one)
+  CUDA_TRY(launch_decode_sites_shrink(sb, 2 * p0->sms, pdl_first, stream));
+  CUDA_TRY(launch_decode_sites(db, shape, p0->sms, true, stream));
+  for (int i = 0; i < n; ++i) {
+    int64_t *info = sites[i].p->last_info;
+    info[0] = i == 0 ? 2 : 0;
+    info[1] = 1;
+    info[2] = p0->sms;
+    info[3] = 1;
+    info[4] = shape.stages;
+    info[5] = N;
+  }
+  p0->total_launches += 2;
   return EDGELORA_OK;
 }
 

@@ -126,6 +126,15 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
                      const void *x_dev, int32_t T, void *y_dev, cudaStream_t stream, Order order = Order::kPool);
 int prefill_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32_t *ids_dev, int32_t T,
                   cudaStream_t stream, bool pdl_first);
+// Decode-sized batches: shrink and base product of a run of sites (at most kDecSites on at most kDecInputs inputs, no
+// pool twice) in one launch each.  ids_dev: the caller's ids; the plan is published.  ws: see DecodeWorkspace.
+struct DecodeWorkspace {
+  float *partial = nullptr;      // two planes [N][128] per CTA
+  int32_t *arrivals = nullptr;   // [CTAs][4]
+};
+size_t decode_workspace_bytes(int32_t sms, int32_t max_tokens, size_t *arrivals_at);
+int decode_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32_t *ids_dev, int32_t T,
+                 const DecodeWorkspace &ws, cudaStream_t stream, bool pdl_first);
 int wait_for_loads(edgelora_pool *p, cudaStream_t stream, bool capturing);
 
 }  // namespace edgelora

@@ -91,6 +91,13 @@ __device__ __forceinline__ void bulk_load_1d(void *smem_dst, const void *gmem_sr
                "l"(reinterpret_cast<uint64_t>(gmem_src)), "r"(bytes), "r"(smem_u32(bar))
                : "memory");
 }
+// Bulk copy from this CTA's shared memory into another CTA's of the cluster (dst and bar: their cluster addresses), counted
+// on a barrier there.  The source must stay until it is complete.
+__device__ __forceinline__ void bulk_copy_cluster(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "r"(smem_u32(src)), "r"(bytes), "r"(bar)
+               : "memory");
+}
 // 2D tiled load, no multicast.  c0 is the innermost (contiguous) coordinate.
 __device__ __forceinline__ void tma_load_2d(void *smem_dst, const CUtensorMap *m, uint64_t *bar,
                                             int32_t c0, int32_t c1) {
@@ -228,6 +235,33 @@ __device__ __forceinline__ void tmem_ld_32x64(uint32_t taddr, float (&v)[64]) {
     v[i] = __uint_as_float(r[i]);
   }
 }
+// Columns of this warp's 32 lanes: loads complete behind tmem_ld_wait, whose values go through tmem_loaded before they are
+// used; stores behind tmem_st_wait.
+__device__ __forceinline__ void tmem_ld_32x1(uint32_t taddr, float &v) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=f"(v) : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld_32x16(uint32_t taddr, float *v) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]), "=f"(v[8]),
+        "=f"(v[9]), "=f"(v[10]), "=f"(v[11]), "=f"(v[12]), "=f"(v[13]), "=f"(v[14]), "=f"(v[15])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_loaded(float &v) { asm volatile("" : "+f"(v)); }
+__device__ __forceinline__ void tmem_st_32x1(uint32_t taddr, const float *v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "f"(v[0]) : "memory");
+}
+__device__ __forceinline__ void tmem_st_32x2(uint32_t taddr, const float *v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x2.b32 [%0], {%1, %2};" ::"r"(taddr), "f"(v[0]), "f"(v[1]) : "memory");
+}
+__device__ __forceinline__ void tmem_st_32x4(uint32_t taddr, const float *v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "f"(v[0]), "f"(v[1]), "f"(v[2]),
+               "f"(v[3])
+               : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // orders this thread's shared-memory writes before later accesses of the async proxy (TMA, tcgen05)
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
@@ -246,9 +280,11 @@ __device__ __forceinline__ uint32_t cluster_rank() {
 }
 // Barrier over every thread of every CTA of the cluster (a hardware barrier: all of them reach it,
 // on the time-out paths too, because no role loop is unbounded).
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  cluster_arrive();
+  cluster_wait();
 }
 // Arrive on a barrier given by its cluster address (see map_to_rank).  What it announces is work of the async
 // proxy in this CTA's own memory (operand rows behind a proxy fence, tensor-memory reads behind
@@ -378,6 +414,31 @@ __device__ __forceinline__ void pdl_launch_dependents() {
 __device__ __forceinline__ float bf16_lo(uint32_t packed) { return __uint_as_float(packed << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t packed) {
   return __uint_as_float(packed & 0xFFFF0000u);
+}
+// Four fp32 values from shared memory, zeros where `live` is 0 (without a branch around the load).
+__device__ __forceinline__ void ld_shared_f32x4_if(uint32_t addr, uint32_t live, uint64_t &lo, uint64_t &hi) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\tmov.b64 %0, 0;\n\tmov.b64 %1, 0;\n\t"
+      "@p ld.shared.v2.b64 {%0, %1}, [%2];\n\t}"
+      : "=&l"(lo), "=&l"(hi)
+      : "r"(addr), "r"(live));
+}
+// Two fp32 values in a register pair, and a fused multiply-add of both in one instruction.
+__device__ __forceinline__ uint64_t f32x2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ float sum_f32x2(uint64_t a, uint64_t b) {  // of all four values
+  float x, y, u, v;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(a));
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(u), "=f"(v) : "l"(b));
+  return (x + u) + (y + v);
 }
 // two fp32 -> packed bf16x2 (lo in the low half), round to nearest even
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {

@@ -3,7 +3,7 @@
 // from adapter ids to samples is worked out once).  The set builds one routing plan per batch and
 // hands its sites to the device in runs: one launch computes the shrink of every site of a run, the next
 // one their base products with the expand, so that launches, ramp-ups and partly empty last waves are paid
-// per run and not per site.  Decode-sized batches go site by site.
+// per run and not per site.
 #include <cuda_runtime.h>
 
 #include <cstring>
@@ -24,6 +24,7 @@ struct edgelora_siteset {
   std::vector<int32_t> in_width;          // h_in of every input
   std::vector<int32_t> first_writer;      // per input, of the call at hand: the first site that writes into its memory
   edgelora_plan *plan = nullptr;
+  DecodeWorkspace ws;                     // of the launches of decode-sized batches
   // host-buffer path (allocated on first use)
   std::vector<uint16_t *> dx;             // [n_inputs] device mirrors of the inputs
   int32_t *dids = nullptr;
@@ -62,8 +63,7 @@ bool overlap(const void *a, size_t na, const void *b, size_t nb) {
 int run_sites(edgelora_siteset *s, const void *const *x_dev, const int32_t *ids_dev, int32_t T,
               void *const *y_dev, cudaStream_t stream, const std::vector<cudaEvent_t> *after = nullptr,
               const std::vector<cudaEvent_t> *before = nullptr) {
-  int rc = edgelora_plan_build(s->plan, ids_dev, T, stream);
-  if (rc != EDGELORA_OK) return rc;
+  int rc = EDGELORA_OK;
   const int n = static_cast<int>(s->pools.size());
   const bool in_capture = capturing(stream);
   // A result that lies in an input's memory is seen by the sites behind it: a site that reads such an input starts
@@ -76,10 +76,20 @@ int run_sites(edgelora_siteset *s, const void *const *x_dev, const int32_t *ids_
     s->first_writer[k] = i;
     chained = chained || i < n;
   }
-  // Large batches: the sites go to the device in runs that share one shrink launch and one base-product
-  // launch, when every pool runs in its default configuration and no result is an input.
-  bool runs = T > kDecodeMaxT && !chained;
-  for (auto *p : s->pools) runs = runs && p->opt_regime == 0 && p->opt_pdl >= 1 && !p->a_q8;
+  // The sites go to the device in runs that share one shrink launch and one base-product launch, when every pool
+  // runs in its default configuration and no result is an input.
+  const bool decode = T <= kDecodeMaxT;
+  bool runs = !chained;
+  for (auto *p : s->pools) {
+    runs = runs && p->opt_regime == 0 && p->opt_pdl >= 1 && !p->a_q8;
+    if (decode)
+      runs = runs && !p->opt_profile && T <= p->opt_gather_min_t && p->opt_decode_splits == 0 && p->opt_shrink_items == 0 &&
+             p->opt_shrink_depth == 0;
+  }
+  if (!runs || !decode) {  // (the decode kernels derive the plan themselves)
+    rc = edgelora_plan_build(s->plan, ids_dev, T, stream);
+    if (rc != EDGELORA_OK) return rc;
+  }
   if (!runs) {
     for (int i = 0; i < n; ++i) {
       if (before && (*before)[i] && cudaStreamWaitEvent(stream, (*before)[i], 0) != cudaSuccess) return EDGELORA_ERR_CUDA;
@@ -132,7 +142,9 @@ int run_sites(edgelora_siteset *s, const void *const *x_dev, const int32_t *ids_
     }
     // (the kernel in front of a run is the plan kernel, launched behind everything before it, or the base
     // product of the run before)
-    rc = prefill_sites(calls, m, s->plan, nullptr, T, stream, true);
+    // (of a decode-sized batch the first kernel stands to the work in front of the set as its first pool says)
+    rc = decode ? decode_sites(calls, m, s->plan, ids_dev, T, s->ws, stream, i0 > 0 || calls[0].p->opt_pdl >= 2)
+                : prefill_sites(calls, m, s->plan, nullptr, T, stream, true);
     if (rc != EDGELORA_OK) return rc;
     for (int i = i0; i < i0 + m; ++i)
       if (after && (*after)[i] && cudaEventRecord((*after)[i], stream) != cudaSuccess) return EDGELORA_ERR_CUDA;
@@ -185,6 +197,15 @@ int edgelora_siteset_create(int32_t n_sites, edgelora_pool_t *const *pools, cons
     delete s;
     return rc;
   }
+  size_t arrivals_at = 0;
+  const size_t ws_bytes = decode_workspace_bytes(pools[0]->sms, max_tokens, &arrivals_at);
+  if (el_malloc(&s->ws.partial, ws_bytes) != cudaSuccess) {
+    cudaGetLastError();
+    edgelora_plan_destroy(s->plan);
+    delete s;
+    return EDGELORA_ERR_CUDA;
+  }
+  s->ws.arrivals = reinterpret_cast<int32_t *>(reinterpret_cast<uint8_t *>(s->ws.partial) + arrivals_at);
   s->dx.assign(n_inputs, nullptr);
   s->dy.assign(n_sites, nullptr);
   *set_out = s;
@@ -199,6 +220,7 @@ int edgelora_siteset_destroy(edgelora_siteset_t *s) {
   for (auto *q : s->dy) if (q) el_free(q);
   for (auto &e : s->dy_scratch) if (e.second) el_free(e.second);
   if (s->dids) el_free(s->dids);
+  if (s->ws.partial) el_free(s->ws.partial);
   for (auto e : s->done_ev) if (e) cudaEventDestroy(e);
   for (auto e : s->up_ev) if (e) cudaEventDestroy(e);
   if (s->copy_stream) cudaStreamDestroy(s->copy_stream);
