@@ -64,3 +64,19 @@ def test_scores_drive_the_cache_aware_selection():
             hits += got[2]
     finally:
         B.edgelora_cache_destroy(cache)
+
+
+@pytest.mark.parametrize("Bn,n,hidden", [
+    (8, 8, 32), (9, 9, 40), (7, 1024, 4096), (2, 1025, 4104), (17, 300, 8192), (3, 1041, 5000), (1, 1500, 8184),
+])
+def test_scores_at_the_edges_of_the_launch_shapes(Bn, n, hidden):
+    # rows and prompts around eight, parts of a row that end inside a chunk of 32 values, rows of one and of two rounds with
+    # eight and with sixteen warps; the bound: fp32 sums of exact products, 2^-23 of the terms' magnitude (|logit| terms
+    # add up to about sqrt(hidden) * 2 / sqrt(hidden) per unit) times the depth of the sum, and the fast exponential's few ulp
+    import torch
+    rng = np.random.Generator(np.random.PCG64(Bn * 7 + n))
+    Wr = wl.normal_bf16(rng, (n, hidden), 2.0 / np.sqrt(hidden))
+    h = wl.normal_bf16(rng, (Bn, hidden), 1.0)
+    bias = rng.normal(0, 1, size=n).astype(np.float32)
+    got = B.edgelora_router_scores(to_dev_bf16(Wr), torch.from_numpy(bias).cuda(), to_dev_bf16(h)).cpu().numpy()
+    assert np.max(np.abs(got - router_scores(Wr, bias, h))) <= 5e-6
