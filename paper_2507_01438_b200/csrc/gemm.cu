@@ -67,6 +67,18 @@ __device__ __forceinline__ int32_t ld_acquire_gpu(const int32_t *ptr) {
   return v;
 }
 
+// Bounded wait of one thread for the shrink teams' arrival counter.
+__device__ __forceinline__ int wait_for_teams(const int32_t *counter, int32_t n, long long wl, uint32_t *status) {
+  const long long t_start = clock64();
+  while (ld_acquire_gpu(counter) < n) {
+    if (clock64() - t_start > wl) {
+      atomicOr(status, EDGELORA_STATUS_TIMEOUT);
+      return 0;
+    }
+  }
+  return 1;
+}
+
 // Fused decode launches (batches of at most 64 tokens): z[t] = s_a A_a x[t] on the CUDA cores, by
 // "teams" of four warps: the four builder warps of every CTA of the decode job (idle there, because
 // the expand is added by the owners of the cluster reduction) and two teams in every spare CTA.
@@ -431,13 +443,12 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
     const bool clustered = p.splits > 1;
     if (kFused && clustered && f.b_stage) {
       // This CTA will finish tokens [rank * cols_per, ...) of its row tile: the B_a rows they need (the
-      // tile's 128 rows of the token's adapter, contiguous in the pool) are copied into shared memory
-      // now, one bulk copy per token, while the main loop runs (the ids are the caller's input, the
-      // pool is not written by this kernel).  One warp per token; cols_per <= 16.
+      // tile's 128 rows of the token's adapter) are copied into shared memory now, one copy per token, while the main
+      // loop runs (the ids are the caller's input, the pool is not written by this kernel).  One warp per token;
+      // cols_per <= 16.
       const int cols_per = p.BN / p.splits;
       const int t0 = static_cast<int>(ptx::cluster_rank()) * cols_per;
       const uint32_t tok_bytes = kTileM * p.R_pad * 2;
-      const uint32_t copy_bytes = static_cast<uint32_t>(min(kTileM, p.h_out - tc_row0(p, bid)) * p.R_pad * 2);
       int32_t a_of[4];
       uint32_t my_bytes = 0;
 #pragma unroll
@@ -455,16 +466,15 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
           s_vid[cl] = a;
           s_lg[cl] = rank;
         }
-        if (a >= 0) my_bytes += copy_bytes;
+        if (a >= 0) my_bytes += tok_bytes;
       }
       if (lane == 0) {
         ptx::mbar_arrive_expect_tx(ep_bar, my_bytes);
 #pragma unroll
         for (int i = 0; i < 4; ++i)
           if (a_of[i] >= 0)
-            ptx::bulk_load_1d(b_stage + static_cast<size_t>(quad + 4 * i) * tok_bytes,
-                              p.B_pool + (static_cast<size_t>(a_of[i]) * p.h_out + tc_row0(p, bid)) * p.R_pad,
-                              copy_bytes, ep_bar);
+            ptx::tma_load_3d(b_stage + static_cast<size_t>(quad + 4 * i) * tok_bytes, &tmap_b, ep_bar, 0, tc_row0(p, bid),
+                             a_of[i]);
       }
     } else if (clustered && p.expand_in_reduce) {
       // This CTA will finish tokens [rank * cols_per, ...) of its row tile; pull the B_a rows they
@@ -493,48 +503,15 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
         }
       }
     }
-    if (kFused && clustered) {
-      // z comes from the shrink teams of this grid (every CTA of the launch is resident, so all of them
-      // run).  These warps have nothing to do until the accumulator is complete: bounded wait for the
-      // teams' arrival counter now, then this thread's share of the owner's z (tokens x R_pad floats,
-      // at most 128 16-byte pieces; the K chunks' planes added in order) goes to shared memory, behind
-      // the staged B_a rows.
-      const int cols_per = p.BN / p.splits, etid = threadIdx.x - 64;
-      const int my_rank = static_cast<int>(ptx::cluster_rank());
-      // the counter belongs to the kernel before this one (another launch of this pool, which leaves it
-      // at zero) until that kernel is done
+    if (kFused && clustered && !f.b_stage) {
+      // z comes from the shrink teams of this grid (every CTA of the launch is resident, so all of them run): bounded wait
+      // for their arrival counter.  The counter belongs to the kernel before this one (another launch of this pool, which
+      // leaves it at zero) until that kernel is done.
       ptx::pdl_wait_prior_grids();
       // one thread of the CTA polls; the named barrier of the four warps passes its acquire on
-      if (warp == 2 && lane == 0) {
-        int got = 1;
-        const long long t_start = clock64();
-        while (ld_acquire_gpu(f.sync) < 2 * cta0 + ngrid) {
-          if (clock64() - t_start > wl) {
-            got = 0;
-            break;
-          }
-        }
-        if (!got) atomicOr(p.status, EDGELORA_STATUS_TIMEOUT);
-        *s_last = got;
-      }
+      if (warp == 2 && lane == 0) *s_last = wait_for_teams(f.sync, 2 * cta0 + ngrid, wl, p.status);
       named_bar_sync(1, 128);
       fused_z_ok = *s_last != 0;
-      const int tok = my_rank * cols_per + etid / (p.R_pad >> 2);
-      if (f.b_stage && fused_z_ok && etid < cols_per * (p.R_pad >> 2)) {
-        float4 z_mine = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (tok < p.T) {
-          const size_t zplane4 = static_cast<size_t>(p.max_tokens) * p.R_pad / 4;
-          const float4 *zp = reinterpret_cast<const float4 *>(f.z) +
-                             static_cast<size_t>(my_rank) * cols_per * (p.R_pad >> 2) + etid;
-          z_mine = __ldcg(zp);
-          for (int sp = 1; sp < f.ks; ++sp) {
-            const float4 w = __ldcg(zp + sp * zplane4);
-            z_mine.x += w.x; z_mine.y += w.y; z_mine.z += w.z; z_mine.w += w.w;
-          }
-        }
-        // read by the expand, behind two cluster barriers
-        reinterpret_cast<float4 *>(b_stage + static_cast<size_t>(cols_per) * kTileM * p.R_pad * 2)[etid] = z_mine;
-      }
     }
     // Earlier kernels may still read y, and z comes from the shrink kernel.  With the expand in
     // the reduction both matter only at the very end, so that wait moves there.
@@ -771,185 +748,241 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
       }
     }
     __syncwarp();
-    ptx::cluster_sync_all();
-    if (epi || wide) {
-      const float *buf = reinterpret_cast<const float *>(red);
-      const int n_units = cols_per * 32;  // unit = (token, 4 adjacent W rows)
-      const int row0 = bid / p.splits * kTileM;
-      auto sum_partials = [&](int cl, int r4) {
-        float4 acc4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int sp = 0; sp < p.splits; ++sp) {
-          const float4 w = *reinterpret_cast<const float4 *>(buf + ((sp * cols_per + cl) * kTileM + r4));
-          acc4.x += w.x; acc4.y += w.y; acc4.z += w.z; acc4.w += w.w;
-        }
-        return acc4;
-      };
-      auto store4 = [&](int t, int j, const float4 &v) {
-        uint2 o;
-        o.x = ptx::pack_bf16x2(v.x, v.y);
-        o.y = ptx::pack_bf16x2(v.z, v.w);
-        *reinterpret_cast<uint2 *>(p.y + static_cast<size_t>(t) * p.h_out + j) = o;
-      };
-      if (!p.expand_in_reduce) {
-        // unit = (token quad, W row): the splits' partial sums are 16 bytes each, lanes take
-        // adjacent rows, so a warp writes 64 bytes in a row of y per token
-        const int qpo = cols_per >> 2;
-        const float4 *buf4 = reinterpret_cast<const float4 *>(red);
-        ptx::pdl_wait_prior_grids();  // warps 0 and 1 have not waited yet; earlier kernels may read y
-        for (int u = threadIdx.x; u < qpo * kTileM; u += kGemmThreads) {
-          const int qd = u >> 7, r = u & (kTileM - 1);
-          const int t0 = static_cast<int>(my_rank) * cols_per + qd * 4, j = row0 + r;
-          if (t0 >= p.T || j >= p.h_out) continue;
-          float4 a4 = make_float4(0.f, 0.f, 0.f, 0.f);
-          for (int sp = 0; sp < p.splits; ++sp) {
-            const float4 w = buf4[(sp * qpo + qd) * kTileM + r];
-            a4.x += w.x; a4.y += w.y; a4.z += w.z; a4.w += w.w;
-          }
-          const float o[4] = {a4.x, a4.y, a4.z, a4.w};
+    if (kFused && f.b_stage) {
+      // Small batches, one launch.  The partial sums are on their way; while the cluster's other CTAs send theirs, the
+      // epilogue and team warps (2..9) work out the expand of this CTA's tokens: wait for the shrink teams, bring z of
+      // their tokens to shared memory, and dot it with the staged B_a rows, a thread per W row and every other token quad.
+      // (With the expand behind the exchange, by the epilogue warps alone, the tail behind the last MMA took 6 us for 32
+      // tokens and 9 for 64: 4096 -> 4096, 32 tokens 15.1 us per call, now 12.3; 64 tokens 18.0 and 14.1; 256 -> 256, 16
+      // tokens 7.9 and 5.7.)
+      ptx::cluster_arrive();
+      const int half = warp >= 6 ? 1 : 0, nq = cols_per >> 2, R4 = p.R_pad >> 2;
+      const int r = (threadIdx.x - 64) & 127;
+      float e[2][4];
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (t0 + i < p.T)
-              p.y[static_cast<size_t>(t0 + i) * p.h_out + j] =
-                  static_cast<uint16_t>(ptx::pack_bf16x2(o[i], 0.f) & 0xFFFFu);
+      for (int i = 0; i < 8; ++i) e[i >> 2][i & 3] = 0.f;
+      int passed = 0;
+      if (warp >= 2) {
+        if (warp == 2) {
+          // the counter belongs to the kernel before this one (another launch of this pool, which leaves it at zero) until
+          // that kernel is done
+          ptx::pdl_wait_prior_grids();
+          // one thread of the CTA polls; the named barrier passes its acquire on
+          if (lane == 0) *s_last = wait_for_teams(f.sync, 2 * cta0 + ngrid, wl, p.status);
         }
-      } else if (kFused && f.b_stage) {
-        // Small batches, one launch: unit = (token quad, W row), as above, and everything the expand
-        // needs is in shared memory by now: B_a[row][0..R_pad) of each token's adapter (lanes take
-        // adjacent rows: 32-byte pieces side by side) and the tokens' z (the same for every lane).
-        const int qpo = cols_per >> 2;
-        const float4 *buf4 = reinterpret_cast<const float4 *>(red);
-        const int n_units = qpo * kTileM;  // at most 4 per thread (cols_per <= 16)
-        const int nch = p.R_pad >> 3;
-        ptx::pdl_wait_prior_grids();  // earlier kernels may still read y
-        bool b_ok = true;
-        {
-          int got = 1;
-          if (lane == 0) got = ptx::mbar_wait(ep_bar, 0, max(wl, ptx::kSettleCycles)) ? 1 : 0;  // the staged B_a rows
-          if (!__shfl_sync(0xffffffffu, got, 0)) {
-            if (lane == 0) atomicOr(p.status, EDGELORA_STATUS_TIMEOUT);
-            b_ok = false;
-          }
-        }
-        const int r = etid & 127, j = row0 + r;
-        // This code runs once per launch: kept as rolled loops, because what it costs is fetching its
-        // instructions, not executing them (fully unrolled it took 2.9 us instead of about 1 us).
-#pragma unroll 1
-        for (int u = etid; u < n_units && j < p.h_out; u += 128) {
-          const int qd = u >> 7;
-          float4 a4 = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 1
-          for (int sp = 0; sp < p.splits; ++sp) {
-            const float4 w = buf4[(sp * qpo + qd) * kTileM + r];
-            a4.x += w.x; a4.y += w.y; a4.z += w.z; a4.w += w.w;
-          }
-          const int t0q = static_cast<int>(my_rank) * cols_per + qd * 4;
-#pragma unroll 1
-          for (int k = 0; k < 4; ++k) {
-            const int cl = qd * 4 + k;
-            const int32_t a = (z_ok && b_ok) ? s_vid[cl] : -1, rank = s_lg[cl];
-            float add = k == 0 ? a4.x : k == 1 ? a4.y : k == 2 ? a4.z : a4.w;
-            if (a >= 0) {
-              const uint4 *Brow =
-                  reinterpret_cast<const uint4 *>(b_stage + static_cast<size_t>(cl) * kTileM * p.R_pad * 2) + r * nch;
-              const float4 *zt = z_stage + cl * (p.R_pad >> 2);
-#pragma unroll 1
-              for (int c = 0; c < nch && c * 8 < rank; ++c) {
-                const uint4 bb = Brow[c];
-                const float4 u0 = zt[2 * c], u1 = zt[2 * c + 1];
-                add = fmaf(ptx::bf16_lo(bb.x), u0.x, add);
-                add = fmaf(ptx::bf16_hi(bb.x), u0.y, add);
-                add = fmaf(ptx::bf16_lo(bb.y), u0.z, add);
-                add = fmaf(ptx::bf16_hi(bb.y), u0.w, add);
-                add = fmaf(ptx::bf16_lo(bb.z), u1.x, add);
-                add = fmaf(ptx::bf16_hi(bb.z), u1.y, add);
-                add = fmaf(ptx::bf16_lo(bb.w), u1.z, add);
-                add = fmaf(ptx::bf16_hi(bb.w), u1.w, add);
+        named_bar_sync(3, 256);
+        // this warp is past its wait for the shrink teams (see the end)
+        if (epi && lane == 0) passed = atomicAdd(f.sync + 1, 1);
+        bool z_ok = *s_last != 0;
+        // z of this CTA's tokens, the K chunks' planes added in order
+        const size_t zplane4 = static_cast<size_t>(p.max_tokens) * R4;
+        for (int i = (threadIdx.x - 64); i < cols_per * R4; i += 256) {
+          const int cl = i / R4, c4 = i - cl * R4, t = static_cast<int>(my_rank) * cols_per + cl;
+          float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (s_vid[cl] >= 0 && z_ok) {
+            const float4 *zp = reinterpret_cast<const float4 *>(f.z) + static_cast<size_t>(t) * R4 + c4;
+            float4 w[8];
+            for (int s0 = 0; s0 < f.ks; s0 += 8) {
+#pragma unroll
+              for (int k = 0; k < 8; ++k) w[k] = s0 + k < f.ks ? __ldcg(zp + (s0 + k) * zplane4) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+              for (int k = 0; k < 8; ++k) {
+                z.x += w[k].x; z.y += w[k].y; z.z += w[k].z; z.w += w[k].w;
               }
             }
-            if (t0q + k < p.T)
-              p.y[static_cast<size_t>(t0q + k) * p.h_out + j] =
-                  static_cast<uint16_t>(ptx::pack_bf16x2(add, 0.f) & 0xFFFFu);
+            const int rank = s_lg[cl];  // (what lies behind the last live group of eight rank rows was not written)
+            if (c4 * 4 + 0 >= rank) z.x = 0.f;
+            if (c4 * 4 + 1 >= rank) z.y = 0.f;
+            if (c4 * 4 + 2 >= rank) z.z = 0.f;
+            if (c4 * 4 + 3 >= rank) z.w = 0.f;
           }
+          z_stage[i] = z;
         }
-        if (lane == 0) {
-          // this warp is past its wait for the shrink teams: the last such warp of the grid puts both
-          // counters back to zero for the next launch
-          if (atomicAdd(f.sync + 1, 1) == ngrid * 4 - 1) {
-            f.sync[0] = 0;
-            f.sync[1] = 0;
-          }
+        int got = 1;
+        if (lane == 0) got = ptx::mbar_wait(ep_bar, 0, max(wl, ptx::kSettleCycles)) ? 1 : 0;  // the staged B_a rows
+        if (!__shfl_sync(0xffffffffu, got, 0)) {
+          if (lane == 0) atomicOr(p.status, EDGELORA_STATUS_TIMEOUT);
+          z_ok = false;
         }
-      } else {
-        // Small batches: wait for the shrink kernel (and for earlier readers of y), then per unit add the
-        // splits' partial sums, fetch z and the B_a rows in one round trip, add B_a[j..j+3][0..r) . z[t]
-        // in fp32 (z carries s_a) and write y.  A rolled loop over the units (at most 4 per thread:
-        // cols_per <= 16): this code runs once per launch, and what it costs is mostly the fetching
-        // of its instructions.
-        ptx::pdl_wait_prior_grids();
-        const int nch = p.R_pad >> 3;
-        const int n_zp = kFused ? f.ks : 1;
-        const size_t zplane4 = static_cast<size_t>(p.max_tokens) * p.R_pad / 4;
-        auto load_z4 = [&](const float4 *ptr) {
-          float4 v = __ldcg(ptr);
-          for (int sp = 1; sp < n_zp; ++sp) {
-            const float4 w = __ldcg(ptr + sp * zplane4);
-            v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
-          }
-          return v;
-        };
-#pragma unroll 1
-        for (int u = etid; u < n_units; u += 128) {
-          const int cl = u >> 5, r4 = (u & 31) << 2;
-          const int t = static_cast<int>(my_rank) * cols_per + cl, j = row0 + r4;
-          if (t >= p.T || j >= p.h_out) continue;
-          float4 acc4 = sum_partials(cl, r4);
-          const int32_t a = z_ok ? s_vid[cl] : -1, rank = s_lg[cl];  // stored by the epilogue warps at the start
-          if (a >= 0) {
-            const uint4 *Brow = reinterpret_cast<const uint4 *>(
-                p.B_pool + (static_cast<size_t>(a) * p.h_out + j) * p.R_pad);
-            const float4 *zt = reinterpret_cast<const float4 *>((kFused ? f.z : p.zws) + static_cast<size_t>(t) * p.R_pad);
-            float add[4] = {0.f, 0.f, 0.f, 0.f};
-            for (int c0 = 0; c0 < nch && c0 * 8 < rank; c0 += 2) {
-              uint4 b[2][4];
-              float4 z4[2][2];
+        named_bar_sync(3, 256);
+        // a row's 16-byte chunks are swizzled as its length of 32, 64 or 128 bytes has it
+        const int sw = p.R_pad == 64 ? r & 7 : p.R_pad == 32 ? (r >> 1) & 3 : (r >> 2) & 1;
+        const uint32_t brow = ptx::smem_u32(b_stage) + r * p.R_pad * 2, tok_bytes = kTileM * p.R_pad * 2;
+        const uint32_t zrow = ptx::smem_u32(z_stage);
 #pragma unroll
-              for (int cc = 0; cc < 2; ++cc) {  // two chunks of 8 rank values: 12 loads in flight
-                const int c = c0 + cc;
-                const bool on = c < nch && c * 8 < rank;
+        for (int i = 0; i < 2; ++i) {
+          const int qd = half + 2 * i;
+          if (qd < nq) {
+            uint32_t live[4];
+            uint64_t s0[4], s1[4];
 #pragma unroll
-                for (int r = 0; r < 4; ++r) b[cc][r] = on ? __ldg(Brow + r * nch + c) : make_uint4(0u, 0u, 0u, 0u);
-                z4[cc][0] = on ? load_z4(zt + 2 * c) : make_float4(0.f, 0.f, 0.f, 0.f);
-                z4[cc][1] = on ? load_z4(zt + 2 * c + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int k = 0; k < 4; ++k) {
+              live[k] = z_ok && s_vid[qd * 4 + k] >= 0 ? 1u : 0u;
+              s0[k] = s1[k] = 0;
+            }
+#pragma unroll 2
+            for (int c = 0; c < p.R_pad / 8; ++c) {
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                const int cl = qd * 4 + k;
+                uint64_t b0, b1, u[4];
+                ptx::ld_shared_f32x4_if(brow + cl * tok_bytes + ((c ^ sw) << 4), live[k], b0, b1);
+                ptx::ld_shared_f32x4_if(zrow + (cl * R4 + 2 * c) * 16, 1u, u[0], u[1]);
+                ptx::ld_shared_f32x4_if(zrow + (cl * R4 + 2 * c + 1) * 16, 1u, u[2], u[3]);
+                const uint32_t w0 = static_cast<uint32_t>(b0), w1 = static_cast<uint32_t>(b0 >> 32);
+                const uint32_t w2 = static_cast<uint32_t>(b1), w3 = static_cast<uint32_t>(b1 >> 32);
+                s0[k] = ptx::fma_f32x2(ptx::f32x2(ptx::bf16_lo(w0), ptx::bf16_hi(w0)), u[0], s0[k]);
+                s1[k] = ptx::fma_f32x2(ptx::f32x2(ptx::bf16_lo(w1), ptx::bf16_hi(w1)), u[1], s1[k]);
+                s0[k] = ptx::fma_f32x2(ptx::f32x2(ptx::bf16_lo(w2), ptx::bf16_hi(w2)), u[2], s0[k]);
+                s1[k] = ptx::fma_f32x2(ptx::f32x2(ptx::bf16_lo(w3), ptx::bf16_hi(w3)), u[3], s1[k]);
               }
+            }
 #pragma unroll
-              for (int cc = 0; cc < 2; ++cc) {
-                const float4 u0 = z4[cc][0], u1 = z4[cc][1];
+            for (int k = 0; k < 4; ++k) e[i][k] = ptx::sum_f32x2(s0[k], s1[k]);
+          }
+        }
+      }
+      ptx::cluster_wait();
+      if (warp >= 2) {
+        const float4 *buf4 = reinterpret_cast<const float4 *>(red);
+        const int j = bid / p.splits * kTileM + r;
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                  const uint4 bb = b[cc][r];
-                  float s4 = add[r];
-                  s4 = fmaf(ptx::bf16_lo(bb.x), u0.x, s4);
-                  s4 = fmaf(ptx::bf16_hi(bb.x), u0.y, s4);
-                  s4 = fmaf(ptx::bf16_lo(bb.y), u0.z, s4);
-                  s4 = fmaf(ptx::bf16_hi(bb.y), u0.w, s4);
-                  s4 = fmaf(ptx::bf16_lo(bb.z), u1.x, s4);
-                  s4 = fmaf(ptx::bf16_hi(bb.z), u1.y, s4);
-                  s4 = fmaf(ptx::bf16_lo(bb.w), u1.z, s4);
-                  s4 = fmaf(ptx::bf16_hi(bb.w), u1.w, s4);
-                  add[r] = s4;
+        for (int i = 0; i < 2; ++i) {
+          const int qd = half + 2 * i, t0 = static_cast<int>(my_rank) * cols_per + qd * 4;
+          if (qd < nq && j < p.h_out) {
+            float4 a4 = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+            for (int sp = 0; sp < p.splits; ++sp) {
+              const float4 w = buf4[(sp * nq + qd) * kTileM + r];
+              a4.x += w.x; a4.y += w.y; a4.z += w.z; a4.w += w.w;
+            }
+            const float o[4] = {a4.x + e[i][0], a4.y + e[i][1], a4.z + e[i][2], a4.w + e[i][3]};
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+              if (t0 + k < p.T)
+                p.y[static_cast<size_t>(t0 + k) * p.h_out + j] = static_cast<uint16_t>(ptx::pack_bf16x2(o[k], 0.f) & 0xFFFFu);
+          }
+        }
+        // the last epilogue warp of the grid to pass its wait puts both counters back to zero for the next launch
+        if (epi && lane == 0 && passed == ngrid * 4 - 1) {
+          f.sync[0] = 0;
+          f.sync[1] = 0;
+        }
+      }
+    } else {
+      ptx::cluster_sync_all();
+      if (epi || wide) {
+        const float *buf = reinterpret_cast<const float *>(red);
+        const int n_units = cols_per * 32;  // unit = (token, 4 adjacent W rows)
+        const int row0 = bid / p.splits * kTileM;
+        auto sum_partials = [&](int cl, int r4) {
+          float4 acc4 = make_float4(0.f, 0.f, 0.f, 0.f);
+          for (int sp = 0; sp < p.splits; ++sp) {
+            const float4 w = *reinterpret_cast<const float4 *>(buf + ((sp * cols_per + cl) * kTileM + r4));
+            acc4.x += w.x; acc4.y += w.y; acc4.z += w.z; acc4.w += w.w;
+          }
+          return acc4;
+        };
+        auto store4 = [&](int t, int j, const float4 &v) {
+          uint2 o;
+          o.x = ptx::pack_bf16x2(v.x, v.y);
+          o.y = ptx::pack_bf16x2(v.z, v.w);
+          *reinterpret_cast<uint2 *>(p.y + static_cast<size_t>(t) * p.h_out + j) = o;
+        };
+        if (!p.expand_in_reduce) {
+          // unit = (token quad, W row): the splits' partial sums are 16 bytes each, lanes take
+          // adjacent rows, so a warp writes 64 bytes in a row of y per token
+          const int qpo = cols_per >> 2;
+          const float4 *buf4 = reinterpret_cast<const float4 *>(red);
+          ptx::pdl_wait_prior_grids();  // warps 0 and 1 have not waited yet; earlier kernels may read y
+          for (int u = threadIdx.x; u < qpo * kTileM; u += kGemmThreads) {
+            const int qd = u >> 7, r = u & (kTileM - 1);
+            const int t0 = static_cast<int>(my_rank) * cols_per + qd * 4, j = row0 + r;
+            if (t0 >= p.T || j >= p.h_out) continue;
+            float4 a4 = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int sp = 0; sp < p.splits; ++sp) {
+              const float4 w = buf4[(sp * qpo + qd) * kTileM + r];
+              a4.x += w.x; a4.y += w.y; a4.z += w.z; a4.w += w.w;
+            }
+            const float o[4] = {a4.x, a4.y, a4.z, a4.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (t0 + i < p.T)
+                p.y[static_cast<size_t>(t0 + i) * p.h_out + j] =
+                    static_cast<uint16_t>(ptx::pack_bf16x2(o[i], 0.f) & 0xFFFFu);
+          }
+        } else {
+          // Small batches: wait for the shrink kernel (and for earlier readers of y), then per unit add the
+          // splits' partial sums, fetch z and the B_a rows in one round trip, add B_a[j..j+3][0..r) . z[t]
+          // in fp32 (z carries s_a) and write y.  A rolled loop over the units (at most 4 per thread:
+          // cols_per <= 16): this code runs once per launch, and what it costs is mostly the fetching
+          // of its instructions.
+          ptx::pdl_wait_prior_grids();
+          const int nch = p.R_pad >> 3;
+          const int n_zp = kFused ? f.ks : 1;
+          const size_t zplane4 = static_cast<size_t>(p.max_tokens) * p.R_pad / 4;
+          auto load_z4 = [&](const float4 *ptr) {
+            float4 v = __ldcg(ptr);
+            for (int sp = 1; sp < n_zp; ++sp) {
+              const float4 w = __ldcg(ptr + sp * zplane4);
+              v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+            }
+            return v;
+          };
+#pragma unroll 1
+          for (int u = etid; u < n_units; u += 128) {
+            const int cl = u >> 5, r4 = (u & 31) << 2;
+            const int t = static_cast<int>(my_rank) * cols_per + cl, j = row0 + r4;
+            if (t >= p.T || j >= p.h_out) continue;
+            float4 acc4 = sum_partials(cl, r4);
+            const int32_t a = z_ok ? s_vid[cl] : -1, rank = s_lg[cl];  // stored by the epilogue warps at the start
+            if (a >= 0) {
+              const uint4 *Brow = reinterpret_cast<const uint4 *>(
+                  p.B_pool + (static_cast<size_t>(a) * p.h_out + j) * p.R_pad);
+              const float4 *zt = reinterpret_cast<const float4 *>((kFused ? f.z : p.zws) + static_cast<size_t>(t) * p.R_pad);
+              float add[4] = {0.f, 0.f, 0.f, 0.f};
+              for (int c0 = 0; c0 < nch && c0 * 8 < rank; c0 += 2) {
+                uint4 b[2][4];
+                float4 z4[2][2];
+#pragma unroll
+                for (int cc = 0; cc < 2; ++cc) {  // two chunks of 8 rank values: 12 loads in flight
+                  const int c = c0 + cc;
+                  const bool on = c < nch && c * 8 < rank;
+#pragma unroll
+                  for (int r = 0; r < 4; ++r) b[cc][r] = on ? __ldg(Brow + r * nch + c) : make_uint4(0u, 0u, 0u, 0u);
+                  z4[cc][0] = on ? load_z4(zt + 2 * c) : make_float4(0.f, 0.f, 0.f, 0.f);
+                  z4[cc][1] = on ? load_z4(zt + 2 * c + 1) : make_float4(0.f, 0.f, 0.f, 0.f);
+                }
+#pragma unroll
+                for (int cc = 0; cc < 2; ++cc) {
+                  const float4 u0 = z4[cc][0], u1 = z4[cc][1];
+#pragma unroll
+                  for (int r = 0; r < 4; ++r) {
+                    const uint4 bb = b[cc][r];
+                    float s4 = add[r];
+                    s4 = fmaf(ptx::bf16_lo(bb.x), u0.x, s4);
+                    s4 = fmaf(ptx::bf16_hi(bb.x), u0.y, s4);
+                    s4 = fmaf(ptx::bf16_lo(bb.y), u0.z, s4);
+                    s4 = fmaf(ptx::bf16_hi(bb.y), u0.w, s4);
+                    s4 = fmaf(ptx::bf16_lo(bb.z), u1.x, s4);
+                    s4 = fmaf(ptx::bf16_hi(bb.z), u1.y, s4);
+                    s4 = fmaf(ptx::bf16_lo(bb.w), u1.z, s4);
+                    s4 = fmaf(ptx::bf16_hi(bb.w), u1.w, s4);
+                    add[r] = s4;
+                  }
                 }
               }
+              acc4.x += add[0]; acc4.y += add[1]; acc4.z += add[2]; acc4.w += add[3];
             }
-            acc4.x += add[0]; acc4.y += add[1]; acc4.z += add[2]; acc4.w += add[3];
+            store4(t, j, acc4);
           }
-          store4(t, j, acc4);
-        }
-        if (kFused && lane == 0) {
-          // this warp is past its wait for the shrink teams: the last such warp of the grid puts both
-          // counters back to zero for the next launch
-          if (atomicAdd(f.sync + 1, 1) == ngrid * 4 - 1) {
-            f.sync[0] = 0;
-            f.sync[1] = 0;
+          if (kFused && lane == 0) {
+            // this warp is past its wait for the shrink teams: the last such warp of the grid puts both
+            // counters back to zero for the next launch
+            if (atomicAdd(f.sync + 1, 1) == ngrid * 4 - 1) {
+              f.sync[0] = 0;
+              f.sync[1] = 0;
+            }
           }
         }
       }
@@ -993,11 +1026,11 @@ cudaError_t launch_gemm(const CUtensorMap &tmap_row, const CUtensorMap &tmap_col
                    tmap_row, tmap_col, tmap_b, p, not_fused());
 }
 
-cudaError_t launch_gemm_fused(const CUtensorMap &tmap_row, const CUtensorMap &tmap_col, const GemmParams &p,
+cudaError_t launch_gemm_fused(const CUtensorMap &tmap_row, const CUtensorMap &tmap_col, const CUtensorMap &tmap_b, const GemmParams &p,
                               const FusedDecode &f, size_t smem_bytes, bool pdl, cudaStream_t stream) {
   const int32_t grid = f.n_ctas + p.n_mtiles * p.splits;
   return launch_ex(lora_gemm_kernel<1, true>, dim3(grid), dim3(kGemmThreads), smem_bytes, stream, pdl, p.splits,
-                   tmap_row, tmap_col, tmap_row, p, f);
+                   tmap_row, tmap_col, tmap_b, p, f);
 }
 
 int32_t gemm_fused_max_ctas(int32_t cluster, size_t smem_bytes) {

@@ -117,7 +117,7 @@ void init_plan_kernel();
 cudaError_t launch_gemm(const CUtensorMap &tmap_row, const CUtensorMap &tmap_col, const CUtensorMap &tmap_b,
                         const GemmParams &p, int32_t grid, size_t smem_bytes, bool pdl, cudaStream_t stream);
 // Decode job with the shrink in the same grid: grid = f.n_ctas + p.n_mtiles * p.splits CTAs.
-cudaError_t launch_gemm_fused(const CUtensorMap &tmap_row, const CUtensorMap &tmap_col, const GemmParams &p,
+cudaError_t launch_gemm_fused(const CUtensorMap &tmap_row, const CUtensorMap &tmap_col, const CUtensorMap &tmap_b, const GemmParams &p,
                               const FusedDecode &f, size_t smem_bytes, bool pdl, cudaStream_t stream);
 // How many CTAs of such a launch (in whole clusters) can be resident at once on the current device.
 int32_t gemm_fused_max_ctas(int32_t cluster, size_t smem_bytes);

@@ -1050,6 +1050,18 @@ int decode_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32_
   return EDGELORA_OK;
 }
 
+// CTAs of a one-launch decode call that the device holds at once, asked once per shape of the last few.
+static int fused_max_ctas(edgelora_pool *p, int splits, size_t smem) {
+  const uint64_t key = (static_cast<uint64_t>(splits) << 32) | static_cast<uint64_t>(smem);
+  for (const auto &f : p->fused_fits)
+    if (f.key == key) return f.ctas;
+  auto &f = p->fused_fits[p->fused_next];
+  p->fused_next = (p->fused_next + 1) % (sizeof(p->fused_fits) / sizeof(p->fused_fits[0]));
+  f.key = key;
+  f.ctas = gemm_fused_max_ctas(splits, smem);
+  return f.ctas;
+}
+
 int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_dev, const void *W_dev,
                      const void *x_dev, int32_t T, void *y_dev, cudaStream_t stream, Order order) {
   if (!p || !plan || T < 0) return EDGELORA_ERR_INVALID_ARG;
@@ -1250,25 +1262,31 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
     // 16.9 against 19.7 us when each call waits for the one before.)
     if (p->opt_fused_decode && !pdl_first && g.expand_in_reduce && T <= 64 && T <= kGatherMinT && ids_dev &&
         !p->a_q8 && h_in % 8 == 0) {
-      FusedDecode f{};
-      // room behind the ring for the B_a rows and z of an owner's tokens, when it fits
-      // (2: and for the cluster reduction's buffer, which then does not have to wait for the ring)
-      size_t stage_extra = static_cast<size_t>(N / splits) * (kTileM * R * 2 + R * 4);
-      f.b_stage = smem_for(g.stages, N, static_cast<int>(stage_extra)) <= kSmemBudget ? 1 : 0;
-      const size_t with_buf = ((stage_extra + 1023) & ~static_cast<size_t>(1023)) + static_cast<size_t>(N) * kTileM * 4;
-      if (f.b_stage && smem_for(g.stages, N, static_cast<int>(with_buf)) <= kSmemBudget) {
-        f.b_stage = 2;
-        stage_extra = with_buf;
-      }
-      const size_t smem = smem_for(g.stages, N, f.b_stage ? static_cast<int>(stage_extra) : 0);
-      const uint64_t key = (static_cast<uint64_t>(splits) << 32) | static_cast<uint64_t>(smem);
-      if (p->fused_key != key) {
-        p->fused_key = key;
-        p->fused_max_ctas = gemm_fused_max_ctas(splits, smem);
-      }
-      const int spare = std::max(0, std::min(p->fused_max_ctas - grid, 32) / splits * splits);
-      if (spare > 0) {  // every CTA resident at once, and a spare CTA to publish the routing plan
-        const int n_teams = 2 * spare + grid;
+      // Fewer K splits when the clusters of all row tiles do not fit beside a spare one (clusters of eight: 16 on this chip;
+      // 2048 -> 2048, 8 tokens: 6.6 us in one launch with 4 splits, 10.4 in two with 8).
+      for (int sp = splits; sp > 1 && !fused; sp >>= 1) {
+        if (N / sp > 16 || (N / sp) * (R / 8) > 64 || (p->opt_decode_splits != 0 && sp != splits)) break;
+        GemmParams gf = g;
+        gf.splits = sp;
+        gf.kb_per = (kb_total + sp - 1) / sp;
+        if (gf.kb_per * (sp - 1) >= kb_total) continue;  // every split needs a K block
+        gf.stages = stages_for(N, gf.kb_per + 8, budget);
+        while (gf.stages * stage_bytes < N * kTileM * 4 + (N / sp) * R * 4 && gf.stages < kMaxStages) ++gf.stages;
+        FusedDecode f{};
+        // room behind the ring for the B_a rows and z of an owner's tokens, when it fits
+        // (2: and for the cluster reduction's buffer, which then does not have to wait for the ring)
+        size_t stage_extra = static_cast<size_t>(N / sp) * (kTileM * R * 2 + R * 4);
+        f.b_stage = smem_for(gf.stages, N, static_cast<int>(stage_extra)) <= kSmemBudget ? 1 : 0;
+        const size_t with_buf = ((stage_extra + 1023) & ~static_cast<size_t>(1023)) + static_cast<size_t>(N) * kTileM * 4;
+        if (f.b_stage && smem_for(gf.stages, N, static_cast<int>(with_buf)) <= kSmemBudget) {
+          f.b_stage = 2;
+          stage_extra = with_buf;
+        }
+        const size_t smem = smem_for(gf.stages, N, f.b_stage ? static_cast<int>(stage_extra) : 0);
+        const int gf_grid = row_tiles * sp;
+        const int spare = std::max(0, std::min(fused_max_ctas(p, sp, smem) - gf_grid, 32) / sp * sp);
+        if (spare == 0) continue;  // every CTA resident at once, and a spare CTA to publish the routing plan
+        const int n_teams = 2 * spare + gf_grid;
         const int n_ksteps = (h_in + kShrinkStepElems - 1) / kShrinkStepElems;
         int ks = std::max(1, std::min(kMaxZSplits, n_ksteps / 4));
         while (ks > 1 && T * (R / 8) * ks > 2 * n_teams) ks >>= 1;
@@ -1280,12 +1298,16 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
         f.z = p->zws;
         f.sync = p->group_counters + kDecodeMaxT * 8 + 8;
         f.pv = plan->pv;
+        CUtensorMap me;  // B_a rows for the expand on the CUDA cores: boxes as wide as the rank stride
+        rc = get_tmap(p, &me, p->B_pool, R, h_out, p->cfg.n_slots, kTileM, R);
+        if (rc) return rc;
         ProfScope ps(p, 3, stream);
-        CUDA_TRY(launch_gemm_fused(mr, mc, g, f, smem, p->opt_pdl != 0, stream));
+        CUDA_TRY(launch_gemm_fused(mr, mc, me, gf, f, smem, p->opt_pdl != 0, stream));
         ++launches;
         fused = true;
-        p->last_info[2] = grid + spare;
-        p->last_info[3] = splits;
+        g = gf;
+        p->last_info[2] = gf_grid + spare;
+        p->last_info[3] = sp;
       }
     }
     if (!fused) {

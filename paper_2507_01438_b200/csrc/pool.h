@@ -83,8 +83,11 @@ struct edgelora_pool {
   std::vector<TmapEntry> tmaps;
   size_t tmap_next = 0;
   int opt_regime = 0, opt_profile = 0, opt_pdl = 1, opt_fused_decode = 1;
-  uint64_t fused_key = 0;  // launch shape the occupancy answer below belongs to
-  int fused_max_ctas = 0;
+  struct {
+    uint64_t key = 0;  // launch shape: K splits and shared memory
+    int ctas = 0;      // the occupancy answer for it
+  } fused_fits[8];
+  int fused_next = 0;
   long long wait_cycles = edgelora::ptx::kWaitLimitCycles;
   int64_t last_info[8] = {0};
   int64_t total_launches = 0;

@@ -105,3 +105,23 @@ def test_status_bits_of_the_one_launch_path():
         assert_parity(from_dev_bf16(y), oracle_of(ref), "bad ids and empty slots fall back to the base product")
     finally:
         pool.close()
+
+
+@pytest.mark.parametrize("T,h_in,h_out,max_rank", [
+    (3, 1024, 136, 64), (16, 512, 1032, 32), (31, 4096, 4096, 32), (32, 1024, 72, 16), (64, 4096, 1000, 16),
+    (64, 1024, 2056, 32), (2, 14336, 512, 16),
+])
+def test_expand_beside_the_exchange_of_partial_sums(T, h_in, h_out, max_rank):
+    # one to four token quads per CTA of a cluster, staged rows of 32, 64 and 128 bytes, row tiles that end inside a tile,
+    # ranks that end inside a group of eight, tokens without an adapter and on an empty slot, K chunks in several planes
+    ranks = [max_rank, max_rank // 2, max_rank - 3, 1, 0, max_rank, 5, max_rank]
+    w = random_workload(7300 + T + h_out, T, h_in, h_out, ranks=ranks, max_rank=max_rank)
+    w.ids = np.random.Generator(np.random.PCG64(T)).integers(-1, len(ranks), size=T).astype(np.int32)
+    w.ids[w.ids == 4] = -1
+    pool = make_pool(w, 64)
+    try:
+        for _ in range(2):
+            assert_parity(run_gpu(w, 1, pool=pool), oracle_of(w), f"T={T} {h_in}->{h_out}")
+            assert B.edgelora_pool_last_launch(pool.handle)["launches"] == 1
+    finally:
+        pool.close()
