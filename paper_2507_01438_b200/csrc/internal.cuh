@@ -123,9 +123,10 @@ cudaError_t launch_gemm_fused(const CUtensorMap &tmap_row, const CUtensorMap &tm
 int32_t gemm_fused_max_ctas(int32_t cluster, size_t smem_bytes);
 cudaError_t gemm_set_smem_limit(size_t smem_bytes);
 cudaError_t shrink_set_smem_limit();
-cudaError_t launch_q8_to_block(const uint8_t *A_q8, const uint8_t *B_q8, uint16_t *A_blk, uint16_t *B_blk,
-                               int32_t rank, int32_t R_pad, int32_t h_in, int32_t h_out, int32_t sms,
-                               cudaStream_t stream);
+// An adapter in Q8_0 form in page-locked host memory (both parts 16-byte aligned, 16 bytes readable behind them) into its slot.
+cudaError_t launch_q8_load(const uint8_t *a_pinned, size_t a_bytes, const uint8_t *b_pinned, size_t b_bytes, uint16_t *A_blk,
+                           uint16_t *B_blk, const SlotRow &row, SlotRow *slot, int32_t R_pad, int32_t h_in, int32_t h_out,
+                           bool keep_q8, cudaStream_t stream);
 void set_last_cuda_error(cudaError_t e, const char *what);
 cudaError_t launch_wait_selftest(uint32_t *status, long long wait_cycles, cudaStream_t stream);
 cudaError_t launch_decode_shrink(const CUtensorMap &tmap_a, const CUtensorMap &tmap_d, const CUtensorMap &tmap_x,

@@ -365,7 +365,6 @@ int edgelora_pool_create(const edgelora_pool_config *cfg, edgelora_pool_t **pool
     POOL_TRY(cudaEventCreateWithFlags(&sb.done, cudaEventDisableTiming));
   }
   POOL_TRY(cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking));
-  POOL_TRY(cudaEventCreateWithFlags(&p->load_ev, cudaEventDisableTiming));
   POOL_TRY(cudaEventCreateWithFlags(&p->use_ev, cudaEventDisableTiming));
   // partial planes [0, kMaxZSplits) plus the final plane of the decode shrink
   POOL_TRY(el_malloc(&p->zws, sizeof(float) * (kMaxZSplits + 1) * static_cast<size_t>(p->cfg.max_tokens) * p->R_pad));
@@ -404,10 +403,8 @@ int edgelora_pool_destroy(edgelora_pool_t *p) {
     if (sb.done) cudaEventDestroy(sb.done);
   }
   if (p->side) cudaStreamDestroy(p->side);
-  if (p->load_ev) cudaEventDestroy(p->load_ev);
   if (p->use_ev) cudaEventDestroy(p->use_ev);
   if (p->zws) el_free(p->zws);
-  if (p->q8_dev) el_free(p->q8_dev);
   if (p->group_counters) el_free(p->group_counters);
   if (p->tile_counters) el_free(p->tile_counters);
   for (auto &r : p->prof) {
@@ -441,6 +438,21 @@ static size_t slot_row_offset(const edgelora_pool *p) {
   return p->a_block * 2 + 16 + std::max(p->b_block * 2, b_q8_bytes);
 }
 
+// Orders the side stream behind the last call that may still read this pool, once per call.
+static int wait_for_use(edgelora_pool *p) {
+  if (p->use_recorded) CUDA_TRY(cudaStreamWaitEvent(p->side, p->use_ev, 0));
+  p->use_recorded = false;
+  return EDGELORA_OK;
+}
+// A load is on the side stream: its staging buffer is free again, and the calls behind it may run, when its event is done.
+static int load_issued(edgelora_pool *p, StagingBuf &sb) {
+  CUDA_TRY(cudaEventRecord(sb.done, p->side));
+  sb.in_flight = true;
+  p->last_load = sb.done;
+  p->load_seq += 1;
+  return EDGELORA_OK;
+}
+
 static int stage_and_copy(edgelora_pool *p, int32_t slot, int32_t rank, float scale,
                           const uint16_t *A_host, const uint16_t *B_host) {
   if (p->a_q8 && rank > 0) return EDGELORA_ERR_INVALID_ARG;  // this pool takes Q8_0 adapters only
@@ -459,8 +471,7 @@ static int stage_and_copy(edgelora_pool *p, int32_t slot, int32_t rank, float sc
   mirror.scale = scale;
   mirror.generation += 1;
   *srow = mirror;
-  // order against the last layer call that may still read this pool
-  if (p->use_recorded) CUDA_TRY(cudaStreamWaitEvent(p->side, p->use_ev, 0));
+  if (const int rc = wait_for_use(p)) return rc;
   if (rank > 0) {
     // A: rows [rank, R) are zero; B: columns [rank, R) are zero
     memcpy(sa, A_host, static_cast<size_t>(rank) * h_in * 2);
@@ -477,11 +488,7 @@ static int stage_and_copy(edgelora_pool *p, int32_t slot, int32_t rank, float sc
     CUDA_TRY(cudaMemcpyAsync(p->B_pool + p->b_block * slot, sbp, p->b_block * 2, cudaMemcpyHostToDevice, p->side));
   }
   CUDA_TRY(cudaMemcpyAsync(p->slots_dev + slot, srow, sizeof(SlotRow), cudaMemcpyHostToDevice, p->side));
-  CUDA_TRY(cudaEventRecord(sb.done, p->side));
-  sb.in_flight = true;
-  CUDA_TRY(cudaEventRecord(p->load_ev, p->side));
-  p->load_seq += 1;
-  return EDGELORA_OK;
+  return load_issued(p, sb);
 }
 
 int edgelora_pool_load_slot(edgelora_pool_t *p, int32_t slot, int32_t rank, float scale,
@@ -517,15 +524,11 @@ int edgelora_pool_load_slot_pinned(edgelora_pool_t *p, int32_t slot, int32_t ran
   mirror.scale = scale;
   mirror.generation += 1;
   *srow = mirror;
-  if (p->use_recorded) CUDA_TRY(cudaStreamWaitEvent(p->side, p->use_ev, 0));
+  if (const int rc = wait_for_use(p)) return rc;
   CUDA_TRY(cudaMemcpyAsync(p->A_pool + p->a_block * slot, A_pinned, p->a_block * 2, cudaMemcpyHostToDevice, p->side));
   CUDA_TRY(cudaMemcpyAsync(p->B_pool + p->b_block * slot, B_pinned, p->b_block * 2, cudaMemcpyHostToDevice, p->side));
   CUDA_TRY(cudaMemcpyAsync(p->slots_dev + slot, srow, sizeof(SlotRow), cudaMemcpyHostToDevice, p->side));
-  CUDA_TRY(cudaEventRecord(sb.done, p->side));
-  sb.in_flight = true;
-  CUDA_TRY(cudaEventRecord(p->load_ev, p->side));
-  p->load_seq += 1;
-  return EDGELORA_OK;
+  return load_issued(p, sb);
 }
 
 int edgelora_pool_load_slot_q8(edgelora_pool_t *p, int32_t slot, int32_t rank, float scale, const void *A_q8,
@@ -538,71 +541,23 @@ int edgelora_pool_load_slot_q8(edgelora_pool_t *p, int32_t slot, int32_t rank, f
   const size_t a_bytes = static_cast<size_t>(rank) * (h_in / 32) * 34;
   const size_t b_bytes = static_cast<size_t>(h_out) * ((rank + 31) / 32) * 34;
   const size_t b_off = (a_bytes + 15) & ~static_cast<size_t>(15);
-  const size_t scratch = static_cast<size_t>(p->cfg.max_rank) * (h_in / 32) * 34 + 16 +
-                         static_cast<size_t>(h_out) * ((p->cfg.max_rank + 31) / 32) * 34;
-  if (!p->q8_dev) CUDA_TRY(el_malloc(&p->q8_dev, scratch));
   StagingBuf &sb = p->staging[p->next_staging];
   p->next_staging = (p->next_staging + 1) % kStagingBuffers;
   if (sb.in_flight) {
     CUDA_TRY(cudaEventSynchronize(sb.done));
     sb.in_flight = false;
   }
-  if (p->a_q8) {
-    // the pool keeps A in Q8_0: rows [rank, R_pad) are zero blocks; only B is converted on the device
-    const size_t a_pad = p->a_block * 2;
-    {  // the pool's layout: the signed bytes of all rows, then the block scales of all rows
-      const int nb = h_in / 32;
-      const uint8_t *src = static_cast<const uint8_t *>(A_q8);
-      uint8_t *qplane = sb.host, *dplane = sb.host + static_cast<size_t>(R) * h_in;
-      memset(sb.host, 0, a_pad);
-      for (int r = 0; r < rank; ++r)
-        for (int b = 0; b < nb; ++b) {
-          const uint8_t *blk = src + (static_cast<size_t>(r) * nb + b) * 34;
-          memcpy(dplane + (static_cast<size_t>(r) * nb + b) * 2, blk, 2);
-          memcpy(qplane + static_cast<size_t>(r) * h_in + b * 32, blk + 2, 32);
-        }
-    }
-    const size_t b_off2 = (a_pad + 15) & ~static_cast<size_t>(15);
-    memcpy(sb.host + b_off2, B_q8, b_bytes);
-    SlotRow *srow2 = reinterpret_cast<SlotRow *>(sb.host + slot_row_offset(p));
-    SlotRow &m2 = p->slots_host[slot];
-    m2.rank = rank;
-    m2.scale = scale;
-    m2.generation += 1;
-    *srow2 = m2;
-    if (p->use_recorded) CUDA_TRY(cudaStreamWaitEvent(p->side, p->use_ev, 0));
-    CUDA_TRY(cudaMemcpyAsync(p->A_pool + p->a_block * slot, sb.host, a_pad, cudaMemcpyHostToDevice, p->side));
-    CUDA_TRY(cudaMemcpyAsync(p->q8_dev, sb.host + b_off2, b_bytes, cudaMemcpyHostToDevice, p->side));
-    CUDA_TRY(launch_q8_to_block(nullptr, p->q8_dev, nullptr, p->B_pool + p->b_block * slot, rank, R, h_in, h_out,
-                                p->sms, p->side));
-    CUDA_TRY(cudaMemcpyAsync(p->slots_dev + slot, srow2, sizeof(SlotRow), cudaMemcpyHostToDevice, p->side));
-    CUDA_TRY(cudaEventRecord(sb.done, p->side));
-    sb.in_flight = true;
-    CUDA_TRY(cudaEventRecord(p->load_ev, p->side));
-    p->load_seq += 1;
-    return EDGELORA_OK;
-  }
   // the 8-bit form is smaller than the block the staging buffer was sized for
   memcpy(sb.host, A_q8, a_bytes);
   memcpy(sb.host + b_off, B_q8, b_bytes);
-  SlotRow *srow = reinterpret_cast<SlotRow *>(sb.host + slot_row_offset(p));
   SlotRow &mirror = p->slots_host[slot];
   mirror.rank = rank;
   mirror.scale = scale;
   mirror.generation += 1;
-  *srow = mirror;
-  if (p->use_recorded) CUDA_TRY(cudaStreamWaitEvent(p->side, p->use_ev, 0));
-  // (the scratch is reused by every load: the copies and conversions of one pool run in order on
-  // its side stream)
-  CUDA_TRY(cudaMemcpyAsync(p->q8_dev, sb.host, b_off + b_bytes, cudaMemcpyHostToDevice, p->side));
-  CUDA_TRY(launch_q8_to_block(p->q8_dev, p->q8_dev + b_off, p->A_pool + p->a_block * slot,
-                              p->B_pool + p->b_block * slot, rank, R, h_in, h_out, p->sms, p->side));
-  CUDA_TRY(cudaMemcpyAsync(p->slots_dev + slot, srow, sizeof(SlotRow), cudaMemcpyHostToDevice, p->side));
-  CUDA_TRY(cudaEventRecord(sb.done, p->side));
-  sb.in_flight = true;
-  CUDA_TRY(cudaEventRecord(p->load_ev, p->side));
-  p->load_seq += 1;
-  return EDGELORA_OK;
+  if (const int rc = wait_for_use(p)) return rc;
+  CUDA_TRY(launch_q8_load(sb.host, a_bytes, sb.host + b_off, b_bytes, p->A_pool + p->a_block * slot,
+                          p->B_pool + p->b_block * slot, mirror, p->slots_dev + slot, R, h_in, h_out, p->a_q8, p->side));
+  return load_issued(p, sb);
 }
 
 int edgelora_pool_evict_slot(edgelora_pool_t *p, int32_t slot) {
@@ -780,7 +735,7 @@ int wait_for_loads(edgelora_pool *p, cudaStream_t stream, bool capturing) {
     it = p->load_waited.end() - 1;
   }
   if (it->second != p->load_seq) {
-    CUDA_TRY(cudaStreamWaitEvent(stream, p->load_ev, 0));
+    CUDA_TRY(cudaStreamWaitEvent(stream, p->last_load, 0));
     it->second = p->load_seq;
   }
   return EDGELORA_OK;

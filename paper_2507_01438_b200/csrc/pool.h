@@ -62,7 +62,6 @@ struct edgelora_pool {
   int R_pad = 0, device = 0, sms = 0;
   bool owns_arena = false, a_q8 = false;  // a_q8: the A blocks are kept in Q8_0 (EDGELORA_FLAG_A_Q8)
   uint8_t *arena = nullptr;
-  uint8_t *q8_dev = nullptr;  // device scratch for one adapter in Q8_0 form (first use of load_slot_q8)
   uint16_t *A_pool = nullptr, *B_pool = nullptr;
   size_t a_block = 0, b_block = 0;  // elements per slot
   SlotRow *slots_dev = nullptr;
@@ -70,7 +69,8 @@ struct edgelora_pool {
   StagingBuf staging[edgelora::kStagingBuffers];
   int next_staging = 0;
   cudaStream_t side = nullptr;
-  cudaEvent_t load_ev = nullptr, use_ev = nullptr;
+  cudaEvent_t use_ev = nullptr;
+  cudaEvent_t last_load = nullptr;  // the event of the staging buffer that the last load went through
   uint64_t load_seq = 0;
   std::vector<std::pair<cudaStream_t, uint64_t>> load_waited;  // per stream: last load it waited for
   bool use_recorded = false;

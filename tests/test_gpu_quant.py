@@ -132,3 +132,46 @@ def test_base_weights_decode_is_bit_exact_and_feeds_the_layer(fmt, code, encode)
     with pytest.raises(B.EdgeLoraError) as e:
         B.edgelora_weights_decode(7, Wq, w.h_out, w.h_in, W)
     assert e.value.code == B.ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("keep_q8", [False, True])
+@pytest.mark.parametrize("h_in,h_out,max_rank,ranks", [
+    (256, 8, 64, [64, 33, 1]), (1024, 1000, 16, [16, 5, 9]), (4096, 120, 32, [32, 9]), (512, 488, 64, [40, 32, 8]),
+])
+def test_a_loaded_slot_bit_for_bit(h_in, h_out, max_rank, ranks, keep_q8):
+    # the slot's blocks in the caller's arena against the decoded values rounded to bfloat16 (or, for a pool that keeps A in
+    # Q8_0, its bytes and scales): CTAs' shares that end inside a row and inside the adapter, one and two blocks per row of B,
+    # padding over what an adapter of a higher rank left behind
+    import torch
+    if not keep_q8:
+        h_in -= 224                                                        # 32 values and odd numbers of blocks too
+    rng = np.random.Generator(np.random.PCG64(h_in + h_out))
+    R = 16 if max_rank <= 16 else 32 if max_rank <= 32 else 64
+    flags = B.FLAG_A_Q8 if keep_q8 else 0
+    a_bytes = R * h_in // 32 * 34 if keep_q8 else R * h_in * 2
+    arena = torch.full((B.edgelora_pool_bytes_required(h_in, h_out, 1, max_rank),), 0x55, dtype=torch.uint8, device="cuda") \
+        if not keep_q8 else torch.full((a_bytes + 2 * R * h_out,), 0x55, dtype=torch.uint8, device="cuda")
+    pool = B.Pool(h_in, h_out, 1, max_rank, max_tokens=16, arena=arena, flags=flags)
+    decode = lambda blocks, n: (np.ascontiguousarray(blocks[..., :2]).view(np.float16).astype(np.float32) *
+                                blocks[..., 2:].view(np.int8).astype(np.float32)).reshape(blocks.shape[0], -1)[:, :n]
+    try:
+        for r in ranks:
+            A, Bm = (wl.q8_0_encode((rng.standard_normal(s) * 0.05).astype(np.float32)) for s in ((r, h_in), (h_out, r)))
+            B.edgelora_pool_load_slot_q8(pool.handle, 0, r, 2.0, A, Bm)
+            B.edgelora_pool_wait_loads(pool.handle)
+            got = arena.cpu().numpy()
+            want = np.zeros((h_out, R), np.float32)
+            want[:, :r] = decode(Bm.reshape(h_out, -1, 34), r)
+            assert np.array_equal(got[a_bytes:a_bytes + 2 * R * h_out].view(np.uint16).reshape(h_out, R), wl.f32_to_bf16_bits(want))
+            blocks = A.reshape(r, -1, 34)
+            if keep_q8:
+                q, d = np.zeros((R, h_in), np.uint8), np.zeros((R, h_in // 32), np.uint16)
+                q[:r], d[:r] = blocks[..., 2:].reshape(r, h_in), np.ascontiguousarray(blocks[..., :2]).view(np.uint16)[..., 0]
+                assert np.array_equal(got[:R * h_in].reshape(R, h_in), q)
+                assert np.array_equal(got[R * h_in:a_bytes].view(np.uint16).reshape(R, -1), d)
+            else:
+                want = np.zeros((R, h_in), np.float32)
+                want[:r] = decode(blocks, h_in)
+                assert np.array_equal(got[:a_bytes].view(np.uint16).reshape(R, h_in), wl.f32_to_bf16_bits(want))
+    finally:
+        pool.close()
