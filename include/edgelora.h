@@ -178,11 +178,9 @@ int edgelora_pool_wait_loads(edgelora_pool_t *pool);
  * adapter_id_dev [T] (slot index or -1), y_dev [T][h_out]; all device memory, 16-byte
  * aligned.  Enqueues, on `stream` (a cudaStream_t; NULL = legacy default stream):
  * routing plan -> shrink (z = s_a A_a x) -> base product W x on the tensor cores with
- * the expand B_a z accumulated into the same tile (z rounded to bfloat16 for it) -> y written
- * once.  Asynchronous; no host synchronisation, no
- * allocation.  An infinity or NaN in an adapter's B reaches the tokens on this adapter only in batches above 256
- * tokens and where the expand runs on the CUDA cores (small decode batches); in the other decode batches it makes
- * the whole batch's y NaN (zeros of z times infinity).  T == 0 is a no-op.  x_dev / y_dev must not alias.  Calls of one pool share its
+ * the expand B_a z added before y is written, once (in batches above 256 tokens z is rounded to bfloat16 for it, in
+ * smaller ones it stays fp32).  Asynchronous; no host synchronisation, no
+ * allocation.  An infinity or NaN in an adapter's B reaches the tokens on this adapter only.  T == 0 is a no-op.  x_dev / y_dev must not alias.  Calls of one pool share its
  * workspaces: they must not overlap on the GPU (one stream, or ordered by events). */
 int edgelora_lora_linear(edgelora_pool_t *pool, const void *W_dev, const void *x_dev,
                          const int32_t *adapter_id_dev, int32_t T, void *y_dev, void *stream);

@@ -40,18 +40,24 @@ __device__ __forceinline__ int block_scan_256(int v, int *wt, int &total) {
 
 // Writes the routing plan of a batch of T <= 256 tokens in canonical order (ids ascending, -1
 // first; segments in token order).  Called by every thread of one CTA; thread t < T passes the
-// validated id `a` of token t (-1 = no adapter), the others -1.  s_id[256] holds those ids already;
+// validated id `a` of token t (-1 = no adapter), the others -1.  s_id[256], 16-byte aligned, holds those ids already;
 // s_cnt[256] and s_wt[9] are scratch.  Everything is worked out in shared memory and registers
 // first; the stores come after griddepcontrol.wait (earlier kernels on the stream may still read the
 // plan).
 __device__ __forceinline__ void publish_decode_plan(const PlanView &pv, int a, int T, int any_bad, int KS,
                                                     const int32_t *s_id, int32_t *s_cnt, int *s_wt) {
   const int tid = threadIdx.x;
-  const uint32_t key = (static_cast<uint32_t>(a + 1) << 16) | static_cast<uint32_t>(tid);
-  int rp = 0;
-  if (tid < T)
-    for (int u = 0; u < T; ++u)
-      rp += (((static_cast<uint32_t>(s_id[u] + 1) << 16) | static_cast<uint32_t>(u)) < key) ? 1 : 0;
+  int rp = 0;  // position of token tid by (id, token); four ids per shared-memory load
+  if (tid < T) {
+    auto in_front = [&](int id, int u) { return static_cast<int>(id < a) | (static_cast<int>(id == a) & static_cast<int>(u < tid)); };
+    const int full = T & ~3;
+#pragma unroll 4
+    for (int u = 0; u < full; u += 4) {
+      const int4 w = *reinterpret_cast<const int4 *>(s_id + u);
+      rp += in_front(w.x, u) + in_front(w.y, u + 1) + in_front(w.z, u + 2) + in_front(w.w, u + 3);
+    }
+    for (int u = full; u < T; ++u) rp += in_front(s_id[u], u);
+  }
   __syncthreads();  // every thread is done with s_cnt as a counter
   if (tid < T) s_cnt[rp] = tid;  // s_cnt now holds the tokens in canonical order
   __syncthreads();
@@ -130,7 +136,7 @@ __device__ __forceinline__ int32_t group_scan(const int32_t (&v)[kPer], int32_t 
     }
     if (lane == 31) wt[k * (kN / 32) + warp] = incl[k];
   }
-  asm volatile("bar.sync %0, %1;" ::"n"(kBar), "n"(kN) : "memory");
+  ptx::named_barrier<kBar, kN>();
   int32_t total = 0;
 #pragma unroll
   for (int i = 0; i < kPer * kN / 32; ++i) {
@@ -146,7 +152,7 @@ __device__ __forceinline__ int32_t group_scan(const int32_t (&v)[kPer], int32_t 
 template <int kBlockTok, int kBar, int kN>
 __device__ __forceinline__ bool derive_groups(Groups &s, const int32_t *ids, int T, int32_t n_slots, int tid) {
   constexpr int kPer = kDecodeMaxT / kN;
-  const auto sync = [] { asm volatile("bar.sync %0, %1;" ::"n"(kBar), "n"(kN) : "memory"); };
+  const auto sync = [] { ptx::named_barrier<kBar, kN>(); };
   int32_t a[kPer], pos[kPer], first[kPer], v[kPer], out[kPer];
   bool bad = false;
 #pragma unroll

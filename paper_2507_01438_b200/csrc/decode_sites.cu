@@ -25,6 +25,7 @@
 
 #include "decode_route.cuh"
 #include "decode_sites.h"
+#include "expand.cuh"
 #include "launch.cuh"
 #include "ptx.cuh"
 #include "shrink_rows.cuh"
@@ -54,6 +55,7 @@ static_assert(sizeof(DecShared) <= kDecTailBytes, "tail of the shared memory");
 // A barrier of the epilogue warps; every thread learns whether any of them passed true.
 __device__ __forceinline__ bool epilogue_any(bool v) {
   uint32_t r;
+  __syncwarp();
   asm volatile(
       "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.or.pred q, 1, 128, p;\n\t"
       "selp.u32 %0, 1, 0, q;\n\t}"
@@ -70,38 +72,6 @@ __device__ __forceinline__ int32_t first_stage(int32_t unit, int32_t n_stages, i
   return min(unit * (64 >> (31 - __clz(R_pad))), n_stages);
 }
 
-// A row of B_a (its 16-byte chunks swizzled by `sw`) against the z rows of kTok tokens.  What bounds a stage is the latency
-// of this chain, in a single warp per scheduler: so no branches (they kept the loads of a chunk behind the sums of the one
-// before it, 75 cycles a chunk and token), and two sums of two values per token.  z is read up to the last live group of
-// eight rank rows; what lies behind it was not written.
-template <int kR, int kTok>
-__device__ __forceinline__ void expand_dots(const uint8_t *brow, int sw, uint32_t z, int rank, float *acc) {
-  uint64_t s0[kTok], s1[kTok];
-#pragma unroll
-  for (int q = 0; q < kTok; ++q) s0[q] = s1[q] = 0;
-#pragma unroll
-  for (int c = 0; c < kR / 8; ++c) {
-    const uint32_t live = c * 8 < rank ? 1u : 0u;
-    const uint4 bb = *reinterpret_cast<const uint4 *>(brow + ((c ^ sw) << 4));
-    uint64_t u[kTok][4];
-#pragma unroll
-    for (int q = 0; q < kTok; ++q) {
-      ptx::ld_shared_f32x4_if(z + q * (kR * 4) + c * 32, live, u[q][0], u[q][1]);
-      ptx::ld_shared_f32x4_if(z + q * (kR * 4) + c * 32 + 16, live, u[q][2], u[q][3]);
-    }
-    const uint64_t f0 = ptx::f32x2(ptx::bf16_lo(bb.x), ptx::bf16_hi(bb.x)), f1 = ptx::f32x2(ptx::bf16_lo(bb.y), ptx::bf16_hi(bb.y));
-    const uint64_t f2 = ptx::f32x2(ptx::bf16_lo(bb.z), ptx::bf16_hi(bb.z)), f3 = ptx::f32x2(ptx::bf16_lo(bb.w), ptx::bf16_hi(bb.w));
-#pragma unroll
-    for (int q = 0; q < kTok; ++q) {
-      s0[q] = ptx::fma_f32x2(f0, u[q][0], s0[q]);
-      s1[q] = ptx::fma_f32x2(f1, u[q][1], s1[q]);
-      s0[q] = ptx::fma_f32x2(f2, u[q][2], s0[q]);
-      s1[q] = ptx::fma_f32x2(f3, u[q][3], s1[q]);
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < kTok; ++q) acc[q] = ptx::sum_f32x2(s0[q], s1[q]);
-}
 // The stage's tokens, four, two or one at a time, into the columns from `taddr` on.
 template <int kR>
 __device__ __forceinline__ void expand_stage(const uint8_t *brow, int sw, uint32_t z, int rank, int nt, uint32_t taddr) {
@@ -352,8 +322,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_sites_kernel(const __gr
       if (expand) {
         if (etid == 0) ptx::mbar_arrive(&sh.lfull[buf]);
         const uint32_t b_bytes = static_cast<uint32_t>(kTileM * st.R_pad * 2);
-        // a row's 16-byte chunks are swizzled as its length of 32, 64 or 128 bytes has it
-        const int sw = st.R_pad == 64 ? row_in_tile & 7 : st.R_pad == 32 ? (row_in_tile >> 1) & 3 : (row_in_tile >> 2) & 1;
+        const int sw = row_swizzle(row_in_tile, st.R_pad);
         const int32_t s0 = first_stage(p.e0, n_stages, st.R_pad), s1 = first_stage(p.e1, n_stages, st.R_pad);
         p0 = s0 < n_stages ? sh.groups.block_pos[s0] : b.T;
         p1 = s1 < n_stages ? sh.groups.block_pos[s1] : b.T;
@@ -379,6 +348,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_sites_kernel(const __gr
           else expand_stage<64>(brow, sw, z, rank, nt, taddr);
           __syncwarp();
           if (lane == 0) ptx::mbar_arrive(&sh.bempty[stage]);
+          __syncwarp();
           if (++stage == nexp) {
             stage = 0;
             phase ^= 1;
@@ -408,6 +378,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_sites_kernel(const __gr
       const uint32_t tacc = tmem_base + lanes + acc_i * static_cast<uint32_t>(Nc), texp = tmem_exp + lanes;
       for (int32_t n0 = 0; n0 < b.N; n0 += 32) {
         float v[32];
+        __syncwarp();
         if (base) {
           ptx::tmem_ld_32x32(tacc + n0, v);
         } else {

@@ -1,26 +1,25 @@
-// tcgen05 / TMEM / TMA bf16 GEMM for decode batches of batch LoRA inference (paper Section 3.4): the base
-// product W [x_0 .. x_n] batched over every token, with the low-rank expand B_a z folded in so that y is
-// written once.  (Batches above 256 tokens: prefill.cu.)
+// Small decode batches (at most 64 tokens) of batch LoRA inference (paper Section 3.4): the base product W [x_0 .. x_n] batched
+// over every token, with the low-rank expand B_a z added in fp32 before y is written once; in the one-launch form the shrink
+// too.  (Larger batches, or too few row tiles to split K: decode_tile.cu.  Runs of sites: decode_sites.cu.  Above 256 tokens:
+// prefill.cu.)
 //
 // D[128 x BN] (fp32, in tensor memory) = R[128 x K] * C[BN x K]^T, both operands K-major bf16 in
 // 128-byte-swizzled shared-memory tiles of 64 K elements ("K blocks"), multiplied by tcgen05.mma
-// issued from one thread.  R = 128 rows of W, C = all tokens (N = T rounded up).  A tile's K blocks of h_in
-// are followed by one "LoRA K block" per adapter of the batch: its operands are B_a rows (fetched by TMA,
-// zero-filled beyond the rank stride) and the tokens' z rounded to bf16, masked to the tokens of that
-// adapter and written into the operand tile by four builder warps.  W is streamed once; K and the LoRA
-// groups are split across CTAs so every SM pulls from HBM.  The K splits of one row tile form a
+// issued from one thread.  R = 128 rows of W, C = all tokens (N = T rounded up to 32 or 64).  W is streamed once; K is split
+// across CTAs so every SM pulls from HBM.  The K splits of one row tile form a
 // thread-block cluster: after the main loop every CTA sends its fp32 partial tile, column block by column
 // block, into the shared memory of the CTA that owns those tokens (distributed shared memory), and each
-// owner adds the partials in a fixed order and writes its part of y.
+// owner adds the partials in a fixed order, adds the expand of its tokens and writes its part of y.
 //
 // Warp roles: warp 0 issues TMA, warp 1 owns TMEM and issues the MMAs, warps 2..5 are the
-// epilogue (each reads the 32 TMEM lanes of its quadrant), warps 6..9 build the z operand.
+// epilogue (each reads the 32 TMEM lanes of its quadrant), warps 6..9 the shrink team of a one-launch call.
 // Every mbarrier wait is bounded; on a timeout the status word gets EDGELORA_STATUS_TIMEOUT and
 // all roles leave their loops.
 #include <cstdio>
 #include <cstdlib>
 
 #include "decode_route.cuh"
+#include "expand.cuh"
 #include "internal.cuh"
 #include "launch.cuh"
 #include "ptx.cuh"
@@ -51,6 +50,7 @@ __device__ __forceinline__ int32_t tc_row0(const GemmParams &p, int32_t bid) {
 }
 
 __device__ __forceinline__ void named_bar_sync(int id, int threads) {
+  __syncwarp();  // (bar.sync is the aligned form)
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 __device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
@@ -215,12 +215,10 @@ __device__ __forceinline__ void fused_shrink_cta(const GemmParams &p, const Fuse
   if (blockIdx.x == 0) publish_decode_plan(f.pv, a, p.T, any_bad, f.ks, s_id, s_cnt, s_wt);
 }
 
-// kMinBlocks = 2 caps the registers so that the CTAs fit beside the shrink kernel's (small decode tiles); with
-// 1 the builder keeps both of its z rows in registers without spilling.
 // kFused: a launch whose first f.n_ctas CTAs are shrink CTAs (fused_shrink_cta); the job's own CTAs are
-// numbered from there.
-template <int kMinBlocks, bool kFused>
-__global__ void __launch_bounds__(kGemmThreads, kMinBlocks)
+// numbered from there.  Without it the registers are capped so that the CTAs fit beside the shrink kernel's.
+template <bool kFused>
+__global__ void __launch_bounds__(kGemmThreads, kFused ? 1 : 2)
 lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_constant__ CUtensorMap tmap_c,
                  const __grid_constant__ CUtensorMap tmap_b, const GemmParams p, const FusedDecode f) {
   extern __shared__ uint8_t smem_raw[];
@@ -239,45 +237,32 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
   uint64_t *bars = reinterpret_cast<uint64_t *>(smem + static_cast<size_t>(p.stages) * stage_bytes);
   uint64_t *full_bar = bars;                      // [stages]  TMA -> MMA
   uint64_t *empty_bar = bars + kMaxStages;        // [stages]  MMA -> TMA
-  uint64_t *zfull_bar = bars + 2 * kMaxStages;    // [stages]  builder -> MMA (LoRA K blocks)
-  uint64_t *zgo_bar = bars + 3 * kMaxStages;      // [stages]  TMA warp -> builder (stage is free)
-  uint64_t *tfull_bar = bars + 4 * kMaxStages;    //           MMA -> epilogue
+  uint64_t *tfull_bar = bars + 2 * kMaxStages;    //           MMA -> epilogue
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(tfull_bar + 4);
   volatile uint32_t *abort_flag = tmem_slot + 1;
-  // 512 bytes after the barriers: the batch's adapter list derived from the ids by the builder warps
+  // 512 bytes after the barriers: what the owner of some tokens keeps of them, scratch of the shrink team
   uint8_t *extra = reinterpret_cast<uint8_t *>(bars) + 512;
-  volatile int32_t *s_nlg = reinterpret_cast<volatile int32_t *>(extra + 64);
-  uint64_t *lg_bar = reinterpret_cast<uint64_t *>(extra + 72);              // builder -> TMA, MMA
-  int32_t *s_lg = reinterpret_cast<int32_t *>(extra + 128);                 // [256] ids ascending
-  int32_t *s_vid = reinterpret_cast<int32_t *>(extra + 1152);               // [256] validated ids
-  uint8_t *s_head = extra + 2176;                                           // [256]
-  uint32_t *s_key = reinterpret_cast<uint32_t *>(extra + 2432);             // [256] sort keys
+  int32_t *s_rank = reinterpret_cast<int32_t *>(extra + 128);               // [16] of each of this CTA's tokens
+  int32_t *s_vid = reinterpret_cast<int32_t *>(extra + 1152);               // [16] adapters, -1: none
+  uint32_t *s_team = reinterpret_cast<uint32_t *>(extra + 2432);            // [256]
   volatile int32_t *s_last = reinterpret_cast<volatile int32_t *>(extra + 80);  // the wait for the shrink teams ended in time
   uint64_t *ep_bar = reinterpret_cast<uint64_t *>(extra + 88);              // the staged B_a rows have landed
   uint8_t *b_stage = reinterpret_cast<uint8_t *>(bars) + 4096;  // fused decode: B_a rows of the owner's tokens, then their z
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long wl = p.wait_cycles;  // limit of every bounded wait below
-  // LoRA K blocks: unless the batch is small enough for the expand to be added by the owners of the cluster
-  // reduction (then z is needed only at the very end and the whole main loop overlaps the shrink kernel)
-  const bool has_lora = !p.expand_in_reduce;
   const TileCoord tc = tile_coord(p, bid);
 
   if (threadIdx.x == 0) {
     ptx::prefetch_tensormap(&tmap_r);
     ptx::prefetch_tensormap(&tmap_c);
-    if (has_lora) ptx::prefetch_tensormap(&tmap_b);
     for (int s = 0; s < p.stages; ++s) {
       ptx::mbar_init(&full_bar[s], 1);
       ptx::mbar_init(&empty_bar[s], 1);
-      ptx::mbar_init(&zfull_bar[s], 4);  // one arrival per builder warp
-      ptx::mbar_init(&zgo_bar[s], 1);
     }
     ptx::mbar_init(tfull_bar, 1);
-    ptx::mbar_init(lg_bar, 1);
     ptx::mbar_init(ep_bar, 4);  // one arrival per epilogue warp
     *abort_flag = 0;
-    *s_nlg = 0;
     ptx::fence_barrier_init();
     if (kFused && f.x_wait) {
       // W is not written by any kernel of this library: this thread (lane 0 of the producer warp, which
@@ -346,24 +331,6 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
         ptx::tma_load_2d(sr + r_bytes, &tmap_c, &full_bar[stage], kb * kBlockK, 0);
         advance();
       }
-      if (ok && has_lora) {
-        ok = ptx::mbar_wait(lg_bar, 0, wl);  // the builder warps derive the adapter list from the ids
-        // the groups are dealt round-robin to the K splits of a row tile
-        for (int32_t e = tc.split; ok && e < *s_nlg; e += p.splits) {
-          const int32_t a = s_lg[e];
-          if (!EL_CHECK(p.status, a >= 0 && a < p.n_slots, 1)) continue;
-          if (!wait_empty()) {
-            ok = false;
-            break;
-          }
-          // The stage is free: let the builder write its half (it follows this warp, never the
-          // stage barriers directly, so it cannot run ahead of the ring).
-          ptx::mbar_arrive(&zgo_bar[stage]);
-          ptx::mbar_arrive_expect_tx(&full_bar[stage], r_bytes);  // rows [row_r, row_r + 128) of B_a
-          ptx::tma_load_3d(smem + static_cast<size_t>(stage) * stage_bytes, &tmap_b, &full_bar[stage], 0, tc.row_r, a);
-          advance();
-        }
-      }
       if (!ok) {
         *abort_flag = 1;
         atomicOr(p.status, EDGELORA_STATUS_TIMEOUT);
@@ -380,9 +347,8 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
     if (ptx::elect_one()) {
-      const int lora_ksteps = p.R_pad / kUmmaK;
       const uint32_t idesc = ptx::umma_idesc_bf16(kTileM, static_cast<uint32_t>(p.BN));
-      uint32_t stage = 0, phase = 0, zphase = 0;  // zphase: one parity bit per stage
+      uint32_t stage = 0, phase = 0;
       bool ok = true;
       for (int32_t kb = tc.kb0; kb < tc.kb1; ++kb) {
         if (!ptx::mbar_wait(&full_bar[stage], phase, wl) || *abort_flag) {
@@ -404,30 +370,6 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
           phase ^= 1;
         }
       }
-      if (ok && has_lora) {
-        ok = ptx::mbar_wait(lg_bar, 0, wl);
-        for (int32_t e = tc.split; ok && e < *s_nlg; e += p.splits) {
-          if (!EL_CHECK(p.status, s_lg[e] >= 0 && s_lg[e] < p.n_slots, 1)) continue;
-          if (!ptx::mbar_wait(&full_bar[stage], phase, wl) ||
-              !ptx::mbar_wait(&zfull_bar[stage], (zphase >> stage) & 1u, wl) || *abort_flag) {
-            ok = false;
-            break;
-          }
-          zphase ^= 1u << stage;
-          ptx::tc_fence_after_sync();
-          const uint32_t sr = ptx::smem_u32(smem + static_cast<size_t>(stage) * stage_bytes);
-          const uint64_t da = ptx::umma_desc_k128(sr);
-          const uint64_t db = ptx::umma_desc_k128(sr + r_bytes);
-          // the whole z operand is there (rows of tokens on other adapters are zero), so one
-          // MMA per 16 rank columns covers every token
-          for (int k = 0; k < lora_ksteps; ++k) ptx::umma_bf16(tmem_base, da + 2 * k, db + 2 * k, idesc, 1u);
-          ptx::umma_commit(&empty_bar[stage]);
-          if (++stage == nstages) {
-            stage = 0;
-            phase ^= 1;
-          }
-        }
-      }
       if (!ok) {
         *abort_flag = 1;
         atomicOr(p.status, EDGELORA_STATUS_TIMEOUT);
@@ -438,10 +380,8 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
     }
   } else if (warp < 6) {
     // ------------------------------------------------------------ epilogue (warps 2..5)
-    const int quad = warp & 3;                      // TMEM lanes [32*quad, 32*quad+32)
-    const int row_in_tile = quad * 32 + lane;
-    const bool clustered = p.splits > 1;
-    if (kFused && clustered && f.b_stage) {
+    const int quad = warp & 3;  // TMEM lanes [32*quad, 32*quad+32)
+    if (kFused && f.b_stage) {
       // This CTA will finish tokens [rank * cols_per, ...) of its row tile: the B_a rows they need (the
       // tile's 128 rows of the token's adapter) are copied into shared memory now, one copy per token, while the main
       // loop runs (the ids are the caller's input, the pool is not written by this kernel).  One warp per token;
@@ -464,7 +404,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
         a_of[i] = a;
         if (cl < cols_per && lane == 0) {  // kept for the expand at the end
           s_vid[cl] = a;
-          s_lg[cl] = rank;
+          s_rank[cl] = rank;
         }
         if (a >= 0) my_bytes += tok_bytes;
       }
@@ -476,7 +416,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
             ptx::tma_load_3d(b_stage + static_cast<size_t>(quad + 4 * i) * tok_bytes, &tmap_b, ep_bar, 0, tc_row0(p, bid),
                              a_of[i]);
       }
-    } else if (clustered && p.expand_in_reduce) {
+    } else {
       // This CTA will finish tokens [rank * cols_per, ...) of its row tile; pull the B_a rows they
       // need into L2 now (the ids are the caller's input, the pool is not written by the shrink).
       const int cols_per = p.BN / p.splits;
@@ -490,7 +430,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
         }
         if (lane == 0) {  // kept for the expand at the end
           s_vid[cl] = rank > 0 ? a : -1;
-          s_lg[cl] = rank;
+          s_rank[cl] = rank;
         }
         if (t0 + cl < p.T) {
           if (a >= 0 && a < p.n_slots) {
@@ -503,7 +443,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
         }
       }
     }
-    if (kFused && clustered && !f.b_stage) {
+    if (kFused && !f.b_stage) {
       // z comes from the shrink teams of this grid (every CTA of the launch is resident, so all of them run): bounded wait
       // for their arrival counter.  The counter belongs to the kernel before this one (another launch of this pool, which
       // leaves it at zero) until that kernel is done.
@@ -513,29 +453,8 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
       named_bar_sync(1, 128);
       fused_z_ok = *s_last != 0;
     }
-    // Earlier kernels may still read y, and z comes from the shrink kernel.  With the expand in
-    // the reduction both matter only at the very end, so that wait moves there.
-    if (!(clustered && p.expand_in_reduce)) ptx::pdl_wait_prior_grids();
     const bool ok = ptx::mbar_wait(tfull_bar, 0, wl) && !*abort_flag;
-    if (__all_sync(0xffffffffu, ok) && !clustered) {  // (with a cluster the accumulator is read after the cluster barrier below)
-      // single K split: row = W row j, columns = tokens c0 + [0, 32), straight to y
-      ptx::tc_fence_after_sync();
-      const int32_t row = tc.row_r + row_in_tile;
-      const uint32_t taddr = tmem_base + (static_cast<uint32_t>(quad * 32) << 16);
-      for (int32_t c0 = 0; c0 < p.BN; c0 += 32) {
-        float v[32];
-        ptx::tmem_ld_32x32(taddr + c0, v);
-        if (row < p.h_out) {
-#pragma unroll
-          for (int jj = 0; jj < 32; ++jj) {
-            const int t = c0 + jj;
-            if (t < p.T)
-              p.y[static_cast<size_t>(t) * p.h_out + row] =
-                  static_cast<uint16_t>(ptx::pack_bf16x2(v[jj], 0.f) & 0xFFFFu);
-          }
-        }
-      }
-    }
+    __syncwarp();
     if (!ok) {
       *abort_flag = 1;
       if (lane == 0) atomicOr(p.status, EDGELORA_STATUS_TIMEOUT);
@@ -543,7 +462,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
   } else if (kFused) {
     // ------------------------------------------------------------ shrink team (warps 6..9)
     const int btid = threadIdx.x - 192;  // 0..127
-    int32_t *s_tid = reinterpret_cast<int32_t *>(s_key) + 64;  // s_key is free: no LoRA K blocks in this launch
+    int32_t *s_tid = reinterpret_cast<int32_t *>(s_team) + 64;
     int32_t *s_trank = s_tid + 64;
     float *s_tscale = reinterpret_cast<float *>(s_trank + 64);
     if (btid < 64) {
@@ -565,132 +484,10 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
       waited = true;
     }
     shrink_team_items<2>(p, f, 2 * cta0 + bid, 2 * cta0 + ngrid, warp - 6, lane, s_tid, s_trank, s_tscale,
-                         reinterpret_cast<float *>(s_key), waited);
-  } else if (has_lora) {
-    // ------------------------------------------------------------ z operand builder (warps 6..9)
-    const int btid = threadIdx.x - 192;  // 0..127
-    const int bwarp = warp - 6;
-    const int nch = p.R_pad >> 3;        // 16-byte chunks of one operand row that the MMAs read
-    uint32_t count = static_cast<uint32_t>(tc.kb1 - tc.kb0);  // K blocks so far: stage = count % stages
-    uint32_t gophase = 0;                // one parity bit per stage for zgo_bar
-    bool ok = true;
-    {
-      // The batch's adapters (paper Section 3.4: one u-batch per adapter), distinct and ascending,
-      // straight from the caller's ids so that the B_a tiles can be fetched before the shrink
-      // kernel has finished.  Thread b looks after tokens b and b + 128.
-      // Keys (id << 8 | token) of the tokens that carry an adapter are sorted (bitonic, BN keys);
-      // the first key of every id that names a loaded slot joins the list.
-      const int nk = p.BN;  // a power of two, 32..256
-      for (int t = btid; t < 256; t += 128) {
-        int32_t a = -1;
-        if (t < p.T) {
-          a = p.ids[t];
-          if (a < -1 || a >= p.n_slots) a = -1;
-        }
-        s_vid[t] = a;
-        s_key[t] = a >= 0 ? ((static_cast<uint32_t>(a) << 8) | static_cast<uint32_t>(t)) : 0xFFFFFFFFu;
-      }
-      named_bar_sync(2, 128);
-      for (int k = 2; k <= nk; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-          for (int i = btid; i < nk; i += 128) {
-            const int ixj = i ^ j;
-            if (ixj > i) {
-              const uint32_t ka = s_key[i], kb = s_key[ixj];
-              if ((ka > kb) == ((i & k) == 0)) {
-                s_key[i] = kb;
-                s_key[ixj] = ka;
-              }
-            }
-          }
-          named_bar_sync(2, 128);
-        }
-      }
-      for (int i = btid; i < nk; i += 128) {
-        const uint32_t key = s_key[i];
-        bool head = key != 0xFFFFFFFFu && (i == 0 || (s_key[i - 1] >> 8) != (key >> 8));
-        if (head) head = p.slots[key >> 8].rank > 0;  // empty slots stay base-only (the shrink flags them)
-        s_head[i] = head ? 1 : 0;
-      }
-      named_bar_sync(2, 128);
-      if (bwarp == 0) {  // 32 lanes x 8 consecutive keys: positions by a warp prefix sum
-        int c = 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) c += (lane * 8 + q < nk) ? s_head[lane * 8 + q] : 0;
-        int incl = c;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-          const int o = __shfl_up_sync(0xffffffffu, incl, d);
-          if (lane >= d) incl += o;
-        }
-        int pos = incl - c;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-          const int i = lane * 8 + q;
-          if (i < nk && s_head[i]) s_lg[pos++] = static_cast<int32_t>(s_key[i] >> 8);
-        }
-        if (lane == 31) *s_nlg = incl;
-      }
-      named_bar_sync(2, 128);
-      if (btid == 0) ptx::mbar_arrive(lg_bar);
-    }
-    ptx::pdl_wait_prior_grids();  // z comes from the kernel before this one
-    // The ids of this thread's tokens do not change over the LoRA blocks, so their z is fetched once
-    // (while the base K blocks stream) and kept as packed bf16.
-    const int32_t id_lo = s_vid[btid];
-    const int32_t id_hi = kMinBlocks == 1 ? s_vid[btid + 128] : -1;  // the other variant runs with BN <= 128
-    uint4 z_lo[8], z_hi[8];
-    if (tc.split < *s_nlg) {
-      if (id_lo >= 0) load_z_packed(p.zws, p.R_pad, p.max_tokens, p.status, btid, p.slots[id_lo].rank, z_lo);
-      if (kMinBlocks == 1 && id_hi >= 0)
-        load_z_packed(p.zws, p.R_pad, p.max_tokens, p.status, btid + 128, p.slots[id_hi].rank, z_hi);
-    }
-    {
-      for (int32_t e = tc.split; e < *s_nlg; e += p.splits) {
-        const int32_t a = s_lg[e];
-        if (!EL_CHECK(p.status, a >= 0 && a < p.n_slots, 1)) continue;
-        const uint32_t stage = count % nstages;
-        ++count;
-        if (!ptx::mbar_wait(&zgo_bar[stage], (gophase >> stage) & 1u, wl) || *abort_flag) {
-          ok = false;
-          break;
-        }
-        gophase ^= 1u << stage;
-        uint8_t *dst = smem + static_cast<size_t>(stage) * stage_bytes + r_bytes;
-        // 128-byte swizzle: the 16-byte chunk index is XORed with the row index modulo 8.
-        // Every token row the MMAs read is written: z of the tokens on this adapter, zeros for
-        // the others (rows btid and btid + 128 below BN).
-        const bool m_lo = id_lo == a, m_hi = id_hi == a;
-        const bool w_lo = btid < p.BN;
-        const bool w_hi = kMinBlocks == 1 && btid + 128 < p.BN;
-        if (w_lo) {
-          uint8_t *drow = dst + btid * 128;
-#pragma unroll
-          for (int c = 0; c < 8; ++c)
-            if (c < nch)
-              *reinterpret_cast<uint4 *>(drow + ((c ^ (btid & 7)) << 4)) =
-                  m_lo ? z_lo[c] : make_uint4(0u, 0u, 0u, 0u);
-        }
-        if (w_hi) {
-          uint8_t *drow = dst + (btid + 128) * 128;
-#pragma unroll
-          for (int c = 0; c < 8; ++c)
-            if (c < nch)
-              *reinterpret_cast<uint4 *>(drow + ((c ^ (btid & 7)) << 4)) =
-                  m_hi ? z_hi[c] : make_uint4(0u, 0u, 0u, 0u);
-        }
-        ptx::fence_proxy_async();  // make the generic-proxy writes visible to the tensor core
-        __syncwarp();
-        if (lane == 0) ptx::mbar_arrive(&zfull_bar[stage]);
-      }
-    }
-    if (!ok && lane == 0) {
-      *abort_flag = 1;
-      atomicOr(p.status, EDGELORA_STATUS_TIMEOUT);
-    }
+                         reinterpret_cast<float *>(s_team), waited);
   }
 
-  if (p.splits > 1) {
+  {
     // ---------------------------------------------------------- split-K reduction in the cluster
     // CTA `rank` of the cluster owns tokens [rank * cols_per, (rank + 1) * cols_per).  Its buffer
     // buf[src split][token][row] overlays the operand ring, which is idle once every CTA of the
@@ -700,13 +497,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
     const uint32_t my_rank = ptx::cluster_rank();
     const int cols_per = p.BN / p.splits;  // a power of two (BN and splits are)
     const int shift = 31 - __clz(cols_per);
-    // Large batches: the builder warps (6..9, the same four lane quadrants) send every other
-    // 32-token block, and all ten warps sum.  The epilogue warps have waited for the accumulator;
-    // the barrier below passes that on to the others.
-    const bool wide = !p.expand_in_reduce;
-    const bool sender = epi || (wide && warp >= 6);
-    const int c_first = (wide && warp >= 6) ? 32 : 0, c_step = wide ? 64 : 32;
-    const bool have_acc = sender && !*abort_flag;  // this CTA's accumulator is complete (tfull waited)
+    const bool have_acc = epi && !*abort_flag;  // this CTA's accumulator is complete (tfull waited)
     const bool z_ok = fused_z_ok;  // fused launches: the wait for the shrink teams ended in time
     float4 *z_stage = reinterpret_cast<float4 *>(b_stage + static_cast<size_t>(cols_per) * kTileM * p.R_pad * 2);
     // The partial tiles land in the operand ring, which is idle once every CTA of the cluster is past
@@ -724,10 +515,10 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
       const uint32_t local = ptx::smem_u32(red) +
                              ((my_rank * cols_per) * kTileM + row_in_tile) * 4u;
       const uint32_t qpo = static_cast<uint32_t>(cols_per) >> 2;  // token quads per owner
-      for (int32_t c0 = c_first; c0 < p.BN; c0 += c_step) {
+      for (int32_t c0 = 0; c0 < p.BN; c0 += 32) {
         float v[32];
         ptx::tmem_ld_32x32(taddr + c0, v);
-        if (p.expand_in_reduce && !(kFused && f.b_stage)) {  // buf[src][token][row]
+        if (!(kFused && f.b_stage)) {  // buf[src][token][row]
 #pragma unroll
           for (int jj = 0; jj < 32; ++jj) {
             const int col = c0 + jj;
@@ -790,7 +581,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
                 z.x += w[k].x; z.y += w[k].y; z.z += w[k].z; z.w += w[k].w;
               }
             }
-            const int rank = s_lg[cl];  // (what lies behind the last live group of eight rank rows was not written)
+            const int rank = s_rank[cl];  // (what lies behind the last live group of eight rank rows was not written)
             if (c4 * 4 + 0 >= rank) z.x = 0.f;
             if (c4 * 4 + 1 >= rank) z.y = 0.f;
             if (c4 * 4 + 2 >= rank) z.z = 0.f;
@@ -805,8 +596,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
           z_ok = false;
         }
         named_bar_sync(3, 256);
-        // a row's 16-byte chunks are swizzled as its length of 32, 64 or 128 bytes has it
-        const int sw = p.R_pad == 64 ? r & 7 : p.R_pad == 32 ? (r >> 1) & 3 : (r >> 2) & 1;
+        const int sw = row_swizzle(r, p.R_pad);
         const uint32_t brow = ptx::smem_u32(b_stage) + r * p.R_pad * 2, tok_bytes = kTileM * p.R_pad * 2;
         const uint32_t zrow = ptx::smem_u32(z_stage);
 #pragma unroll
@@ -871,7 +661,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
       }
     } else {
       ptx::cluster_sync_all();
-      if (epi || wide) {
+      if (epi) {
         const float *buf = reinterpret_cast<const float *>(red);
         const int n_units = cols_per * 32;  // unit = (token, 4 adjacent W rows)
         const int row0 = bid / p.splits * kTileM;
@@ -889,29 +679,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
           o.y = ptx::pack_bf16x2(v.z, v.w);
           *reinterpret_cast<uint2 *>(p.y + static_cast<size_t>(t) * p.h_out + j) = o;
         };
-        if (!p.expand_in_reduce) {
-          // unit = (token quad, W row): the splits' partial sums are 16 bytes each, lanes take
-          // adjacent rows, so a warp writes 64 bytes in a row of y per token
-          const int qpo = cols_per >> 2;
-          const float4 *buf4 = reinterpret_cast<const float4 *>(red);
-          ptx::pdl_wait_prior_grids();  // warps 0 and 1 have not waited yet; earlier kernels may read y
-          for (int u = threadIdx.x; u < qpo * kTileM; u += kGemmThreads) {
-            const int qd = u >> 7, r = u & (kTileM - 1);
-            const int t0 = static_cast<int>(my_rank) * cols_per + qd * 4, j = row0 + r;
-            if (t0 >= p.T || j >= p.h_out) continue;
-            float4 a4 = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int sp = 0; sp < p.splits; ++sp) {
-              const float4 w = buf4[(sp * qpo + qd) * kTileM + r];
-              a4.x += w.x; a4.y += w.y; a4.z += w.z; a4.w += w.w;
-            }
-            const float o[4] = {a4.x, a4.y, a4.z, a4.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-              if (t0 + i < p.T)
-                p.y[static_cast<size_t>(t0 + i) * p.h_out + j] =
-                    static_cast<uint16_t>(ptx::pack_bf16x2(o[i], 0.f) & 0xFFFFu);
-          }
-        } else {
+        {
           // Small batches: wait for the shrink kernel (and for earlier readers of y), then per unit add the
           // splits' partial sums, fetch z and the B_a rows in one round trip, add B_a[j..j+3][0..r) . z[t]
           // in fp32 (z carries s_a) and write y.  A rolled loop over the units (at most 4 per thread:
@@ -935,7 +703,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
             const int t = static_cast<int>(my_rank) * cols_per + cl, j = row0 + r4;
             if (t >= p.T || j >= p.h_out) continue;
             float4 acc4 = sum_partials(cl, r4);
-            const int32_t a = z_ok ? s_vid[cl] : -1, rank = s_lg[cl];  // stored by the epilogue warps at the start
+            const int32_t a = z_ok ? s_vid[cl] : -1, rank = s_rank[cl];  // stored by the epilogue warps at the start
             if (a >= 0) {
               const uint4 *Brow = reinterpret_cast<const uint4 *>(
                   p.B_pool + (static_cast<size_t>(a) * p.h_out + j) * p.R_pad);
@@ -997,39 +765,28 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
   }
 }
 
-static FusedDecode not_fused() {
-  FusedDecode f{};
-  return f;
-}
-
 cudaError_t gemm_set_smem_limit(size_t smem_bytes) {
   cudaError_t e = cudaSuccess;
   const int bytes = static_cast<int>(smem_bytes);
-#define EDGELORA_SMEM(MB, FU)                                                                               \
+#define EDGELORA_SMEM(FU)                                                                                       \
   if (e == cudaSuccess)                                                                                     \
-    e = cudaFuncSetAttribute(lora_gemm_kernel<MB, FU>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  EDGELORA_SMEM(1, false)
-  EDGELORA_SMEM(2, false)
-  EDGELORA_SMEM(1, true)
+    e = cudaFuncSetAttribute(lora_gemm_kernel<FU>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  EDGELORA_SMEM(false)
+  EDGELORA_SMEM(true)
 #undef EDGELORA_SMEM
   return e;
 }
 
-cudaError_t launch_gemm(const CUtensorMap &tmap_row, const CUtensorMap &tmap_col, const CUtensorMap &tmap_b,
-                        const GemmParams &p, int32_t grid, size_t smem_bytes, bool pdl, cudaStream_t stream) {
-  const int cluster = p.splits;
-  // small shared memory and at most 128 tokens: the variant whose CTAs fit beside the shrink kernel's
-  if (smem_bytes * 2 <= 225 * 1024 && p.BN <= 128)
-    return launch_ex(lora_gemm_kernel<2, false>, dim3(grid), dim3(kGemmThreads), smem_bytes, stream, pdl, cluster,
-                     tmap_row, tmap_col, tmap_b, p, not_fused());
-  return launch_ex(lora_gemm_kernel<1, false>, dim3(grid), dim3(kGemmThreads), smem_bytes, stream, pdl, cluster,
-                   tmap_row, tmap_col, tmap_b, p, not_fused());
+cudaError_t launch_gemm(const CUtensorMap &tmap_row, const CUtensorMap &tmap_col, const GemmParams &p, int32_t grid,
+                        size_t smem_bytes, bool pdl, cudaStream_t stream) {
+  return launch_ex(lora_gemm_kernel<false>, dim3(grid), dim3(kGemmThreads), smem_bytes, stream, pdl, p.splits, tmap_row, tmap_col,
+                   tmap_row, p, FusedDecode{});
 }
 
 cudaError_t launch_gemm_fused(const CUtensorMap &tmap_row, const CUtensorMap &tmap_col, const CUtensorMap &tmap_b, const GemmParams &p,
                               const FusedDecode &f, size_t smem_bytes, bool pdl, cudaStream_t stream) {
   const int32_t grid = f.n_ctas + p.n_mtiles * p.splits;
-  return launch_ex(lora_gemm_kernel<1, true>, dim3(grid), dim3(kGemmThreads), smem_bytes, stream, pdl, p.splits,
+  return launch_ex(lora_gemm_kernel<true>, dim3(grid), dim3(kGemmThreads), smem_bytes, stream, pdl, p.splits,
                    tmap_row, tmap_col, tmap_b, p, f);
 }
 
@@ -1046,7 +803,7 @@ int32_t gemm_fused_max_ctas(int32_t cluster, size_t smem_bytes) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, lora_gemm_kernel<1, true>, &cfg);
+  const cudaError_t e = cudaOccupancyMaxActiveClusters(&n, lora_gemm_kernel<true>, &cfg);
   if (getenv("EDGELORA_LOG"))
     fprintf(stderr, "edgelora: one-launch decode, clusters of %d, %zu bytes of shared memory: %s, %d clusters fit\n",
             cluster, smem_bytes, cudaGetErrorString(e), n);

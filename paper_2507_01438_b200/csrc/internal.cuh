@@ -16,7 +16,7 @@ constexpr int kMaxStages = 12;
 constexpr int kSegMin = 32;        // prefill: runs at least this long go through the segment shrink
 constexpr int kDecodeMaxT = 256;   // decode regime: all tokens are one UMMA N tile
 constexpr int kMaxTokensLimit = 32768;
-constexpr int kGemmThreads = 320;  // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue, warps 6..9 z operand
+constexpr int kGemmThreads = 320;  // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue, warps 6..9 shrink team
 constexpr int kMaxZSplits = 16;    // partial z planes (K splits of the shrink); plane 16 = summed z
 constexpr int kShrinkThreads = 256;
 constexpr int kShrinkStepElems = 256;  // K elements of one shrink step (512 bytes of a row)
@@ -71,7 +71,7 @@ struct PlanView {
 // A decode launch of the tile kernel (gemm.cu).
 struct GemmParams {
   int32_t T, h_in, h_out;
-  int32_t BN;          // UMMA N = tokens rounded up to a power of two (32 .. 256)
+  int32_t BN;          // UMMA N = tokens rounded up to 32 or 64
   int32_t stages;      // TMA pipeline depth
   int32_t tmem_cols;   // power of two >= BN
   int32_t kb_total;    // K blocks of 64 covering h_in
@@ -79,8 +79,6 @@ struct GemmParams {
   int32_t splits;
   int32_t n_mtiles;    // W row tiles
   int32_t R_pad;       // slot block rank stride
-  int32_t expand_in_reduce;  // small batches: B_a z is added by the owners of the cluster
-                             // reduction on the CUDA cores instead of by LoRA K blocks
   int32_t max_tokens;  // row stride of the z workspace
   long long wait_cycles;  // limit of the bounded in-kernel waits, in SM clock cycles
   const int32_t *ids;       // the caller's ids (validated again inside the kernel)
@@ -114,8 +112,8 @@ struct FusedDecode {
 void launch_plan(const int32_t *ids, int32_t T, int32_t n_slots, const PlanView &pv, bool pdl,
                  cudaStream_t stream);
 void init_plan_kernel();
-cudaError_t launch_gemm(const CUtensorMap &tmap_row, const CUtensorMap &tmap_col, const CUtensorMap &tmap_b,
-                        const GemmParams &p, int32_t grid, size_t smem_bytes, bool pdl, cudaStream_t stream);
+cudaError_t launch_gemm(const CUtensorMap &tmap_row, const CUtensorMap &tmap_col, const GemmParams &p, int32_t grid,
+                        size_t smem_bytes, bool pdl, cudaStream_t stream);
 // Decode job with the shrink in the same grid: grid = f.n_ctas + p.n_mtiles * p.splits CTAs.
 cudaError_t launch_gemm_fused(const CUtensorMap &tmap_row, const CUtensorMap &tmap_col, const CUtensorMap &tmap_b, const GemmParams &p,
                               const FusedDecode &f, size_t smem_bytes, bool pdl, cudaStream_t stream);

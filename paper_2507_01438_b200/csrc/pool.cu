@@ -15,6 +15,7 @@
 #include <vector>
 
 #include "decode_sites.h"
+#include "decode_tile.h"
 #include "guard.h"
 #include "pool.h"
 #include "prefill.h"
@@ -381,6 +382,7 @@ int edgelora_pool_create(const edgelora_pool_config *cfg, edgelora_pool_t **pool
   POOL_TRY(shrink_tiles_set_smem_limit());
   POOL_TRY(pair_set_smem_limit());
   POOL_TRY(decode_sites_set_smem_limit());
+  POOL_TRY(decode_tile_set_smem_limit());
   rc = edgelora_plan_create(p->cfg.max_tokens, cfg->n_slots, &p->plan);
   if (rc != EDGELORA_OK) {
     edgelora_pool_destroy(p);
@@ -1005,6 +1007,70 @@ int decode_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32_
   return EDGELORA_OK;
 }
 
+// ---- decode-sized batch of one site (decode_tile.cu)
+//
+// CTAs that share a tile: the count whose launch is done first.  A K block takes a CTA about a third of a microsecond, and so
+// does an adapter of its own tokens in the expand beside it (the device knows their number; six tenths of the tokens are
+// assumed); the exchange of the parts takes 1.5, and a count whose clusters are not all resident at once pays its ramp-up of 4 us
+// again.  Us per call, before (an expand on the tensor cores, tokens padded to a power of two) and now: 3080 -> 5000, 77 tokens:
+// 27.4 and 26.1; 14336 -> 4096, 256 tokens on 109 adapters of rank 64: 91.2 and 83.3; 4096 -> 12000, 90 tokens: 48.8 and 41.6;
+// 8192 -> 8192, 128 tokens: 48.6 and 43.0; 1024 -> 4096, 160 tokens: 39.7 and 32.7; 664 -> 864, 226 tokens: 33.7 and 35.6.
+static int decode_parts(edgelora_pool *p, int n_tiles, int kb, int32_t T) {
+  if (p->tile_clusters[1] == 0)
+    for (int c = 1; c <= kTileMaxParts; ++c) p->tile_clusters[c] = std::max(1, decode_tile_max_clusters(c));
+  const int most = std::max(1, std::min(p->opt_decode_splits > 0 ? p->opt_decode_splits : kTileMaxParts, kb / 2));
+  const int quads = (T + 3) / 4;
+  int best = 1;
+  double best_cost = 0;
+  for (int c = 1; c <= most; ++c) {
+    if (!decode_tile_parts_fit(T, c)) continue;
+    const int waves = (n_tiles + p->tile_clusters[c] - 1) / p->tile_clusters[c];
+    const int own = std::min((quads + c - 1) / c * 4, p->cfg.n_slots);
+    const double cost = waves * (std::max((kb + c - 1) / c * 0.33, own * 0.6 * 0.33) + 4.0) + (c > 1 ? 1.5 : 0.0);
+    if (c == 1 || cost < best_cost || p->opt_decode_splits > 0) {
+      best = c;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
+static int decode_tile(const SiteCall &c, const edgelora_plan *plan, const int32_t *ids_dev, int32_t T, bool pdl,
+                       cudaStream_t stream) {
+  edgelora_pool *p = c.p;
+  const int h_in = p->cfg.h_in, h_out = p->cfg.h_out, R = p->R_pad;
+  const int32_t N = decode_columns(T);
+  DecTile d{};
+  int rc = get_tmap(p, &d.w, c.W, h_in, h_out, 0, kTileM);
+  if (!rc) rc = get_tmap(p, &d.x, c.x, h_in, T, 0, N);
+  if (!rc) rc = get_tmap(p, &d.b, p->B_pool, R, h_out, p->cfg.n_slots, kTileM, R);
+  if (rc) return rc;
+  d.y = static_cast<uint16_t *>(c.y);
+  d.slots = p->slots_dev;
+  d.z = p->zws + static_cast<size_t>(kMaxZSplits) * p->cfg.max_tokens * R;
+  d.status = p->status_dev;
+  d.ids = ids_dev;
+  d.T = T;
+  d.h_out = h_out;
+  d.kb = (h_in + kBlockK - 1) / kBlockK;
+  d.R_pad = R;
+  d.n_slots = plan->n_slots;
+  d.N = N;
+  const int n_tiles = (h_out + kTileM - 1) / kTileM;
+  const DecTileShape shape = decode_tile_shape(N, R);
+  d.parts = decode_parts(p, n_tiles, d.kb, T);
+  d.stages = shape.stages;
+  d.exp_bytes = shape.exp_bytes;
+  d.tmem_cols = shape.tmem_cols;
+  d.wait_cycles = p->wait_cycles;
+  CUDA_TRY(launch_decode_tile(d, pdl, stream));
+  p->last_info[2] = n_tiles * d.parts;
+  p->last_info[3] = d.parts;
+  p->last_info[4] = shape.stages;
+  p->last_info[5] = N;
+  return EDGELORA_OK;
+}
+
 // CTAs of a one-launch decode call that the device holds at once, asked once per shape of the last few.
 static int fused_max_ctas(edgelora_pool *p, int splits, size_t smem) {
   const uint64_t key = (static_cast<uint64_t>(splits) << 32) | static_cast<uint64_t>(smem);
@@ -1015,6 +1081,18 @@ static int fused_max_ctas(edgelora_pool *p, int splits, size_t smem) {
   f.key = key;
   f.ctas = gemm_fused_max_ctas(splits, smem);
   return f.ctas;
+}
+
+// A call is on the stream: slot loads issued later wait for it.
+static int call_issued(edgelora_pool *p, int launches, int regime, bool capturing, cudaStream_t stream) {
+  if (!capturing) {
+    CUDA_TRY(cudaEventRecord(p->use_ev, stream));
+    p->use_recorded = true;
+  }
+  p->last_info[0] = launches;
+  p->last_info[1] = regime;
+  p->total_launches += launches;
+  return EDGELORA_OK;
 }
 
 int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_dev, const void *W_dev,
@@ -1127,7 +1205,7 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
         const int target = p->opt_shrink_items > 0 ? p->opt_shrink_items : (overlapped ? 1 : auto_target);
         // at most T token blocks x (R / 8) row groups x K chunks warp items, eight warps per CTA
         const int n_ksteps = (h_in + kShrinkStepElems - 1) / kShrinkStepElems;
-        const int max_chunks = target == 1 ? 1 : std::max(1, std::min(kMaxZSplits, n_ksteps / 4));
+        const int max_chunks = target == 1 ? 1 : std::max(1, std::min(kMaxZSplits, n_ksteps / 2));
         const int max_items = std::min(T, p->cfg.n_slots) * (R / 8) * max_chunks;
         const int grid = std::max(1, std::min(cta_cap - 1, (max_items + 7) / 8)) + 1;  // + the publishing CTA
         CUtensorMap ma, mx, md;
@@ -1155,52 +1233,54 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
       }
       return 0;
     };
-    int N = 32;  // tokens on the UMMA N axis: a power of two so that the cluster's owners get
-    while (N < T) N <<= 1;  // equal power-of-two column blocks
-    const int row_tiles = (h_out + kTileM - 1) / kTileM;
+    // Up to 64 tokens whose row tiles leave SMs for K splits: the K splits of a row tile form a cluster, and the expand moves
+    // to the owners of the cluster reduction (at most 16 tokens and 64 16-byte loads of B per thread), so the main loop does not
+    // depend on the shrink at all.
+    const int N = T <= 32 ? 32 : 64;  // tokens on the UMMA N axis: a power of two so that the cluster's owners get
+    const int row_tiles = (h_out + kTileM - 1) / kTileM;  // equal power-of-two column blocks
     const int stage_bytes = kTileM * kBlockK * 2 + N * kBlockK * 2;
-    const int ctas_per_sm = (stage_bytes * 4 + 5120 <= static_cast<int>(kSmemBudget / 2)) ? 2 : 1;
-    int want = p->opt_decode_splits > 0 ? p->opt_decode_splits
-                                        : std::max(1, (p->sms * ctas_per_sm) / row_tiles);
+    int want = p->opt_decode_splits > 0 ? p->opt_decode_splits : std::max(1, 2 * p->sms / row_tiles);
     want = std::min({want, kMaxDecodeSplits, std::max(1, kb_total / 2)});
     int splits = 1;
     while (splits * 2 <= want) splits <<= 1;
-    int kb_per = (kb_total + splits - 1) / splits;
-    while (splits > 1 && kb_per * (splits - 1) >= kb_total) {  // every split needs a K block
-      splits >>= 1;
-      kb_per = (kb_total + splits - 1) / splits;
+    while (splits > 1 && (kb_total + splits - 1) / splits * (splits - 1) >= kb_total) splits >>= 1;  // every split needs a K block
+    auto owners_expand = [&](int sp) { return T <= 64 && sp > 1 && N / sp <= 16 && N / sp * (R / 8) <= 64; };
+    // one CTA per SM leaves room for the shrink kernel's CTAs, so that the two kernels run side
+    // by side (measured on 4096 -> 4096, T = 32: 18.4 us per step with 4 splits, 24.4 with 8)
+    if (owners_expand(splits) && p->opt_decode_splits == 0)
+      while (splits > 1 && row_tiles * splits > p->sms) splits >>= 1;
+    if (!owners_expand(splits)) {
+      int rc = launch_shrink();
+      if (rc) return rc;
+      {
+        // Launched under the shrink's tail: its CTAs end at different times, and on the SMs that are free early the K
+        // blocks, which need no z, start at once.
+        ProfScope ps(p, 3, stream);
+        rc = decode_tile(SiteCall{p, W_dev, x, y_dev}, plan, ids_in, T, pdl, stream);
+        if (rc) return rc;
+        ++launches;
+      }
+      return call_issued(p, launches, regime, capturing, stream);
     }
     g.BN = N;
     g.splits = splits;
-    g.kb_per = kb_per;
+    g.kb_per = (kb_total + splits - 1) / splits;
     g.n_mtiles = row_tiles;
     // the decode shrink leaves the summed z in the plane after the partial ones
     g.zws = p->zws + static_cast<size_t>(kMaxZSplits) * p->cfg.max_tokens * R;
-    const size_t budget = ctas_per_sm == 2 ? kSmemBudget / 2 : kSmemBudget;
-    g.stages = stages_for(N, kb_per + 8, budget);
-    // Small batches: the expand moves to the owners of the cluster reduction (at most 64 16-byte
-    // loads of B per thread), so the main loop does not depend on the shrink at all.
-    g.expand_in_reduce = (splits > 1 && N <= 64 && (N / splits) <= 16 && (N / splits) * (R / 8) <= 64) ? 1 : 0;
-    if (g.expand_in_reduce && p->opt_decode_splits == 0) {
-      // one CTA per SM leaves room for the shrink kernel's CTAs, so that the two kernels run side
-      // by side (measured on 4096 -> 4096, T = 32: 18.4 us per step with 4 splits, 24.4 with 8)
-      while (splits > 1 && row_tiles * splits > p->sms) splits >>= 1;
-      kb_per = (kb_total + splits - 1) / splits;
-      g.splits = splits;
-      g.kb_per = kb_per;
-      g.expand_in_reduce = (splits > 1 && (N / splits) <= 16 && (N / splits) * (R / 8) <= 64) ? 1 : 0;
-      g.stages = stages_for(N, kb_per + 8, budget);
-    }
+    const size_t budget = kSmemBudget / 2;
     // the cluster's reduction buffer (N x 128 fp32, plus z of the owner's tokens) overlays the ring
-    while (splits > 1 && g.stages * stage_bytes < N * kTileM * 4 + (N / splits) * R * 4 && g.stages < kMaxStages)
-      ++g.stages;
+    auto stages_of = [&](int sp, int kb_per) {
+      int st = stages_for(N, kb_per + 8, budget);
+      while (st * stage_bytes < N * kTileM * 4 + (N / sp) * R * 4 && st < kMaxStages) ++st;
+      return st;
+    };
+    g.stages = stages_of(splits, g.kb_per);
     g.tmem_cols = pow2_cols(N);
-    CUtensorMap mr, mc, mb;
+    CUtensorMap mr, mc;
     int rc = get_tmap(p, &mr, W_dev, h_in, h_out, 0, kTileM);
     if (rc) return rc;
     rc = get_tmap(p, &mc, x, h_in, T, 0, N);
-    if (rc) return rc;
-    rc = get_tmap(p, &mb, p->B_pool, R, h_out, p->cfg.n_slots, kTileM);
     if (rc) return rc;
     const int grid = row_tiles * splits;
     // Small batches in one launch: the shrink runs on the idle builder warps of the base product's CTAs
@@ -1209,24 +1289,22 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
     // cluster of the launch must be resident at once: checked against the device's occupancy figure.
     bool fused = false;
     if (getenv("EDGELORA_LOG"))
-      fprintf(stderr, "edgelora: decode T %d N %d splits %d grid %d expand_in_reduce %d ctas_per_sm %d\n", T, N, splits,
-              grid, g.expand_in_reduce, ctas_per_sm);
+      fprintf(stderr, "edgelora: decode T %d N %d splits %d grid %d\n", T, N, splits, grid);
     // (Calls that may overlap the call before them keep the two launches: a one-launch grid holds every
     // SM until its last CTA is done, so consecutive calls cannot overlap; measured on 4096 -> 4096,
     // T = 32: 17.0 us per step in one launch against 9.7 us in two when the calls are independent, and
     // 16.9 against 19.7 us when each call waits for the one before.)
-    if (p->opt_fused_decode && !pdl_first && g.expand_in_reduce && T <= 64 && T <= kGatherMinT && ids_dev &&
+    if (p->opt_fused_decode && !pdl_first && T <= kGatherMinT && ids_dev &&
         !p->a_q8 && h_in % 8 == 0) {
       // Fewer K splits when the clusters of all row tiles do not fit beside a spare one (clusters of eight: 16 on this chip;
       // 2048 -> 2048, 8 tokens: 6.6 us in one launch with 4 splits, 10.4 in two with 8).
       for (int sp = splits; sp > 1 && !fused; sp >>= 1) {
-        if (N / sp > 16 || (N / sp) * (R / 8) > 64 || (p->opt_decode_splits != 0 && sp != splits)) break;
+        if (!owners_expand(sp) || (p->opt_decode_splits != 0 && sp != splits)) break;
         GemmParams gf = g;
         gf.splits = sp;
         gf.kb_per = (kb_total + sp - 1) / sp;
         if (gf.kb_per * (sp - 1) >= kb_total) continue;  // every split needs a K block
-        gf.stages = stages_for(N, gf.kb_per + 8, budget);
-        while (gf.stages * stage_bytes < N * kTileM * 4 + (N / sp) * R * 4 && gf.stages < kMaxStages) ++gf.stages;
+        gf.stages = stages_of(sp, gf.kb_per);
         FusedDecode f{};
         // room behind the ring for the B_a rows and z of an owner's tokens, when it fits
         // (2: and for the cluster reduction's buffer, which then does not have to wait for the ring)
@@ -1263,6 +1341,8 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
         g = gf;
         p->last_info[2] = gf_grid + spare;
         p->last_info[3] = sp;
+        p->last_info[4] = g.stages;
+        p->last_info[5] = g.BN;
       }
     }
     if (!fused) {
@@ -1271,15 +1351,12 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
     }
     if (!fused) {
       ProfScope ps(p, 3, stream);
-      // Launched under the shrink's tail: a base-product CTA cannot share an SM with the shrink's CTAs
-      // (shared memory), but the shrink's CTAs end at different times, and on the SMs that are free
-      // early the base K blocks, which need no z, start at once (14336 -> 4096, T = 256: 99 us per
-      // step against 104; with the one-CTA-per-SM shrink of four ring stages it was the other way
-      // round, 178 against 122 us).
-      CUDA_TRY(launch_gemm(mr, mc, mb, g, grid, smem_for(g.stages, N), pdl, stream));
+      CUDA_TRY(launch_gemm(mr, mc, g, grid, smem_for(g.stages, N), pdl, stream));
       ++launches;
       p->last_info[2] = grid;
       p->last_info[3] = splits;
+      p->last_info[4] = g.stages;
+      p->last_info[5] = g.BN;
     }
   } else {
     // ---------------------------------------------------------------- prefill
@@ -1293,16 +1370,7 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
     return EDGELORA_OK;
   }
 
-  if (!capturing) {
-    CUDA_TRY(cudaEventRecord(p->use_ev, stream));
-    p->use_recorded = true;
-  }
-  p->last_info[0] = launches;
-  p->last_info[1] = regime;
-  p->last_info[4] = g.stages;
-  p->last_info[5] = g.BN;
-  p->total_launches += launches;
-  return EDGELORA_OK;
+  return call_issued(p, launches, regime, capturing, stream);
 }
 }  // namespace edgelora
 

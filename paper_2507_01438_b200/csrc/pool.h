@@ -88,6 +88,7 @@ struct edgelora_pool {
     int ctas = 0;      // the occupancy answer for it
   } fused_fits[8];
   int fused_next = 0;
+  int tile_clusters[9] = {0};  // clusters of each size of the tile launch that the device holds at once; 0: not asked yet
   long long wait_cycles = edgelora::ptx::kWaitLimitCycles;
   int64_t last_info[8] = {0};
   int64_t total_launches = 0;

@@ -22,6 +22,14 @@ __device__ __forceinline__ uint32_t elect_one() {
   return pred;
 }
 
+// A barrier of kThreads threads (whole warps).  bar.sync is the aligned form: a warp that a loop or a branch in front of it
+// has left apart comes together first.
+template <int kId, int kThreads>
+__device__ __forceinline__ void named_barrier() {
+  __syncwarp();
+  asm volatile("bar.sync %0, %1;" ::"n"(kId), "n"(kThreads) : "memory");
+}
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
@@ -260,6 +268,14 @@ __device__ __forceinline__ void tmem_st_32x4(uint32_t taddr, const float *v) {
   asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1, %2, %3, %4};" ::"r"(taddr), "f"(v[0]), "f"(v[1]), "f"(v[2]),
                "f"(v[3])
                : "memory");
+}
+__device__ __forceinline__ void tmem_fill_32x32(uint32_t taddr, float v) {  // 32 columns of one value
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
+      "{%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, "
+      "%1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr),
+      "r"(__float_as_uint(v))
+      : "memory");
 }
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 // orders this thread's shared-memory writes before later accesses of the async proxy (TMA, tcgen05)

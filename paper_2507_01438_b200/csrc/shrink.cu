@@ -27,7 +27,6 @@ namespace edgelora {
 // fixed order into the final plane zws[kMaxZSplits] that the base-product kernel reads.  The last CTA also
 // writes the routing plan in its canonical form for the base-product kernel and for export.
 
-constexpr int kDsBlockTok = kDsTok;  // tokens of one group handled by one work item (one pass)
 constexpr int kDsTicket = kDecodeMaxT * 8;  // index of the work-item ticket counter in group_counters
 
 constexpr size_t ds_ring_bytes(int depth) {
@@ -46,17 +45,9 @@ decode_shrink_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
                      int32_t target_items, int32_t late_ticket, uint32_t *status) {
   extern __shared__ uint8_t s_ring_raw[];  // [warp][stage][8 A rows + 4 x rows][512 bytes]
   __shared__ uint64_t s_bars[kShrinkThreads / 32][kDsMaxDepth];
-  __shared__ __align__(16) int32_t s_id[256];  // validated id of each token
-  __shared__ int32_t s_grp[256];       // group (in order of first appearance) of a group's first token
-  __shared__ int32_t s_gadapter[256];  // adapter of each group
-  __shared__ int32_t s_gstart[257];    // token list boundaries
-  __shared__ int32_t s_gtok[256];      // tokens ordered by (group, token)
-  __shared__ int32_t s_cnt[256];
-  __shared__ int32_t s_bgrp[256];      // token blocks: group and first position in s_gtok
-  __shared__ int32_t s_btok[256];
+  __shared__ Groups s_groups;
   __shared__ int32_t s_grank[256];     // rank and scale of each group's slot
   __shared__ float s_gscale[256];
-  __shared__ int s_wt[9];
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   ptx::pdl_launch_dependents();
@@ -70,78 +61,24 @@ decode_shrink_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
   }
 
   // ---- routing, in shared memory (reads only the caller's ids)
-  int a = -1;
-  bool bad = false;
-  if (tid < T) {
-    a = ids[tid];
-    if (a < -1 || a >= n_slots) {
-      a = -1;
-      bad = true;
-    }
+  const bool bad = derive_groups<kDsTok, 1, kShrinkThreads>(s_groups, ids, T, n_slots, tid);
+  const int G = s_groups.n_groups, NB = s_groups.n_blocks;
+  if (tid < G) {
+    const SlotRow row = slots[s_groups.adapter[tid]];
+    s_grank[tid] = row.rank;
+    s_gscale[tid] = row.scale;
   }
-  SlotRow myrow = {0, 0.f, 0, 0};
-  if (a >= 0) myrow = slots[a];  // in flight during the duplicate scan below
-  s_id[tid] = a;
-  s_cnt[tid] = 0;
-  __syncthreads();
-  int pos = 0, first = tid;
-  if (a >= 0) {  // earlier tokens on the same adapter, four ids per shared-memory load
-    auto see = [&](int id, int u) {
-      if (id == a) {
-        if (pos == 0) first = u;
-        ++pos;
-      }
-    };
-    const int full = tid & ~3;
-    for (int u = 0; u < full; u += 4) {
-      const int4 w = *reinterpret_cast<const int4 *>(&s_id[u]);
-      see(w.x, u);
-      see(w.y, u + 1);
-      see(w.z, u + 2);
-      see(w.w, u + 3);
-    }
-    for (int u = full; u < tid; ++u) see(s_id[u], u);
-  }
-  const bool leader = a >= 0 && pos == 0;
-  int G;
-  const int g = block_scan_256(leader ? 1 : 0, s_wt, G);
-  if (leader) {
-    s_grp[tid] = g;
-    s_gadapter[g] = a;
-    s_grank[g] = myrow.rank;
-    s_gscale[g] = myrow.scale;
-  }
-  __syncthreads();
-  int mygrp = -1;
-  if (a >= 0) {
-    mygrp = s_grp[first];
-    atomicAdd(&s_cnt[mygrp], 1);
-  }
-  __syncthreads();
-  int tot;
-  const int n_mine = tid < G ? s_cnt[tid] : 0;
-  const int gs = block_scan_256(n_mine, s_wt, tot);
-  if (tid < G) s_gstart[tid] = gs;
-  if (tid == 0) s_gstart[G] = tot;
-  // token blocks of at most kDsBlockTok tokens
-  const int nb_mine = (n_mine + kDsBlockTok - 1) / kDsBlockTok;
-  int NB;
-  const int b0 = block_scan_256(nb_mine, s_wt, NB);
-  for (int b = 0; b < nb_mine; ++b) {
-    s_bgrp[b0 + b] = tid;
-    s_btok[b0 + b] = gs + b * kDsBlockTok;
-  }
-  __syncthreads();
-  if (mygrp >= 0) s_gtok[s_gstart[mygrp] + pos] = tid;
   const int any_bad = __syncthreads_or(bad ? 1 : 0);
 
   // Work items are per warp: (token block, K chunk, group of eight rank rows).  K chunks: enough
   // items for every warp of the grid, but a chunk keeps at least four K steps (1024 elements)
-  // unless h_in is shorter, so that the ring's ramp-up is amortised.
-  const int n_ksteps = (h_in + 255) >> 8;
+  // unless h_in is shorter, so that the ring's ramp-up is amortised; or two, as long as a warp has no more than one item.
+  const int n_ksteps = (h_in + 255) >> 8, warps_total = (gridDim.x - 1) * (kShrinkThreads / 32);
   const int n_rgn = R_pad >> 3;  // row groups of the rank stride: 2, 4 or 8
   int KS = (target_items + max(NB * n_rgn, 1) - 1) / max(NB * n_rgn, 1);
   KS = max(1, min(min(KS, kMaxZSplits), n_ksteps / 4));
+  if (target_items > 1 && NB * n_rgn * KS < warps_total)
+    KS = max(KS, min(min(kMaxZSplits, n_ksteps / 2), warps_total / max(NB * n_rgn, 1)));
   const int spc = (n_ksteps + KS - 1) / KS;
   KS = (n_ksteps + spc - 1) / spc;
 
@@ -152,7 +89,7 @@ decode_shrink_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
 
   // ---- the last CTA publishes the plan in canonical order (ids ascending, -1 first): everything
   // is worked out in shared memory and registers first, the stores come after the wait
-  if (publisher) publish_decode_plan(pv, a, T, any_bad, KS, s_id, s_cnt, s_wt);
+  if (publisher) publish_decode_plan(pv, s_groups.id[tid], T, any_bad, KS, s_groups.id, s_groups.cnt, s_groups.wt);
 
   // ---- per-warp work items, no CTA-wide synchronisation from here on
   const int n_items = NB * KS * n_rgn;
@@ -166,7 +103,6 @@ decode_shrink_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
   // next ticket is drawn before the current item is processed.  The very last draw of the launch
   // (item number n_items + warps - 1) puts the counter back to zero.
   // (the publishing CTA takes no items: nothing that the next kernel waits for queues behind it)
-  const int warps_total = (gridDim.x - 1) * (kShrinkThreads / 32);
   int32_t *ticket = group_counters + kDsTicket;
   int item = publisher ? n_items : blockIdx.x * (kShrinkThreads / 32) + warp;  // first round is static
   // The warp that completes a (group, row group) adds the K chunks in order into the final plane;
@@ -176,7 +112,7 @@ decode_shrink_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
   int pend_gi = -1, pend_rg = 0, pend_gt0 = 0, pend_gend = 0;
   auto finalize = [&]() {
     if (pend_gi < 0) return;
-    const int arrivals = KS * ((pend_gend - pend_gt0 + kDsBlockTok - 1) / kDsBlockTok);
+    const int arrivals = KS * ((pend_gend - pend_gt0 + kDsTok - 1) / kDsTok);
     __syncwarp();  // the lanes' z stores happen before lane 0's release
     int old = 0;
     if (lane == 0) old = atomic_add_acq_rel(&group_counters[pend_gi * 8 + pend_rg], 1);
@@ -185,7 +121,7 @@ decode_shrink_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
       if (lane == 0) group_counters[pend_gi * 8 + pend_rg] = 0;  // ready for the next launch
       for (int idx = lane; idx < (pend_gend - pend_gt0) * 8; idx += 32) {
         const int tq = idx >> 3;
-        const size_t off = static_cast<size_t>(s_gtok[pend_gt0 + tq]) * R_pad + pend_rg * 8 + (idx & 7);
+        const size_t off = static_cast<size_t>(s_groups.tok[pend_gt0 + tq]) * R_pad + pend_rg * 8 + (idx & 7);
         float part[kMaxZSplits];
 #pragma unroll
         for (int sp = 0; sp < kMaxZSplits; ++sp) part[sp] = sp < KS ? __ldcg(zws + sp * zplane + off) : 0.f;
@@ -224,12 +160,12 @@ decode_shrink_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
     const int c = cur % KS;
     const int br = cur / KS;
     const int bi = br / n_rgn, rg = br - bi * n_rgn;
-    const int gi = s_bgrp[bi];
-    const int ad = s_gadapter[gi];
+    const int gi = s_groups.block_group[bi];
+    const int ad = s_groups.adapter[gi];
     const int rank = s_grank[gi];
     const float scale = s_gscale[gi];
-    const int gt0 = s_gstart[gi], g_end = s_gstart[gi + 1];
-    const int t0 = s_btok[bi], t1 = min(t0 + kDsBlockTok, g_end);
+    const int gt0 = s_groups.start[gi], g_end = s_groups.start[gi + 1];
+    const int t0 = s_groups.block_pos[bi], t1 = min(t0 + kDsTok, g_end);
     if (rank <= 0) {
       if (lane == 0 && c == 0 && rg == 0 && t0 == gt0) atomicOr(status, EDGELORA_STATUS_SLOT_EMPTY);
       item = late_ticket ? draw() : next;
@@ -249,7 +185,7 @@ decode_shrink_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
       for (int i = 0; i < 8 * kDsTok; ++i) acc[i] = 0.f;
       int32_t tok[kDsTok];
 #pragma unroll
-      for (int qq = 0; qq < kDsTok; ++qq) tok[qq] = s_gtok[tb + min(qq, nt - 1)];
+      for (int qq = 0; qq < kDsTok; ++qq) tok[qq] = s_groups.tok[tb + min(qq, nt - 1)];
       if (nt == 1) ok = shrink_rows8<1, kDsDepth, kQ8>(&tmap_a, &tmap_d, &tmap_x, ad, rg * 8, tok, step0, step1, KS, ring, bars, phase, lane, acc);
       else if (nt == 2) ok = shrink_rows8<2, kDsDepth, kQ8>(&tmap_a, &tmap_d, &tmap_x, ad, rg * 8, tok, step0, step1, KS, ring, bars, phase, lane, acc);
       else if (nt == 3) ok = shrink_rows8<3, kDsDepth, kQ8>(&tmap_a, &tmap_d, &tmap_x, ad, rg * 8, tok, step0, step1, KS, ring, bars, phase, lane, acc);
@@ -271,8 +207,8 @@ decode_shrink_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
         ptx::pdl_wait_prior_grids();
         waited = true;
       }
-      if (q < nt && EL_CHECK(status, s_gtok[tb + q] >= 0 && s_gtok[tb + q] < max_tokens && ad >= 0 && ad < n_slots, 20))
-        zws[(KS > 1 ? c : kMaxZSplits) * zplane + static_cast<size_t>(s_gtok[tb + q]) * R_pad + r] =
+      if (q < nt && EL_CHECK(status, s_groups.tok[tb + q] < max_tokens && ad >= 0 && ad < n_slots, 20))
+        zws[(KS > 1 ? c : kMaxZSplits) * zplane + static_cast<size_t>(s_groups.tok[tb + q]) * R_pad + r] =
             scale * acc[0];
     }
     if (!ok) break;
