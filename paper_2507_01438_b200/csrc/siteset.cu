@@ -140,10 +140,10 @@ int run_sites(edgelora_siteset *s, const void *const *x_dev, const int32_t *ids_
       calls[m++] = call;
       read_back = read_back || (after && (*after)[i]);
     }
-    // (the kernel in front of a run is the plan kernel, launched behind everything before it, or the base
-    // product of the run before)
-    // (of a decode-sized batch the first kernel stands to the work in front of the set as its first pool says)
-    rc = decode ? decode_sites(calls, m, s->plan, ids_dev, T, s->ws, stream, i0 > 0 || calls[0].p->opt_pdl >= 2)
+    // The kernel in front of a run is the plan kernel, launched behind everything before it, or the base product of the run
+    // before.  A decode-sized batch has no plan kernel: its first run starts behind everything before the set, whatever
+    // overlap its pools allow (the sites read inputs of their own, which no pool's option speaks for).
+    rc = decode ? decode_sites(calls, m, s->plan, ids_dev, T, s->ws, stream, i0 > 0)
                 : prefill_sites(calls, m, s->plan, nullptr, T, stream, true);
     if (rc != EDGELORA_OK) return rc;
     for (int i = i0; i < i0 + m; ++i)

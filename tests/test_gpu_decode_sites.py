@@ -124,3 +124,35 @@ def test_sites_that_share_a_pool_or_a_result_keep_their_order():
     finally:
         B.edgelora_siteset_destroy(h)
         pool.close()
+
+
+@pytest.mark.parametrize("options", [[2, 1], [2, 2], [1, 2]])
+def test_a_run_starts_behind_the_work_in_front_of_the_set(options):
+    # The input of every run but the first is a result of the run before it, and the GPU is still busy when the runs are
+    # issued: a run that starts early reads what the buffers held before.  Same bits as with a wait behind every run.
+    import torch
+    ids = np.random.Generator(np.random.PCG64(12)).integers(-1, 3, size=40).astype(np.int32)
+    xs, sites = make_sites(13, 40, [(1024, 1024), (1024, 392)], [16, 8, 4], 16, ids)
+    with SetOf(sites, [0, 0]) as s:
+        for p, value in zip(s.pools, options):
+            B.edgelora_pool_set_option(p.handle, B.OPT_PDL, value)
+        first, busy = to_dev_bf16(xs[1024]), torch.randn(4096, 4096, device="cuda")
+
+        def chain(wait):
+            outs = [[torch.full_like(y, float("nan")) for y in s.ys] for _ in range(6)]
+            torch.cuda.synchronize()
+            for _ in range(4):
+                torch.mm(busy, busy)
+            x = first
+            for ys in outs:
+                B.edgelora_siteset_run(s.handle, [x], s.ids, ys)
+                x = ys[0]
+                if wait:
+                    torch.cuda.synchronize()
+            torch.cuda.synchronize()
+            return [[from_dev_bf16(y) for y in ys] for ys in outs]
+
+        for got, want in zip(chain(False), chain(True)):
+            for a, b in zip(got, want):
+                assert np.array_equal(a, b) and np.isfinite(b).all()
+        assert [p.status() for p in s.pools] == [(0, 0)] * 2
