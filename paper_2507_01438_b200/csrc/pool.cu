@@ -262,6 +262,7 @@ int edgelora_plan_build(edgelora_plan_t *plan, const int32_t *ids_dev, int32_t T
   if (T > plan->max_tokens) return EDGELORA_ERR_TOO_MANY_TOKENS;
   plan->last_T = T;
   if (T == 0) return EDGELORA_OK;
+  plan->unread = true;
   launch_plan(ids_dev, T, plan->n_slots, plan->pv, false, static_cast<cudaStream_t>(stream));
   CUDA_TRY(cudaGetLastError());
   return EDGELORA_OK;
@@ -898,6 +899,7 @@ int prefill_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32
   if (ids_dev) {
     ProfScope ps(p0, 0, stream);
     plan->last_T = T;
+    plan->unread = true;
     launch_plan(ids_dev, T, plan->n_slots, plan->pv, pdl_first, stream);
     CUDA_TRY(cudaGetLastError());
     ++launches;
@@ -991,6 +993,7 @@ int decode_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32_
     s.max_tokens = q->cfg.max_tokens;
   }
   plan->last_T = T;
+  plan->unread = true;
   // (two CTAs of the shrink per SM, 98 KB of ring each: 333 us for the 28 sites, 336 with one)
   CUDA_TRY(launch_decode_sites_shrink(sb, 2 * p0->sms, pdl_first, stream));
   CUDA_TRY(launch_decode_sites(db, shape, p0->sms, true, stream));
@@ -1111,8 +1114,8 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
   const bool pdl = p->opt_pdl >= 1 && !p->opt_profile;        // between the kernels of this call
   // first kernel vs earlier stream work (see Order): a set of sites knows whether a call consumes what the calls
   // before it produce
-  const bool pdl_first = !p->opt_profile && ((order == Order::kPool && p->opt_pdl >= 2) ||
-                                             (order == Order::kIndependent && p->opt_pdl >= 1));
+  bool pdl_first = !p->opt_profile && ((order == Order::kPool && p->opt_pdl >= 2) ||
+                                       (order == Order::kIndependent && p->opt_pdl >= 1));
   const uint16_t *x = static_cast<const uint16_t *>(x_dev);
   int launches = 0;
 
@@ -1166,6 +1169,8 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
     // ---------------------------------------------------------------- decode
     const int32_t *ids_in = ids_dev ? ids_dev : plan->pv.ids_valid;
     plan->last_T = T;
+    if (!ids_dev && plan->unread) pdl_first = false;  // (the ids are the library's own)
+    plan->unread = plan->unread || ids_dev;
     auto launch_shrink = [&]() -> int {
       if (T > kGatherMinT) {
         if (ids_dev) {
@@ -1231,6 +1236,7 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
                                       p->status_dev, pdl_first, p->a_q8, shrink_depth, stream));
         ++launches;
       }
+      if (!ids_dev) plan->unread = false;
       return 0;
     };
     // Up to 64 tokens whose row tiles leave SMs for K splits: the K splits of a row tile form a cluster, and the expand moves

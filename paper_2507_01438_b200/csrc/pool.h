@@ -49,6 +49,10 @@ struct ProfRec {
 struct edgelora_plan {
   using PlanView = edgelora::PlanView;
   int32_t max_tokens = 0, n_slots = 0, last_T = 0;
+  // The kernel that writes the plan lets its dependents start at once, and the decode kernels of a planned call read the
+  // plan's ids before their dependency wait.  True until a planned decode call started behind that kernel: the first one
+  // does, whatever overlap the pool allows, and those after it are behind it too.
+  bool unread = false;
   void *block = nullptr;
   PlanView pv{};
 };

@@ -79,6 +79,47 @@ def test_a_result_that_is_an_input_of_later_sites(T, options):
             s.check(f"T={T}")
 
 
+@pytest.mark.parametrize("how", ["chained set", "planned calls"])
+@pytest.mark.parametrize("T", [24, 150])
+def test_the_first_reader_of_a_plan_starts_behind_the_kernel_that_wrote_it(T, how):
+    # Other ids in every step, steps issued while the GPU is busy, pools that allow overlap with earlier work: a kernel that
+    # starts under the plan kernel reads the ids of the step before.  Same bits as with a wait behind every launch.
+    import torch
+    rng = np.random.Generator(np.random.PCG64(71))
+    xs, sites = make_sites(72, T, [(1024, 256), (256, 264), (1024, 136)], [16, 8, 4, 16, 12], 16,
+                           rng.integers(-1, 5, size=T).astype(np.int32))
+    steps = [torch.from_numpy(rng.integers(-1, 5, size=T).astype(np.int32)).cuda() for _ in range(6)]
+    with SetOf(sites, [0, 1, 0]) as s:
+        plan = B.edgelora_plan_create(T, 5)
+        for p in s.pools:
+            B.edgelora_pool_set_option(p.handle, B.OPT_PDL, 2)
+        x, busy = to_dev_bf16(xs[1024]), torch.randn(4096, 4096, device="cuda")
+
+        def run(wait):
+            sync = torch.cuda.synchronize if wait else (lambda: None)
+            outs = [[torch.full_like(y, float("nan")) for y in s.ys] for _ in steps]
+            torch.cuda.synchronize()
+            for _ in range(4):
+                torch.mm(busy, busy)
+            for ids, ys in zip(steps, outs):
+                if how == "chained set":
+                    B.edgelora_siteset_run(s.handle, [x, ys[0]], ids, ys)
+                else:
+                    B.edgelora_plan_build(plan, ids)
+                    for i in (0, 2):
+                        sync()
+                        B.edgelora_lora_linear_planned(s.pools[i].handle, plan, s.Ws[i], x, ys[i])
+                sync()
+            torch.cuda.synchronize()
+            return [[y.view(torch.int16).cpu().numpy() for y in ys] for ys in outs]
+
+        for got, want in zip(run(False), run(True)):
+            for a, b in zip(got, want):
+                assert np.array_equal(a, b)
+        assert [p.status() for p in s.pools] == [(0, 0)] * 3
+        B.edgelora_plan_destroy(plan)
+
+
 def shorten_waits(pool, on=True):
     # 1024 cycles, and what a single try of a barrier may take: far less than the longest waits of these calls.  The
     # kernels give up, wait for what they have in flight, report and return; sync_status brings the pool back
