@@ -994,6 +994,7 @@ int decode_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32_
   }
   plan->last_T = T;
   plan->unread = true;
+  if (getenv("EDGELORA_LOG")) fprintf(stderr, "edgelora: decode T %d N %d sites %d grid %d\n", T, N, n, p0->sms);
   // (two CTAs of the shrink per SM, 98 KB of ring each: 333 us for the 28 sites, 336 with one)
   CUDA_TRY(launch_decode_sites_shrink(sb, 2 * p0->sms, pdl_first, stream));
   CUDA_TRY(launch_decode_sites(db, shape, p0->sms, true, stream));
@@ -1066,6 +1067,8 @@ static int decode_tile(const SiteCall &c, const edgelora_plan *plan, const int32
   d.exp_bytes = shape.exp_bytes;
   d.tmem_cols = shape.tmem_cols;
   d.wait_cycles = p->wait_cycles;
+  if (getenv("EDGELORA_LOG"))
+    fprintf(stderr, "edgelora: decode T %d N %d splits %d grid %d\n", T, N, d.parts, n_tiles * d.parts);
   CUDA_TRY(launch_decode_tile(d, pdl, stream));
   p->last_info[2] = n_tiles * d.parts;
   p->last_info[3] = d.parts;

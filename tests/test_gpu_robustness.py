@@ -186,3 +186,22 @@ def test_the_log_switch_is_read_at_every_decode_call(monkeypatch, capfd):
             assert ("edgelora: decode T 20" in capfd.readouterr().err) == on
     finally:
         pool.close()
+
+
+@pytest.mark.parametrize("T,as_set", [(20, False), (100, False), (20, True), (100, True)])
+def test_every_decode_call_writes_its_log_line(T, as_set, monkeypatch, capfd):
+    import torch
+    w = random_workload(48, T, 256, 256, ranks=[16, 8], max_rank=16)
+    pool = make_pool(w)
+    try:
+        W, x, ids = to_dev_bf16(w.W), to_dev_bf16(w.x), torch.from_numpy(w.ids).cuda()
+        monkeypatch.setenv("EDGELORA_LOG", "1")
+        if as_set:
+            s = B.edgelora_siteset_create([pool.handle], [W], [0], 1, T)
+            B.edgelora_siteset_run(s, [x], ids, [torch.empty(T, 256, dtype=torch.bfloat16, device="cuda")])
+            B.edgelora_siteset_destroy(s)
+        else:
+            pool.linear(W, x, ids)
+        assert f"edgelora: decode T {T} " in capfd.readouterr().err
+    finally:
+        pool.close()
