@@ -85,7 +85,7 @@ __device__ __forceinline__ void publish_decode_plan(const PlanView &pv, int a, i
       pv.group_start[gi] = tid;
       pv.gs_short[gi] = tid;
       pv.group_adapter[gi] = ida;
-      if (ida >= 0) pv.lg_adapter[gi - has_base] = ida;
+      if (ida >= 0) pv.lg_adapter[gi - has_base] = pv.mt_list[gi - has_base] = ida;  // (all tokens are one tile of the list)
     }
     pv.tok_seg[tid] = si + (shead ? 1 : 0) - 1;
     if (shead) {
@@ -104,6 +104,7 @@ __device__ __forceinline__ void publish_decode_plan(const PlanView &pv, int a, i
     pv.counts[4] = n_groups - has_base;
     pv.counts[5] = KS;
     pv.counts[6] = 0;
+    pv.mt_count[0] = n_groups - has_base;
   }
 }
 

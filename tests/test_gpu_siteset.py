@@ -171,3 +171,33 @@ def test_host_buffer_call_twice_on_one_set():
         B.edgelora_siteset_destroy(s)
         for p in pools:
             p.close()
+
+
+@pytest.mark.parametrize("T", [20, 200, 256])
+@pytest.mark.parametrize("by", ["set", "fused call", "call"])
+def test_a_plan_left_by_a_decode_sized_step_serves_a_planned_call_of_the_prefill_regime(by, T):
+    # The handles of a set's and of a pool's plan are open to planned calls: the adapter lists of the step are all there, not
+    # those of a step before it.
+    import torch
+    ranks = [16, 8, 12, 16, 16, 4, 16, 16]
+    old, ids = mixed_ids(81, T - 9, [(1, 9)], 3), mixed_ids(82, T - 9, [(7, 9)], len(ranks))
+    xs, sites = make_sites(83, T, [(256, 264), (256, 136)], ranks, 16, ids)
+    pools, Ws, x = [make_pool(w, T) for w in sites], [to_dev_bf16(w.W) for w in sites], to_dev_bf16(xs[256])
+    s = B.edgelora_siteset_create([p.handle for p in pools], Ws, [0, 0], 1, T)
+    try:
+        B.edgelora_pool_set_option(pools[0].handle, B.OPT_FUSED_DECODE, 1 if by == "fused call" else 0)
+        ys = [torch.full((T, w.h_out), float("nan"), dtype=torch.bfloat16, device="cuda") for w in sites]
+        for step in (old, ids):
+            if by == "set":
+                B.edgelora_siteset_run(s, [x], torch.from_numpy(step).cuda(), ys)
+            else:
+                pools[0].linear(Ws[0], x, torch.from_numpy(step).cuda(), ys[0])
+        plan = B.edgelora_siteset_plan(s) if by == "set" else B.edgelora_pool_plan(pools[0].handle)
+        B.edgelora_pool_set_option(pools[1].handle, B.OPT_REGIME, 2)
+        B.edgelora_lora_linear_planned(pools[1].handle, plan, Ws[1], x, ys[1])
+        assert_parity(from_dev_bf16(ys[1]), oracle_of(sites[1]), "planned")
+        assert [p.status() for p in pools] == [(0, 0)] * 2
+    finally:
+        B.edgelora_siteset_destroy(s)
+        for p in pools:
+            p.close()
