@@ -1206,14 +1206,17 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
         // the 200-adapter down_proj: 45.8 us against 49.8 us with depth 4)
         const int shrink_depth = T <= 64 ? 2 : (p->opt_shrink_depth == 4 ? 4 : 2);
         const int cta_cap = shrink_depth == 2 && T > 64 ? 2 * p->sms : p->sms;
-        // Large batches: few, long items (about 0.6 per warp) beat many short ones, whose ring ramp-up and
-        // chunk sums add up: 92 us per step with 2 K chunks on the 1000-adapter down_proj, 96 with 3-4,
-        // 100 with 12, 104 with 1.  Small batches: four items per warp.
+        // Large batches: few, long items beat many short ones, whose ring ramp-up and chunk sums add up: 92 us per step
+        // with 2 K chunks on the 1000-adapter down_proj, 96 with 3-4, 100 with 12, 104 with 1.  About 0.6 per warp are
+        // aimed for, and where they leave warps without one, K is cut further, to about one per warp (6144 -> 3432 with A
+        // in Q8_0, 145 tokens on six adapters: 42.7 us per call, 53.9 without; 1656 -> 328, 69 tokens on four: 21.6 and
+        // 27.3; 984 -> 11960, four tokens, one of the few that lose: 10.3 and 9.8).  Small batches: four items per warp.
         const int auto_target = T > 64 ? 5 * cta_cap : 4 * 8 * cta_cap;
         const int target = p->opt_shrink_items > 0 ? p->opt_shrink_items : (overlapped ? 1 : auto_target);
         // at most T token blocks x (R / 8) row groups x K chunks warp items, eight warps per CTA
         const int n_ksteps = (h_in + kShrinkStepElems - 1) / kShrinkStepElems;
-        const int max_chunks = target == 1 ? 1 : std::max(1, std::min(kMaxZSplits, n_ksteps / 2));
+        const bool fill_warps = p->opt_shrink_items == 0 && !overlapped;
+        const int max_chunks = target == 1 ? 1 : std::max(1, std::min(kMaxZSplits, n_ksteps / (fill_warps ? 2 : 4)));
         const int max_items = std::min(T, p->cfg.n_slots) * (R / 8) * max_chunks;
         const int grid = std::max(1, std::min(cta_cap - 1, (max_items + 7) / 8)) + 1;  // + the publishing CTA
         CUtensorMap ma, mx, md;
@@ -1235,7 +1238,7 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
         rc = get_tmap(p, &mx, x, h_in, T, 0, 1, kShrinkStepElems);
         if (rc) return rc;
         CUDA_TRY(launch_decode_shrink(ma, md, mx, ids_in, p->slots_dev, plan->pv, p->zws, p->group_counters,
-                                      T, h_in, R, p->cfg.n_slots, p->cfg.max_tokens, target, grid,
+                                      T, h_in, R, p->cfg.n_slots, p->cfg.max_tokens, target, fill_warps, grid,
                                       p->status_dev, pdl_first, p->a_q8, shrink_depth, stream));
         ++launches;
       }

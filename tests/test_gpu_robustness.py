@@ -205,3 +205,23 @@ def test_every_decode_call_writes_its_log_line(T, as_set, monkeypatch, capfd):
         assert f"edgelora: decode T {T} " in capfd.readouterr().err
     finally:
         pool.close()
+
+
+def test_a_given_number_of_shrink_items_is_kept():
+    # 40 tokens on four adapters have more (token block, eight rank rows) items than one or two: K stays whole for both numbers,
+    # and so do the sums; the library's own choice cuts it
+    import torch
+    w = random_workload(49, 40, 8192, 264, ranks=[16, 16, 16, 16], max_rank=16)
+    pool = make_pool(w)
+    try:
+        B.edgelora_pool_set_option(pool.handle, B.OPT_FUSED_DECODE, 0)
+        W, x, ids = to_dev_bf16(w.W), to_dev_bf16(w.x), torch.from_numpy(w.ids).cuda()
+        got = {}
+        for items in (1, 2, 0):
+            B.edgelora_pool_set_option(pool.handle, B.OPT_SHRINK_ITEMS, items)
+            got[items] = from_dev_bf16(pool.linear(W, x, ids))
+            assert_parity(got[items], oracle_of(w), f"{items} items")
+        assert np.array_equal(got[1], got[2]) and not np.array_equal(got[1], got[0])
+        assert pool.status() == (0, 0)
+    finally:
+        pool.close()
