@@ -24,7 +24,6 @@
 #include "launch.cuh"
 #include "ptx.cuh"
 #include "tile_order.h"
-#include "zload.cuh"
 
 namespace edgelora {
 
@@ -80,8 +79,7 @@ __device__ __forceinline__ int wait_for_teams(const int32_t *counter, int32_t n,
 }
 
 // Fused decode launches (batches of at most 64 tokens): z[t] = s_a A_a x[t] on the CUDA cores, by
-// "teams" of four warps: the four builder warps of every CTA of the decode job (idle there, because
-// the expand is added by the owners of the cluster reduction) and two teams in every spare CTA.
+// "teams" of four warps: warps 6..9 of every CTA of the decode job and two teams in every spare CTA.
 // A team item is (token, eight rank rows, K chunk): chunk c covers the K steps c, c + ks, ... of 256
 // elements; warp w of the team takes every fourth of them, lane l the elements [8 l, 8 l + 8) of a
 // step (one 16-byte load of x and eight of A in flight per lane).  The four warps' sums meet in

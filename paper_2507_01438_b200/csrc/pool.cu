@@ -1295,7 +1295,7 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
     rc = get_tmap(p, &mc, x, h_in, T, 0, N);
     if (rc) return rc;
     const int grid = row_tiles * splits;
-    // Small batches in one launch: the shrink runs on the idle builder warps of the base product's CTAs
+    // Small batches in one launch: the shrink runs on team warps of the base product's CTAs
     // and on spare CTAs in front of them (SMs the grid leaves empty), and the owners of the cluster
     // reduction wait for its arrival counter.  CTAs of one grid wait for one another here, so every
     // cluster of the launch must be resident at once: checked against the device's occupancy figure.

@@ -23,9 +23,18 @@
 #include "ptx.cuh"
 #include "shrink_tiles.h"
 #include "tile_order.h"
-#include "zload.cuh"
 
 namespace edgelora {
+
+// Eight consecutive values of z, from rank index r0 on, as one 16-byte chunk of the operand: values at or past the
+// true rank forced to zero.
+__device__ __forceinline__ uint4 pack_z_chunk(const float (&v)[8], int32_t r0, int32_t rank) {
+  float m[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) m[i] = r0 + i < rank ? v[i] : 0.f;
+  return make_uint4(ptx::pack_bf16x2(m[0], m[1]), ptx::pack_bf16x2(m[2], m[3]), ptx::pack_bf16x2(m[4], m[5]),
+                    ptx::pack_bf16x2(m[6], m[7]));
+}
 
 namespace {
 
