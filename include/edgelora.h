@@ -243,7 +243,9 @@ int edgelora_plan_sync_status(edgelora_plan_t *plan, void *stream, uint32_t *bit
  * to 32 sites share one shrink launch and one base-product launch.  A site's result may lie in the memory of
  * an input: the sites behind it that read this input read the result (they start when it is written, one
  * launch per site, also with EDGELORA_OPT_PDL = 2); only a site's own input must not overlap its result.  The set
- * borrows the pools and W (the caller keeps them alive) and owns its plan and the device mirrors of the
+ * borrows the pools and W (the caller keeps them alive) and owns its plan, a device workspace for batches of at most 256
+ * tokens (allocated here: two fp32 tiles of 128 rows x min(max_tokens, 256) columns per SM, or per four K blocks of work
+ * where the sites have less than that for every SM: 38.8 MB at most on 148 SMs) and the device mirrors of the
  * host-buffer call.  One thread at a time per set; runs of one set (and of its pools) must not overlap on
  * the GPU. */
 typedef struct edgelora_siteset edgelora_siteset_t;

@@ -65,8 +65,6 @@ __device__ __forceinline__ bool epilogue_any(bool v) {
   return r != 0;
 }
 
-// Expand units of a tile (one for 64 rank columns of B: as many bytes as a K block of W), of NS stages.
-__device__ __forceinline__ int32_t expand_units(int32_t n_stages, int32_t R_pad) { return (n_stages * R_pad + 63) >> 6; }
 // Stages of the units [e0, e1).
 __device__ __forceinline__ int32_t first_stage(int32_t unit, int32_t n_stages, int32_t R_pad) {
   return min(unit * (64 >> (31 - __clz(R_pad))), n_stages);
@@ -177,7 +175,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_sites_kernel(const __gr
   __syncthreads();
   const uint32_t tmem_base = sh.tmem_slot, tmem_exp = tmem_base + static_cast<uint32_t>(b.n_acc * Nc);
   const int32_t n_units = sh.site_end[b.n_sites - 1];
-  const int32_t n_runs = min(static_cast<int32_t>(gridDim.x), max(1, n_units >> 2));
+  const int32_t n_runs = run_count(n_units, static_cast<int32_t>(gridDim.x));
   const Runs runs(n_units, n_runs);
   const int32_t u_begin = me < n_runs ? runs.begin(me) : n_units, u_end = me < n_runs ? runs.begin(me + 1) : n_units;
   int32_t site = 0;

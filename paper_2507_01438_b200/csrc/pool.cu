@@ -21,6 +21,7 @@
 #include "prefill.h"
 #include "shrink_tiles.h"
 #include "tile_order.h"
+#include "units.h"
 
 using namespace edgelora;
 
@@ -916,10 +917,18 @@ int prefill_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32
 // ---- decode-sized batches of a run of sites (decode_sites.cu)
 static int32_t decode_columns(int32_t T) { return std::max(16, (T + 15) / 16 * 16); }
 
-size_t decode_workspace_bytes(int32_t sms, int32_t max_tokens, size_t *arrivals_at) {
-  const size_t planes = static_cast<size_t>(sms) * 2 * kTileM * decode_columns(std::min(max_tokens, kDecodeMaxT)) * sizeof(float);
-  *arrivals_at = planes;
-  return planes + static_cast<size_t>(sms) * 4 * sizeof(int32_t);
+int32_t decode_workspace_ctas(edgelora_pool *const *pools, int32_t n, int32_t max_tokens) {
+  const int32_t T = std::min(max_tokens, kDecodeMaxT), stages = expand_stages_max(T, pools[0]->cfg.n_slots, kExpTok);
+  int64_t units = 0;
+  for (int32_t i = 0; i < n; ++i) {
+    const edgelora_pool_config &c = pools[i]->cfg;
+    units += static_cast<int64_t>((c.h_out + kTileM - 1) / kTileM) *
+             ((c.h_in + kBlockK - 1) / kBlockK + expand_units(stages, pools[i]->R_pad));
+  }
+  return run_count(static_cast<int32_t>(std::min<int64_t>(units, INT32_MAX)), pools[0]->sms);
+}
+size_t decode_workspace_planes(int32_t ctas, int32_t max_tokens) {
+  return static_cast<size_t>(ctas) * 2 * kTileM * decode_columns(std::min(max_tokens, kDecodeMaxT));
 }
 
 static int fill_decode_site(const SiteCall &c, int x_index, DecSite *d) {
@@ -953,7 +962,7 @@ int decode_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32_
   sb.ids = ids_dev;
   sb.pv = plan->pv;
   sb.zero = db.arrivals = ws.arrivals;
-  sb.n_zero = 4 * p0->sms;
+  sb.n_zero = 4 * ws.ctas;
   db.T = T;
   db.N = N;
   db.ids = ids_dev;
@@ -994,15 +1003,15 @@ int decode_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32_
   }
   plan->last_T = T;
   plan->unread = true;
-  if (getenv("EDGELORA_LOG")) fprintf(stderr, "edgelora: decode T %d N %d sites %d grid %d\n", T, N, n, p0->sms);
+  if (getenv("EDGELORA_LOG")) fprintf(stderr, "edgelora: decode T %d N %d sites %d grid %d\n", T, N, n, ws.ctas);
   // (two CTAs of the shrink per SM, 98 KB of ring each: 333 us for the 28 sites, 336 with one)
   CUDA_TRY(launch_decode_sites_shrink(sb, 2 * p0->sms, pdl_first, stream));
-  CUDA_TRY(launch_decode_sites(db, shape, p0->sms, true, stream));
+  CUDA_TRY(launch_decode_sites(db, shape, ws.ctas, true, stream));
   for (int i = 0; i < n; ++i) {
     int64_t *info = sites[i].p->last_info;
     info[0] = i == 0 ? 2 : 0;
     info[1] = 1;
-    info[2] = p0->sms;
+    info[2] = ws.ctas;
     info[3] = 1;
     info[4] = shape.stages;
     info[5] = N;

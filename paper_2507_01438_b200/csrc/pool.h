@@ -139,8 +139,11 @@ int prefill_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32
 struct DecodeWorkspace {
   float *partial = nullptr;      // two planes [N][128] per CTA
   int32_t *arrivals = nullptr;   // [CTAs][4]
+  int32_t ctas = 0;              // one per SM, or as many as the set's sites have work for
 };
-size_t decode_workspace_bytes(int32_t sms, int32_t max_tokens, size_t *arrivals_at);
+// The CTAs of a set of these pools, and the fp32 values of their planes.
+int32_t decode_workspace_ctas(edgelora_pool *const *pools, int32_t n, int32_t max_tokens);
+size_t decode_workspace_planes(int32_t ctas, int32_t max_tokens);
 int decode_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32_t *ids_dev, int32_t T,
                  const DecodeWorkspace &ws, cudaStream_t stream, bool pdl_first);
 int wait_for_loads(edgelora_pool *p, cudaStream_t stream, bool capturing);

@@ -197,15 +197,17 @@ int edgelora_siteset_create(int32_t n_sites, edgelora_pool_t *const *pools, cons
     delete s;
     return rc;
   }
-  size_t arrivals_at = 0;
-  const size_t ws_bytes = decode_workspace_bytes(pools[0]->sms, max_tokens, &arrivals_at);
-  if (el_malloc(&s->ws.partial, ws_bytes) != cudaSuccess) {
+  s->ws.ctas = decode_workspace_ctas(pools, n_sites, max_tokens);
+  const size_t planes = decode_workspace_planes(s->ws.ctas, max_tokens);
+  const cudaError_t e = el_malloc(&s->ws.partial, (planes + static_cast<size_t>(s->ws.ctas) * 4) * 4);
+  if (e != cudaSuccess) {
+    set_last_cuda_error(e, "workspace of a site set");
     cudaGetLastError();
     edgelora_plan_destroy(s->plan);
     delete s;
     return EDGELORA_ERR_CUDA;
   }
-  s->ws.arrivals = reinterpret_cast<int32_t *>(reinterpret_cast<uint8_t *>(s->ws.partial) + arrivals_at);
+  s->ws.arrivals = reinterpret_cast<int32_t *>(s->ws.partial + planes);
   s->dx.assign(n_inputs, nullptr);
   s->dy.assign(n_sites, nullptr);
   *set_out = s;

@@ -18,6 +18,19 @@ struct Runs {
   }
 };
 
+// Expand units of a tile (one for 64 rank columns of B: as many bytes as a K block of W), of n stages.
+EDGELORA_HD int32_t expand_units(int32_t n_stages, int32_t R_pad) { return (n_stages * R_pad + 63) >> 6; }
+// Stages that T tokens on adapters of n_slots slots make at most, `tok` tokens of an adapter in a stage.
+EDGELORA_HD int32_t expand_stages_max(int32_t T, int32_t n_slots, int32_t tok) {
+  const int32_t g = T < n_slots ? T : n_slots;
+  return g + (T - g) / tok;
+}
+// Runs of a launch of n units on a device of p SMs: four units each at least.
+EDGELORA_HD int32_t run_count(int32_t n, int32_t p) {
+  const int32_t most = n / 4 > 1 ? n / 4 : 1;
+  return most < p ? most : p;
+}
+
 // What a run does of one tile: its expand stages' units first, the units of its K blocks behind them.
 struct Piece {
   int32_t s, tile;   // site, W row tile of the site

@@ -201,3 +201,17 @@ def test_a_plan_left_by_a_decode_sized_step_serves_a_planned_call_of_the_prefill
         B.edgelora_siteset_destroy(s)
         for p in pools:
             p.close()
+
+
+def test_the_workspace_of_a_small_set_is_small():
+    import torch
+    _, sites = make_sites(84, 256, [(264, 136), (264, 8)], [16, 8, 4], 16, np.zeros(256, np.int32))
+    pools, Ws = [make_pool(w, 256) for w in sites], [to_dev_bf16(w.W) for w in sites]
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    s = B.edgelora_siteset_create([p.handle for p in pools], Ws, [0, 0], 1, 256)
+    used = free - torch.cuda.mem_get_info()[0]
+    B.edgelora_siteset_destroy(s)
+    for p in pools:
+        p.close()
+    assert used <= 8 << 20      # two tiles each of ten CTAs, in the driver's granules; for every SM they are 38.8 MB

@@ -36,6 +36,12 @@ extern "C" int32_t pieces(int32_t n_sites, const int32_t *tiles, const int32_t *
 """
 
 
+SOURCE += r"""
+extern "C" int32_t stages_max(int32_t T, int32_t n_slots, int32_t tok) { return edgelora::expand_stages_max(T, n_slots, tok); }
+extern "C" int32_t run_count(int32_t n, int32_t p) { return edgelora::run_count(n, p); }
+"""
+
+
 @pytest.fixture(scope="module")
 def units(tmp_path_factory):
     d = tmp_path_factory.mktemp("units")
@@ -68,3 +74,23 @@ def test_every_unit_of_every_tile_is_done_once(units, tiles, expand, kb, runs):
     assert len(starts) == len(set(starts))           # a run begins one shared tile at most
     for (_, _, r0, r1), who in by_tile.items():
         assert who == list(range(r0, r1 + 1))        # the runs that add up a tile, a piece each
+
+
+@pytest.mark.parametrize("T,n_slots", [(1, 1), (8, 1), (9, 1), (27, 64), (256, 3), (256, 40), (256, 1000)])
+def test_a_workspace_for_the_most_stages_holds_every_batch(units, T, n_slots):
+    # as many stages as the bound says are reached, none more; and a grid of the runs of the largest batch cuts a smaller one
+    # as a grid of the whole device would
+    rng = np.random.Generator(np.random.PCG64(T + n_slots))
+    most = units.stages_max(T, n_slots, 8)
+    worst = 0
+    for k in range(60):
+        few = rng.integers(1, n_slots + 1)
+        n = np.bincount(rng.integers(0, few, size=rng.integers(1, T + 1)) if k else np.arange(T) % n_slots)
+        worst = max(worst, int((-(-n // 8)).sum()))
+        assert worst <= most
+    groups = np.ones(min(T, n_slots), int)           # one token each, the others by whole stages on the first
+    groups[0] += T - len(groups)
+    assert int((-(-groups // 8)).sum()) == most or (T - len(groups)) % 8
+    for n_max in (1, 7, 40, 590, 592, 10000):
+        for n in {1, n_max // 3 + 1, n_max - 1 or 1, n_max}:
+            assert units.run_count(n, units.run_count(n_max, 148)) == units.run_count(n, 148)
