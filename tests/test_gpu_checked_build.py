@@ -18,7 +18,8 @@ pytestmark = pytest.mark.gpu
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 CASES = ["tests/test_gpu_parity.py", "tests/test_gpu_fused_decode.py", "tests/test_gpu_gather_tiles.py",
-         "tests/test_gpu_siteset.py", "tests/test_gpu_routing.py", "tests/test_gpu_quant.py"]
+         "tests/test_gpu_siteset.py", "tests/test_gpu_routing.py", "tests/test_gpu_quant.py",
+         "tests/test_gpu_decode_sites.py", "tests/test_gpu_decode_tile.py"]
 
 
 def test_parity_cases_under_the_checked_build():

@@ -156,3 +156,33 @@ def test_a_run_starts_behind_the_work_in_front_of_the_set(options):
             for a, b in zip(got, want):
                 assert np.array_equal(a, b) and np.isfinite(b).all()
         assert [p.status() for p in s.pools] == [(0, 0)] * 2
+
+
+@pytest.mark.parametrize("pdl", [1, 2])
+@pytest.mark.parametrize("T", [12, 130])
+def test_several_runs_of_a_step_and_steps_in_a_row(T, pdl):
+    # a pool that comes twice cuts a step into two runs, which use one workspace and one z in turn; nothing waits in between
+    import torch
+    ids = np.random.Generator(np.random.PCG64(14)).integers(-1, 4, size=T).astype(np.int32)
+    xs, sites = make_sites(15, T, [(1032, 520), (1032, 136), (1032, 264)], [16, 8, 4, 16], 16, ids)
+    pools, Ws, x = [make_pool(w, T) for w in sites], [to_dev_bf16(w.W) for w in sites], to_dev_bf16(xs[1032])
+    order = [0, 1, 0, 2, 1]
+    s = B.edgelora_siteset_create([pools[i].handle for i in order], [Ws[i] for i in order], [0] * 5, 1, T)
+    try:
+        for p in pools:
+            B.edgelora_pool_set_option(p.handle, B.OPT_PDL, pdl)
+        idt = torch.from_numpy(ids).cuda()
+        steps = [[torch.full((T, sites[i].h_out), float("nan"), dtype=torch.bfloat16, device="cuda") for i in order]
+                 for _ in range(4)]
+        torch.cuda.synchronize()
+        for ys in steps:
+            B.edgelora_siteset_run(s, [x], idt, ys)
+        for k, i in enumerate(order):
+            got = [from_dev_bf16(ys[k]) for ys in steps]
+            assert_parity(got[0], oracle_of(sites[i]), sites[i].name)
+            assert all(np.array_equal(got[0], g) for g in got[1:])
+        assert [p.status() for p in pools] == [(0, 0)] * 3
+    finally:
+        B.edgelora_siteset_destroy(s)
+        for p in pools:
+            p.close()

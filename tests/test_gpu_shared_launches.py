@@ -131,7 +131,7 @@ def shorten_waits(pool, on=True):
     (513, 1032, 40000, {}),                      # tiles off the launch queue
     (40, 2048, 264, {B.OPT_REGIME: 2}),          # gather tiles only
     (24, 4096, 512, {}),                         # decode in one launch
-    (200, 14336, 520, {}),                       # decode with LoRA K blocks
+    (200, 14336, 520, {}),                       # decode, shrink and tile kernel
 ])
 def test_a_call_whose_waits_run_out_reports_and_leaves_the_pool_usable(T, h_in, h_out, options):
     import torch

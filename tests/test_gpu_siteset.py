@@ -1,5 +1,5 @@
 """A set of linear sites over one batch (edgelora_siteset_*): one routing plan, the sites of a large
-batch in shared launches, those of a decode-sized batch one after the other.  Every site's
+batch in shared launches, those of a decode-sized batch in others of their own.  Every site's
 result is compared with the CPU oracle of that site, element by element; the plan bit for bit.
 """
 import numpy as np
