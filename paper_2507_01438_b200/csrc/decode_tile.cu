@@ -9,8 +9,12 @@
 // its own tokens' ids only.  Figures: see decode_parts in pool.cu.
 //
 // Warp roles: warp 0 issues the loads of W and x (the first round of the ring before anything else), warp 1 owns tensor memory
-// and issues the MMAs, warp 2 issues the copies of the expand, warps 4..11 (two to a lane quadrant: a single warp per scheduler
-// cannot keep up with the latency of its sums) work out the u-batches, the expand and y.  Every mbarrier wait is bounded; on a
+// and issues the MMAs, warps 2 and 3 issue the copies of the expand, each those of one of the two groups of expand warps,
+// warps 4..11 (two to a lane quadrant: a single warp per scheduler cannot keep up with the latency of its sums) work out the
+// u-batches, the expand and y.  (A thread takes 0.3 us to issue the copies of a stage; with all stages issued by one warp that
+// was the pace of an expand of rank stride 16 or 32: 336 -> 13208, 209 tokens on 17 adapters: 37.1 us per call, now 31.7; 512 ->
+// 11744, 119 tokens on 25, A in Q8_0: 28.9 and 25.5; 1848 -> 288, 255 tokens on 56: 36.0 and 34.4.  At stride 64 the reads of z
+// from shared memory are: 680 -> 9576, 97 tokens on seven adapters: 32.0 with either.)  Every mbarrier wait is bounded; on a
 // timeout the status word gets EDGELORA_STATUS_TIMEOUT and all roles leave.
 #include <algorithm>
 
@@ -50,6 +54,12 @@ struct Shared {
   Groups groups;
 };
 static_assert(sizeof(Shared) <= kTailBytes, "tail of the shared memory");
+
+// Rank, tokens and first position of an expand stage, in one word.
+__device__ __forceinline__ uint32_t stage_info(const Shared &sh, int s) {
+  const int g = sh.groups.block_group[s], pos = sh.groups.block_pos[s];
+  return sh.rank[g] | min(kExpTok, sh.groups.start[g + 1] - pos) << 8 | pos << 16;
+}
 
 // The stage's tokens, four, two or one at a time, each into its column.
 template <int kR>
@@ -166,31 +176,42 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tile_kernel(const __grid_c
       }
       ptx::umma_commit(&sh.tfull);  // accumulator complete, or as far as it came
     }
-  } else if (warp == 2) {
-    // ------------------------------------------------------------ copies of the expand (B_a rows and z)
-    if (ptx::elect_one()) {
-      ok = ptx::mbar_wait(&sh.groups_ready, 0, wl);
-      ptx::pdl_wait_prior_grids();  // z comes from the kernel before this one
-      const uint32_t b_bytes = static_cast<uint32_t>(kTileM * p.R_pad * 2), z_bytes = static_cast<uint32_t>(p.R_pad) * 4;
-      uint32_t stage = 0, phase = 0;
-      for (int32_t s = 0; ok && s < sh.groups.n_blocks; ++s) {
-        const int g = sh.groups.block_group[s], pos = sh.groups.block_pos[s];
-        if (sh.rank[g] == 0) continue;  // an empty slot: its tokens stay base-only
-        const int nt = min(kExpTok, sh.groups.start[g + 1] - pos);
-        if (!ptx::mbar_wait(&sh.bempty[stage], phase ^ 1, wl) || sh.abort_flag) {
-          ok = false;
-          break;
+  } else if (warp < 4) {
+    // ------------------------------------------------------------ copies of the expand (B_a rows and z; warps 2 and 3)
+    const int half = warp - 2;
+    ok = __all_sync(0xffffffffu, ptx::mbar_wait(&sh.groups_ready, 0, wl));
+    ptx::pdl_wait_prior_grids();  // z comes from the kernel before this one
+    const uint32_t b_bytes = static_cast<uint32_t>(kTileM * p.R_pad * 2), z_bytes = static_cast<uint32_t>(p.R_pad) * 4;
+    uint32_t stage = 0, phase = 0, info = 0;  // lane l: rank, tokens and first position of the stage l of the next 32
+    int32_t adapter = 0;                      // and its adapter
+    int live = 0;
+    const int n_blocks = sh.groups.n_blocks;
+    for (int s = 0; ok && s < n_blocks; ++s) {
+      if ((s & 31) == 0 && s + lane < n_blocks) {
+        info = stage_info(sh, s + lane);
+        adapter = sh.groups.adapter[sh.groups.block_group[s + lane]];
+      }
+      const uint32_t mine = __shfl_sync(0xffffffffu, info, s & 31);
+      const int32_t a = __shfl_sync(0xffffffffu, adapter, s & 31);
+      const int rank = mine & 255, nt = (mine >> 8) & 255, pos = mine >> 16;
+      if (rank == 0) continue;  // an empty slot: its tokens stay base-only
+      if ((live++ & 1) == half) {
+        if (ptx::elect_one()) {
+          ok = ptx::mbar_wait(&sh.bempty[stage], phase ^ 1, wl) && !sh.abort_flag;
+          if (ok) {
+            uint8_t *dst = exp_ring + static_cast<size_t>(stage) * p.exp_bytes;
+            ptx::mbar_arrive_expect_tx(&sh.bfull[stage], b_bytes + nt * z_bytes);
+            ptx::tma_load_3d(dst, &p.b, &sh.bfull[stage], 0, row0, a);
+            for (int q = 0; q < nt; ++q)
+              ptx::bulk_load_1d(dst + b_bytes + q * z_bytes, p.z + static_cast<size_t>(t0 + sh.groups.tok[pos + q]) * p.R_pad,
+                                z_bytes, &sh.bfull[stage]);
+          }
         }
-        uint8_t *dst = exp_ring + static_cast<size_t>(stage) * p.exp_bytes;
-        ptx::mbar_arrive_expect_tx(&sh.bfull[stage], b_bytes + nt * z_bytes);
-        ptx::tma_load_3d(dst, &p.b, &sh.bfull[stage], 0, row0, sh.groups.adapter[g]);
-        for (int q = 0; q < nt; ++q)
-          ptx::bulk_load_1d(dst + b_bytes + q * z_bytes, p.z + static_cast<size_t>(t0 + sh.groups.tok[pos + q]) * p.R_pad, z_bytes,
-                            &sh.bfull[stage]);
-        if (++stage == nexp) {
-          stage = 0;
-          phase ^= 1;
-        }
+        ok = __all_sync(0xffffffffu, ok);
+      }
+      if (++stage == nexp) {
+        stage = 0;
+        phase ^= 1;
       }
     }
   } else if (warp >= 4) {
@@ -215,10 +236,7 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tile_kernel(const __grid_c
     int live = 0;
     const int n_blocks = sh.groups.n_blocks;
     for (int s = 0; s < n_blocks; ++s) {
-      if ((s & 31) == 0 && s + lane < n_blocks) {
-        const int g = sh.groups.block_group[s + lane], pos = sh.groups.block_pos[s + lane];
-        info = sh.rank[g] | min(kExpTok, sh.groups.start[g + 1] - pos) << 8 | pos << 16;
-      }
+      if ((s & 31) == 0 && s + lane < n_blocks) info = stage_info(sh, s + lane);
       const uint32_t mine = __shfl_sync(0xffffffffu, info, s & 31);
       const int rank = mine & 255, nt = (mine >> 8) & 255, pos = mine >> 16;
       if (rank == 0) continue;
