@@ -1022,24 +1022,29 @@ int decode_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32_
 
 // ---- decode-sized batch of one site (decode_tile.cu)
 //
-// CTAs that share a tile: the count whose launch is done first.  A K block takes a CTA about a third of a microsecond, and so
-// does an adapter of its own tokens in the expand beside it (the device knows their number; six tenths of the tokens are
-// assumed); the exchange of the parts takes 1.5, and a count whose clusters are not all resident at once pays its ramp-up of 4 us
-// again.  Us per call, before (an expand on the tensor cores, tokens padded to a power of two) and now: 3080 -> 5000, 77 tokens:
-// 27.4 and 26.1; 14336 -> 4096, 256 tokens on 109 adapters of rank 64: 91.2 and 83.3; 4096 -> 12000, 90 tokens: 48.8 and 41.6;
-// 8192 -> 8192, 128 tokens: 48.6 and 43.0; 1024 -> 4096, 160 tokens: 39.7 and 32.7; 664 -> 864, 226 tokens: 33.7 and 35.6.
+// CTAs that share a tile: the count whose launch is done first.  A K block takes a CTA about a third of a microsecond.  Beside
+// the K blocks it works out the expand of its own tokens: a sixth for every stage (one for each of their adapters, whose number
+// the device knows, six tenths of the tokens are assumed, and one for every eight tokens more), and 0.028, 0.036 or 0.052 for
+// every token, by the rank stride.  All of that is little beside a wave: clusters that are not resident at once begin their launch over, with
+// its u-batches and its first round of copies, which takes 16, and 1.5 more with parts to exchange.
+// (Residency, by count: 148, 74, 45, 33, 26, 22, 15 and 15 clusters.)  In 130 drawn calls of 33 to 256 tokens the count taken
+// was 0.6 % slower than the best of all eight on average, 7 % at most.  Us per call, with the rule before (the tokens of an adapter
+// free, four per wave, two K blocks for each CTA) and now: 608 -> 1280, 106 tokens on 19 adapters of rank 64: 31.7 and 22.0; 5216 -> 11224,
+// 64 tokens: 49.7 and 39.8; 9440 -> 6184, 142 tokens: 53.8 and 38.2; 664 -> 864, 226 tokens on 34: 43.1 and 30.8.
 static int decode_parts(edgelora_pool *p, int n_tiles, int kb, int32_t T) {
   if (p->tile_clusters[1] == 0)
     for (int c = 1; c <= kTileMaxParts; ++c) p->tile_clusters[c] = std::max(1, decode_tile_max_clusters(c));
-  const int most = std::max(1, std::min(p->opt_decode_splits > 0 ? p->opt_decode_splits : kTileMaxParts, kb / 2));
+  const int most = std::max(1, std::min(p->opt_decode_splits > 0 ? p->opt_decode_splits : kTileMaxParts, kb));
   const int quads = (T + 3) / 4;
   int best = 1;
   double best_cost = 0;
   for (int c = 1; c <= most; ++c) {
     if (!decode_tile_parts_fit(T, c)) continue;
     const int waves = (n_tiles + p->tile_clusters[c] - 1) / p->tile_clusters[c];
-    const int own = std::min((quads + c - 1) / c * 4, p->cfg.n_slots);
-    const double cost = waves * (std::max((kb + c - 1) / c * 0.33, own * 0.6 * 0.33) + 4.0) + (c > 1 ? 1.5 : 0.0);
+    const int own = std::min((quads + c - 1) / c * 4, T);
+    const double stages = std::min(0.6 * own, static_cast<double>(p->cfg.n_slots)) + own / 8.0;
+    const double expand = 0.17 * stages + (0.02 + 0.0005 * p->R_pad) * own;
+    const double cost = waves * (std::max((kb + c - 1) / c * 0.33, expand) + (c > 1 ? 17.5 : 16.0));
     if (c == 1 || cost < best_cost || p->opt_decode_splits > 0) {
       best = c;
       best_cost = cost;

@@ -77,3 +77,29 @@ def test_a_non_finite_adapter_reaches_its_own_tokens_only():
         assert not np.isfinite(got[bad]).any()
     finally:
         pool.close()
+
+
+@pytest.mark.parametrize("h_in,h_out,T,slots,rank", [
+    (664, 864, 226, 40, 16),        # few adapters with many tokens each: their tokens count too
+    (344, 344, 202, 38, 64),        # as many CTAs as K blocks
+    (5216, 11224, 65, 254, 64),     # more row tiles than clusters of two: nothing is gained by a second wave
+    (9440, 6184, 142, 12, 16),
+])
+def test_the_count_of_parts_taken(h_in, h_out, T, slots, rank):
+    # every row tile's cluster is resident at once, and the count leaves no SM empty that another whole part could use where K or
+    # the expand is long
+    n_tiles, held = -(-h_out // 128), {1: 148, 2: 74, 3: 45, 4: 33, 5: 26, 6: 22, 7: 15, 8: 15}
+    import torch
+    pool = B.Pool(h_in, h_out, slots, rank, max_tokens=T)   # (no adapter loaded: the host knows no more than the slots)
+    try:
+        dev = lambda *shape: torch.zeros(shape, dtype=torch.bfloat16, device="cuda")
+        pool.linear(dev(h_out, h_in), dev(T, h_in), torch.full((T,), -1, dtype=torch.int32, device="cuda"))
+        got = B.edgelora_pool_last_launch(pool.handle)["split_k"]
+        assert pool.status() == (0, 0)
+    finally:
+        pool.close()
+    assert n_tiles <= held[got]
+    if n_tiles > 74:
+        assert got == 1
+    else:
+        assert got > 1 and (got >= 5 or n_tiles > held[got + 1])
