@@ -534,17 +534,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_sites_shrink_kernel(con
 #undef EDGELORA_ROWS
     ok = __all_sync(0xffffffffu, ok);
     if (!ok) break;
-    // lane L ends with the sum over lanes of value L (= row L / 4, token L % 4)
-#pragma unroll
-    for (int off = 16, cnt = 16; off >= 1; off >>= 1, cnt >>= 1) {
-      const bool upper = (lane & off) != 0;
-#pragma unroll
-      for (int i = 0; i < cnt; ++i) {
-        const float send = upper ? acc[i] : acc[i + cnt];
-        const float keep = upper ? acc[i + cnt] : acc[i];
-        acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-      }
-    }
+    sum_over_lanes(acc, lane);  // value L: row L / 4, token L % 4
     if (!waited) {  // first write of this warp to memory that earlier kernels may read
       ptx::pdl_wait_prior_grids();
       waited = true;
@@ -564,13 +554,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_sites_shrink_kernel(con
         if (lane == 0) st.counters[gi * 8 + rg] = 0;  // ready for the next launch
         for (int idx = lane; idx < (g_end - g_begin) * 8; idx += 32) {
           const size_t off = static_cast<size_t>(s_groups.tok[g_begin + (idx >> 3)]) * st.R_pad + rg * 8 + (idx & 7);
-          float part[kMaxZSplits];
-#pragma unroll
-          for (int sp = 0; sp < kMaxZSplits; ++sp) part[sp] = sp < st.ks ? __ldcg(st.zws + sp * zplane + off) : 0.f;
-          float sum = 0.f;
-#pragma unroll
-          for (int sp = 0; sp < kMaxZSplits; ++sp) sum += part[sp];
-          st.zws[kMaxZSplits * zplane + off] = sum;
+          add_z_planes(st.zws, zplane, st.ks, off);
         }
       }
     }

@@ -9,7 +9,6 @@ constexpr int kDecInputs = 4;   // distinct inputs of one launch at most
 constexpr int kDecThreads = 256;
 constexpr int kDecMaxStages = 12;
 constexpr int kDecMaxExpStages = 4;
-constexpr int kExpTok = 8;      // tokens of an expand stage at most
 constexpr size_t kDecTailBytes = 8192;
 
 struct DecSite {

@@ -29,7 +29,6 @@ namespace edgelora {
 namespace {
 
 constexpr int kThreads = 384, kExpandThreads = 256;
-constexpr int kExpTok = 8;  // tokens of an expand stage at most
 // Stages of the expand's ring.  Even: the two groups of warps take alternate stages, and a group may wait for the second use of
 // a ring position only if it was the one that saw the first (a wait for the phase behind one that is not over passes at once).
 constexpr int kExpStages = 4;

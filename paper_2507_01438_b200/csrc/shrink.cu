@@ -123,13 +123,7 @@ decode_shrink_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
       for (int idx = lane; idx < (pend_gend - pend_gt0) * 8; idx += 32) {
         const int tq = idx >> 3;
         const size_t off = static_cast<size_t>(s_groups.tok[pend_gt0 + tq]) * R_pad + pend_rg * 8 + (idx & 7);
-        float part[kMaxZSplits];
-#pragma unroll
-        for (int sp = 0; sp < kMaxZSplits; ++sp) part[sp] = sp < KS ? __ldcg(zws + sp * zplane + off) : 0.f;
-        float sum = 0.f;
-#pragma unroll
-        for (int sp = 0; sp < kMaxZSplits; ++sp) sum += part[sp];
-        zws[kMaxZSplits * zplane + off] = sum;
+        add_z_planes(zws, zplane, KS, off);
       }
     }
     pend_gi = -1;
@@ -193,17 +187,7 @@ decode_shrink_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
       else ok = shrink_rows8<4, kDsDepth, kQ8>(&tmap_a, &tmap_d, &tmap_x, ad, rg * 8, tok, step0, step1, KS, ring, bars, phase, lane, acc);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
-      // lane L ends with the sum over lanes of value L (= row L / 4, token L % 4)
-#pragma unroll
-      for (int off = 16, cnt = 16; off >= 1; off >>= 1, cnt >>= 1) {
-        const bool upper = (lane & off) != 0;
-#pragma unroll
-        for (int i = 0; i < cnt; ++i) {
-          const float send = upper ? acc[i] : acc[i + cnt];
-          const float keep = upper ? acc[i + cnt] : acc[i];
-          acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
-        }
-      }
+      sum_over_lanes(acc, lane);  // value L: row L / 4, token L % 4
       if (!waited) {  // first write of this warp to memory that earlier kernels may read
         ptx::pdl_wait_prior_grids();
         waited = true;

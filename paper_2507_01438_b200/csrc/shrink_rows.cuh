@@ -118,6 +118,31 @@ __device__ __forceinline__ bool shrink_rows8(const CUtensorMap *tmap_a, const CU
   return true;
 }
 
+// The sums over the warp's lanes of 32 values at once: lane L ends with that of value L, in acc[0].
+__device__ __forceinline__ void sum_over_lanes(float (&acc)[8 * kDsTok], int lane) {
+#pragma unroll
+  for (int off = 16, cnt = 16; off >= 1; off >>= 1, cnt >>= 1) {
+    const bool upper = (lane & off) != 0;
+#pragma unroll
+    for (int i = 0; i < cnt; ++i) {
+      const float send = upper ? acc[i] : acc[i + cnt];
+      const float keep = upper ? acc[i + cnt] : acc[i];
+      acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+    }
+  }
+}
+
+// The K chunks' partial planes at `off`, added in order into the plane that the expand reads.
+__device__ __forceinline__ void add_z_planes(float *zws, size_t zplane, int ks, size_t off) {
+  float part[kMaxZSplits];
+#pragma unroll
+  for (int sp = 0; sp < kMaxZSplits; ++sp) part[sp] = sp < ks ? __ldcg(zws + sp * zplane + off) : 0.f;
+  float sum = 0.f;
+#pragma unroll
+  for (int sp = 0; sp < kMaxZSplits; ++sp) sum += part[sp];
+  zws[kMaxZSplits * zplane + off] = sum;
+}
+
 __device__ __forceinline__ int atomic_add_acq_rel(int32_t *p, int v) {
   int old;
   asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
