@@ -554,7 +554,7 @@ def bench_site(name, ctx, steps=None, warmup=None, pdl=None, graph=True, cpu_bud
         # writes y once; its fp32 split-K partials are not counted
         gemm_bytes = 2 * w.h_in * w.h_out + 2 * w.T * (w.h_in + w.h_out) + \
             sum(2 * w.adapters[a].rank * w.h_out for a in w.distinct_adapters())
-        kernel_name = "lora_gemm_kernel (decode mode)"
+        kernel_name = "decode_tile_kernel" if w.T > 64 else "lora_gemm_kernel (decode mode)"
         if not any(kt.get(k, {}).get("launches", 0) for k in ("shrink_small_decode", "shrink_tiles", "plan")):
             # one launch per call: the same kernel also reads every distinct A_a (its shrink teams)
             gemm_bytes = ws_bytes

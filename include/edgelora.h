@@ -92,7 +92,9 @@ typedef struct {
                                     kernels of one call; 2 also lets the first kernel of a call
                                     start under the tail of earlier work on the stream -- only
                                     valid when W, x and the ids of a call are not produced by the
-                                    call before it (independent sites / batches)                  */
+                                    call before it (independent sites / batches).  A planned call
+                                    never starts under the kernel that writes its plan, and a set's
+                                    run never under the work in front of it                       */
 #define EDGELORA_OPT_DECODE_SPLITS 4 /* tuning: K splits per W row tile in decode, 0 = automatic  */
 #define EDGELORA_OPT_SHRINK_ITEMS 5  /* tuning: work items the decode shrink aims for, 0 = auto   */
 #define EDGELORA_OPT_GATHER_SPLITS 7 /* tuning: K splits of the tensor-core gather shrink in decode, 0 = chosen
@@ -161,9 +163,9 @@ int edgelora_pool_load_slot_pinned(edgelora_pool_t *pool, int32_t slot, int32_t 
  * d * q.  A_q8 is [rank][h_in / 32] blocks (h_in % 32 == 0), B_q8 is [h_out][ceil(rank / 32)]
  * blocks whose entries past `rank` are ignored.  The 8-bit form crosses to the device (about half
  * the bytes of the bfloat16 form) and is converted there, on the pool's side stream, into the
- * block's bfloat16 layout (each value rounded to nearest even), so the layer calls are unchanged.
- * Ordering, ownership and errors as for edgelora_pool_load_slot; the first call allocates a
- * device scratch for one adapter. */
+ * block's bfloat16 layout (each value rounded to nearest even; a kernel that reads the page-locked staging buffer),
+ * so the layer calls are unchanged.
+ * Ordering, ownership and errors as for edgelora_pool_load_slot. */
 int edgelora_pool_load_slot_q8(edgelora_pool_t *pool, int32_t slot, int32_t rank, float scale,
                                const void *A_q8, const void *B_q8);
 
@@ -238,9 +240,14 @@ int edgelora_plan_sync_status(edgelora_plan_t *plan, void *stream, uint32_t *bit
  * sees the same mixed batch; Section 4.3: the id -> sample mapping is worked out once).  Site i is
  * (pools[i], W_dev[i]) and reads input number input_of_site[i] (sites with the same input width
  * may share an input, e.g. q/k/v/o/gate/up of a decoder layer); all pools have the same n_slots
- * and max_tokens >= the set's.  A run builds ONE routing plan from the ids and evaluates the sites
- * in order; the sites are independent given their inputs, so in batches above 256 tokens runs of up
- * to 32 sites share one shrink launch and one base-product launch.  A site's result may lie in the memory of
+ * and max_tokens >= the set's.  A run makes ONE routing plan from the ids and evaluates the sites in order; the sites are
+ * independent given their inputs, so runs of up to 32 sites on up to 4 inputs share one shrink launch and one base-product
+ * launch, behind a plan kernel in batches above 256 tokens; in smaller ones the shrink launch derives the plan and leaves it
+ * in the set's plan object.  A launch is counted at the first site of its run (edgelora_pool_last_launch: 2, and 0 at the
+ * others).  A set goes site by site instead, the plan kernel first, when a result lies in an input's memory, when a pool has
+ * EDGELORA_FLAG_A_Q8, EDGELORA_OPT_REGIME other than 0 or EDGELORA_OPT_PDL = 0, and for at most 256 tokens also when one has
+ * EDGELORA_OPT_PROFILE, _DECODE_SPLITS, _SHRINK_ITEMS or _SHRINK_DEPTH set or an EDGELORA_OPT_GATHER_MIN_T below the batch.
+ * Whatever EDGELORA_OPT_PDL says, a run starts behind all work in front of it on the stream.  A site's result may lie in the memory of
  * an input: the sites behind it that read this input read the result (they start when it is written, one
  * launch per site, also with EDGELORA_OPT_PDL = 2); only a site's own input must not overlap its result.  The set
  * borrows the pools and W (the caller keeps them alive) and owns its plan, a device workspace for batches of at most 256
