@@ -80,3 +80,17 @@ def test_scores_at_the_edges_of_the_launch_shapes(Bn, n, hidden):
     bias = rng.normal(0, 1, size=n).astype(np.float32)
     got = B.edgelora_router_scores(to_dev_bf16(Wr), torch.from_numpy(bias).cuda(), to_dev_bf16(h)).cpu().numpy()
     assert np.max(np.abs(got - router_scores(Wr, bias, h))) <= 5e-6
+
+
+@pytest.mark.parametrize("n,hidden", [(1, 2056), (9, 4096), (1000, 4096), (1023, 3080), (1025, 8192), (2001, 4104)])
+def test_one_prompt_on_long_rows(n, hidden):
+    # a warp per row: a last CTA that is not full, rows that end inside a load, rows of two rounds; the bound of the test above
+    # (the longest chain is 128 sums of a lane, whose partial sums stay below 2, and the tree over the lanes)
+    import torch
+    rng = np.random.Generator(np.random.PCG64(n + hidden))
+    Wr = wl.normal_bf16(rng, (n, hidden), 2.0 / np.sqrt(hidden))
+    h = wl.normal_bf16(rng, (1, hidden), 1.0)
+    bias = rng.normal(0, 1, size=n).astype(np.float32)
+    for b in (bias, None):
+        got = B.edgelora_router_scores(to_dev_bf16(Wr), None if b is None else torch.from_numpy(b).cuda(), to_dev_bf16(h)).cpu().numpy()
+        assert np.max(np.abs(got - router_scores(Wr, b, h))) <= 5e-6
