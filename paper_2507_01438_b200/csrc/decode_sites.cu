@@ -552,10 +552,7 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_sites_shrink_kernel(con
       old = __shfl_sync(0xffffffffu, old, 0);
       if (old == arrivals - 1) {
         if (lane == 0) st.counters[gi * 8 + rg] = 0;  // ready for the next launch
-        for (int idx = lane; idx < (g_end - g_begin) * 8; idx += 32) {
-          const size_t off = static_cast<size_t>(s_groups.tok[g_begin + (idx >> 3)]) * st.R_pad + rg * 8 + (idx & 7);
-          add_z_planes(st.zws, zplane, st.ks, off);
-        }
+        add_z_planes(st.zws, zplane, st.ks, s_groups.tok + g_begin, g_end - g_begin, st.R_pad, rg * 8, lane);
       }
     }
   }

@@ -120,11 +120,7 @@ decode_shrink_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
     old = __shfl_sync(0xffffffffu, old, 0);
     if (old == arrivals - 1) {
       if (lane == 0) group_counters[pend_gi * 8 + pend_rg] = 0;  // ready for the next launch
-      for (int idx = lane; idx < (pend_gend - pend_gt0) * 8; idx += 32) {
-        const int tq = idx >> 3;
-        const size_t off = static_cast<size_t>(s_groups.tok[pend_gt0 + tq]) * R_pad + pend_rg * 8 + (idx & 7);
-        add_z_planes(zws, zplane, KS, off);
-      }
+      add_z_planes(zws, zplane, KS, s_groups.tok + pend_gt0, pend_gend - pend_gt0, R_pad, pend_rg * 8, lane);
     }
     pend_gi = -1;
   };

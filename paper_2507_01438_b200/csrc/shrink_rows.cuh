@@ -132,15 +132,51 @@ __device__ __forceinline__ void sum_over_lanes(float (&acc)[8 * kDsTok], int lan
   }
 }
 
-// The K chunks' partial planes at `off`, added in order into the plane that the expand reads.
-__device__ __forceinline__ void add_z_planes(float *zws, size_t zplane, int ks, size_t off) {
-  float part[kMaxZSplits];
+// The K chunks' partial planes added in order into the plane that the expand reads, by one warp: eight rank rows from r0 on of
+// the n tokens `tok` of an adapter.  What bounds it is the latency of a round of loads, behind everything else of the launch:
+// 16 planes of up to four tokens in one round, four planes of 16 tokens where an adapter has more of them.  (A token's planes are
+// added by the last warp of its adapter alone, so an adapter with many tokens is what the launch ends on.  Four tokens in a
+// round whatever their number, and now, us per call: 4616 -> 4136, 225 tokens on seven adapters: 49.0 and 40.9; 2584 -> 3264, 158
+// on four: 47.4 and 41.4; 1848 -> 288, 255 on 56: 35.7 and 31.4; 14336 -> 4096, 256 on about 100: 87.1 and 85.8.)
+__device__ __forceinline__ void add_z_planes(float *zws, size_t zplane, int ks, const uint8_t *tok, int n, int R_pad, int r0,
+                                             int lane) {
+  if (n <= 4) {
+    if (lane >= n * 8) return;
+    const size_t off = static_cast<size_t>(tok[lane >> 3]) * R_pad + r0 + (lane & 7);
+    float part[kMaxZSplits];
 #pragma unroll
-  for (int sp = 0; sp < kMaxZSplits; ++sp) part[sp] = sp < ks ? __ldcg(zws + sp * zplane + off) : 0.f;
-  float sum = 0.f;
+    for (int sp = 0; sp < kMaxZSplits; ++sp) part[sp] = sp < ks ? __ldcg(zws + sp * zplane + off) : 0.f;
+    float sum = 0.f;
 #pragma unroll
-  for (int sp = 0; sp < kMaxZSplits; ++sp) sum += part[sp];
-  zws[kMaxZSplits * zplane + off] = sum;
+    for (int sp = 0; sp < kMaxZSplits; ++sp) sum += part[sp];
+    zws[kMaxZSplits * zplane + off] = sum;
+    return;
+  }
+#pragma unroll 1
+  for (int i0 = lane; i0 < n * 8; i0 += 128) {
+    size_t off[4];
+    float sum[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      off[e] = static_cast<size_t>(tok[min(i0 + 32 * e, n * 8 - 1) >> 3]) * R_pad + r0 + (lane & 7);
+      sum[e] = 0.f;
+    }
+#pragma unroll 1
+    for (int s0 = 0; s0 < ks; s0 += 4) {
+      float part[4][4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) part[k][e] = s0 + k < ks ? __ldcg(zws + (s0 + k) * zplane + off[e]) : 0.f;
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sum[e] += part[k][e];
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (i0 + 32 * e < n * 8) zws[kMaxZSplits * zplane + off[e]] = sum[e];
+  }
 }
 
 __device__ __forceinline__ int atomic_add_acq_rel(int32_t *p, int v) {

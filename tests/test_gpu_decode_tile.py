@@ -103,3 +103,13 @@ def test_the_count_of_parts_taken(h_in, h_out, T, slots, rank):
         assert got == 1
     else:
         assert got > 1 and (got >= 5 or n_tiles > held[got + 1])
+
+
+@pytest.mark.parametrize("items", [0, 60, 20000])
+def test_sums_of_k_chunks_for_all_counts_of_tokens(items):
+    # groups around the four tokens and the sixteen of a round of loads, few and many K chunks (8192: 32 steps)
+    counts = [1, 3, 4, 5, 15, 16, 17, 32, 33, 47]
+    ids = np.random.Generator(np.random.PCG64(9)).permutation(np.repeat(np.arange(len(counts)), counts))
+    w = workload(8, len(ids), 8192, 136, 32, len(counts), ids)
+    y = run_gpu(w, 1, options={B.OPT_SHRINK_ITEMS: items})
+    assert_parity(y, oracle_of(w), w.name)
