@@ -71,22 +71,23 @@ __device__ __forceinline__ int32_t first_stage(int32_t unit, int32_t n_stages, i
 }
 
 // The stage's tokens, four, two or one at a time, into the columns from `taddr` on.
-template <int kR>
-__device__ __forceinline__ void expand_stage(const uint8_t *brow, int sw, uint32_t z, int rank, int nt, uint32_t taddr) {
+template <int kChunks>
+__device__ __forceinline__ void expand_stage(const uint8_t *brow, int sw, uint32_t z, uint32_t z_bytes, int rank, int nt,
+                                             uint32_t taddr) {
   float acc[4];
 #pragma unroll 1
-  for (; nt >= 4; nt -= 4, z += 4 * kR * 4, taddr += 4) {
-    expand_dots<kR, 4>(brow, sw, z, rank, acc);
+  for (; nt >= 4; nt -= 4, z += 4 * z_bytes, taddr += 4) {
+    expand_dots<kChunks, 4>(brow, sw, z, z_bytes, rank, acc);
     ptx::tmem_st_32x4(taddr, acc);
   }
   if (nt & 2) {
-    expand_dots<kR, 2>(brow, sw, z, rank, acc);
+    expand_dots<kChunks, 2>(brow, sw, z, z_bytes, rank, acc);
     ptx::tmem_st_32x2(taddr, acc);
-    z += 2 * kR * 4;
+    z += 2 * z_bytes;
     taddr += 2;
   }
   if (nt & 1) {
-    expand_dots<kR, 1>(brow, sw, z, rank, acc);
+    expand_dots<kChunks, 1>(brow, sw, z, z_bytes, rank, acc);
     ptx::tmem_st_32x1(taddr, acc);
   }
 }
@@ -341,9 +342,11 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_sites_kernel(const __gr
           const uint8_t *src = exp_ring + static_cast<size_t>(stage) * b.exp_bytes;
           const uint8_t *brow = src + row_in_tile * st.R_pad * 2;
           const uint32_t z = ptx::smem_u32(src + b_bytes), taddr = tmem_exp + lanes + pos;
-          if (st.R_pad == 16) expand_stage<16>(brow, sw, z, rank, nt, taddr);
-          else if (st.R_pad == 32) expand_stage<32>(brow, sw, z, rank, nt, taddr);
-          else expand_stage<64>(brow, sw, z, rank, nt, taddr);
+          const uint32_t z_bytes = static_cast<uint32_t>(st.R_pad) * 4;
+          if (rank <= 8) expand_stage<1>(brow, sw, z, z_bytes, rank, nt, taddr);
+          else if (rank <= 16) expand_stage<2>(brow, sw, z, z_bytes, rank, nt, taddr);
+          else if (rank <= 32) expand_stage<4>(brow, sw, z, z_bytes, rank, nt, taddr);
+          else expand_stage<8>(brow, sw, z, z_bytes, rank, nt, taddr);
           __syncwarp();
           if (lane == 0) ptx::mbar_arrive(&sh.bempty[stage]);
           __syncwarp();

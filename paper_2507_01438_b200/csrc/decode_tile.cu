@@ -13,8 +13,8 @@
 // warps 4..11 (two to a lane quadrant: a single warp per scheduler cannot keep up with the latency of its sums) work out the
 // u-batches, the expand and y.  (A thread takes 0.3 us to issue the copies of a stage; with all stages issued by one warp that
 // was the pace of an expand of rank stride 16 or 32: 336 -> 13208, 209 tokens on 17 adapters: 37.1 us per call, now 31.7; 512 ->
-// 11744, 119 tokens on 25, A in Q8_0: 28.9 and 25.5; 1848 -> 288, 255 tokens on 56: 36.0 and 34.4.  At stride 64 the reads of z
-// from shared memory are: 680 -> 9576, 97 tokens on seven adapters: 32.0 with either.)  Every mbarrier wait is bounded; on a
+// 11744, 119 tokens on 25, A in Q8_0: 28.9 and 25.5; 1848 -> 288, 255 tokens on 56: 36.0 and 34.4.  At stride 64 the reads of
+// z and B from shared memory are.)  Every mbarrier wait is bounded; on a
 // timeout the status word gets EDGELORA_STATUS_TIMEOUT and all roles leave.
 #include <algorithm>
 
@@ -61,25 +61,25 @@ __device__ __forceinline__ uint32_t stage_info(const Shared &sh, int s) {
 }
 
 // The stage's tokens, four, two or one at a time, each into its column.
-template <int kR>
-__device__ __forceinline__ void expand_stage(const uint8_t *brow, int sw, uint32_t z, int rank, int nt, uint32_t texp,
-                                             const uint8_t *columns) {
+template <int kChunks>
+__device__ __forceinline__ void expand_stage(const uint8_t *brow, int sw, uint32_t z, uint32_t z_bytes, int rank, int nt,
+                                             uint32_t texp, const uint8_t *columns) {
   float acc[4];
 #pragma unroll 1
-  for (; nt >= 4; nt -= 4, z += 4 * kR * 4, columns += 4) {
-    expand_dots<kR, 4>(brow, sw, z, rank, acc);
+  for (; nt >= 4; nt -= 4, z += 4 * z_bytes, columns += 4) {
+    expand_dots<kChunks, 4>(brow, sw, z, z_bytes, rank, acc);
 #pragma unroll
     for (int q = 0; q < 4; ++q) ptx::tmem_st_32x1(texp + columns[q], &acc[q]);
   }
   if (nt & 2) {
-    expand_dots<kR, 2>(brow, sw, z, rank, acc);
+    expand_dots<kChunks, 2>(brow, sw, z, z_bytes, rank, acc);
     ptx::tmem_st_32x1(texp + columns[0], &acc[0]);
     ptx::tmem_st_32x1(texp + columns[1], &acc[1]);
-    z += 2 * kR * 4;
+    z += 2 * z_bytes;
     columns += 2;
   }
   if (nt & 1) {
-    expand_dots<kR, 1>(brow, sw, z, rank, acc);
+    expand_dots<kChunks, 1>(brow, sw, z, z_bytes, rank, acc);
     ptx::tmem_st_32x1(texp + columns[0], &acc[0]);
   }
 }
@@ -247,9 +247,11 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tile_kernel(const __grid_c
         const uint8_t *src = exp_ring + static_cast<size_t>(stage) * p.exp_bytes;
         const uint8_t *brow = src + row_in_tile * p.R_pad * 2;
         const uint32_t z = ptx::smem_u32(src + b_bytes);
-        if (p.R_pad == 16) expand_stage<16>(brow, sw, z, rank, nt, texp, sh.groups.tok + pos);
-        else if (p.R_pad == 32) expand_stage<32>(brow, sw, z, rank, nt, texp, sh.groups.tok + pos);
-        else expand_stage<64>(brow, sw, z, rank, nt, texp, sh.groups.tok + pos);
+        const uint32_t z_bytes = static_cast<uint32_t>(p.R_pad) * 4;
+        if (rank <= 8) expand_stage<1>(brow, sw, z, z_bytes, rank, nt, texp, sh.groups.tok + pos);
+        else if (rank <= 16) expand_stage<2>(brow, sw, z, z_bytes, rank, nt, texp, sh.groups.tok + pos);
+        else if (rank <= 32) expand_stage<4>(brow, sw, z, z_bytes, rank, nt, texp, sh.groups.tok + pos);
+        else expand_stage<8>(brow, sw, z, z_bytes, rank, nt, texp, sh.groups.tok + pos);
         __syncwarp();
         if (lane == 0) ptx::mbar_arrive(&sh.bempty[stage]);
       }
