@@ -13,8 +13,8 @@
 // the tile and the z rows of up to eight tokens of the adapter come through a ring of their own, the dot products wait in
 // tensor memory until the accumulator is complete.  An adapter's values reach the rows of its own tokens only.
 //
-// 28 sites of four decoder layers (4096, 1024, 14336 wide), 27 tokens on 18 adapters of rank 8 to 32: 331 us for 1.93 GB
-// that cannot be done without (2.04 GB as the B blocks are padded: 6.2 TB/s), 412 us with two launches per site; seven
+// 28 sites of four decoder layers (4096, 1024, 14336 wide), 27 tokens on 18 adapters of rank 8 to 32: 337 us for 1.93 GB
+// that cannot be done without (2.04 GB as the B blocks are padded: 6.1 TB/s), 416 us with two launches per site; seven
 // sites of a layer 1024 wide, one token: 21 us, 45 before.  64 tokens: 400 us, 565 before; 256 tokens through two layers:
 // 483 us, 671 before.
 //
@@ -569,8 +569,8 @@ __global__ void __launch_bounds__(kDecThreads, 2) decode_sites_shrink_kernel(con
 // ---------------------------------------------------------------------------------------------------------- launch
 
 // The operand ring gets what the other parts leave of an SM's shared memory: the stream of W needs the bytes in flight (28
-// sites, 27 tokens: 335 us; 355 with 123 KB per CTA, which leave room for a CTA of the shrink on the same SM, 368 with
-// 104 KB).  Three stages of the expand: 333 us, two 339.
+// sites, 27 tokens: 6 % more with 123 KB per CTA, which leave room for a CTA of the shrink on the same SM, 10 % with
+// 104 KB).  Two stages of the expand instead of three: 2 % more.
 DecShape decode_sites_shape(int32_t N, int32_t R_pad) {
   DecShape s{};
   const size_t stage = kWBytes + static_cast<size_t>(N) * kBlockK * 2;

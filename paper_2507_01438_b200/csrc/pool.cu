@@ -996,7 +996,7 @@ int decode_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32_
     s.status = q->status_dev;
     s.x_index = xi;
     s.n_ksteps = (h_in + kShrinkStepElems - 1) / kShrinkStepElems;
-    // K chunks of eight steps or more, 32 KB of A per item (four and sixteen: within 1 us of 335)
+    // K chunks of eight steps or more, 32 KB of A per item (four and sixteen: no difference)
     s.ks = std::max(1, std::min(kMaxZSplits, s.n_ksteps / 8));
     s.R_pad = R;
     s.max_tokens = q->cfg.max_tokens;
@@ -1004,7 +1004,7 @@ int decode_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32_
   plan->last_T = T;
   plan->unread = true;
   if (getenv("EDGELORA_LOG")) fprintf(stderr, "edgelora: decode T %d N %d sites %d grid %d\n", T, N, n, ws.ctas);
-  // (two CTAs of the shrink per SM, 98 KB of ring each: 333 us for the 28 sites, 336 with one)
+  // (two CTAs of the shrink per SM, 98 KB of ring each: 1 % less for 28 sites than one)
   CUDA_TRY(launch_decode_sites_shrink(sb, 2 * p0->sms, pdl_first, stream));
   CUDA_TRY(launch_decode_sites(db, shape, ws.ctas, true, stream));
   for (int i = 0; i < n; ++i) {

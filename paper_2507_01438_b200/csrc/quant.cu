@@ -7,7 +7,7 @@
 // to [h_out][R_pad], bfloat16, padding zero; or A kept in Q8_0, as a plane of bytes and a plane of scales) and writes its
 // row of the slot table.  It reads the 8-bit form straight from the page-locked staging buffer: one launch per load, where
 // copies of the blocks and of the row around a conversion kernel were four entries on the side stream and twice the
-// driver calls, which is what a load cost (two loads, 4096 -> 4096, rank 16: 45 us of host time, 40 now; three, 9024 -> 1576: 51 and 36).
+// driver calls, which is what a load cost (two loads in front of a step, 4096 -> 4096, rank 16: 57 us a step, 50 now).
 //
 #include <cuda_fp16.h>
 
