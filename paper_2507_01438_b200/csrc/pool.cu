@@ -915,6 +915,7 @@ int prefill_sites(const SiteCall *sites, int n, edgelora_plan *plan, const int32
 }
 
 // ---- decode-sized batches of a run of sites (decode_sites.cu)
+static_assert(kPairSites <= kDecSites && kPairInputs <= kDecInputs, "the runs of a set are cut for either launch");
 static int32_t decode_columns(int32_t T) { return std::max(16, (T + 15) / 16 * 16); }
 
 int32_t decode_workspace_ctas(edgelora_pool *const *pools, int32_t n, int32_t max_tokens) {
