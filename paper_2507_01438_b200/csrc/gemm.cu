@@ -539,8 +539,8 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
     __syncwarp();
     if (kFused && f.b_stage) {
       // Small batches, one launch.  The partial sums are on their way; while the cluster's other CTAs send theirs, the
-      // epilogue and team warps (2..9) work out the expand of this CTA's tokens: wait for the shrink teams, bring z of
-      // their tokens to shared memory, and dot it with the staged B_a rows, a thread per W row and every other token quad.
+      // epilogue and team warps (2..9) work out the expand of this CTA's tokens: z, which the team has brought to shared
+      // memory, against the staged B_a rows, a thread per W row and every other token quad.
       // (With the expand behind the exchange, by the epilogue warps alone, the tail behind the last MMA took 6 us for 32
       // tokens and 9 for 64: 4096 -> 4096, 32 tokens 15.1 us per call, now 12.3; 64 tokens 18.0 and 14.1; 256 -> 256, 16
       // tokens 7.9 and 5.7.)
@@ -551,24 +551,26 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
 #pragma unroll
       for (int i = 0; i < 8; ++i) e[i >> 2][i & 3] = 0.f;
       int passed = 0;
-      if (warp >= 2) {
-        if (warp == 2) {
+      if (warp >= 6) {
+        // Behind its items the team waits for the others and brings z of the tokens that this CTA will finish to shared memory,
+        // the K chunks' planes added in order.  With a long K that is over before the accumulator is.  (By the epilogue warps, behind
+        // it, and here, us per call: 8192 -> 512, one token on rank 32: 7.9 and 6.9; 14336 -> 1024, one token on rank 16: 11.4 and
+        // 10.4; 4096 -> 4096, four tokens: 10.8 and 9.8, 32 tokens: 11.9 and 11.2; 2048 -> 2048, eight tokens: 7.1 and 6.2.)
+        const int32_t *s_tid = reinterpret_cast<const int32_t *>(s_team) + 64, *s_trank = s_tid + 64;
+        if (warp == 6) {
           // the counter belongs to the kernel before this one (another launch of this pool, which leaves it at zero) until
           // that kernel is done
           ptx::pdl_wait_prior_grids();
-          // one thread of the CTA polls; the named barrier passes its acquire on
+          // one thread of the CTA polls; the named barriers pass its acquire on
           if (lane == 0) *s_last = wait_for_teams(f.sync, 2 * cta0 + ngrid, wl, p.status);
         }
-        named_bar_sync(3, 256);
-        // this warp is past its wait for the shrink teams (see the end)
-        if (epi && lane == 0) passed = atomicAdd(f.sync + 1, 1);
-        bool z_ok = *s_last != 0;
-        // z of this CTA's tokens, the K chunks' planes added in order
+        named_bar_sync(2, 128);
+        const bool in_time = *s_last != 0;
         const size_t zplane4 = static_cast<size_t>(p.max_tokens) * R4;
-        for (int i = (threadIdx.x - 64); i < cols_per * R4; i += 256) {
-          const int cl = i / R4, c4 = i - cl * R4, t = static_cast<int>(my_rank) * cols_per + cl;
+        for (int i = static_cast<int>(threadIdx.x) - 192; i < cols_per * R4; i += 128) {
+          const int cl = i / R4, c4 = i - cl * R4, t = static_cast<int>(my_rank) * cols_per + cl, rank = s_trank[t];
           float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (s_vid[cl] >= 0 && z_ok) {
+          if (s_tid[t] >= 0 && rank > 0 && in_time) {
             const float4 *zp = reinterpret_cast<const float4 *>(f.z) + static_cast<size_t>(t) * R4 + c4;
             float4 w[8];
             for (int s0 = 0; s0 < f.ks; s0 += 8) {
@@ -579,7 +581,7 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
                 z.x += w[k].x; z.y += w[k].y; z.z += w[k].z; z.w += w[k].w;
               }
             }
-            const int rank = s_rank[cl];  // (what lies behind the last live group of eight rank rows was not written)
+            // (what lies behind the last live group of eight rank rows was not written)
             if (c4 * 4 + 0 >= rank) z.x = 0.f;
             if (c4 * 4 + 1 >= rank) z.y = 0.f;
             if (c4 * 4 + 2 >= rank) z.z = 0.f;
@@ -587,13 +589,16 @@ lora_gemm_kernel(const __grid_constant__ CUtensorMap tmap_r, const __grid_consta
           }
           z_stage[i] = z;
         }
-        int got = 1;
-        if (lane == 0) got = ptx::mbar_wait(ep_bar, 0, max(wl, ptx::kSettleCycles)) ? 1 : 0;  // the staged B_a rows
-        if (!__shfl_sync(0xffffffffu, got, 0)) {
+      }
+      if (warp >= 2) {
+        named_bar_sync(3, 256);  // z of this CTA's tokens is there
+        // the wait for the shrink teams is over in this CTA (see the end)
+        if (epi && lane == 0) passed = atomicAdd(f.sync + 1, 1);
+        bool z_ok = *s_last != 0;
+        if (!__all_sync(0xffffffffu, ptx::mbar_wait(ep_bar, 0, max(wl, ptx::kSettleCycles)))) {  // the staged B_a rows
           if (lane == 0) atomicOr(p.status, EDGELORA_STATUS_TIMEOUT);
           z_ok = false;
         }
-        named_bar_sync(3, 256);
         const int sw = row_swizzle(r, p.R_pad);
         const uint32_t brow = ptx::smem_u32(b_stage) + r * p.R_pad * 2, tok_bytes = kTileM * p.R_pad * 2;
         const uint32_t zrow = ptx::smem_u32(z_stage);
