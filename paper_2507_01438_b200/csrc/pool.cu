@@ -1189,7 +1189,7 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
     plan->last_T = T;
     if (!ids_dev && plan->unread) pdl_first = false;  // (the ids are the library's own)
     plan->unread = plan->unread || ids_dev;
-    auto launch_shrink = [&]() -> int {
+    auto launch_shrink = [&](int base_ctas) -> int {  // base_ctas: CTAs that run beside it
       if (T > kGatherMinT) {
         if (ids_dev) {
           ProfScope ps(p, 0, stream);
@@ -1225,15 +1225,20 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
         // with 2 K chunks on the 1000-adapter down_proj, 96 with 3-4, 100 with 12, 104 with 1.  About 0.6 per warp are
         // aimed for, and where they leave warps without one, K is cut further, to about one per warp (6144 -> 3432 with A
         // in Q8_0, 145 tokens on six adapters: 42.7 us per call, 53.9 without; 1656 -> 328, 69 tokens on four: 21.6 and
-        // 27.3; 984 -> 11960, four tokens, one of the few that lose: 10.3 and 9.8).  Small batches: four items per warp.
+        // 27.3), in small batches on the SMs that the base product beside it leaves only (1752 -> 4136, 54 tokens, 132 CTAs of the base
+        // product: 15.5 with all SMs, 14.1; 5120 -> 1608, 58 tokens, A in Q8_0: 16.7 and 13.7).  Small batches: four items per warp.
         const int auto_target = T > 64 ? 5 * cta_cap : 4 * 8 * cta_cap;
         const int target = p->opt_shrink_items > 0 ? p->opt_shrink_items : (overlapped ? 1 : auto_target);
         // at most T token blocks x (R / 8) row groups x K chunks warp items, eight warps per CTA
         const int n_ksteps = (h_in + kShrinkStepElems - 1) / kShrinkStepElems;
-        const bool fill_warps = p->opt_shrink_items == 0 && !overlapped;
-        const int max_chunks = target == 1 ? 1 : std::max(1, std::min(kMaxZSplits, n_ksteps / (fill_warps ? 2 : 4)));
-        const int max_items = std::min(T, p->cfg.n_slots) * (R / 8) * max_chunks;
-        const int grid = std::max(1, std::min(cta_cap - 1, (max_items + 7) / 8)) + 1;  // + the publishing CTA
+        auto ctas_for = [&](int chunk) {  // K chunks of so many steps at least
+          const int chunks = target == 1 ? 1 : std::max(1, std::min(kMaxZSplits, n_ksteps / chunk));
+          return std::max(1, std::min(cta_cap - 1, (std::min(T, p->cfg.n_slots) * (R / 8) * chunks + 7) / 8));
+        };
+        const int spare = p->opt_shrink_items > 0 || overlapped ? 0 : std::max(0, cta_cap - base_ctas);
+        const int workers = std::max(ctas_for(4), std::min(ctas_for(2), spare));
+        const int grid = workers + 1;  // + the publishing CTA
+        const int fill_warps = std::min(workers, spare) * 8;
         CUtensorMap ma, mx, md;
         // A rows: bfloat16, or for a pool that keeps A in Q8_0 two planes per slot: the signed bytes
         // [R_pad][h_in] (taken as 16-bit elements: 128 per K step) and the half-precision block scales
@@ -1277,7 +1282,7 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
     if (owners_expand(splits) && p->opt_decode_splits == 0)
       while (splits > 1 && row_tiles * splits > p->sms) splits >>= 1;
     if (!owners_expand(splits)) {
-      int rc = launch_shrink();
+      int rc = launch_shrink(0);
       if (rc) return rc;
       {
         // Launched under the shrink's tail: its CTAs end at different times, and on the SMs that are free early the K
@@ -1373,7 +1378,7 @@ int lora_linear_impl(edgelora_pool *p, edgelora_plan *plan, const int32_t *ids_d
       }
     }
     if (!fused) {
-      rc = launch_shrink();
+      rc = launch_shrink(grid);
       if (rc) return rc;
     }
     if (!fused) {

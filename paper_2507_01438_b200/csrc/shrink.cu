@@ -73,13 +73,13 @@ decode_shrink_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_co
   // Work items are per warp: (token block, K chunk, group of eight rank rows).  K chunks: enough
   // items for every warp of the grid, but a chunk keeps at least four K steps (1024 elements)
   // unless h_in is shorter, so that the ring's ramp-up is amortised; or two, as long as a warp has no more than one item
-  // (fill_warps: the host chose the number of items itself).
+  // (fill_warps: so many of them, none where the caller gave the number of items).
   const int n_ksteps = (h_in + 255) >> 8, warps_total = (gridDim.x - 1) * (kShrinkThreads / 32);
   const int n_rgn = R_pad >> 3;  // row groups of the rank stride: 2, 4 or 8
   int KS = (target_items + max(NB * n_rgn, 1) - 1) / max(NB * n_rgn, 1);
   KS = max(1, min(min(KS, kMaxZSplits), n_ksteps / 4));
-  if (fill_warps && NB * n_rgn * KS < warps_total)
-    KS = max(KS, min(min(kMaxZSplits, n_ksteps / 2), warps_total / max(NB * n_rgn, 1)));
+  if (NB * n_rgn * KS < fill_warps)
+    KS = max(KS, min(min(kMaxZSplits, n_ksteps / 2), fill_warps / max(NB * n_rgn, 1)));
   const int spc = (n_ksteps + KS - 1) / KS;
   KS = (n_ksteps + spc - 1) / spc;
 
@@ -231,13 +231,13 @@ cudaError_t launch_decode_shrink(const CUtensorMap &tmap_a, const CUtensorMap &t
                                  const int32_t *ids, const SlotRow *slots, const PlanView &pv,
                                  float *zws, int32_t *group_counters, int32_t T, int32_t h_in,
                                  int32_t R_pad, int32_t n_slots, int32_t max_tokens,
-                                 int32_t target_items, bool fill_warps, int32_t grid, uint32_t *status, bool pdl, bool a_q8,
+                                 int32_t target_items, int32_t fill_warps, int32_t grid, uint32_t *status, bool pdl, bool a_q8,
                                  int32_t depth, cudaStream_t stream) {
   const int32_t late_ticket = pdl ? 1 : 0;  // pdl here = this launch may start under the call before it
 #define EDGELORA_SHRINK(D, Q)                                                                                     \
   launch_ex(decode_shrink_kernel<D, Q>, dim3(grid), dim3(kShrinkThreads), ds_ring_bytes(D), stream, pdl, 1, tmap_a, \
             tmap_d, tmap_x, ids, slots, pv, zws, group_counters, T, h_in, R_pad, n_slots, max_tokens, target_items,        \
-            fill_warps ? 1 : 0, late_ticket, status)
+            fill_warps, late_ticket, status)
   if (depth == 2) return a_q8 ? EDGELORA_SHRINK(2, true) : EDGELORA_SHRINK(2, false);
   return a_q8 ? EDGELORA_SHRINK(4, true) : EDGELORA_SHRINK(4, false);
 #undef EDGELORA_SHRINK
