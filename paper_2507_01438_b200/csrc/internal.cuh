@@ -19,6 +19,7 @@ constexpr int kMaxTokensLimit = 32768;
 constexpr int kGemmThreads = 320;  // warp 0 TMA, warp 1 MMA, warps 2..5 epilogue, warps 6..9 shrink team
 constexpr int kMaxZSplits = 16;    // partial z planes (K splits of the shrink); plane 16 = summed z
 constexpr int kShrinkThreads = 256;
+constexpr int kDecShrinkTok = 4;   // decode shrink: tokens of a block
 constexpr int kExpTok = 8;         // decode: tokens of an expand stage at most
 constexpr int kShrinkStepElems = 256;  // K elements of one shrink step (512 bytes of a row)
 

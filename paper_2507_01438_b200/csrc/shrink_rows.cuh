@@ -8,7 +8,7 @@
 
 namespace edgelora {
 
-constexpr int kDsTok = 4;
+constexpr int kDsTok = kDecShrinkTok;
 
 __device__ __forceinline__ void unpack8(const uint4 &v, float (&f)[8]) {
   f[0] = ptx::bf16_lo(v.x); f[1] = ptx::bf16_hi(v.x);
