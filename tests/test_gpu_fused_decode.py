@@ -125,3 +125,22 @@ def test_expand_beside_the_exchange_of_partial_sums(T, h_in, h_out, max_rank):
             assert B.edgelora_pool_last_launch(pool.handle)["launches"] == 1
     finally:
         pool.close()
+
+
+@pytest.mark.parametrize("T,h_in,h_out,max_rank,stages", [
+    (32, 4096, 4096, 64, 4), (7, 5216, 1944, 64, 4), (64, 4096, 4096, 32, 3), (40, 1024, 2056, 32, 3), (64, 4096, 1000, 64, 3),
+    (32, 4096, 4096, 32, 5), (64, 4096, 4096, 16, 4),
+])
+def test_a_ring_stage_makes_room_for_the_staged_rows(T, h_in, h_out, max_rank, stages):
+    # the last two have room for both
+    ranks = [max_rank, max_rank // 2, max_rank - 3, 1, 0, max_rank, 5, max_rank]
+    w = random_workload(7500 + T, T, h_in, h_out, ranks=ranks, max_rank=max_rank)
+    w.ids = np.random.Generator(np.random.PCG64(T)).integers(-1, len(ranks), size=T).astype(np.int32)
+    w.ids[w.ids == 4] = -1
+    pool = make_pool(w, 64)
+    try:
+        assert_parity(run_gpu(w, 1, pool=pool), oracle_of(w), f"T={T} {h_in}->{h_out}")
+        info = B.edgelora_pool_last_launch(pool.handle)
+        assert (info["launches"], info["stages"]) == (1, stages), info
+    finally:
+        pool.close()
