@@ -240,7 +240,9 @@ __global__ void __launch_bounds__(kThreads, 1) decode_tile_kernel(const __grid_c
       const int rank = mine & 255, nt = (mine >> 8) & 255, pos = mine >> 16;
       if (rank == 0) continue;
       if ((live++ & 1) == half) {  // the groups of four warps take every other stage
-        if (!__all_sync(0xffffffffu, ptx::mbar_wait(&sh.bfull[stage], phase, wl) && !sh.abort_flag)) {
+        // (the first one is for z, too: it ends behind the shrink)
+        const bool there = live <= 2 ? ptx::mbar_wait_timed(&sh.bfull[stage], phase, wl) : ptx::mbar_wait(&sh.bfull[stage], phase, wl);
+        if (!__all_sync(0xffffffffu, there && !sh.abort_flag)) {
           ok = false;
           break;
         }

@@ -76,6 +76,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity,
   return true;
 }
 
+// The same, and a wait that lasted longer counts as one that ran out, although it ended within a try (which may last as long
+// as a short kernel).
+__device__ __forceinline__ bool mbar_wait_timed(uint64_t *bar, uint32_t parity, long long limit_cycles) {
+  const long long t0 = clock64();
+  return mbar_wait(bar, parity, limit_cycles) && clock64() - t0 <= limit_cycles;
+}
+
 // For a role that gives up a wait, behind the last thing it issued: copies, tensor operations and launch-queue answers
 // may still be on their way into shared and tensor memory, and which of them will ever be counted on a barrier depends on
 // where each role gave up.  They take microseconds; the role stays for about half a millisecond before it goes to the
